@@ -6,11 +6,11 @@ A case is a dict of plain values; ``prepare`` makes its inputs on the GPU from a
 
 Particle sets are those of the benchmark: uniform in the periodic unit cube, or
 clustered (half uniform, half in 256 Plummer spheres); equal masses 1/N, Gaussian
-velocities, log-normal internal energies.  Smoothing lengths come from the analytic
-number density of the set, h = (3 64 / (4 pi n(x)))^(1/3), so that a particle has 64
-neighbours up to the Poisson scatter of the set (the spread of h before a timestep's
-iteration); density and f, where a case takes them as inputs, are that density and 1 with
-a scatter.  Active subsets are runs along the curve of mean length 32.
+velocities, log-normal internal energies.  Smoothing lengths come from particle counts
+on a hierarchy of grids, so that a sphere of radius h holds about 64 particles with a
+scatter of some 10% in h (the spread of h before a timestep's iteration); density and f,
+where a case takes them as inputs, are 64 m / (4 pi h^3 / 3) and 1 with a scatter.
+Active subsets are runs along the curve of mean length 32.
 """
 
 import math
@@ -139,18 +139,53 @@ def _inputs(case, seed, dev):
     rng = np.random.default_rng(seed)
     n = case["n"]
     pos, dens = _particles(case["set"], n, gen, rng, dev)
-    s = _fields(n, dens, gen, dev)
+    s = _fields(n, pos, dens, gen, dev)
     s["pos"] = pos
     return s, gen
 
 
-def _fields(n, dens, gen, dev):
-    m = torch.full((n,), 1.0 / n, device=dev)
+def _smoothing(pos, dens):
+    """h with about 64 particles in its sphere: the counts of ever finer grids, taken at the
+    particle by trilinear interpolation, give the number expected within one cell size;
+    h lies where that crosses 64.  Cores too dense for the grids take the analytic density."""
+    n = pos.shape[0]
     h = (3.0 * NNGB / (4.0 * math.pi * dens)) ** (1.0 / 3.0)
-    h.clamp_(max=0.45)
+    found = torch.zeros(n, dtype=torch.bool, device=pos.device)
+    last = torch.full_like(h, n * 4.0 * math.pi / 3.0 / 8.0)   # within half the box
+    for level in range(2, 10):
+        size = 1 << level
+        x = pos * size - 0.5
+        cell = torch.floor(x)
+        w = (x - cell).float()
+        i0 = torch.remainder(cell.long(), size)
+        i1 = torch.remainder(i0 + 1, size)
+        own = torch.floor(pos * size).long().clamp_(max=size - 1)
+        count = torch.bincount((own[:, 0] * size + own[:, 1]) * size + own[:, 2], minlength=size ** 3)
+        c = torch.zeros(n, device=pos.device)
+        for a in range(8):
+            ix, iy, iz = ((i1 if a >> q & 1 else i0)[:, q] for q in range(3))
+            f = torch.ones(n, device=pos.device)
+            for q in range(3):
+                f *= w[:, q] if a >> q & 1 else 1.0 - w[:, q]
+            c += f * count[(ix * size + iy) * size + iz]
+        c = (c.double() * (4.0 * math.pi / 3.0)).clamp_(min=1e-3)
+        cross = ~found & (c < NNGB)
+        t = (torch.log(last) - math.log(NNGB)) / (torch.log(last) - torch.log(c)).clamp(min=1e-9)
+        h = torch.where(cross, 2.0 ** (1.0 - level) * 0.5 ** t.clamp(0.0, 1.0), h)
+        found |= cross
+        last = c
+        if 8 ** (level + 1) > 64 * n:
+            break
+    h = torch.where(found, h, torch.clamp(h, max=0.5 ** level))
+    return h.clamp_(max=0.45)
+
+
+def _fields(n, pos, dens, gen, dev):
+    m = torch.full((n,), 1.0 / n, device=dev)
+    h = _smoothing(pos, dens)
     vel = torch.randn((n, 3), generator=gen, device=dev) * 0.1
     u = torch.exp(torch.randn(n, generator=gen, device=dev))
-    rho = (dens / n * torch.exp(0.1 * torch.randn(n, generator=gen, device=dev).double())).float()
+    rho = (3.0 * NNGB / (4.0 * math.pi * n) / h ** 3).float() * torch.exp(0.1 * torch.randn(n, generator=gen, device=dev))
     fgrad = 1.0 + 0.1 * torch.randn(n, generator=gen, device=dev).clamp_(-3, 3)
     return {"m": m, "h": h, "vel": vel, "u": u, "rho": rho, "fgrad": fgrad}
 
@@ -190,7 +225,7 @@ def _prepare_batch(case, seed, dev):
     parts = []
     for n, kind, frac in zip(sizes, kinds, fracs):
         pos, dens = _particles(kind, int(n), gen, srng, dev)
-        f = _fields(int(n), dens, gen, dev)
+        f = _fields(int(n), pos, dens, gen, dev)
         f["pos"] = pos
         act = torch.rand(int(n), generator=gen, device=dev) < frac
         act[0] = True
