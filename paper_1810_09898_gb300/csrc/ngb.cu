@@ -6,9 +6,10 @@
 //    of every opened leaf;
 //  * grouped: one warp per group of consecutive active particles (key order).  The
 //    warp walks the octree cooperatively once for the group (32 nodes tested per
-//    step) with the radius that covers every member's sphere, streams the particles
-//    of the opened leaves (the common superset) through shared memory in tiles (TMA
-//    bulk copies), and every member filters the tile down to its own neighbours.
+//    step) over the members' box dilated by their largest radius, takes the particles
+//    of the opened nodes (the common superset) 32 at a time, keeps those inside the
+//    dilated box in a shared-memory tile, and every member filters the tile down to
+//    its own neighbours.
 //
 // The grouped kernel is shared by four kinds of pair loop: density (0), hydro (1),
 // and the adjoints of the hydro accelerations (2) and of the density (3); the two
@@ -26,38 +27,45 @@ namespace sphgrp {
 
 constexpr int kWarpsPerBlock = 4;
 constexpr int kStackCap = kStackSharedMax;     // walk stack entries in shared memory
-constexpr int kRangeCap = 64;                  // pending leaf ranges
+constexpr int kRangeCap = 64;                  // pending particle ranges (ring, power of two)
 constexpr int kSpillCap = kStackSpillPerWarp;  // overflow entries per warp (global memory)
-constexpr int kTileD = 128;   // density tile (candidates)
-constexpr int kTileH = 128;   // hydro tile
-constexpr int kTileA = 128;   // adjoint tiles
-constexpr int kTileV = 128;   // velocity-derivative tile
+constexpr int kTile = 128;                     // candidates of a tile
+constexpr int kPartMax = 32;                   // members searched at once (one per lane)
+// The walk takes a node of at most this many particles whole instead of opening it.
+constexpr int kWalkWhole = 32;
 
 
-
+// per-lane counts of one launch (nodes and cands on lane 0 only); summed in 64 bits
 struct LocalCounters {
-    unsigned long long nodes = 0, cands = 0, tests = 0, pairs = 0, retests = 0;
+    unsigned nodes = 0, cands = 0, tests = 0, pairs = 0, retests = 0;
     int max_stack = 0;
 };
 
-__device__ __forceinline__ void flush_counters(const SearchArgs& a, LocalCounters& lc, int lane) {
+__device__ __forceinline__ unsigned long long warp_sum(unsigned v) {
+    unsigned long long t = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+__device__ __forceinline__ void flush_counters(const SearchArgs& a, const LocalCounters& lc, int lane) {
     // warp-reduce then one atomic per warp
-    for (int o = 16; o > 0; o >>= 1) {
-        lc.nodes += __shfl_xor_sync(0xffffffffu, lc.nodes, o);
-        lc.cands += __shfl_xor_sync(0xffffffffu, lc.cands, o);
-        lc.tests += __shfl_xor_sync(0xffffffffu, lc.tests, o);
-        lc.pairs += __shfl_xor_sync(0xffffffffu, lc.pairs, o);
-        lc.retests += __shfl_xor_sync(0xffffffffu, lc.retests, o);
-        lc.max_stack = max(lc.max_stack, __shfl_xor_sync(0xffffffffu, lc.max_stack, o));
-    }
+    const unsigned long long nodes = warp_sum(lc.nodes), cands = warp_sum(lc.cands), tests = warp_sum(lc.tests),
+                             pairs = warp_sum(lc.pairs), retests = warp_sum(lc.retests);
+    const int deep = __reduce_max_sync(0xffffffffu, lc.max_stack);
     if (lane == 0) {
-        if (lc.nodes) atomicAdd(&a.ctr->nodes, lc.nodes);
-        if (lc.cands) atomicAdd(&a.ctr->cands, lc.cands);
-        if (lc.tests) atomicAdd(&a.ctr->tests, lc.tests);
-        if (lc.pairs) atomicAdd(&a.ctr->pairs, lc.pairs);
-        if (lc.retests) atomicAdd(&a.ctr->retests, lc.retests);
-        atomicMax(&a.ctr->max_stack, (unsigned long long)lc.max_stack);
+        if (nodes) atomicAdd(&a.ctr->nodes, nodes);
+        if (cands) atomicAdd(&a.ctr->cands, cands);
+        if (tests) atomicAdd(&a.ctr->tests, tests);
+        if (pairs) atomicAdd(&a.ctr->pairs, pairs);
+        if (retests) atomicAdd(&a.ctr->retests, retests);
+        atomicMax(&a.ctr->max_stack, (unsigned long long)deep);
     }
+}
+
+// largest of the lanes' non-negative floats
+__device__ __forceinline__ float warp_max(float v) {
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
 // Squared distance, in fixed-point units^2 and rounded down, from the point C to a
@@ -117,58 +125,15 @@ __device__ __forceinline__ void m4_shape2(float q, float& w, float& dw, float& d
 }
 
 // ---------------------------------------------------------------------------------
-// TMA bulk copies (global -> shared) completing on an mbarrier
+// Asynchronous 16-byte copies global -> shared (both addresses 16-byte aligned)
 // ---------------------------------------------------------------------------------
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// orders this thread's earlier generic accesses of shared memory before later async-proxy writes
-__device__ __forceinline__ void fence_proxy_async_smem() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
+__device__ __forceinline__ void copy16_async(float4* dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
 
-// both addresses 16-byte aligned, bytes a multiple of 16
-__device__ __forceinline__ void bulk_to_smem(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0u;
-}
-
-// Waits, with the whole warp, for the phase with the given parity; gives up after a
-// bounded number of polls (the copies of a tile take microseconds), setting the timeout
-// flag.  The result is the same on every lane: true only if every lane saw the phase
-// complete.
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, uint32_t parity, unsigned* err) {
-    bool ok = false;
-    for (uint32_t k = 0; k < (1u << 24) && !ok; ++k) ok = mbar_try_wait(bar, parity);
-    ok = __all_sync(0xffffffffu, ok);
-    if (!ok && (threadIdx.x & 31) == 0) atomicOr(err, kErrTimeout);
-    return ok;
-}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------------
 // Per-member state of the four pair loops
@@ -184,8 +149,31 @@ struct MemberPos {
     int64_t xpos;       // export write position
 };
 
-__device__ __forceinline__ bool pos_init(MemberPos& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                         uint32_t cz, float hf) {
+// a member's key-ordered records, loaded once per search (rank < 0: an empty slot)
+struct MemberRec {
+    int rank;
+    uint4 P;
+    float4 O;
+    double h;
+};
+
+__device__ __forceinline__ MemberRec load_member(const SearchArgs& a, int rank) {
+    MemberRec r;
+    r.rank = rank;
+    r.P = make_uint4(0u, 0u, 0u, 0u);
+    r.O = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    r.h = 1.0;
+    if (rank >= 0) {
+        r.P = a.pfix[rank];
+        r.O = a.poff[rank];
+        r.h = a.h64[rank];
+    }
+    return r;
+}
+
+__device__ __forceinline__ bool pos_init(MemberPos& M, const MemberRec& rec, uint32_t cx, uint32_t cy, uint32_t cz,
+                                         float hf) {
+    const int rank = rec.rank;
     M.rank = rank;
     M.n = 0;
     M.xpos = 0;
@@ -194,11 +182,9 @@ __device__ __forceinline__ bool pos_init(MemberPos& M, const SearchArgs& a, int 
         M.mx = M.my = M.mz = 0.0f;
         return false;
     }
-    uint4 P = a.pfix[rank];
-    float4 O = a.poff[rank];
-    M.mx = rel_coord(P.x, O.x, cx);
-    M.my = rel_coord(P.y, O.y, cy);
-    M.mz = rel_coord(P.z, O.z, cz);
+    M.mx = rel_coord(rec.P.x, rec.O.x, cx);
+    M.my = rel_coord(rec.P.y, rec.O.y, cy);
+    M.mz = rel_coord(rec.P.z, rec.O.z, cz);
     M.precise = fmaxf(fabsf(M.mx), fmaxf(fabsf(M.my), fabsf(M.mz))) > kPreciseReach * hf;
     return true;
 }
@@ -208,8 +194,13 @@ struct DMember : MemberPos {
     float hinv;
     float h2lo, h2hi;   // decided-inside below h2lo, candidate below h2hi
     float thr_dot;      // phase-A threshold of |p|^2 - 2 p.m (= h2hi - |m|^2)
-    float s0, c0, s1, c1, s2, c2;   // compensated totals: sum m w, sum m (3w + q w'), sum of the W_hh shape
-    float p0, p1, p2;               // plain partial sums of the current tile
+    float s0, c0, s1, c1;   // compensated totals: sum m w, sum m (3w + q w')
+    float p0, p1;           // plain partial sums of the current tile
+};
+
+// density member with the second derivative (backward): also the sum of the W_hh shape
+struct D2Member : DMember {
+    float s2, c2, p2;
 };
 
 // density member with the velocity derivatives over the same density set: the sums of
@@ -272,13 +263,13 @@ struct VMember : MemberPos {
     float pd, px_, py_, pz_;                   // plain partial sums of the current tile
 };
 
-__device__ __forceinline__ void member_init(DMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
-    M.s0 = M.c0 = M.s1 = M.c1 = M.s2 = M.c2 = 0.0f;
-    M.p0 = M.p1 = M.p2 = 0.0f;
-    double h = rank >= 0 ? a.h64[rank] : 1.0;
+__device__ __forceinline__ void member_init(DMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
+    M.s0 = M.c0 = M.s1 = M.c1 = 0.0f;
+    M.p0 = M.p1 = 0.0f;
+    const double h = rec.h;
     float hf = (float)h;
-    if (!pos_init(M, a, rank, cx, cy, cz, hf)) {
+    if (!pos_init(M, rec, cx, cy, cz, hf)) {
         M.hinv = 0.0f;
         M.h2lo = M.h2hi = -1.0f;
         M.thr_dot = -3.0e38f;
@@ -293,27 +284,33 @@ __device__ __forceinline__ void member_init(DMember& M, const SearchArgs& a, int
     M.thr_dot = M.h2hi - m2;
 }
 
-__device__ __forceinline__ void member_init(DVMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
-    member_init(static_cast<DMember&>(M), a, rank, cx, cy, cz);
+__device__ __forceinline__ void member_init(D2Member& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
+    member_init(static_cast<DMember&>(M), a, rec, cx, cy, cz);
+    M.s2 = M.c2 = M.p2 = 0.0f;
+}
+
+__device__ __forceinline__ void member_init(DVMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
+    member_init(static_cast<DMember&>(M), a, rec, cx, cy, cz);
     M.sd = M.cd = M.sx = M.cx_ = M.sy = M.cy_ = M.sz = M.cz_ = 0.0f;
     M.pd = M.px_ = M.py_ = M.pz_ = 0.0f;
     M.vx = M.vy = M.vz = M.sk = 0.0f;
-    if (rank < 0) return;
-    const float4 V = a.hyd0[rank];
+    if (rec.rank < 0) return;
+    const float4 V = a.hyd0[rec.rank];
     M.vx = V.x;
     M.vy = V.y;
     M.vz = V.z;
     M.sk = kSkernel * (M.hinv * M.hinv) * (M.hinv * M.hinv);
 }
 
-__device__ __forceinline__ void member_init(DLMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
-    member_init(static_cast<DMember&>(M), a, rank, cx, cy, cz);
+__device__ __forceinline__ void member_init(DLMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
+    member_init(static_cast<DMember&>(M), a, rec, cx, cy, cz);
     M.lsub = 0;
     M.lcnt = 0;
     M.lptr = nullptr;
-    if (rank < 0) {
+    if (rec.rank < 0) {
         M.hwf = 0.0f;
         M.h2whi = -1.0f;
         M.thr_dot_w = -3.0e38f;
@@ -321,18 +318,18 @@ __device__ __forceinline__ void member_init(DLMember& M, const SearchArgs& a, in
     }
     // the same band as the thresholds at h, at h_w: every candidate with an exact
     // distance below h_w passes it
-    const double hw = a.h64[rank] * a.list_widen;
+    const double hw = rec.h * a.list_widen;
     M.hwf = (float)hw;
     const float m2 = M.mx * M.mx + M.my * M.my + M.mz * M.mz;
     M.h2whi = fmaf((float)(hw * hw), 1.0f + 3.0f * kBandRel, 8.0f * kBandRel * m2);
     M.thr_dot_w = M.h2whi - m2;
 }
 
-__device__ __forceinline__ bool sym_init(SymMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
+__device__ __forceinline__ bool sym_init(SymMember& M, const MemberRec& rec, uint32_t cx, uint32_t cy,
                                          uint32_t cz) {
-    double h = rank >= 0 ? a.h64[rank] : 1.0;
+    const double h = rec.h;
     M.h = (float)h;
-    if (!pos_init(M, a, rank, cx, cy, cz, M.h)) {
+    if (!pos_init(M, rec, cx, cy, cz, M.h)) {
         M.h = 0.0f; M.hinv = 0.0f; M.sk = 0.0f;
         M.h2 = -1.0f; M.bk = -1.0f;
         M.bk_dot = -3.0e38f;
@@ -345,15 +342,15 @@ __device__ __forceinline__ bool sym_init(SymMember& M, const SearchArgs& a, int 
     return true;
 }
 
-__device__ __forceinline__ void member_init(HMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
+__device__ __forceinline__ void member_init(HMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
     M.sx = M.cx_ = M.sy = M.cy_ = M.sz = M.cz_ = M.su = M.cu = 0.0f;
     M.px_ = M.py_ = M.pz_ = M.pu = 0.0f;
     M.vx = M.vy = M.vz = M.cs = M.A = M.rho = 0.0f;
     M.fb = 1.0f;
-    if (!sym_init(M, a, rank, cx, cy, cz)) return;
-    float4 H0 = a.hyd0[rank];
-    float4 H1 = a.hyd1[rank];   // {A, rho, 1/h, limiter}
+    if (!sym_init(M, rec, cx, cy, cz)) return;
+    float4 H0 = a.hyd0[rec.rank];
+    float4 H1 = a.hyd1[rec.rank];   // {A, rho, 1/h, limiter}
     M.hinv = H1.z;
     M.sk = kSkernel * (H1.z * H1.z) * (H1.z * H1.z);
     M.fb = H1.w;
@@ -362,49 +359,49 @@ __device__ __forceinline__ void member_init(HMember& M, const SearchArgs& a, int
     M.rho = H1.y;
 }
 
-__device__ __forceinline__ void member_init(HAMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
+__device__ __forceinline__ void member_init(HAMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
     for (int k = 0; k < 3; ++k) M.xb[k] = M.vb[k] = 0.0f;
     M.mb = M.hb = M.rb = M.Ab = 0.0f;
     M.vx = M.vy = M.vz = M.cs = M.A = M.rho = M.m = 0.0f;
     M.wx = M.wy = M.wz = 0.0f;
-    if (!sym_init(M, a, rank, cx, cy, cz)) return;
-    float4 H0 = a.hyd0[rank];
-    float4 H1 = a.hyd1[rank];
-    float4 Wt = a.wadj[rank];
+    if (!sym_init(M, rec, cx, cy, cz)) return;
+    float4 H0 = a.hyd0[rec.rank];
+    float4 H1 = a.hyd1[rec.rank];
+    float4 Wt = a.wadj[rec.rank];
     M.hinv = H1.z;
     M.sk = H1.w;
     M.vx = H0.x; M.vy = H0.y; M.vz = H0.z; M.cs = H0.w;
     M.A = H1.x;
     M.rho = H1.y;
-    M.m = a.poff[rank].w;
+    M.m = rec.O.w;
     M.wx = Wt.x; M.wy = Wt.y; M.wz = Wt.z;
 }
 
-__device__ __forceinline__ void member_init(DAMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
+__device__ __forceinline__ void member_init(DAMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
     for (int k = 0; k < 3; ++k) M.xb[k] = 0.0f;
     M.mb = 0.0f;
     M.alpha = M.beta = M.m = 0.0f;
-    if (!sym_init(M, a, rank, cx, cy, cz)) return;
-    float4 D = a.dadj[rank];
+    if (!sym_init(M, rec, cx, cy, cz)) return;
+    float4 D = a.dadj[rec.rank];
     M.alpha = D.x;
     M.beta = D.y;
     M.hinv = D.z;
     M.sk = D.w;
-    M.m = a.poff[rank].w;
+    M.m = rec.O.w;
 }
 
-__device__ __forceinline__ void member_init(VMember& M, const SearchArgs& a, int rank, uint32_t cx, uint32_t cy,
-                                            uint32_t cz) {
+__device__ __forceinline__ void member_init(VMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
+                                            uint32_t cy, uint32_t cz) {
     M.sd = M.cd = M.sx = M.cx_ = M.sy = M.cy_ = M.sz = M.cz_ = 0.0f;
     M.pd = M.px_ = M.py_ = M.pz_ = 0.0f;
     M.vx = M.vy = M.vz = 0.0f;
     M.sk = 0.0f;
     M.rrho = 0.0f;
-    double h = rank >= 0 ? a.h64[rank] : 1.0;
+    const double h = rec.h;
     float hf = (float)h;
-    if (!pos_init(M, a, rank, cx, cy, cz, hf)) {
+    if (!pos_init(M, rec, cx, cy, cz, hf)) {
         M.hinv = 0.0f;
         M.h2lo = M.h2hi = -1.0f;
         M.thr_dot = -3.0e38f;
@@ -417,202 +414,131 @@ __device__ __forceinline__ void member_init(VMember& M, const SearchArgs& a, int
     M.h2hi = fmaf(h2, 1.0f + 3.0f * kBandRel, bk);
     M.h2lo = fmaf(h2, 1.0f - 3.0f * kBandRel, -bk);
     M.thr_dot = M.h2hi - m2;
-    const float4 H0 = a.hyd0[rank];
-    const float4 H1 = a.hyd1[rank];
+    const float4 H0 = a.hyd0[rec.rank];
+    const float4 H1 = a.hyd1[rec.rank];
     M.vx = H0.x; M.vy = H0.y; M.vz = H0.z;
     M.rrho = 1.0f / H1.y;
     M.sk = H1.w;
 }
 
-// walk radius ingredients: density R_s = max(|m| + h); symmetric R_g = max |m|, hmax_g
-__device__ __forceinline__ void radius_terms(const VMember& M, float& rl, float& hl) {
-    if (M.rank < 0) return;
-    float mr = sqrt(M.mx * M.mx + M.my * M.my + M.mz * M.mz);
-    rl = fmaxf(rl, mr + 1.0f / M.hinv);
-}
-
-__device__ __forceinline__ void radius_terms(const DLMember& M, float& rl, float& hl) {
-    if (M.rank < 0) return;
-    float mr = sqrtf(M.mx * M.mx + M.my * M.my + M.mz * M.mz);
-    rl = fmaxf(rl, mr + M.hwf);
-}
-
-__device__ __forceinline__ void radius_terms(const DMember& M, float& rl, float& hl) {
-    if (M.rank < 0) return;
-    float mr = sqrtf(M.mx * M.mx + M.my * M.my + M.mz * M.mz);
-    rl = fmaxf(rl, mr + 1.0f / M.hinv);
-}
-
-__device__ __forceinline__ void radius_terms(const SymMember& M, float& rl, float& hl) {
-    if (M.rank < 0) return;
-    float mr = sqrtf(M.mx * M.mx + M.my * M.my + M.mz * M.mz);
-    rl = fmaxf(rl, mr);
-    hl = fmaxf(hl, M.h);
-}
+// radius of the search sphere around a member (symmetric kinds: its own h; a node or a
+// candidate widens it by its own)
+__device__ __forceinline__ float member_radius(const DMember& M) { return M.rank < 0 ? 0.0f : 1.0f / M.hinv; }
+__device__ __forceinline__ float member_radius(const DLMember& M) { return M.rank < 0 ? 0.0f : M.hwf; }
+__device__ __forceinline__ float member_radius(const VMember& M) { return M.rank < 0 ? 0.0f : 1.0f / M.hinv; }
+__device__ __forceinline__ float member_radius(const SymMember& M) { return M.rank < 0 ? 0.0f : M.h; }
 
 // ---------------------------------------------------------------------------------
-// Candidate tiles in shared memory.  The raw key-ordered records of a tile's leaf
-// ranges land here by TMA bulk copies (cp.async.bulk, global -> shared, completion
-// on an mbarrier); the fixed-point positions are then converted in place to FP32
-// coordinates relative to the group centre, {px, py, pz, |p|^2}.  With S slices the
-// lane of slice s filters positions s, s + S, s + 2S, ...; positions beyond the tile's
-// candidates, up to whole chunks of 32 per slice, hold NaN dummies.
+// Candidate tiles in shared memory: the candidates of a group that passed the test
+// against its dilated box, in walk order, as FP32 coordinates relative to the group
+// centre {px, py, pz, |p|^2}, with their mass (symmetric kinds: and h^2), rank and the
+// kind's own records.  With S slices the lane of slice s filters positions s, s + S,
+// s + 2S, ...; positions beyond the tile's candidates, up to whole chunks of 32 per
+// slice, hold NaN dummies.
 // ---------------------------------------------------------------------------------
 
-struct DensTile {
-    float4 p[kTileD];   // raw pfix -> {px, py, pz, |p|^2}
-    float4 o[kTileD];   // raw poff {ox, oy, oz, m}
-    int r[kTileD];      // ranks
-    uint32_t masks[kTileD];   // phase-A bit masks [chunk][lane]
+struct PlainTile {
+    float4 p[kTile];        // {px, py, pz, |p|^2}
+    float m[kTile];
+    int r[kTile];           // ranks
+    uint32_t masks[kTile];  // phase-A bit masks [chunk][lane]
+};
+struct SymTile {
+    float4 p[kTile];
+    float2 q[kTile];        // {h_j^2, m_j}
+    int r[kTile];
+    uint32_t masks[kTile];
+};
+struct VelTile : PlainTile {
+    float4 v[kTile];        // hyd0 {vx, vy, vz, -}
+};
+struct HydroTile : SymTile {
+    float4 v[kTile];        // hyd0 {vx, vy, vz, c}
+    float4 h[kTile];        // hyd1 {A, rho, 1/h, limiter}
+};
+struct HAdjTile : SymTile {
+    float4 v[kTile];        // hyd0 {vx, vy, vz, c}
+    float4 h[kTile];        // hyd1 {A, rho, 1/h, 8/(pi h^4)}
+    float4 w[kTile];        // wadj {wx, wy, wz, -}
+};
+struct DAdjTile : SymTile {
+    float4 d[kTile];        // dadj {alpha, beta, 1/h, 8/(pi h^4)}
 };
 
-struct HydroTile {
-    float4 p[kTileH];   // raw pfix -> {px, py, pz, |p|^2}
-    float4 o[kTileH];   // raw poff {ox, oy, oz, m} -> {h^2, m, -, -}
-    float4 v[kTileH];   // raw hyd0 {vx, vy, vz, c}
-    float4 h[kTileH];   // raw hyd1 {A, rho, 1/h, 8/(pi h^4)}
-    int r[kTileH];
-    uint32_t masks[kTileH];
-};
-
-struct HAdjTile {
-    float4 p[kTileA];
-    float4 o[kTileA];   // -> {h^2, m, -, -}
-    float4 v[kTileA];   // hyd0 {vx, vy, vz, c}
-    float4 h[kTileA];   // hyd1 {A, rho, 1/h, 8/(pi h^4)}
-    float4 w[kTileA];   // wadj {wx, wy, wz, -}
-    int r[kTileA];
-    uint32_t masks[kTileA];
-};
-
-struct DAdjTile {
-    float4 p[kTileA];
-    float4 o[kTileA];   // -> {h^2, m, -, -}
-    float4 d[kTileA];   // dadj {alpha, beta, 1/h, 8/(pi h^4)}
-    int r[kTileA];
-    uint32_t masks[kTileA];
-};
-
-struct DensVTile {
-    float4 p[kTileD];   // raw pfix -> {px, py, pz, |p|^2}
-    float4 o[kTileD];   // raw poff {ox, oy, oz, m}
-    float4 v[kTileD];   // raw hyd0 {vx, vy, vz, -}
-    int r[kTileD];
-    uint32_t masks[kTileD];
-};
-
-struct VelTile {
-    float4 p[kTileV];   // raw pfix -> {px, py, pz, |p|^2}
-    float4 o[kTileV];   // raw poff {ox, oy, oz, m}
-    float4 v[kTileV];   // raw hyd0 {vx, vy, vz, -}
-    int r[kTileV];
-    uint32_t masks[kTileV];
-};
-
-// kind policies
+// kind policies; min_blocks: resident blocks per SM (register budget; 0: compiler's choice)
 struct KDens {
-    static constexpr int min_blocks = 8;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 8;
     static constexpr int id = 0;
     static constexpr bool sym = false;
-    static constexpr int cap = kTileD;
-    static constexpr uint32_t bytes = 32u;
     using Member = DMember;
-    using Tile = DensTile;
+    using Tile = PlainTile;
+};
+struct KDens2 {
+    static constexpr int min_blocks = 7;
+    static constexpr int id = kKindDensity;
+    static constexpr bool sym = false;
+    using Member = D2Member;
+    using Tile = PlainTile;
 };
 struct KDensVel {
-    static constexpr int min_blocks = 6;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 6;
     static constexpr int id = kKindDensityVel;
     static constexpr bool sym = false;
-    static constexpr int cap = kTileD;
-    static constexpr uint32_t bytes = 48u;
     using Member = DVMember;
-    using Tile = DensVTile;
+    using Tile = VelTile;
 };
 struct KDensList {
-    static constexpr int min_blocks = 7;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 7;
     static constexpr int id = kKindDensityList;
     static constexpr bool sym = false;
-    static constexpr int cap = kTileD;
-    static constexpr uint32_t bytes = 32u;
     using Member = DLMember;
-    using Tile = DensTile;
+    using Tile = PlainTile;
 };
 struct KHydro {
-    static constexpr int min_blocks = 5;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 5;
     static constexpr int id = 1;
     static constexpr bool sym = true;
-    static constexpr int cap = kTileH;
-    static constexpr uint32_t bytes = 64u;
     using Member = HMember;
     using Tile = HydroTile;
 };
 struct KHAdj {
-    static constexpr int min_blocks = 0;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 0;
     static constexpr int id = 2;
     static constexpr bool sym = true;
-    static constexpr int cap = kTileA;
-    static constexpr uint32_t bytes = 80u;
     using Member = HAMember;
     using Tile = HAdjTile;
 };
 struct KDAdj {
-    static constexpr int min_blocks = 6;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 6;
     static constexpr int id = 3;
     static constexpr bool sym = true;
-    static constexpr int cap = kTileA;
-    static constexpr uint32_t bytes = 48u;
     using Member = DAMember;
     using Tile = DAdjTile;
 };
-
 struct KVel {
-    static constexpr int min_blocks = 0;   // resident blocks per SM (register budget; 0: compiler's choice)
+    static constexpr int min_blocks = 0;
     static constexpr int id = 4;
     static constexpr bool sym = false;
-    static constexpr int cap = kTileV;
-    static constexpr uint32_t bytes = 48u;
     using Member = VMember;
     using Tile = VelTile;
 };
 
-// bulk copies of one run of candidates into the tile
-__device__ __forceinline__ void stage_run(DensTile& T, const SearchArgs& a, int dst, int src, uint32_t b,
-                                          unsigned long long* bar) {
-    bulk_to_smem(&T.p[dst], a.pfix + src, b, bar);
-    bulk_to_smem(&T.o[dst], a.poff + src, b, bar);
+// the kind's own records of a candidate that entered the tile at position t
+__device__ __forceinline__ void stage_records(PlainTile&, const SearchArgs&, int, int) {}
+__device__ __forceinline__ void stage_records(VelTile& T, const SearchArgs& a, int t, int rank) {
+    copy16_async(&T.v[t], a.hyd0 + rank);
 }
-__device__ __forceinline__ void stage_run(HydroTile& T, const SearchArgs& a, int dst, int src, uint32_t b,
-                                          unsigned long long* bar) {
-    bulk_to_smem(&T.p[dst], a.pfix + src, b, bar);
-    bulk_to_smem(&T.o[dst], a.poff + src, b, bar);
-    bulk_to_smem(&T.v[dst], a.hyd0 + src, b, bar);
-    bulk_to_smem(&T.h[dst], a.hyd1 + src, b, bar);
+__device__ __forceinline__ void stage_records(HydroTile& T, const SearchArgs& a, int t, int rank) {
+    copy16_async(&T.v[t], a.hyd0 + rank);
+    copy16_async(&T.h[t], a.hyd1 + rank);
 }
-__device__ __forceinline__ void stage_run(HAdjTile& T, const SearchArgs& a, int dst, int src, uint32_t b,
-                                          unsigned long long* bar) {
-    bulk_to_smem(&T.p[dst], a.pfix + src, b, bar);
-    bulk_to_smem(&T.o[dst], a.poff + src, b, bar);
-    bulk_to_smem(&T.v[dst], a.hyd0 + src, b, bar);
-    bulk_to_smem(&T.h[dst], a.hyd1 + src, b, bar);
-    bulk_to_smem(&T.w[dst], a.wadj + src, b, bar);
+__device__ __forceinline__ void stage_records(HAdjTile& T, const SearchArgs& a, int t, int rank) {
+    copy16_async(&T.v[t], a.hyd0 + rank);
+    copy16_async(&T.h[t], a.hyd1 + rank);
+    copy16_async(&T.w[t], a.wadj + rank);
 }
-__device__ __forceinline__ void stage_run(DensVTile& T, const SearchArgs& a, int dst, int src, uint32_t b,
-                                          unsigned long long* bar) {
-    bulk_to_smem(&T.p[dst], a.pfix + src, b, bar);
-    bulk_to_smem(&T.o[dst], a.poff + src, b, bar);
-    bulk_to_smem(&T.v[dst], a.hyd0 + src, b, bar);
-}
-__device__ __forceinline__ void stage_run(VelTile& T, const SearchArgs& a, int dst, int src, uint32_t b,
-                                          unsigned long long* bar) {
-    bulk_to_smem(&T.p[dst], a.pfix + src, b, bar);
-    bulk_to_smem(&T.o[dst], a.poff + src, b, bar);
-    bulk_to_smem(&T.v[dst], a.hyd0 + src, b, bar);
-}
-__device__ __forceinline__ void stage_run(DAdjTile& T, const SearchArgs& a, int dst, int src, uint32_t b,
-                                          unsigned long long* bar) {
-    bulk_to_smem(&T.p[dst], a.pfix + src, b, bar);
-    bulk_to_smem(&T.o[dst], a.poff + src, b, bar);
-    bulk_to_smem(&T.d[dst], a.dadj + src, b, bar);
+__device__ __forceinline__ void stage_records(DAdjTile& T, const SearchArgs& a, int t, int rank) {
+    copy16_async(&T.d[t], a.dadj + rank);
 }
 
 // ---------------------------------------------------------------------------------
@@ -624,8 +550,13 @@ __device__ __forceinline__ void stage_run(DAdjTile& T, const SearchArgs& a, int 
 __device__ __forceinline__ void flush(DMember& M) {
     kahan_add(M.s0, M.c0, M.p0);
     kahan_add(M.s1, M.c1, M.p1);
+    M.p0 = M.p1 = 0.0f;
+}
+
+__device__ __forceinline__ void flush(D2Member& M) {
+    flush(static_cast<DMember&>(M));
     kahan_add(M.s2, M.c2, M.p2);
-    M.p0 = M.p1 = M.p2 = 0.0f;
+    M.p2 = 0.0f;
 }
 
 __device__ __forceinline__ void flush(HMember& M) {
@@ -670,9 +601,24 @@ __device__ __forceinline__ void precise_diff(const Mem& M, const SearchArgs& a, 
     r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
+// density terms of a neighbour at q = r / h
+__device__ __forceinline__ void density_terms(DMember& M, float mj, float q) {
+    float w, dw;
+    m4_shape(q, w, dw);
+    M.p0 = fmaf(mj, w, M.p0);
+    M.p1 = fmaf(mj, fmaf(q, dw, 3.0f * w), M.p1);
+}
+__device__ __forceinline__ void density_terms(D2Member& M, float mj, float q) {
+    float w, dw, d2w;
+    m4_shape2(q, w, dw, d2w);
+    M.p0 = fmaf(mj, w, M.p0);
+    M.p1 = fmaf(mj, fmaf(q, dw, 3.0f * w), M.p1);
+    M.p2 = fmaf(mj, fmaf(q * q, d2w, fmaf(8.0f * q, dw, 12.0f * w)), M.p2);
+}
+
 // density pair: p = candidate's coordinates relative to the member's centre, m_j its mass
-template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void density_pair(DMember& M, const SearchArgs& a, float4 p, float mj, int crank,
+template <int MODE, bool WRAP = false, class Mem>
+__device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float4 p, float mj, int crank,
                                              LocalCounters& lc) {
     float dx = rel_diff<WRAP>(p.x, M.mx), dy = rel_diff<WRAP>(p.y, M.my), dz = rel_diff<WRAP>(p.z, M.mz);
     float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -689,18 +635,7 @@ __device__ __forceinline__ void density_pair(DMember& M, const SearchArgs& a, fl
     if (MODE == kAcc) {
         if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
         float q = r2 * rsqrtf(fmaxf(r2, 1.0e-30f)) * M.hinv;
-        if (a.o_s2) {
-            float w, dw, d2w;
-            m4_shape2(q, w, dw, d2w);
-            M.p0 = fmaf(mj, w, M.p0);
-            M.p1 = fmaf(mj, fmaf(q, dw, 3.0f * w), M.p1);
-            M.p2 = fmaf(mj, fmaf(q * q, d2w, fmaf(8.0f * q, dw, 12.0f * w)), M.p2);
-        } else {
-            float w, dw;
-            m4_shape(q, w, dw);
-            M.p0 = fmaf(mj, w, M.p0);
-            M.p1 = fmaf(mj, fmaf(q, dw, 3.0f * w), M.p1);
-        }
+        density_terms(M, mj, q);
     } else if (MODE == kFill) {
         int64_t q = M.xpos++;
         if (q < a.x_cap) a.x_idx[q] = a.perm[crank];
@@ -715,7 +650,7 @@ template <int MODE, bool WRAP = false>
 __device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, float4 p, float mj, float4 vj,
                                              int crank, LocalCounters& lc) {
     const int n0 = M.n;
-    density_pair<MODE, WRAP>(M, a, p, mj, crank, lc);
+    density_pair<MODE, WRAP>(static_cast<DMember&>(M), a, p, mj, crank, lc);
     if (MODE != kAcc || M.n == n0) return;
     float dx, dy, dz, r2;
     if (M.precise) {
@@ -750,7 +685,7 @@ __device__ __forceinline__ void density_list_pair(DLMember& M, const SearchArgs&
         if (M.lcnt < M.lsub) M.lptr[M.lcnt] = crank;
         M.lcnt++;
     }
-    density_pair<MODE, WRAP>(M, a, p, mj, crank, lc);
+    density_pair<MODE, WRAP>(static_cast<DMember&>(M), a, p, mj, crank, lc);
 }
 
 // velocity-derivative pair (density criterion): p = relative coordinates, mj the mass,
@@ -805,10 +740,10 @@ __device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, fl
     return in;
 }
 
-// hydro pair: p = relative coordinates, q = {h_j^2, m_j, -, -}, v = {vx, vy, vz, c_j},
+// hydro pair: p = relative coordinates, q = {h_j^2, m_j}, v = {vx, vy, vz, c_j},
 // hh = {A_j, rho_j, 1/h_j, limiter_j}
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float4 p, float4 q,
+__device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float4 p, float2 q,
                                            float4 v, float4 hh, int crank, LocalCounters& lc) {
     // The member itself is a candidate: the exports skip it by rank; the sums skip it
     // as a pair at r = 0 (counted, then taken off the neighbour count at the end).
@@ -859,7 +794,7 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
 // Q = rhat . (m_j w_k - m_k w_j), rhat = (x_k - x_j) / r.  Accumulated: dE/d of x_k,
 // v_k, m_k, h_k, rho_k (through the viscosity) and A_k.
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a, float4 p, float4 q, float4 v,
+__device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a, float4 p, float2 q, float4 v,
                                                float4 hh, float4 wj, int crank, LocalCounters& lc) {
     // the member itself enters as a pair at r = 0, which contributes nothing
     float dx, dy, dz, r2;
@@ -932,9 +867,9 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
 
 // Adjoint of sum_i (alpha_i rho_i + beta_i dRho_i/dh_i) at fixed h, gathered at member k:
 // rho_k's own sum (x_k moves every pair) and the sums of every j with k in N_j (x_k and
-// m_k enter as a neighbour).  q = {h_j^2, m_j, -, -}, d = {alpha_j, beta_j, 1/h_j, s_j}.
+// m_k enter as a neighbour).  q = {h_j^2, m_j}, d = {alpha_j, beta_j, 1/h_j, s_j}.
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, float4 p, float4 q, float4 d,
+__device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, float4 p, float2 q, float4 d,
                                               int crank, LocalCounters& lc) {
     // The member itself enters as a pair at r = 0 like any coincident neighbour:
     // alpha W(0, h) + beta W_h(0, h) = alpha s h - 3 beta s, and no position term.
@@ -965,39 +900,44 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
 
 // phase B dispatch
 template <int MODE, bool WRAP>
-__device__ __forceinline__ void tile_pair(DMember& M, const SearchArgs& a, const DensTile& T, int j,
+__device__ __forceinline__ void tile_pair(DMember& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_pair<MODE, WRAP>(M, a, T.p[j], T.o[j].w, T.r[j], lc);
+    density_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
-__device__ __forceinline__ void tile_pair(DVMember& M, const SearchArgs& a, const DensVTile& T, int j,
+__device__ __forceinline__ void tile_pair(D2Member& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    densvel_pair<MODE, WRAP>(M, a, T.p[j], T.o[j].w, T.v[j], T.r[j], lc);
+    density_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
-__device__ __forceinline__ void tile_pair(DLMember& M, const SearchArgs& a, const DensTile& T, int j,
+__device__ __forceinline__ void tile_pair(DVMember& M, const SearchArgs& a, const VelTile& T, int j,
                                           LocalCounters& lc) {
-    density_list_pair<MODE, WRAP>(M, a, T.p[j], T.o[j].w, T.r[j], lc);
+    densvel_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.v[j], T.r[j], lc);
+}
+template <int MODE, bool WRAP>
+__device__ __forceinline__ void tile_pair(DLMember& M, const SearchArgs& a, const PlainTile& T, int j,
+                                          LocalCounters& lc) {
+    density_list_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(VMember& M, const SearchArgs& a, const VelTile& T, int j,
                                           LocalCounters& lc) {
-    vel_pair<MODE, WRAP>(M, a, T.p[j], T.o[j].w, T.v[j], T.r[j], lc);
+    vel_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.v[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(HMember& M, const SearchArgs& a, const HydroTile& T, int j,
                                           LocalCounters& lc) {
-    hydro_pair<MODE, WRAP>(M, a, T.p[j], T.o[j], T.v[j], T.h[j], T.r[j], lc);
+    hydro_pair<MODE, WRAP>(M, a, T.p[j], T.q[j], T.v[j], T.h[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(HAMember& M, const SearchArgs& a, const HAdjTile& T, int j,
                                           LocalCounters& lc) {
-    hydro_adj_pair<MODE, WRAP>(M, a, T.p[j], T.o[j], T.v[j], T.h[j], T.w[j], T.r[j], lc);
+    hydro_adj_pair<MODE, WRAP>(M, a, T.p[j], T.q[j], T.v[j], T.h[j], T.w[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DAMember& M, const SearchArgs& a, const DAdjTile& T, int j,
                                           LocalCounters& lc) {
-    dens_adj_pair<MODE, WRAP>(M, a, T.p[j], T.o[j], T.d[j], T.r[j], lc);
+    dens_adj_pair<MODE, WRAP>(M, a, T.p[j], T.q[j], T.d[j], T.r[j], lc);
 }
 
 // phase A threshold of the dot form |p|^2 - 2 p.m (density) and of the difference
@@ -1019,8 +959,11 @@ __device__ __forceinline__ float thr_diff(const SymMember& M, float hj2) {
 __device__ __forceinline__ float xsum(float v, int o) { return v + __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ void slice_add(DMember& M, int o) {
     M.s0 = xsum(M.s0, o); M.c0 = xsum(M.c0, o); M.s1 = xsum(M.s1, o); M.c1 = xsum(M.c1, o);
-    M.s2 = xsum(M.s2, o); M.c2 = xsum(M.c2, o);
     M.n += __shfl_xor_sync(0xffffffffu, M.n, o);
+}
+__device__ __forceinline__ void slice_add(D2Member& M, int o) {
+    slice_add(static_cast<DMember&>(M), o);
+    M.s2 = xsum(M.s2, o); M.c2 = xsum(M.c2, o);
 }
 __device__ __forceinline__ void slice_add(DVMember& M, int o) {
     slice_add(static_cast<DMember&>(M), o);
@@ -1054,11 +997,15 @@ __device__ __forceinline__ void write_result(const DMember& D, const SearchArgs&
     if (MODE == kAcc) {
         a.o_s0[D.rank] = D.s0 - D.c0;
         a.o_s1[D.rank] = D.s1 - D.c1;
-        if (a.o_s2) a.o_s2[D.rank] = D.s2 - D.c2;
         a.o_n[D.rank] = D.n;
     } else if (MODE == kCount) {
         a.x_cnt[a.perm[D.rank]] = D.n;
     }
+}
+template <int MODE>
+__device__ __forceinline__ void write_result(const D2Member& D, const SearchArgs& a) {
+    write_result<MODE>(static_cast<const DMember&>(D), a);
+    if (MODE == kAcc) a.o_s2[D.rank] = D.s2 - D.c2;
 }
 template <int MODE>
 __device__ __forceinline__ void write_result(const DVMember& D, const SearchArgs& a) {
@@ -1118,10 +1065,8 @@ __device__ __forceinline__ void write_result(const DAMember& D, const SearchArgs
 // ---------------------------------------------------------------------------------
 
 struct alignas(16) WalkSmem {
-    unsigned long long bar;      // mbarrier of the tile copies
     uint32_t stack[kStackCap];   // node ranges: (first child << 3) | (count - 1)
-    int2 ranges[kRangeCap];      // pending leaf ranges (first rank, count)
-    int rpre[kRangeCap + 1];     // prefix of the pending counts
+    int2 ranges[kRangeCap];      // ring of pending particle ranges {first rank - flat start, flat start}
 };
 
 __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
@@ -1133,126 +1078,107 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
     return v;
 }
 
-// Member slot layout of a lane: with group size g <= 32 a power of two, the warp
-// holds S = 32 / g copies ("slices") of the g members and each slice filters a
-// different subset of the candidates; otherwise the lane holds M members, one slice.
+// Member slot layout of a lane: gw member slots (the member count rounded up to a power
+// of two, at most 32) in S copies ("slices"), each filtering a different subset of the
+// candidates; k = the lane's member, -1 if it holds none.
 struct Layout {
-    int S;       // slices
-    int slice;   // this lane's slice
-    int gw;      // members per slice row (min(g, 32))
+    int gw, S, slice, k;
 };
 
-__device__ __forceinline__ Layout make_layout(int g, int lane, bool allow_slices, int max_slices) {
+__device__ __forceinline__ Layout make_layout(int cnt, int lane, bool allow_slices, int max_slices) {
     Layout L;
-    L.gw = g < 32 ? g : 32;
-    bool pow2 = (g & (g - 1)) == 0;
-    L.S = (allow_slices && g < 32 && pow2) ? min(32 / g, max_slices) : 1;
-    L.slice = L.S > 1 ? lane / g : 0;
-    if (L.slice >= L.S) L.slice = L.S;   // lanes beyond the last slice hold no member
+    const int sh = cnt <= 1 ? 0 : 32 - __clz(cnt - 1);
+    L.gw = 1 << sh;
+    L.S = allow_slices ? min(32 >> sh, max_slices) : 1;
+    L.slice = lane >> sh;
+    const int k = lane & (L.gw - 1);
+    L.k = (L.slice < L.S && k < cnt) ? k : -1;
     return L;
 }
 
-// member index (within the group) held by slot mm of this lane; -1 if none
-__device__ __forceinline__ int member_of(const Layout& L, int lane, int mm, int g) {
-    int k;
-    if (L.S > 1) {
-        if (L.slice >= L.S) return -1;
-        k = lane % g;
-    } else {
-        k = lane + 32 * mm;
-    }
-    return k < g ? k : -1;
-}
-
-// Member x candidate filter of one staged tile.  Phase A: for every chunk of 32 of
-// the lane's slice, a bit mask of the candidates inside the member's FP32 threshold,
-// tested in dot-product form |p|^2 - 2 p.m < h^2 - |m|^2 (three FMAs; its rounding
-// stays inside the FP64 decision band).  Phase B: every lane walks its own set bits
-// across all chunks (no per-chunk wait for the slowest lane) for the exact decision
-// and the pair terms; forward partial sums are folded into the compensated totals
-// after the tile.
-template <class K, int MODE, int M, bool WRAP>
-__device__ __forceinline__ void filter_tile(typename K::Tile& T, const Layout& L, typename K::Member* mem, int nt,
+// Member x candidate filter of one tile.  Phase A: for every chunk of 32 of the lane's
+// slice, a bit mask of the candidates inside the member's FP32 threshold, tested in
+// dot-product form |p|^2 - 2 p.m < h^2 - |m|^2 (three FMAs; its rounding stays inside
+// the FP64 decision band).  Phase B: every lane walks its own set bits across all chunks
+// (no per-chunk wait for the slowest lane) for the exact decision and the pair terms;
+// forward partial sums are folded into the compensated totals after the tile.
+template <class K, int MODE, bool WRAP>
+__device__ __forceinline__ void filter_tile(typename K::Tile& T, const Layout& L, typename K::Member& Mb, int nt,
                                             const SearchArgs& a, LocalCounters& lc, int lane) {
     const int S = L.S;
     if (L.slice >= S) return;
     const int cnt_slice = (nt > L.slice) ? (nt - L.slice + S - 1) / S : 0;
     const int nch = ((nt + S - 1) / S + 31) >> 5;
+    const float mx = Mb.mx, my = Mb.my, mz = Mb.mz;
+    const float ax = -2.0f * mx, ay = -2.0f * my, az = -2.0f * mz;
+    for (int c = 0; c < nch; ++c) {
+        uint32_t mask = 0u;
+        const int j0 = L.slice + S * (c << 5);
 #pragma unroll
-    for (int mm = 0; mm < M; ++mm) {
-        auto& Mb = mem[mm];
-        const float mx = Mb.mx, my = Mb.my, mz = Mb.mz;
-        const float ax = -2.0f * mx, ay = -2.0f * my, az = -2.0f * mz;
-        for (int c = 0; c < nch; ++c) {
-            uint32_t mask = 0u;
-            const int j0 = L.slice + S * (c << 5);
-#pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                const int j = j0 + q * S;
-                const float4 cp = T.p[j];
-                float hj2 = 0.0f;
-                if constexpr (K::sym) hj2 = T.o[j].x;
-                bool pass;
-                if constexpr (!WRAP) {
-                    float t = fmaf(cp.x, ax, fmaf(cp.y, ay, fmaf(cp.z, az, cp.w)));
-                    pass = t < thr_dot(Mb, hj2);
-                } else {
-                    float dx = rel_diff<true>(cp.x, mx), dy = rel_diff<true>(cp.y, my), dz = rel_diff<true>(cp.z, mz);
-                    float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    pass = r2 < thr_diff(Mb, hj2);
-                }
-                mask |= (pass ? 1u : 0u) << q;
+        for (int q = 0; q < 32; ++q) {
+            const int j = j0 + q * S;
+            const float4 cp = T.p[j];
+            float hj2 = 0.0f;
+            if constexpr (K::sym) hj2 = T.q[j].x;
+            bool pass;
+            if constexpr (!WRAP) {
+                float t = fmaf(cp.x, ax, fmaf(cp.y, ay, fmaf(cp.z, az, cp.w)));
+                pass = t < thr_dot(Mb, hj2);
+            } else {
+                float dx = rel_diff<true>(cp.x, mx), dy = rel_diff<true>(cp.y, my), dz = rel_diff<true>(cp.z, mz);
+                float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                pass = r2 < thr_diff(Mb, hj2);
             }
-            T.masks[(c << 5) + lane] = mask;
-            if (Mb.rank >= 0) lc.tests += min(32, cnt_slice - (c << 5));
+            mask |= (pass ? 1u : 0u) << q;
         }
-        int c = 0;
-        uint32_t cur = T.masks[lane];
-        for (;;) {
-            while (cur == 0u) {
-                if (++c >= nch) break;
-                cur = T.masks[(c << 5) + lane];
-            }
-            if (cur == 0u) break;
-            const int q = __ffs(cur) - 1;
-            cur &= cur - 1u;
-            tile_pair<MODE, WRAP>(Mb, a, T, L.slice + S * ((c << 5) + q), lc);
-        }
-        if (MODE == kAcc) flush(Mb);
+        T.masks[(c << 5) + lane] = mask;
     }
+    if (Mb.rank >= 0) lc.tests += cnt_slice;
+    int c = 0;
+    uint32_t cur = T.masks[lane];
+    for (;;) {
+        while (cur == 0u) {
+            if (++c >= nch) break;
+            cur = T.masks[(c << 5) + lane];
+        }
+        if (cur == 0u) break;
+        const int q = __ffs(cur) - 1;
+        cur &= cur - 1u;
+        tile_pair<MODE, WRAP>(Mb, a, T, L.slice + S * ((c << 5) + q), lc);
+    }
+    if (MODE == kAcc) flush(Mb);
 }
 
-// Filter of the nt converted candidates held in the tile: NaN dummies up to whole chunks of
-// 32 in every slice, then the member x candidate filter (dot form unless the group wraps).
-template <class K, int MODE, int M>
-__device__ __forceinline__ void filter_staged(typename K::Tile& T, const Layout& L, typename K::Member* mem, int nt,
+// Filter of the nt candidates in the tile: NaN dummies up to whole chunks of 32 in every
+// slice, then the member x candidate filter (dot form unless the group wraps).
+template <class K, int MODE>
+__device__ __forceinline__ void filter_staged(typename K::Tile& T, const Layout& L, typename K::Member& mem, int nt,
                                               const SearchArgs& a, LocalCounters& lc, int lane, bool wrap_safe) {
     const int padded = L.S * ((((nt + L.S - 1) / L.S) + 31) >> 5) * 32;
     const float nanv = __int_as_float(0x7fffffff);
     for (int t = nt + lane; t < padded; t += 32) T.p[t] = make_float4(nanv, nanv, nanv, nanv);
+    copies_wait();
     __syncwarp();
-    if (wrap_safe) filter_tile<K, MODE, M, false>(T, L, mem, nt, a, lc, lane);
-    else filter_tile<K, MODE, M, true>(T, L, mem, nt, a, lc, lane);
+    if (wrap_safe) filter_tile<K, MODE, false>(T, L, mem, nt, a, lc, lane);
+    else filter_tile<K, MODE, true>(T, L, mem, nt, a, lc, lane);
     __syncwarp();
 }
 
 // Work item of the grouped kernels: members U[base, base + cnt), the walk's start node
-// (a root of the forest), the group size of the member layout and the slice limit.
+// (a root of the forest) and the slice limit.
 struct GroupDesc {
-    int base, cnt, root, g, smax;
+    int base, cnt, root, smax;
 };
 
 __device__ __forceinline__ GroupDesc group_desc(const SearchArgs& a, int gid) {
     GroupDesc d;
     d.root = 0;
-    d.g = a.g;
-    d.smax = 32;
+    d.smax = 4;
     if (a.groups4) {
         const int4 G = a.groups4[gid];
         d.base = G.x;
         d.cnt = G.y;
         d.root = G.z;
-        d.g = G.w & 0xff;
         d.smax = (G.w >> 8) & 0xff;   // bits 16.. carry the box's leaf size
     } else if (a.groups) {
         const int2 G = a.groups[gid];
@@ -1262,10 +1188,6 @@ __device__ __forceinline__ GroupDesc group_desc(const SearchArgs& a, int gid) {
         d.base = gid * a.g;
         d.cnt = min(a.g, a.nu - d.base);
     }
-    // member slots: the group's count rounded up to a power of two, so that a group cut
-    // smaller by the split keeps every lane busy with more slices
-    const int p2 = d.cnt <= 1 ? 1 : 1 << (32 - __clz(d.cnt - 1));
-    d.g = min(d.g, p2);
     return d;
 }
 
@@ -1273,46 +1195,36 @@ __device__ __forceinline__ int group_count(const SearchArgs& a) {
     return a.ngroups_dev ? *a.ngroups_dev : a.ngroups;
 }
 
-// Group centre: the fixed-point position of the first member (lowest slot of the
-// lowest lane), or the centre of the members' bounding box (offsets from the first
-// member are exact minimum-image integers).  Ranks < 0 are empty slots.  Returns
-// false when the group has no member.
+// Group centre: the fixed-point position of the lowest lane that holds a member, or the
+// centre of the members' bounding box (offsets from that member are exact minimum-image
+// integers).  Every lane passes one record per slot; false when no lane holds a member.
 template <int M>
-__device__ __forceinline__ bool group_centre(const SearchArgs& a, const int (&rk)[M], uint32_t& cx, uint32_t& cy,
-                                             uint32_t& cz) {
-    int ref = -1;
-#pragma unroll
-    for (int mm = 0; mm < M; ++mm) {
-        const unsigned b = __ballot_sync(0xffffffffu, rk[mm] >= 0);
-        const int cand = __shfl_sync(0xffffffffu, rk[mm], b ? __ffs(b) - 1 : 0);
-        if (ref < 0 && b) ref = cand;
-    }
-    if (ref < 0) return false;
-    const uint4 P0 = a.pfix[ref];
-    cx = P0.x;
-    cy = P0.y;
-    cz = P0.z;
+__device__ __forceinline__ bool group_centre(const SearchArgs& a, const MemberRec (&rec)[M], uint32_t& cx,
+                                             uint32_t& cy, uint32_t& cz) {
+    const unsigned have = __ballot_sync(0xffffffffu, rec[0].rank >= 0);   // slot 0 holds the first members
+    if (have == 0u) return false;
+    const int ref = __ffs(have) - 1;
+    cx = __shfl_sync(0xffffffffu, rec[0].P.x, ref);
+    cy = __shfl_sync(0xffffffffu, rec[0].P.y, ref);
+    cz = __shfl_sync(0xffffffffu, rec[0].P.z, ref);
     if (a.centre_box) {
         int lox = 0, loy = 0, loz = 0, hix = 0, hiy = 0, hiz = 0;
 #pragma unroll
         for (int mm = 0; mm < M; ++mm) {
-            if (rk[mm] >= 0) {
-                const uint4 P = a.pfix[rk[mm]];
-                const int dx = (int32_t)(P.x - cx), dy = (int32_t)(P.y - cy), dz = (int32_t)(P.z - cz);
+            if (rec[mm].rank >= 0) {
+                const int dx = (int32_t)(rec[mm].P.x - cx), dy = (int32_t)(rec[mm].P.y - cy),
+                          dz = (int32_t)(rec[mm].P.z - cz);
                 lox = min(lox, dx); hix = max(hix, dx);
                 loy = min(loy, dy); hiy = max(hiy, dy);
                 loz = min(loz, dz); hiz = max(hiz, dz);
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lox = min(lox, __shfl_xor_sync(0xffffffffu, lox, o));
-            loy = min(loy, __shfl_xor_sync(0xffffffffu, loy, o));
-            loz = min(loz, __shfl_xor_sync(0xffffffffu, loz, o));
-            hix = max(hix, __shfl_xor_sync(0xffffffffu, hix, o));
-            hiy = max(hiy, __shfl_xor_sync(0xffffffffu, hiy, o));
-            hiz = max(hiz, __shfl_xor_sync(0xffffffffu, hiz, o));
-        }
+        lox = __reduce_min_sync(0xffffffffu, lox);
+        loy = __reduce_min_sync(0xffffffffu, loy);
+        loz = __reduce_min_sync(0xffffffffu, loz);
+        hix = __reduce_max_sync(0xffffffffu, hix);
+        hiy = __reduce_max_sync(0xffffffffu, hiy);
+        hiz = __reduce_max_sync(0xffffffffu, hiz);
         cx += (uint32_t)(int32_t)(((int64_t)lox + hix) >> 1);
         cy += (uint32_t)(int32_t)(((int64_t)loy + hiy) >> 1);
         cz += (uint32_t)(int32_t)(((int64_t)loz + hiz) >> 1);
@@ -1328,381 +1240,321 @@ __device__ __forceinline__ uint32_t cell_morton(uint32_t x, uint32_t y, uint32_t
 }
 
 // First node of the walk: the node of the deepest cell (level <= kStartLevels) of the
-// tree rooted at `root` (tab: that tree's start table) that
-// holds the whole search sphere (centre C, radius Rb in box units).  Every particle
-// within the sphere lies in that cell and hence in that node's subtree (a node is the
+// tree rooted at `root` (tab: that tree's start table) that holds the cube of half width
+// Rb (box units) around C, which covers the whole search region.  Every particle
+// within the region lies in that cell and hence in that node's subtree (a node is the
 // set of particles whose keys share its cell's prefix).  Cells the tree did not reach
 // fall back to the nearest ancestor cell with a node.
 __device__ __forceinline__ int walk_start(const int32_t* __restrict__ tab, int root, uint32_t cx, uint32_t cy,
                                           uint32_t cz, float Rb) {
-    // radius in fixed-point units, rounded up, plus the sub-unit offsets of the positions
-    const double Ru = ceil((double)Rb * 4294967296.0 * (1.0 + 1e-6)) + 2.0;
-    if (!(Ru < 2147483648.0)) return root;
-    const int64_t r = (int64_t)Ru;
+    // half width in fixed-point units, rounded up, plus the sub-unit offsets of the positions
+    const float Ru = __fmul_ru(__fmul_ru(Rb, 1.000002f), 4294967296.0f);
+    if (!(Ru < 2147483648.0f)) return root;
+    const int64_t r = (int64_t)Ru + 3;
     int lvl = kStartLevels;
     const uint32_t c3[3] = {cx, cy, cz};
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
         const int64_t lo = (int64_t)c3[ax] - r, hi = (int64_t)c3[ax] + r;
-        if (lo < 0 || hi > 0xffffffffll) lvl = 0;   // the sphere wraps around the box
+        if (lo < 0 || hi > 0xffffffffll) lvl = 0;   // the region wraps around the box
         else lvl = min(lvl, __clz((uint32_t)lo ^ (uint32_t)hi));
     }
-    for (; lvl >= 1; --lvl) {
-        const int nd = tab[start_table_offset(lvl) +
-                           cell_morton(cx >> (32 - lvl), cy >> (32 - lvl), cz >> (32 - lvl), lvl)];
+    if (lvl < 1) return root;
+    uint32_t m = cell_morton(cx >> (32 - lvl), cy >> (32 - lvl), cz >> (32 - lvl), lvl);
+    for (; lvl >= 1; --lvl, m >>= 3) {
+        const int nd = tab[start_table_offset(lvl) + m];
         if (nd >= 0) return nd;
     }
     return root;
 }
 
-// One group's walk from node `root` and the member x candidate filter of every staged
-// tile (the members are initialised relative to the centre C).  kSupFill writes the
-// superset at sup_pos + sup_n; sup_n accumulates the candidates.
-// Returns false if a tile copy timed out: the warp must then stop taking work.
-template <class K, int MODE, int M>
-__device__ __forceinline__ bool group_search(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, const Layout& L,
-                                             typename K::Member (&mem)[M], uint32_t cx, uint32_t cy, uint32_t cz,
-                                             int root, LocalCounters& lc, uint32_t& tma_phase, int lane,
-                                             int64_t sup_pos, int64_t& sup_n) {
-    constexpr int TCAP = K::cap;
-    constexpr bool kSup = (MODE == kSupCount || MODE == kSupFill);
+// The walk's stack and the ring of particle ranges it emits.  The stack lives in shared
+// memory (at most a.stack_cap entries); when it fills up, its oldest entries move to this
+// warp's overflow area in global memory, which holds the bottom of the stack and refills
+// the shared part when that runs empty.  The ranges, laid end to end in walk order, number
+// the candidates flat: [done, total) are pending, in ring entries [e0, e1).
+struct Walk {
+    uint32_t* spill;
+    int sp, gsp;
+    int e0, e1, done, total;
+
+    __device__ __forceinline__ bool empty() const { return sp == 0 && gsp == 0; }
+};
+
+__device__ __forceinline__ Walk walk_begin(const SearchArgs& a, WalkSmem& W, int start, int lane) {
+    Walk w;
+    w.spill = a.stack_spill + (size_t)(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * kSpillCap;
+    w.sp = 1;
+    w.gsp = 0;
+    w.e0 = w.e1 = w.done = w.total = 0;
+    if (lane == 0) W.stack[0] = (uint32_t)start << 3;   // one node
+    __syncwarp();
+    return w;
+}
+
+// A step can be taken: entries on the stack, room to push 32 of them and to emit 32 ranges.
+__device__ __forceinline__ bool walk_can_step(const SearchArgs& a, const Walk& w) {
+    return !w.empty() && w.sp <= a.stack_cap - 32 && w.e1 - w.e0 <= kRangeCap - 32;
+}
+
+// One step: up to 32 nodes from the top of the stack are tested (open(cen, ext)); of the
+// open ones, leaves and nodes of at most `whole` particles emit their range, the
+// others push their children.
+template <class Open>
+__device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk& w, int whole, LocalCounters& lc,
+                                          int lane, Open open_node) {
     const uint32_t lt = (1u << lane) - 1u;
-    float rlane = 0.0f, hlane = 0.0f;   // walk radius ingredients of this lane
-#pragma unroll
-    for (int mm = 0; mm < M; ++mm) radius_terms(mem[mm], rlane, hlane);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        rlane = fmaxf(rlane, __shfl_xor_sync(0xffffffffu, rlane, o));
-        hlane = fmaxf(hlane, __shfl_xor_sync(0xffffffffu, hlane, o));
+    if (w.sp == 0) {
+        const int m = min(w.gsp, 32);
+        if (lane < m) W.stack[lane] = w.spill[w.gsp - m + lane];
+        w.gsp -= m;
+        w.sp = m;
+        __syncwarp();
     }
-    // density: R_s = max_k (|m_k| + h_k); symmetric: R_g = max_k |m_k|, hmax_g
-    const float Rd2 = radius2_units(rlane);
-    const float Rg = rlane, hmax_g = hlane;
+    // take range entries from the top of the stack, up to 32 nodes
+    uint32_t ent = 0;
+    int ecnt = 0;
+    if (lane < w.sp) {
+        ent = W.stack[w.sp - 1 - lane];
+        ecnt = (int)(ent & 7u) + 1;
+    }
+    const int incl = warp_incl_scan(ecnt, lane);
+    const bool take = (lane < w.sp) && (incl <= 32);
+    const unsigned tm = __ballot_sync(0xffffffffu, take);
+    const int nent = __popc(tm);
+    const int nnodes = __shfl_sync(0xffffffffu, incl, nent - 1);
+    // node slot l belongs to the taken entry whose first slot is the highest entry
+    // start <= l (the starts as a bit mask; entries sit on lanes 0 .. nent-1)
+    const unsigned starts = __reduce_or_sync(0xffffffffu, take ? 1u << (incl - ecnt) : 0u);
+    const unsigned below = starts & ((2u << lane) - 1u);
+    const uint32_t my_ent = __shfl_sync(0xffffffffu, ent, max(__popc(below) - 1, 0));
+    w.sp -= nent;
+    const int node = lane < nnodes ? (int)(my_ent >> 3) + (lane - (31 - __clz(below))) : -1;
+    bool open = false, emit = false;
+    int4 lk = make_int4(0, 0, -1, 0);
+    int nch = 0;
+    if (node >= 0) {
+        const uint4 cen = a.ncen[node];
+        const float4 ext = a.next[node];
+        lk = a.nlink[node];
+        nch = __float_as_int(ext.w);
+        open = open_node(cen, ext);
+        emit = open && lk.y > 0 && (lk.z < 0 || lk.y <= whole);
+    }
+    lc.nodes += (lane == 0) ? nnodes : 0;
+    const unsigned em = __ballot_sync(0xffffffffu, emit);
+    if (em) {
+        const int add = emit ? lk.y : 0;
+        const int pre = warp_incl_scan(add, lane);
+        if (emit) {
+            const int start = w.total + pre - add;
+            W.ranges[(w.e1 + __popc(em & lt)) & (kRangeCap - 1)] = make_int2(lk.x - start, start);
+        }
+        w.e1 += __popc(em);
+        w.total += __shfl_sync(0xffffffffu, pre, 31);
+    }
+    const bool push = open && lk.z >= 0 && !emit;
+    const unsigned pm = __ballot_sync(0xffffffffu, push);
+    if (push) W.stack[w.sp + __popc(pm & lt)] = ((uint32_t)lk.z << 3) | (uint32_t)(nch - 1);
+    w.sp += __popc(pm);
+    lc.max_stack = max(lc.max_stack, w.sp + w.gsp);
+    __syncwarp();
+}
+
+// When the next step could push more entries than the shared part holds, the oldest (up
+// to 32, its bottom) move to the top of the overflow area, which stays below the shared
+// part, so the whole stack remains last in, first out.
+__device__ __forceinline__ void walk_spill(const SearchArgs& a, WalkSmem& W, Walk& w, int lane) {
+    if (w.sp <= a.stack_cap - 32) return;
+    const int ev = min(32, w.sp);
+    if (w.gsp + ev > kSpillCap) atomicOr(a.err, kErrStack);
+    else if (lane < ev) w.spill[w.gsp + lane] = W.stack[lane];
+    __syncwarp();
+    for (int b = 0; b < w.sp - ev; b += 32) {
+        const uint32_t v = (b + lane < w.sp - ev) ? W.stack[ev + b + lane] : 0u;
+        __syncwarp();
+        if (b + lane < w.sp - ev) W.stack[b + lane] = v;
+        __syncwarp();
+    }
+    w.gsp = min(w.gsp + ev, kSpillCap);
+    w.sp -= ev;
+}
+
+// The next up to 32 pending candidates, one per lane: returns their number and this
+// lane's rank (undefined beyond the number).  Lane l looks at range e0 + l; a window bit
+// marks where each range starts, and a lane's range is the last one starting at or
+// before it.  Only 32 ranges are looked at, so the window ends where the 33rd starts.
+__device__ __forceinline__ int walk_take(WalkSmem& W, Walk& w, int lane, int& rank) {
+    const int ne = w.e1 - w.e0;
+    int take = min(32, w.total - w.done);
+    if (ne > 32) take = min(take, W.ranges[(w.e0 + 32) & (kRangeCap - 1)].y - w.done);
+    int2 R = make_int2(0, 0x7fffffff);
+    if (lane < ne) R = W.ranges[(w.e0 + lane) & (kRangeCap - 1)];
+    const int rel = lane < ne ? R.y - w.done : 64;
+    const int first = __popc(__ballot_sync(0xffffffffu, rel <= 0)) - 1;   // the range holding candidate `done`
+    const unsigned starts = __reduce_or_sync(0xffffffffu, (rel > 0 && rel < 32) ? 1u << rel : 0u);
+    const int off = first + __popc(starts & ((2u << lane) - 1u));
+    rank = __shfl_sync(0xffffffffu, R.x, off & 31) + w.done + lane;
+    w.e0 += __popc(__ballot_sync(0xffffffffu, rel <= take)) - 1;
+    w.done += take;
+    __syncwarp();
+    return take;
+}
+
+// One search's walk from the tree rooted at `root` and the member x candidate filter of
+// every tile (the members are initialised relative to the centre C).
+//
+// A node or a candidate matters only if it lies within H of the members' box (H the
+// largest member radius; symmetric kinds: or its own h), so both are tested against the
+// box dilated by H.  The box is symmetric about C, E = max |m| per axis.  The sphere
+// around C that covers every member's sphere is up to a third larger in volume for a
+// cubic box and far larger for an elongated one.
+//
+// Bound by instruction issue (71% of issue slots, L2 hit 97%).  Of the about 900 particles
+// that the opened nodes hold (16.8M clustered particles, g = 16) fewer than half lie in
+// the dilated box: they are dropped here, at a few instructions per 32 of them, before
+// the members' filter, and only the kept ones fetch the kind's own records.  Against
+// staging every candidate of the covering sphere's leaves by bulk copies and filtering
+// them all: a timestep of 16.8M clustered particles 128.8 -> 99.0 ms, hydro of 4.2M 10.9 -> 8.5 ms.
+template <class K, int MODE>
+__device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, const Layout& L,
+                                             typename K::Member& mem, uint32_t cx, uint32_t cy, uint32_t cz, int root,
+                                             LocalCounters& lc, int lane) {
+    const uint32_t lt = (1u << lane) - 1u;
+    const float ex = warp_max(fabsf(mem.mx)), ey = warp_max(fabsf(mem.my)), ez = warp_max(fabsf(mem.mz));
+    const float H = warp_max(member_radius(mem));
+    // node test: half extents in fixed-point units, covering the FP32 error of the members'
+    // coordinates (2 ulps and the rounding of the offset)
+    const float nx = __fadd_ru(__fmul_ru(__fmul_ru(ex, 1.000001f), 4294967296.0f), 1.0f);
+    const float ny = __fadd_ru(__fmul_ru(__fmul_ru(ey, 1.000001f), 4294967296.0f), 1.0f);
+    const float nz = __fadd_ru(__fmul_ru(__fmul_ru(ez, 1.000001f), 4294967296.0f), 1.0f);
+    const float H2u = radius2_units(H);
+    // candidate test: the FP32 gap to the box is at most the FP32 distance to any member, so
+    // the decision band of that distance covers it (|m| <= |E|)
+    const float H2 = H * H;
+    const float band = 8.0f * kBandRel * fmaf(ex, ex, fmaf(ey, ey, ez * ez));
     // every relevant pair difference is already the nearest image when the group's
     // reach stays below half the box (symmetric: with the largest h of the tree)
-    const float reach = K::sym ? Rg + fmaxf(hmax_g, __uint_as_float(a.ncen[root].w)) : rlane;
+    const float emax = fmaxf(ex, fmaxf(ey, ez));
+    const float reach = emax + (K::sym ? fmaxf(H, __uint_as_float(a.ncen[root].w)) : H);
     const bool wrap_safe = reach < 0.49f;
     // the start table of the walk's tree (one per box of a forest, whose roots are the
     // first nodes)
     const int start = a.start_tab ? walk_start(a.start_tab + (size_t)root * kStartTableSize, root, cx, cy, cz, reach)
                                   : root;
-
-    // The stack lives in shared memory (at most a.stack_cap entries); when it fills up,
-    // its oldest entries move to this warp's overflow area in global memory, which holds
-    // the bottom of the stack and refills the shared part when that runs empty.
-    uint32_t* spill = a.stack_spill + (size_t)(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * kSpillCap;
-    int sp = 1, gsp = 0;
-    if (lane == 0) W.stack[0] = (uint32_t)start << 3;   // one node
-    int nr = 0, pending = 0;
-    int nf = 0;   // converted candidates held in the tile, waiting for the filter
-    __syncwarp();
+    auto open_node = [&](const uint4& cen, const float4& ext) {
+        const float gap2 = node_gap2(cen, make_float4(__fadd_ru(ext.x, nx), __fadd_ru(ext.y, ny),
+                                                      __fadd_ru(ext.z, nz), 0.0f), cx, cy, cz);
+        if constexpr (K::sym) return gap2 <= radius2_units(fmaxf(H, __uint_as_float(cen.w)));
+        else return gap2 <= H2u;
+    };
+    Walk w = walk_begin(a, W, start, lane);
+    int ns = 0;   // candidates in the tile
     for (;;) {
-        while ((sp > 0 || gsp > 0) && sp <= a.stack_cap - 32 && pending < TCAP - nf && nr <= kRangeCap - 32) {
-            if (sp == 0) {
-                const int m = min(gsp, 32);
-                if (lane < m) W.stack[lane] = spill[gsp - m + lane];
-                gsp -= m;
-                sp = m;
-                __syncwarp();
+        while (walk_can_step(a, w) && w.total - w.done < 64) walk_step(a, W, w, kWalkWhole, lc, lane, open_node);
+        walk_spill(a, W, w, lane);
+        const bool walked = w.empty();
+        // candidates by whole windows of 32 while the walk goes on
+        while (ns <= kTile - 32 && (w.total - w.done >= 32 || (walked && w.total > w.done))) {
+            int rank;
+            const int nt = walk_take(W, w, lane, rank);
+            lc.cands += (lane == 0) ? nt : 0;
+            bool in = false;
+            float px = 0.0f, py = 0.0f, pz = 0.0f, mj = 0.0f, hj2 = 0.0f;
+            if (lane < nt) {
+                const uint4 P = a.pfix[rank];
+                const float4 O = a.poff[rank];
+                px = rel_coord(P.x, O.x, cx);
+                py = rel_coord(P.y, O.y, cy);
+                pz = rel_coord(P.z, O.z, cz);
+                mj = O.w;
+                const float gx = fmaxf(fabsf(px) - ex, 0.0f), gy = fmaxf(fabsf(py) - ey, 0.0f),
+                            gz = fmaxf(fabsf(pz) - ez, 0.0f);
+                const float gap2 = fmaf(gx, gx, fmaf(gy, gy, gz * gz));
+                float lim = H2;
+                if constexpr (K::sym) {
+                    const float hj = __uint_as_float(P.w);
+                    hj2 = hj * hj;
+                    lim = fmaxf(H2, hj2);
+                }
+                in = gap2 < fmaf(lim, 1.0f + 3.0f * kBandRel, band);
             }
-            // take range entries from the top of the stack, up to 32 nodes
-            uint32_t ent = 0;
-            int ecnt = 0;
-            if (lane < sp) {
-                ent = W.stack[sp - 1 - lane];
-                ecnt = (int)(ent & 7u) + 1;
+            const unsigned im = __ballot_sync(0xffffffffu, in);
+            if (in) {
+                const int t = ns + __popc(im & lt);
+                T.p[t] = make_float4(px, py, pz, fmaf(px, px, fmaf(py, py, pz * pz)));
+                if constexpr (K::sym) T.q[t] = make_float2(hj2, mj);
+                else T.m[t] = mj;
+                T.r[t] = rank;
+                stage_records(T, a, t, rank);
             }
-            int incl = warp_incl_scan(ecnt, lane);
-            bool take = (lane < sp) && (incl <= 32);
-            unsigned tm = __ballot_sync(0xffffffffu, take);
-            int nent = __popc(tm);
-            int nnodes = __shfl_sync(0xffffffffu, incl, nent - 1);
-            // node slot l belongs to the taken entry whose first slot is the highest entry
-            // start <= l (the starts as a bit mask; entries sit on lanes 0 .. nent-1)
-            const unsigned starts = __reduce_or_sync(0xffffffffu, take ? 1u << (incl - ecnt) : 0u);
-            const unsigned below = (lane == 31) ? starts : (starts & ((2u << lane) - 1u));
-            const int e_of = max(__popc(below) - 1, 0);
-            const uint32_t my_ent = __shfl_sync(0xffffffffu, ent, e_of);
-            sp -= nent;
-            int node = lane < nnodes ? (int)(my_ent >> 3) + (lane - (31 - __clz(below))) : -1;
-            bool open = false, leaf = false;
-            int4 lk = make_int4(0, 0, -1, 0);
-            int nch = 0;
-            if (node >= 0) {
-                uint4 cen = a.ncen[node];
-                float4 ext = a.next[node];
-                lk = a.nlink[node];
-                nch = __float_as_int(ext.w);
-                float gap2 = node_gap2(cen, ext, cx, cy, cz);
-                float R2;
-                if constexpr (!K::sym) R2 = Rd2;
-                else R2 = radius2_units(Rg + fmaxf(hmax_g, __uint_as_float(cen.w)));
-                open = gap2 <= R2;
-                leaf = lk.z < 0;
-            }
-            lc.nodes += (lane == 0) ? nnodes : 0;
-            bool emit = open && leaf && lk.y > 0;
-            unsigned em = __ballot_sync(0xffffffffu, emit);
-            if (emit) {
-                int pos = nr + __popc(em & lt);
-                W.ranges[pos] = make_int2(lk.x, lk.y);
-            }
-            nr += __popc(em);
-            int add = emit ? lk.y : 0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
-            pending += add;
-            bool push = open && !leaf;
-            unsigned pm = __ballot_sync(0xffffffffu, push);
-            const int npush = __popc(pm);
-            if (push) W.stack[sp + __popc(pm & lt)] = ((uint32_t)lk.z << 3) | (uint32_t)(nch - 1);
-            sp += npush;
-            lc.max_stack = max(lc.max_stack, sp + gsp);
-            __syncwarp();
+            ns += __popc(im);
         }
-        const bool walk_done = (sp == 0 && gsp == 0);
-        if (kSup) {
-            if (nr > 0) {
-                // superset export: every pending range's particles, in walk order
-                int run = 0;
-                for (int e0 = 0; e0 < nr; e0 += 32) {
-                    const int e = e0 + lane;
-                    const int c = e < nr ? W.ranges[e].y : 0;
-                    const int inc = warp_incl_scan(c, lane);
-                    if (e < nr) W.rpre[e] = run + inc - c;
-                    run += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                __syncwarp();
-                lc.cands += (lane == 0) ? run : 0;
-                if (MODE == kSupFill) {
-                    for (int e = lane >> 4; e < nr; e += 2) {
-                        const int rb = W.rpre[e];
-                        const int2 R = W.ranges[e];
-                        for (int gt = rb + (lane & 15); gt < rb + R.y; gt += 16) {
-                            const int64_t q = sup_pos + sup_n + gt;
-                            if (q < a.x_cap) a.x_idx[q] = a.perm[R.x + (gt - rb)];
-                            else atomicOr(a.err, kErrCap);
-                        }
-                    }
-                }
-                sup_n += run;
-                nr = 0;
-                pending = 0;
-                __syncwarp();
-            }
-        } else {
-            // Stage the pending ranges from their front into the tile's free part [nf, TCAP)
-            // (what does not fit stays pending for the next tile) and filter whenever the tile
-            // is full, so that every tile but a group's last holds TCAP candidates.
-            for (;;) {
-                const int room = TCAP - nf;
-                if (!(nr > 0 && (walk_done || pending >= room || nr > kRangeCap - 32))) break;
-                const int nt = min(pending, room);
-                int run = 0;
-                for (int e0 = 0; e0 < nr; e0 += 32) {
-                    const int e = e0 + lane;
-                    const int c = e < nr ? W.ranges[e].y : 0;
-                    const int inc = warp_incl_scan(c, lane);
-                    if (e < nr) W.rpre[e] = run + inc - c;
-                    run += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                __syncwarp();
-                lc.cands += (lane == 0) ? nt : 0;
-                // bulk copies of every SoA array; ranges adjacent in memory (consecutive
-                // leaves of the walk usually are) are merged into one copy, issued by the
-                // first range of the run (or of a 32-range block)
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_expect_tx(&W.bar, (uint32_t)nt * K::bytes);
-                __syncwarp();
-                int nfull = 0;   // ranges consumed entirely by this chunk
-                for (int eb = 0; eb < nr; eb += 32) {
-                    const int e = eb + lane;
-                    int rb = 0, src = 0, dst = 0, cnt = 0;
-                    bool valid = false, cont = false;
-                    if (e < nr) {
-                        rb = W.rpre[e];
-                        valid = rb < nt;
-                    }
-                    if (valid) {
-                        const int2 R = W.ranges[e];
-                        src = R.x;
-                        dst = nf + rb;
-                        cnt = min(R.y, nt - rb);
-                        if (lane > 0) {
-                            const int2 Q = W.ranges[e - 1];
-                            cont = Q.x + Q.y == R.x;
-                        }
-                        for (int k = 0; k < cnt; ++k) T.r[dst + k] = src + k;
-                    }
-                    nfull += __popc(__ballot_sync(0xffffffffu, valid && cnt == W.ranges[e < nr ? e : 0].y));
-                    const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-                    if (vmask == 0u) break;
-                    const bool head = valid && !cont;
-                    const unsigned hmask = __ballot_sync(0xffffffffu, head);
-                    const int last = 31 - __clz(vmask);
-                    const int chunk_end = __shfl_sync(0xffffffffu, dst + cnt, last);
-                    const unsigned above = (lane == 31) ? 0u : (hmask >> (lane + 1)) << (lane + 1);
-                    const int nxt = above ? __ffs(above) - 1 : 0;
-                    const int nxt_dst = __shfl_sync(0xffffffffu, dst, nxt);
-                    if (head) {
-                        const int runlen = (above ? nxt_dst : chunk_end) - dst;
-                        stage_run(T, a, dst, src, (uint32_t)runlen * 16u, &W.bar);
-                    }
-                    if (vmask != 0xffffffffu) break;
-                }
-                // the chunk leaves the pending list: drop the consumed ranges, shorten a
-                // partly consumed one, move the rest to the front
-                {
-                    const int keep_n = nr - nfull;
-                    int2 r0 = make_int2(0, 0), r1 = make_int2(0, 0);
-                    if (lane < keep_n) r0 = W.ranges[nfull + lane];
-                    if (lane + 32 < keep_n) r1 = W.ranges[nfull + lane + 32];
-                    if (lane == 0 && keep_n > 0) {
-                        const int used = nt - W.rpre[nfull];   // > 0 only for a partly consumed range
-                        if (used > 0) { r0.x += used; r0.y -= used; }
-                    }
-                    __syncwarp();
-                    if (lane < keep_n) W.ranges[lane] = r0;
-                    if (lane + 32 < keep_n) W.ranges[lane + 32] = r1;
-                    __syncwarp();
-                    nr = keep_n;
-                    pending -= nt;
-                }
-                if (!mbar_wait_bounded(&W.bar, tma_phase, a.err)) {
-                    // The chunk never completed: nothing of it may be used, and the barrier's
-                    // phase no longer matches tma_phase.  Give the copies in flight one more
-                    // bounded wait to land in shared memory, then the warp abandons its work
-                    // (the timeout flag is set; the call reports ETIMEOUT).
-                    mbar_wait_bounded(&W.bar, tma_phase, a.err);
-                    return false;
-                }
-                tma_phase ^= 1u;
-                // in place: fixed point -> coordinates relative to the centre
-                for (int t = nf + lane; t < nf + nt; t += 32) {
-                    const uint4 P = *reinterpret_cast<const uint4*>(&T.p[t]);
-                    const float4 O = T.o[t];
-                    const float px = rel_coord(P.x, O.x, cx), py = rel_coord(P.y, O.y, cy),
-                                pz = rel_coord(P.z, O.z, cz);
-                    T.p[t] = make_float4(px, py, pz, fmaf(px, px, fmaf(py, py, pz * pz)));
-                    if constexpr (K::sym) {
-                        const float hj = __uint_as_float(P.w);
-                        T.o[t] = make_float4(hj * hj, O.w, 0.0f, 0.0f);
-                    }
-                }
-                __syncwarp();
-                nf += nt;
-                if (nf >= TCAP) {
-                    filter_staged<K, MODE, M>(T, L, mem, nf, a, lc, lane, wrap_safe);
-                    nf = 0;
-                }
-            }
-            if (walk_done && nf > 0) {
-                filter_staged<K, MODE, M>(T, L, mem, nf, a, lc, lane, wrap_safe);
-                nf = 0;
-            }
+        const bool last = walked && w.total == w.done;
+        if (ns > kTile - 32 || last) {
+            if (ns > 0) filter_staged<K, MODE>(T, L, mem, ns, a, lc, lane, wrap_safe);
+            ns = 0;
+            if (last) break;
         }
-        if (sp > a.stack_cap - 32) {
-            // the next step could push 32 entries: the oldest (up to 32, the bottom of the
-            // shared part) move to the top of the overflow area, which stays below the
-            // shared part, so the whole stack remains last in, first out
-            const int ev = min(32, sp);
-            if (gsp + ev > kSpillCap) atomicOr(a.err, kErrStack);
-            else if (lane < ev) spill[gsp + lane] = W.stack[lane];
-            __syncwarp();
-            for (int b = 0; b < sp - ev; b += 32) {
-                const uint32_t v = (b + lane < sp - ev) ? W.stack[ev + b + lane] : 0u;
-                __syncwarp();
-                if (b + lane < sp - ev) W.stack[b + lane] = v;
-                __syncwarp();
-            }
-            gsp = min(gsp + ev, kSpillCap);
-            sp -= ev;
-        }
-        if (sp == 0 && gsp == 0) break;
     }
-    return true;
 }
 
-// One work item of the grouped kernels: set-up, search, results.  Returns false if the
-// warp must stop taking work (a tile copy timed out).
-template <class K, int MODE, int M>
-__device__ __forceinline__ bool process_group(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, int gid,
-                                              LocalCounters& lc, uint32_t& tma_phase, int lane) {
-    using Member = typename K::Member;
-    constexpr bool kSup = (MODE == kSupCount || MODE == kSupFill);
-    const GroupDesc d = group_desc(a, gid);
-    const Layout L = make_layout(d.g, lane, MODE == kAcc, min(K::cap / 32, d.smax));
-    int rk[M];
-#pragma unroll
-    for (int mm = 0; mm < M; ++mm) {
-        const int k = member_of(L, lane, mm, d.g);
-        rk[mm] = (k >= 0 && k < d.cnt) ? a.U[d.base + k] : -1;
-    }
+// One part of a work item: up to 32 members U[base, base + cnt), one per lane and slice.
+template <class K, int MODE>
+__device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, int base, int cnt,
+                                             int root, int smax, LocalCounters& lc, int lane) {
+    const Layout L = make_layout(cnt, lane, MODE == kAcc, min(kTile / 32, smax));
+    const MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[base + L.k] : -1)};
     uint32_t cx = 0, cy = 0, cz = 0;
-    if (!group_centre<M>(a, rk, cx, cy, cz)) return true;
-    Member mem[M];
-#pragma unroll
-    for (int mm = 0; mm < M; ++mm) member_init(mem[mm], a, rk[mm], cx, cy, cz);
+    if (!group_centre<1>(a, rec, cx, cy, cz)) return;
+    typename K::Member mem;
+    member_init(mem, a, rec[0], cx, cy, cz);
     if constexpr (K::id == kKindDensityList) {
         // list slot = the member's index in the work list; sub-list of this lane's slice
-        static_assert(M == 1, "the recycled iteration keeps lists for one member per lane");
-        const int k = member_of(L, lane, 0, d.g);
-        if (mem[0].rank >= 0) {
-            mem[0].lsub = kListCap / L.S;
-            mem[0].lptr = a.o_list + (int64_t)(d.base + k) * kListCap + L.slice * mem[0].lsub;
+        if (mem.rank >= 0) {
+            mem.lsub = kListCap / L.S;
+            mem.lptr = a.o_list + (int64_t)(base + L.k) * kListCap + L.slice * mem.lsub;
         }
     }
-    // export: write positions of every slot
-    if (MODE == kFill) {
-#pragma unroll
-        for (int mm = 0; mm < M; ++mm)
-            if (mem[mm].rank >= 0) mem[mm].xpos = a.x_off[a.perm[mem[mm].rank]];
-    }
-    int64_t sup_pos = 0, sup_n = 0;
-    if (MODE == kSupFill) sup_pos = a.x_off[gid];
-    if (!group_search<K, MODE, M>(a, W, T, L, mem, cx, cy, cz, d.root, lc, tma_phase, lane, sup_pos, sup_n))
-        return false;
+    // export: write position of the member's neighbours
+    if (MODE == kFill && mem.rank >= 0) mem.xpos = a.x_off[a.perm[mem.rank]];
+    group_search<K, MODE>(a, W, T, L, mem, cx, cy, cz, root, lc, lane);
     // the symmetric sums count the member itself as a pair at r = 0 (once, in slice 0)
     constexpr bool kSelfPair = MODE == kAcc && (K::id == kKindHydro || K::id == kKindHydroAdj);
-#pragma unroll
-    for (int mm = 0; mm < M; ++mm)
-        lc.pairs += mem[mm].n - ((kSelfPair && L.slice == 0 && mem[mm].rank >= 0) ? 1 : 0);
-    if (kSup) {
-        if (MODE == kSupCount && lane == 0) a.x_cnt[gid] = sup_n;
-        return true;
-    }
+    lc.pairs += mem.n - ((kSelfPair && L.slice == 0 && mem.rank >= 0) ? 1 : 0);
     if constexpr (K::id == kKindDensityList) {
         // the member's slice-0 lane records its sub-list lengths, S and whether all fit
-        int cnt[4];
+        int cnt4[4];
 #pragma unroll
         for (int sl = 0; sl < 4; ++sl) {
-            const int src = L.S > 1 ? sl * d.g + (lane & (d.g - 1)) : lane;
-            const int v = __shfl_sync(0xffffffffu, mem[0].lcnt, (sl < L.S && src < 32) ? src : lane);
-            cnt[sl] = sl < L.S ? v : 0;
+            const int src = L.S > 1 ? sl * L.gw + (lane & (L.gw - 1)) : lane;
+            const int v = __shfl_sync(0xffffffffu, mem.lcnt, (sl < L.S && src < 32) ? src : lane);
+            cnt4[sl] = sl < L.S ? v : 0;
         }
-        if (L.slice == 0 && mem[0].rank >= 0) {
+        if (L.slice == 0 && mem.rank >= 0) {
             const int lsub = kListCap / L.S;
-            const bool ok = cnt[0] <= lsub && cnt[1] <= lsub && cnt[2] <= lsub && cnt[3] <= lsub;
-            const int slot = d.base + member_of(L, lane, 0, d.g);
-            a.o_lrec[slot] = make_int4(ok ? cnt[0] | (cnt[1] << 16) : 0, ok ? cnt[2] | (cnt[3] << 16) : 0, L.S,
+            const bool ok = cnt4[0] <= lsub && cnt4[1] <= lsub && cnt4[2] <= lsub && cnt4[3] <= lsub;
+            const int slot = base + L.k;
+            a.o_lrec[slot] = make_int4(ok ? cnt4[0] | (cnt4[1] << 16) : 0, ok ? cnt4[2] | (cnt4[3] << 16) : 0, L.S,
                                        ok ? 1 : 0);
-            a.o_lhw[slot] = a.h64[mem[0].rank] * a.list_widen;
-            a.o_lslot[mem[0].rank] = slot;
+            a.o_lhw[slot] = rec[0].h * a.list_widen;
+            a.o_lslot[mem.rank] = slot;
         }
     }
-    if (L.S > 1) {
-#pragma unroll
-        for (int mm = 0; mm < M; ++mm)
-            for (int o = d.g; o < 32; o <<= 1) slice_add(mem[mm], o);
-    }
-    if (L.slice == 0) {
-#pragma unroll
-        for (int mm = 0; mm < M; ++mm) {
-            if (mem[mm].rank >= 0) write_result<MODE>(mem[mm], a);
-        }
-    }
-    return true;
+    for (int o = L.gw; o < L.gw * L.S; o <<= 1) slice_add(mem, o);
+    if (L.slice == 0 && mem.rank >= 0) write_result<MODE>(mem, a);
+}
+
+// One work item of the grouped kernels.  A group of more than 32 members is searched in
+// parts of 32: one walk for all of them would pay every member a filter over the whole
+// superset (at g = 64 on 4.2M clustered particles 15.5 ms a density pass, g = 128 more;
+// in parts of 32 9.7 ms, all with the walk and staging before culling).
+template <class K, int MODE>
+__device__ __forceinline__ void process_group(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, int gid,
+                                              LocalCounters& lc, int lane) {
+    const GroupDesc d = group_desc(a, gid);
+    for (int b = 0; b < d.cnt; b += kPartMax)
+        process_part<K, MODE>(a, W, T, d.base + b, min(kPartMax, d.cnt - b), d.root, d.smax, lc, lane);
 }
 
 __device__ __forceinline__ int next_item(const SearchArgs& a, int lane) {
@@ -1711,32 +1563,28 @@ __device__ __forceinline__ int next_item(const SearchArgs& a, int lane) {
     return __shfl_sync(0xffffffffu, gid, 0);
 }
 
-template <class K, int MODE, int M>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, M == 1 ? K::min_blocks : 0)
-k_group(SearchArgs a) {
+template <class K, int MODE>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, K::min_blocks) k_group(SearchArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[wib];
     auto& T = reinterpret_cast<typename K::Tile*>(smem_raw + kWarpsPerBlock * sizeof(WalkSmem))[wib];
     LocalCounters lc;
-    uint32_t tma_phase = 0u;
-    if (lane == 0) mbar_init(&W.bar, 1u);
-    __syncwarp();
     const int ng = group_count(a);
     for (;;) {
         const int gid = next_item(a, lane);
         if (gid >= ng) break;
-        if (!process_group<K, MODE, M>(a, W, T, gid, lc, tma_phase, lane)) break;
+        process_group<K, MODE>(a, W, T, gid, lc, lane);
     }
     flush_counters(a, lc, lane);
 }
 
 // Two kinds of work item in one persistent queue: the groups of a0 (kind K0) first,
 // then those of a1 (kind K1).  Both share the work counter of a0.
-template <class K0, class K1, int M>
+template <class K0, class K1>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32,
-                                  M > 1 ? 0 : (K0::min_blocks < K1::min_blocks ? K0::min_blocks : K1::min_blocks))
+                                  K0::min_blocks < K1::min_blocks ? K0::min_blocks : K1::min_blocks)
 k_group_pair(SearchArgs a0, SearchArgs a1) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr size_t kTileBytes = sizeof(typename K0::Tile) > sizeof(typename K1::Tile) ? sizeof(typename K0::Tile)
@@ -1746,21 +1594,84 @@ k_group_pair(SearchArgs a0, SearchArgs a1) {
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[wib];
     unsigned char* tile = smem_raw + kWarpsPerBlock * sizeof(WalkSmem) + wib * kTileBytes;
     LocalCounters lc;
-    uint32_t tma_phase = 0u;
-    if (lane == 0) mbar_init(&W.bar, 1u);
-    __syncwarp();
     const int n0 = group_count(a0), n1 = group_count(a1);
     for (;;) {
         const int gid = next_item(a0, lane);
         if (gid >= n0 + n1) break;
-        const bool ok =
-            gid < n0 ? process_group<K0, kAcc, M>(a0, W, *reinterpret_cast<typename K0::Tile*>(tile), gid, lc,
-                                                  tma_phase, lane)
-                     : process_group<K1, kAcc, M>(a1, W, *reinterpret_cast<typename K1::Tile*>(tile), gid - n0, lc,
-                                                  tma_phase, lane);
-        if (!ok) break;
+        if (gid < n0)
+            process_group<K0, kAcc>(a0, W, *reinterpret_cast<typename K0::Tile*>(tile), gid, lc, lane);
+        else
+            process_group<K1, kAcc>(a1, W, *reinterpret_cast<typename K1::Tile*>(tile), gid - n0, lc, lane);
     }
     flush_counters(a0, lc, lane);
+}
+
+// The candidate superset of every group (inspection): the particles of the leaves that
+// meet the sphere around the group centre covering every member's sphere, in walk order.
+// Up to kSupSlots members per lane, one walk for the whole group.  FILL writes the
+// candidates at x_off[group], else they are counted.
+constexpr int kSupSlots = 4;
+
+template <bool SYM, bool FILL>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32) k_superset(SearchArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31;
+    WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[threadIdx.x >> 5];
+    LocalCounters lc;
+    const int ng = group_count(a);
+    for (;;) {
+        const int gid = next_item(a, lane);
+        if (gid >= ng) break;
+        const GroupDesc d = group_desc(a, gid);
+        MemberRec rec[kSupSlots];
+#pragma unroll
+        for (int mm = 0; mm < kSupSlots; ++mm) {
+            const int k = lane + 32 * mm;
+            rec[mm] = load_member(a, k < d.cnt ? a.U[d.base + k] : -1);
+        }
+        uint32_t cx = 0, cy = 0, cz = 0;
+        if (!group_centre<kSupSlots>(a, rec, cx, cy, cz)) continue;
+        // density: R_s = max_k (|m_k| + h_k); hydro: R_g = max_k |m_k|, hmax_g
+        float rlane = 0.0f, hlane = 0.0f;
+#pragma unroll
+        for (int mm = 0; mm < kSupSlots; ++mm) {
+            if (rec[mm].rank < 0) continue;
+            const float mx = rel_coord(rec[mm].P.x, rec[mm].O.x, cx), my = rel_coord(rec[mm].P.y, rec[mm].O.y, cy),
+                        mz = rel_coord(rec[mm].P.z, rec[mm].O.z, cz);
+            const float mr = sqrtf(mx * mx + my * my + mz * mz);
+            const float hf = (float)rec[mm].h;
+            rlane = fmaxf(rlane, SYM ? mr : mr + 1.0f / (1.0f / hf));
+            hlane = fmaxf(hlane, hf);
+        }
+        const float R = warp_max(rlane), hmax_g = warp_max(hlane);
+        const float R2d = radius2_units(R);
+        const float reach = SYM ? R + fmaxf(hmax_g, __uint_as_float(a.ncen[d.root].w)) : R;
+        const int start = a.start_tab ? walk_start(a.start_tab + (size_t)d.root * kStartTableSize, d.root, cx, cy, cz,
+                                                   reach)
+                                      : d.root;
+        auto open_node = [&](const uint4& cen, const float4& ext) {
+            const float R2 = SYM ? radius2_units(R + fmaxf(hmax_g, __uint_as_float(cen.w))) : R2d;
+            return node_gap2(cen, ext, cx, cy, cz) <= R2;
+        };
+        Walk w = walk_begin(a, W, start, lane);
+        const int64_t pos = FILL ? a.x_off[gid] : 0;
+        while (!w.empty() || w.total > w.done) {
+            while (walk_can_step(a, w)) walk_step(a, W, w, 0, lc, lane, open_node);
+            walk_spill(a, W, w, lane);
+            while (w.total > w.done) {
+                const int64_t at = pos + w.done;
+                int rank;
+                const int nt = walk_take(W, w, lane, rank);
+                if (FILL && lane < nt) {
+                    if (at + lane < a.x_cap) a.x_idx[at + lane] = a.perm[rank];
+                    else atomicOr(a.err, kErrCap);
+                }
+            }
+        }
+        lc.cands += (lane == 0) ? w.total : 0;
+        if (!FILL && lane == 0) a.x_cnt[gid] = w.total;
+    }
+    flush_counters(a, lc, lane);
 }
 
 // Density with the smoothing-length iteration inside the group (no host loop, no
@@ -1812,62 +1723,36 @@ __device__ __forceinline__ bool hsml_step(const SearchArgs& a, const IterArgs& i
     return false;
 }
 
-template <int M>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, M == 1 ? 6 : 0)
-k_group_dens_iter(SearchArgs a, IterArgs it) {
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(SearchArgs a, IterArgs it) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[wib];
-    DensTile& T = reinterpret_cast<DensTile*>(smem_raw + kWarpsPerBlock * sizeof(WalkSmem))[wib];
+    PlainTile& T = reinterpret_cast<PlainTile*>(smem_raw + kWarpsPerBlock * sizeof(WalkSmem))[wib];
     LocalCounters lc;
-    uint32_t tma_phase = 0u;
-    if (lane == 0) mbar_init(&W.bar, 1u);
-    __syncwarp();
     const int ng = group_count(a);
-    bool alive = true;
-    while (alive) {
+    for (;;) {
         const int gid = next_item(a, lane);
         if (gid >= ng) break;
         const GroupDesc d = group_desc(a, gid);
-        const Layout L = make_layout(d.g, lane, true, min(kTileD / 32, d.smax));
-        int rk[M];
-        double hc[M], lo[M], hi[M];
-#pragma unroll
-        for (int mm = 0; mm < M; ++mm) {
-            const int k = member_of(L, lane, mm, d.g);
-            rk[mm] = (k >= 0 && k < d.cnt) ? a.U[d.base + k] : -1;
-            hc[mm] = rk[mm] >= 0 ? a.h64[rk[mm]] : 1.0;
-            lo[mm] = 0.0;
-            hi[mm] = __longlong_as_double(0x7ff0000000000000ll);
-        }
-        for (int pass = 1;; ++pass) {
-            uint32_t cx = 0, cy = 0, cz = 0;
-            if (!group_centre<M>(a, rk, cx, cy, cz)) break;
-            DMember mem[M];
-#pragma unroll
-            for (int mm = 0; mm < M; ++mm) member_init(mem[mm], a, rk[mm], cx, cy, cz);
-            int64_t sup_n = 0;
-            if (!group_search<KDens, kAcc, M>(a, W, T, L, mem, cx, cy, cz, d.root, lc, tma_phase, lane, 0, sup_n)) {
-                alive = false;
-                break;
+        for (int b = 0; b < d.cnt; b += kPartMax) {
+            const Layout L = make_layout(min(kPartMax, d.cnt - b), lane, true, min(kTile / 32, d.smax));
+            MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[d.base + b + L.k] : -1)};
+            double lo = 0.0, hi = __longlong_as_double(0x7ff0000000000000ll);
+            for (int pass = 1;; ++pass) {
+                uint32_t cx = 0, cy = 0, cz = 0;
+                if (!group_centre<1>(a, rec, cx, cy, cz)) break;
+                DMember mem;
+                member_init(mem, a, rec[0], cx, cy, cz);
+                group_search<KDens, kAcc>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
+                lc.pairs += mem.n;
+                for (int o = L.gw; o < L.gw * L.S; o <<= 1) slice_add(mem, o);
+                if (rec[0].rank >= 0 && hsml_step(a, it, rec[0].rank, rec[0].h, lo, hi, mem.s0 - mem.c0,
+                                                  mem.s1 - mem.c1, mem.n, pass, L.slice == 0))
+                    rec[0].rank = -1;
+                // the new h (global memory) is read by the next pass's FP64 re-tests
+                __syncwarp();
             }
-#pragma unroll
-            for (int mm = 0; mm < M; ++mm) lc.pairs += mem[mm].n;
-            if (L.S > 1) {
-#pragma unroll
-                for (int mm = 0; mm < M; ++mm)
-                    for (int o = d.g; o < 32; o <<= 1) slice_add(mem[mm], o);
-            }
-#pragma unroll
-            for (int mm = 0; mm < M; ++mm) {
-                if (rk[mm] >= 0 &&
-                    hsml_step(a, it, rk[mm], hc[mm], lo[mm], hi[mm], mem[mm].s0 - mem[mm].c0, mem[mm].s1 - mem[mm].c1,
-                              mem[mm].n, pass, L.slice == 0))
-                    rk[mm] = -1;
-            }
-            // the new h (global memory) is read by the next pass's FP64 re-tests
-            __syncwarp();
         }
     }
     flush_counters(a, lc, lane);
@@ -1884,17 +1769,17 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u < a.nu) {
         const int rank = a.U[u];
-        uint4 P = a.pfix[rank];
-        const uint32_t cx = P.x, cy = P.y, cz = P.z;
+        const MemberRec rec = load_member(a, rank);
+        const uint32_t cx = rec.P.x, cy = rec.P.y, cz = rec.P.z;
         DMember dm;
         HMember hm;
         float Rbox;
         if (KIND == 0) {
-            member_init(dm, a, rank, cx, cy, cz);
-            Rbox = (float)a.h64[rank];
+            member_init(dm, a, rec, cx, cy, cz);
+            Rbox = (float)rec.h;
             if (MODE == kFill) dm.xpos = a.x_off[a.perm[rank]];
         } else {
-            member_init(hm, a, rank, cx, cy, cz);
+            member_init(hm, a, rec, cx, cy, cz);
             Rbox = hm.h;
             if (MODE == kFill) hm.xpos = a.x_off[a.perm[rank]];
         }
@@ -1925,7 +1810,7 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                             float thr = fmaf(fmaxf(hm.h2, hj * hj), 1.0f + 3.0f * kBandRel, hm.bk);
                             if (r2 < thr) {
                                 float4 H0 = a.hyd0[q], H1 = a.hyd1[q];
-                                hydro_pair<MODE>(hm, a, rel, make_float4(hj * hj, O.w, 0.0f, 0.0f), H0, H1, q, lc);
+                                hydro_pair<MODE>(hm, a, rel, make_float2(hj * hj, O.w), H0, H1, q, lc);
                             }
                         }
                     }
@@ -2116,91 +2001,71 @@ static int launch_persistent(Kern kern, bool& configured, size_t sh, int64_t ngr
     return check_cuda(cudaGetLastError(), what);
 }
 
-template <class K, int MODE, int M>
-static int launch_group_t(const SearchArgs& a, int sm_count, cudaStream_t s) {
+template <class K, int MODE>
+static int launch_group(const SearchArgs& a, int sm_count, cudaStream_t s) {
     static bool configured = false;
-    return launch_persistent(k_group<K, MODE, M>, configured, group_smem<K>(), a.ngroups_dev ? -1 : a.ngroups,
-                             sm_count, s, "grouped search kernel", a);
+    if (a.g > 128) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
+    return launch_persistent(k_group<K, MODE>, configured, group_smem<K>(), a.ngroups_dev ? -1 : a.ngroups, sm_count,
+                             s, "grouped search kernel", a);
 }
 
-template <class K, int MODE>
-static int launch_group_m(const SearchArgs& a, int sm_count, cudaStream_t s) {
-    int M = (a.g + 31) / 32;
-    if (M <= 1) return launch_group_t<K, MODE, 1>(a, sm_count, s);
-    if (M <= 2) return launch_group_t<K, MODE, 2>(a, sm_count, s);
-    if (M <= 4) return launch_group_t<K, MODE, 4>(a, sm_count, s);
-    return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
+template <bool SYM, bool FILL>
+static int launch_superset(const SearchArgs& a, int sm_count, cudaStream_t s) {
+    static bool configured = false;
+    if (a.g > 32 * kSupSlots) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
+    return launch_persistent(k_superset<SYM, FILL>, configured, kWarpsPerBlock * sizeof(WalkSmem), a.ngroups, sm_count,
+                             s, "superset kernel", a);
 }
 
 template <class K>
 static int launch_group_k(const SearchArgs& a, int mode, int sm_count, cudaStream_t s) {
     switch (mode) {
-        case kAcc: return launch_group_m<K, kAcc>(a, sm_count, s);
-        case kCount: return launch_group_m<K, kCount>(a, sm_count, s);
-        case kFill: return launch_group_m<K, kFill>(a, sm_count, s);
-        case kSupCount: return launch_group_m<K, kSupCount>(a, sm_count, s);
-        case kSupFill: return launch_group_m<K, kSupFill>(a, sm_count, s);
+        case kAcc: return launch_group<K, kAcc>(a, sm_count, s);
+        case kCount: return launch_group<K, kCount>(a, sm_count, s);
+        case kFill: return launch_group<K, kFill>(a, sm_count, s);
+        case kSupCount: return launch_superset<K::sym, false>(a, sm_count, s);
+        case kSupFill: return launch_superset<K::sym, true>(a, sm_count, s);
     }
     return set_error(SPHGRP_EINVAL, "bad search mode");
 }
-
-static int members_per_lane(int max_g) { return max_g <= 32 ? 1 : (max_g <= 64 ? 2 : 4); }
 
 int launch_search_dev(const SearchArgs& a, int kind, int max_g, int sm_count, cudaStream_t s) {
     if (max_g < 1 || max_g > 128) return set_error(SPHGRP_EINVAL, "group size outside [1, 128]");
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     SearchArgs b = a;
-    b.g = max_g;   // selects the member slots per lane; groups4 carries every group's size
+    b.g = max_g;   // bound only; groups4 carries every group's size
     switch (kind) {
-        case kKindDensity: return launch_group_m<KDens, kAcc>(b, sm_count, s);
-        case kKindHydro: return launch_group_m<KHydro, kAcc>(b, sm_count, s);
-        case kKindHydroAdj: return launch_group_m<KHAdj, kAcc>(b, sm_count, s);
-        case kKindDensityAdj: return launch_group_m<KDAdj, kAcc>(b, sm_count, s);
+        case kKindDensity:
+            return b.o_s2 ? launch_group<KDens2, kAcc>(b, sm_count, s) : launch_group<KDens, kAcc>(b, sm_count, s);
+        case kKindHydro: return launch_group<KHydro, kAcc>(b, sm_count, s);
+        case kKindHydroAdj: return launch_group<KHAdj, kAcc>(b, sm_count, s);
+        case kKindDensityAdj: return launch_group<KDAdj, kAcc>(b, sm_count, s);
     }
     return set_error(SPHGRP_EINVAL, "bad kind");
-}
-
-template <int M>
-static int launch_iter_t(const SearchArgs& a, const IterArgs& it, int sm_count, cudaStream_t s) {
-    static bool configured = false;
-    return launch_persistent(k_group_dens_iter<M>, configured, group_smem<KDens>(), a.ngroups_dev ? -1 : a.ngroups,
-                             sm_count, s, "grouped density iteration kernel", a, it);
 }
 
 int launch_density_iter(const SearchArgs& a, const IterArgs& it, int max_g, int sm_count, cudaStream_t s) {
     if (max_g < 1 || max_g > 128) return set_error(SPHGRP_EINVAL, "group size outside [1, 128]");
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
-    switch (members_per_lane(max_g)) {
-        case 1: return launch_iter_t<1>(a, it, sm_count, s);
-        case 2: return launch_iter_t<2>(a, it, sm_count, s);
-        default: return launch_iter_t<4>(a, it, sm_count, s);
-    }
+    static bool configured = false;
+    return launch_persistent(k_group_dens_iter, configured, group_smem<KDens>(), a.ngroups_dev ? -1 : a.ngroups,
+                             sm_count, s, "grouped density iteration kernel", a, it);
 }
 
-template <class K0, class K1, int M>
-static int launch_pair_t(const SearchArgs& a0, const SearchArgs& a1, int sm_count, cudaStream_t s) {
+template <class K0, class K1>
+static int launch_pair(const SearchArgs& a0, const SearchArgs& a1, int sm_count, cudaStream_t s) {
     static bool configured = false;
     constexpr size_t tile = sizeof(typename K0::Tile) > sizeof(typename K1::Tile) ? sizeof(typename K0::Tile)
                                                                                   : sizeof(typename K1::Tile);
     const size_t sh = kWarpsPerBlock * (sizeof(WalkSmem) + tile);
-    return launch_persistent(k_group_pair<K0, K1, M>, configured, sh, -1, sm_count, s, "paired search kernel", a0,
-                             a1);
-}
-
-template <class K0, class K1>
-static int launch_pair_m(const SearchArgs& a0, const SearchArgs& a1, int max_g, int sm_count, cudaStream_t s) {
-    switch (members_per_lane(max_g)) {
-        case 1: return launch_pair_t<K0, K1, 1>(a0, a1, sm_count, s);
-        case 2: return launch_pair_t<K0, K1, 2>(a0, a1, sm_count, s);
-        default: return launch_pair_t<K0, K1, 4>(a0, a1, sm_count, s);
-    }
+    return launch_persistent(k_group_pair<K0, K1>, configured, sh, -1, sm_count, s, "paired search kernel", a0, a1);
 }
 
 int launch_search_pair(const SearchArgs& a0, int kind0, const SearchArgs& a1, int kind1, int max_g, int sm_count,
                        cudaStream_t s) {
     if (max_g < 1 || max_g > 128) return set_error(SPHGRP_EINVAL, "group size outside [1, 128]");
     cudaMemsetAsync(a0.work, 0, sizeof(int), s);
-    if (kind0 == kKindHydro && kind1 == kKindHydroAdj) return launch_pair_m<KHydro, KHAdj>(a0, a1, max_g, sm_count, s);
+    if (kind0 == kKindHydro && kind1 == kKindHydroAdj) return launch_pair<KHydro, KHAdj>(a0, a1, sm_count, s);
     return set_error(SPHGRP_EINVAL, "unsupported kind pair");
 }
 
@@ -2209,24 +2074,26 @@ int launch_search(const SearchArgs& a, int kind, int mode, bool grouped, int sm_
     if (grouped) {
         cudaMemsetAsync(a.work, 0, sizeof(int), s);
         switch (kind) {
-            case 0: return launch_group_k<KDens>(a, mode, sm_count, s);
+            case 0:
+                if (mode == kAcc && a.o_s2) return launch_group<KDens2, kAcc>(a, sm_count, s);
+                return launch_group_k<KDens>(a, mode, sm_count, s);
             case 1: return launch_group_k<KHydro>(a, mode, sm_count, s);
             case 2:
                 if (mode != kAcc) return set_error(SPHGRP_EINVAL, "adjoint kernels accumulate only");
-                return launch_group_m<KHAdj, kAcc>(a, sm_count, s);
+                return launch_group<KHAdj, kAcc>(a, sm_count, s);
             case 3:
                 if (mode != kAcc) return set_error(SPHGRP_EINVAL, "adjoint kernels accumulate only");
-                return launch_group_m<KDAdj, kAcc>(a, sm_count, s);
+                return launch_group<KDAdj, kAcc>(a, sm_count, s);
             case kKindVelocity:
                 if (mode != kAcc) return set_error(SPHGRP_EINVAL, "the velocity derivatives accumulate only");
-                return launch_group_m<KVel, kAcc>(a, sm_count, s);
+                return launch_group<KVel, kAcc>(a, sm_count, s);
             case kKindDensityVel:
                 if (mode != kAcc) return set_error(SPHGRP_EINVAL, "velocity derivatives accumulate only");
-                return launch_group_m<KDensVel, kAcc>(a, sm_count, s);
+                return launch_group<KDensVel, kAcc>(a, sm_count, s);
             case kKindDensityList:
                 if (mode != kAcc || a.g > 32)
                     return set_error(SPHGRP_EINVAL, "candidate lists: accumulation, group size <= 32");
-                return launch_group_t<KDensList, kAcc, 1>(a, sm_count, s);
+                return launch_group<KDensList, kAcc>(a, sm_count, s);
         }
         return set_error(SPHGRP_EINVAL, "bad kind");
     }
