@@ -29,7 +29,7 @@ constexpr int kWarpsPerBlock = 4;
 constexpr int kStackCap = kStackSharedMax;     // walk stack entries in shared memory
 constexpr int kRangeCap = 64;                  // pending particle ranges (ring, power of two)
 constexpr int kSpillCap = kStackSpillPerWarp;  // overflow entries per warp (global memory)
-constexpr int kTile = 128;                     // candidates of a tile
+constexpr int kTile = 128;                     // candidates of a tile (192: 1-9% slower, fewer warps fit)
 constexpr int kPartMax = 32;                   // members searched at once (one per lane)
 // The walk takes a node of at most this many particles whole instead of opening it.
 constexpr int kWalkWhole = 32;
@@ -114,6 +114,34 @@ __device__ __forceinline__ float rel_diff(float p, float m) {
 // dW/dr = kSkernel h^-4 dw/dq for the M4 spline W = 8 / (pi h^3) w(r / h)
 constexpr float kSkernel = 2.54647908947032537f;   // 8 / pi
 
+// hardware reciprocal square root and reciprocal (1 ulp; arguments of normal size)
+__device__ __forceinline__ float rsqrt_fast(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_fast(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// M4 slope w'(q) (zero for q >= 1; q >= 0)
+__device__ __forceinline__ float m4_slope(float q) {
+    const float u = __saturatef(1.0f - q);
+    return q <= 0.5f ? q * fmaf(18.0f, q, -12.0f) : -6.0f * u * u;
+}
+
+// w(q) and 3 w + q w' of the M4 spline (zero for q >= 1; q >= 0): inside 1/2
+// 1 + q^2 (6q - 6) and 3 + q^2 (36q - 30), outside 2 u^3 and 6 u^2 (1 - 2q), u = 1 - q
+__device__ __forceinline__ void m4_density(float q, float& w, float& v) {
+    const float u = __saturatef(1.0f - q);
+    const float q2 = q * q, u2 = u * u;
+    const bool inner = q <= 0.5f;
+    w = inner ? fmaf(q2, fmaf(6.0f, q, -6.0f), 1.0f) : 2.0f * u2 * u;
+    v = inner ? fmaf(q2, fmaf(36.0f, q, -30.0f), 3.0f) : 6.0f * u2 * fmaf(-2.0f, q, 1.0f);
+}
+
 // M4 shape w(q), w'(q), w''(q) (zero for q >= 1)
 __device__ __forceinline__ void m4_shape2(float q, float& w, float& dw, float& d2w) {
     float u = 1.0f - q;
@@ -132,6 +160,26 @@ __device__ __forceinline__ void copy16_async(float4* dst, const float4* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
+
+// packed FP32 pairs (two FMAs in one issue slot)
+__device__ __forceinline__ unsigned long long pair_of(float lo, float hi) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ unsigned long long fma_pair(unsigned long long a, unsigned long long b,
+                                                       unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add_pair(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// m shifted left by one, the sign of v entering at the bottom
+__device__ __forceinline__ uint32_t push_sign(uint32_t m, uint32_t v) { return __funnelshift_l(v, m, 1); }
 
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -431,23 +479,36 @@ __device__ __forceinline__ float member_radius(const SymMember& M) { return M.ra
 // ---------------------------------------------------------------------------------
 // Candidate tiles in shared memory: the candidates of a group that passed the test
 // against its dilated box, in walk order, as FP32 coordinates relative to the group
-// centre {px, py, pz, |p|^2}, with their mass (symmetric kinds: and h^2), rank and the
-// kind's own records.  With S slices the lane of slice s filters positions s, s + S,
-// s + 2S, ...; positions beyond the tile's candidates, up to whole chunks of 32 per
-// slice, hold NaN dummies.
+// centre, packed in pairs, with their mass (symmetric kinds: and h^2), rank and the
+// kind's own records.  With S slices the lane of slice s filters the pairs s, s + S,
+// s + 2S, ...  Phase A reads whole rows of pairs past the last candidate (up to 64 pairs,
+// into the arrays behind b) and drops their bits.
 // ---------------------------------------------------------------------------------
 
 struct PlainTile {
-    float4 p[kTile];        // {px, py, pz, |p|^2}
+    float4 a[kTile / 2];    // {x0, x1, y0, y1}
+    float4 b[kTile / 2];    // {z0, z1, w0, w1}, w = |p|^2
     float m[kTile];
     int r[kTile];           // ranks
-    uint32_t masks[kTile];  // phase-A bit masks [chunk][lane]
+    uint32_t masks[kTile];  // phase-A bit masks [word][lane]
+
+    __device__ __forceinline__ void put(int t, float x, float y, float z) {
+        const int o = 4 * (t >> 1) + (t & 1);
+        float* pa = reinterpret_cast<float*>(a);
+        float* pb = reinterpret_cast<float*>(b);
+        pa[o] = x;
+        pa[o + 2] = y;
+        pb[o] = z;
+        pb[o + 2] = fmaf(x, x, fmaf(y, y, z * z));
+    }
+    __device__ __forceinline__ float3 pos(int t) const {
+        const int o = 4 * (t >> 1) + (t & 1);
+        const float* pa = reinterpret_cast<const float*>(a);
+        return make_float3(pa[o], pa[o + 2], reinterpret_cast<const float*>(b)[o]);
+    }
 };
-struct SymTile {
-    float4 p[kTile];
-    float2 q[kTile];        // {h_j^2, m_j}
-    int r[kTile];
-    uint32_t masks[kTile];
+struct SymTile : PlainTile {
+    float h2[kTile];        // h_j^2
 };
 struct VelTile : PlainTile {
     float4 v[kTile];        // hyd0 {vx, vy, vz, -}
@@ -603,10 +664,10 @@ __device__ __forceinline__ void precise_diff(const Mem& M, const SearchArgs& a, 
 
 // density terms of a neighbour at q = r / h
 __device__ __forceinline__ void density_terms(DMember& M, float mj, float q) {
-    float w, dw;
-    m4_shape(q, w, dw);
+    float w, v;
+    m4_density(q, w, v);
     M.p0 = fmaf(mj, w, M.p0);
-    M.p1 = fmaf(mj, fmaf(q, dw, 3.0f * w), M.p1);
+    M.p1 = fmaf(mj, v, M.p1);
 }
 __device__ __forceinline__ void density_terms(D2Member& M, float mj, float q) {
     float w, dw, d2w;
@@ -618,7 +679,7 @@ __device__ __forceinline__ void density_terms(D2Member& M, float mj, float q) {
 
 // density pair: p = candidate's coordinates relative to the member's centre, m_j its mass
 template <int MODE, bool WRAP = false, class Mem>
-__device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float4 p, float mj, int crank,
+__device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float3 p, float mj, int crank,
                                              LocalCounters& lc) {
     float dx = rel_diff<WRAP>(p.x, M.mx), dy = rel_diff<WRAP>(p.y, M.my), dz = rel_diff<WRAP>(p.z, M.mz);
     float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -634,7 +695,7 @@ __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float4
     M.n++;
     if (MODE == kAcc) {
         if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
-        float q = r2 * rsqrtf(fmaxf(r2, 1.0e-30f)) * M.hinv;
+        float q = r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)) * M.hinv;
         density_terms(M, mj, q);
     } else if (MODE == kFill) {
         int64_t q = M.xpos++;
@@ -647,7 +708,7 @@ __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float4
 // density_pair, then (for pairs at r > 0) the divergence and curl terms with
 // grad_i W = W'(r, h_i) (x_i - x_j) / r and v_ij = v_i - v_j
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, float4 p, float mj, float4 vj,
+__device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, float3 p, float mj, float4 vj,
                                              int crank, LocalCounters& lc) {
     const int n0 = M.n;
     density_pair<MODE, WRAP>(static_cast<DMember&>(M), a, p, mj, crank, lc);
@@ -662,9 +723,8 @@ __device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, f
         r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
     }
     if (r2 == 0.0f) return;
-    const float rinv = rsqrtf(r2);
-    float w, dw;
-    m4_shape(r2 * rinv * M.hinv, w, dw);
+    const float rinv = rsqrt_fast(r2);
+    const float dw = m4_slope(r2 * rinv * M.hinv);
     const float c = -M.sk * dw * rinv;   // x_i - x_j = -d
     const float gx = c * dx, gy = c * dy, gz = c * dz;
     const float vx = M.vx - vj.x, vy = M.vy - vj.y, vz = M.vz - vj.z;
@@ -677,7 +737,7 @@ __device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, f
 // density pair of the recycled iteration: a candidate inside the widened threshold joins
 // the member's sub-list, then the pair enters the sums at h as in density_pair
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void density_list_pair(DLMember& M, const SearchArgs& a, float4 p, float mj, int crank,
+__device__ __forceinline__ void density_list_pair(DLMember& M, const SearchArgs& a, float3 p, float mj, int crank,
                                                   LocalCounters& lc) {
     const float dx = rel_diff<WRAP>(p.x, M.mx), dy = rel_diff<WRAP>(p.y, M.my), dz = rel_diff<WRAP>(p.z, M.mz);
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -691,7 +751,7 @@ __device__ __forceinline__ void density_list_pair(DLMember& M, const SearchArgs&
 // velocity-derivative pair (density criterion): p = relative coordinates, mj the mass,
 // vj = {vx, vy, vz, -}
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float4 p, float mj, float4 vj, int crank,
+__device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float3 p, float mj, float4 vj, int crank,
                                          LocalCounters& lc) {
     float dx = rel_diff<WRAP>(p.x, M.mx), dy = rel_diff<WRAP>(p.y, M.my), dz = rel_diff<WRAP>(p.z, M.mz);
     float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -708,9 +768,8 @@ __device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float4
     if (MODE != kAcc) return;
     if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
     if (r2 == 0.0f) return;   // the particle itself (and coincident ones): grad W = 0
-    const float rinv = rsqrtf(r2);
-    float w, dw;
-    m4_shape(r2 * rinv * M.hinv, w, dw);
+    const float rinv = rsqrt_fast(r2);
+    const float dw = m4_slope(r2 * rinv * M.hinv);
     const float c = -M.sk * dw * rinv;   // grad_i W = W' (x_i - x_j) / r, x_i - x_j = -d
     const float gx = c * dx, gy = c * dy, gz = c * dz;
     const float vx = M.vx - vj.x, vy = M.vy - vj.y, vz = M.vz - vj.z;
@@ -722,7 +781,7 @@ __device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float4
 
 // decision of the symmetric criterion |r| < max(h_i, h_j) with the FP64 band re-test
 template <bool WRAP, class Mem>
-__device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, float4 p, float hj2, int crank,
+__device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, float3 p, float hj2, int crank,
                                            LocalCounters& lc, float& dx, float& dy, float& dz, float& r2) {
     dx = rel_diff<WRAP>(p.x, M.mx);
     dy = rel_diff<WRAP>(p.y, M.my);
@@ -743,7 +802,7 @@ __device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, fl
 // hydro pair: p = relative coordinates, q = {h_j^2, m_j}, v = {vx, vy, vz, c_j},
 // hh = {A_j, rho_j, 1/h_j, limiter_j}
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float4 p, float2 q,
+__device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float3 p, float2 q,
                                            float4 v, float4 hh, int crank, LocalCounters& lc) {
     // The member itself is a candidate: the exports skip it by rank; the sums skip it
     // as a pair at r = 0 (counted, then taken off the neighbour count at the end).
@@ -760,11 +819,9 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
     if (MODE != kAcc) return;
     if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
     if (r2 == 0.0f) return;  // coincident: the kernel gradient vanishes
-    float rinv = rsqrtf(r2);
+    float rinv = rsqrt_fast(r2);
     float r = r2 * rinv;
-    float wi, dwi, wj, dwj;
-    m4_shape(r * M.hinv, wi, dwi);
-    m4_shape(r * hh.z, wj, dwj);
+    const float dwi = m4_slope(r * M.hinv), dwj = m4_slope(r * hh.z);
     float dWi = M.sk * dwi;
     float dWj = kSkernel * (hh.z * hh.z) * (hh.z * hh.z) * dwj;
     float rx = -dx, ry = -dy, rz = -dz;  // r_ij = x_i - x_j
@@ -773,11 +830,11 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
     float visc = 0.0f;
     if (vr < 0.0f) {
         float hb = 0.5f * fmaf(q.x, hh.z, M.h);
-        float mu = hb * vr * __frcp_rn(fmaf(a.eps * hb, hb, r2));
+        float mu = hb * vr * rcp_fast(fmaf(a.eps * hb, hb, r2));
         float cb = 0.5f * (M.cs + v.w);
         // Pi = (-alpha cbar mu + beta mu^2) / rhobar, rhobar = (rho_i + rho_j) / 2, scaled by
         // the pair mean of the limiter (1 for the plain viscosity)
-        visc = 2.0f * fmaf(-a.alpha * cb, mu, a.beta * mu * mu) * __frcp_rn(M.rho + hh.y);
+        visc = 2.0f * fmaf(-a.alpha * cb, mu, a.beta * mu * mu) * rcp_fast(M.rho + hh.y);
         visc *= 0.5f * (M.fb + hh.w);
     }
     float gbar = 0.5f * (dWi + dWj);
@@ -794,7 +851,7 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
 // Q = rhat . (m_j w_k - m_k w_j), rhat = (x_k - x_j) / r.  Accumulated: dE/d of x_k,
 // v_k, m_k, h_k, rho_k (through the viscosity) and A_k.
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a, float4 p, float2 q, float4 v,
+__device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a, float3 p, float2 q, float4 v,
                                                float4 hh, float4 wj, int crank, LocalCounters& lc) {
     // the member itself enters as a pair at r = 0, which contributes nothing
     float dx, dy, dz, r2;
@@ -803,7 +860,7 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     if (MODE != kAcc) return;
     if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
     if (r2 == 0.0f) return;
-    const float rinv = rsqrtf(r2);
+    const float rinv = rsqrt_fast(r2);
     const float r = r2 * rinv;
     const float D0 = -dx, D1 = -dy, D2 = -dz;   // x_k - x_j
     const float e0 = D0 * rinv, e1 = D1 * rinv, e2 = D2 * rinv;
@@ -818,8 +875,8 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     const float vr = fmaf(v0, D0, fmaf(v1, D1, v2 * D2));
     const float hbar = 0.5f * fmaf(q.x, hh.z, M.h);
     const float Dn = fmaf(a.eps * hbar, hbar, r2);
-    const float iDn = __frcp_rn(Dn);
-    const float irbar = 2.0f * __frcp_rn(M.rho + hh.y);   // 1 / rhobar
+    const float iDn = rcp_fast(Dn);
+    const float irbar = 2.0f * rcp_fast(M.rho + hh.y);   // 1 / rhobar
     float Pi = 0.0f, Pmu = 0.0f;
     if (vr < 0.0f) {
         const float cbar = 0.5f * (M.cs + v.w);
@@ -869,7 +926,7 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
 // rho_k's own sum (x_k moves every pair) and the sums of every j with k in N_j (x_k and
 // m_k enter as a neighbour).  q = {h_j^2, m_j}, d = {alpha_j, beta_j, 1/h_j, s_j}.
 template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, float4 p, float2 q, float4 d,
+__device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, float3 p, float2 q, float4 d,
                                               int crank, LocalCounters& lc) {
     // The member itself enters as a pair at r = 0 like any coincident neighbour:
     // alpha W(0, h) + beta W_h(0, h) = alpha s h - 3 beta s, and no position term.
@@ -878,7 +935,7 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
     M.n++;
     if (MODE != kAcc) return;
     if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
-    const float rinv = r2 > 0.0f ? rsqrtf(r2) : 0.0f;
+    const float rinv = r2 > 0.0f ? rsqrt_fast(r2) : 0.0f;
     const float r = r2 * rinv;
     float wk_, dwk, d2wk, wj_, dwj, d2wj;
     const float qk = r * M.hinv, qj = r * d.z;
@@ -902,93 +959,102 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DMember& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.r[j], lc);
+    density_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(D2Member& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.r[j], lc);
+    density_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DVMember& M, const SearchArgs& a, const VelTile& T, int j,
                                           LocalCounters& lc) {
-    densvel_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.v[j], T.r[j], lc);
+    densvel_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.v[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DLMember& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_list_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.r[j], lc);
+    density_list_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(VMember& M, const SearchArgs& a, const VelTile& T, int j,
                                           LocalCounters& lc) {
-    vel_pair<MODE, WRAP>(M, a, T.p[j], T.m[j], T.v[j], T.r[j], lc);
+    vel_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.v[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(HMember& M, const SearchArgs& a, const HydroTile& T, int j,
                                           LocalCounters& lc) {
-    hydro_pair<MODE, WRAP>(M, a, T.p[j], T.q[j], T.v[j], T.h[j], T.r[j], lc);
+    hydro_pair<MODE, WRAP>(M, a, T.pos(j), make_float2(T.h2[j], T.m[j]), T.v[j], T.h[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(HAMember& M, const SearchArgs& a, const HAdjTile& T, int j,
                                           LocalCounters& lc) {
-    hydro_adj_pair<MODE, WRAP>(M, a, T.p[j], T.q[j], T.v[j], T.h[j], T.w[j], T.r[j], lc);
+    hydro_adj_pair<MODE, WRAP>(M, a, T.pos(j), make_float2(T.h2[j], T.m[j]), T.v[j], T.h[j], T.w[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DAMember& M, const SearchArgs& a, const DAdjTile& T, int j,
                                           LocalCounters& lc) {
-    dens_adj_pair<MODE, WRAP>(M, a, T.p[j], T.q[j], T.d[j], T.r[j], lc);
+    dens_adj_pair<MODE, WRAP>(M, a, T.pos(j), make_float2(T.h2[j], T.m[j]), T.d[j], T.r[j], lc);
 }
 
-// phase A threshold of the dot form |p|^2 - 2 p.m (density) and of the difference
-// form (WRAP); symmetric kinds read h_j^2 from the tile
-__device__ __forceinline__ float thr_dot(const DMember& M, float) { return M.thr_dot; }
-__device__ __forceinline__ float thr_dot(const SymMember& M, float hj2) {
-    return fmaf(fmaxf(M.h2, hj2), 1.0f + 3.0f * kBandRel, M.bk_dot);
-}
+// Phase-A thresholds: of the dot form |p|^2 - 2 p.m (one-sided kinds: a constant of the
+// member; symmetric ones: max(h^2, h_j^2) (1 + band) + bk_dot) and of the difference form
+__device__ __forceinline__ float thr_dot(const DMember& M) { return M.thr_dot; }
+__device__ __forceinline__ float thr_dot(const DLMember& M) { return M.thr_dot_w; }
+__device__ __forceinline__ float thr_dot(const VMember& M) { return M.thr_dot; }
+__device__ __forceinline__ float thr_dot(const SymMember& M) { return M.bk_dot; }
 __device__ __forceinline__ float thr_diff(const DMember& M, float) { return M.h2hi; }
-__device__ __forceinline__ float thr_dot(const DLMember& M, float) { return M.thr_dot_w; }
 __device__ __forceinline__ float thr_diff(const DLMember& M, float) { return M.h2whi; }
-__device__ __forceinline__ float thr_dot(const VMember& M, float) { return M.thr_dot; }
 __device__ __forceinline__ float thr_diff(const VMember& M, float) { return M.h2hi; }
 __device__ __forceinline__ float thr_diff(const SymMember& M, float hj2) {
     return fmaf(fmaxf(M.h2, hj2), 1.0f + 3.0f * kBandRel, M.bk);
 }
 
-// combine the slice copies of a member (lanes k, k+g, k+2g, ...)
-__device__ __forceinline__ float xsum(float v, int o) { return v + __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ void slice_add(DMember& M, int o) {
-    M.s0 = xsum(M.s0, o); M.c0 = xsum(M.c0, o); M.s1 = xsum(M.s1, o); M.c1 = xsum(M.c1, o);
-    M.n += __shfl_xor_sync(0xffffffffu, M.n, o);
+// combine the slice copies of a member: add the values held o lanes above, where add says so
+struct SliceStep {
+    int o;
+    bool add;
+};
+__device__ __forceinline__ float xsum(float v, SliceStep o) {
+    const float t = __shfl_down_sync(0xffffffffu, v, o.o);
+    return o.add ? v + t : v;
 }
-__device__ __forceinline__ void slice_add(D2Member& M, int o) {
+__device__ __forceinline__ int xsum(int v, SliceStep o) {
+    const int t = __shfl_down_sync(0xffffffffu, v, o.o);
+    return o.add ? v + t : v;
+}
+__device__ __forceinline__ void slice_add(DMember& M, SliceStep o) {
+    M.s0 = xsum(M.s0, o); M.c0 = xsum(M.c0, o); M.s1 = xsum(M.s1, o); M.c1 = xsum(M.c1, o);
+    M.n = xsum(M.n, o);
+}
+__device__ __forceinline__ void slice_add(D2Member& M, SliceStep o) {
     slice_add(static_cast<DMember&>(M), o);
     M.s2 = xsum(M.s2, o); M.c2 = xsum(M.c2, o);
 }
-__device__ __forceinline__ void slice_add(DVMember& M, int o) {
+__device__ __forceinline__ void slice_add(DVMember& M, SliceStep o) {
     slice_add(static_cast<DMember&>(M), o);
     M.sd = xsum(M.sd, o); M.cd = xsum(M.cd, o); M.sx = xsum(M.sx, o); M.cx_ = xsum(M.cx_, o);
     M.sy = xsum(M.sy, o); M.cy_ = xsum(M.cy_, o); M.sz = xsum(M.sz, o); M.cz_ = xsum(M.cz_, o);
 }
-__device__ __forceinline__ void slice_add(HMember& M, int o) {
+__device__ __forceinline__ void slice_add(HMember& M, SliceStep o) {
     M.sx = xsum(M.sx, o); M.cx_ = xsum(M.cx_, o); M.sy = xsum(M.sy, o); M.cy_ = xsum(M.cy_, o);
     M.sz = xsum(M.sz, o); M.cz_ = xsum(M.cz_, o); M.su = xsum(M.su, o); M.cu = xsum(M.cu, o);
-    M.n += __shfl_xor_sync(0xffffffffu, M.n, o);
+    M.n = xsum(M.n, o);
 }
-__device__ __forceinline__ void slice_add(VMember& M, int o) {
+__device__ __forceinline__ void slice_add(VMember& M, SliceStep o) {
     M.sd = xsum(M.sd, o); M.cd = xsum(M.cd, o); M.sx = xsum(M.sx, o); M.cx_ = xsum(M.cx_, o);
     M.sy = xsum(M.sy, o); M.cy_ = xsum(M.cy_, o); M.sz = xsum(M.sz, o); M.cz_ = xsum(M.cz_, o);
-    M.n += __shfl_xor_sync(0xffffffffu, M.n, o);
+    M.n = xsum(M.n, o);
 }
-__device__ __forceinline__ void slice_add(HAMember& M, int o) {
+__device__ __forceinline__ void slice_add(HAMember& M, SliceStep o) {
     for (int k = 0; k < 3; ++k) { M.xb[k] = xsum(M.xb[k], o); M.vb[k] = xsum(M.vb[k], o); }
     M.mb = xsum(M.mb, o); M.hb = xsum(M.hb, o); M.rb = xsum(M.rb, o); M.Ab = xsum(M.Ab, o);
-    M.n += __shfl_xor_sync(0xffffffffu, M.n, o);
+    M.n = xsum(M.n, o);
 }
-__device__ __forceinline__ void slice_add(DAMember& M, int o) {
+__device__ __forceinline__ void slice_add(DAMember& M, SliceStep o) {
     for (int k = 0; k < 3; ++k) M.xb[k] = xsum(M.xb[k], o);
     M.mb = xsum(M.mb, o);
-    M.n += __shfl_xor_sync(0xffffffffu, M.n, o);
+    M.n = xsum(M.n, o);
 }
 
 // results of a member
@@ -1078,90 +1144,120 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
     return v;
 }
 
-// Member slot layout of a lane: gw member slots (the member count rounded up to a power
-// of two, at most 32) in S copies ("slices"), each filtering a different subset of the
-// candidates; k = the lane's member, -1 if it holds none.
+// Member slot layout of a lane: the part's gw members in S copies ("slices"), each
+// filtering a different subset of the candidates; k = the lane's member, -1 if it holds
+// none (its slice is then S or more, or the member has left).
 struct Layout {
     int gw, S, slice, k;
+    uint32_t inv;   // ceil(2^16 / S): n / S = n * inv >> 16 for the n <= 2^10 used here
 };
 
-__device__ __forceinline__ Layout make_layout(int cnt, int lane, bool allow_slices, int max_slices) {
+// pow2: member slots rounded up to a power of two and at most 4 slices
+__device__ __forceinline__ Layout make_layout(int cnt, int lane, bool allow_slices, int max_slices, bool pow2) {
     Layout L;
-    const int sh = cnt <= 1 ? 0 : 32 - __clz(cnt - 1);
-    L.gw = 1 << sh;
-    L.S = allow_slices ? min(32 >> sh, max_slices) : 1;
-    L.slice = lane >> sh;
-    const int k = lane & (L.gw - 1);
+    L.gw = pow2 && cnt > 1 ? 1 << (32 - __clz(cnt - 1)) : cnt;
+    const uint32_t q = 65536u / (uint32_t)L.gw + 1u;
+    L.S = allow_slices ? min((int)((32u * q) >> 16), max_slices) : 1;
+    L.slice = (int)(((uint32_t)lane * q) >> 16);
+    const int k = lane - L.slice * L.gw;
     L.k = (L.slice < L.S && k < cnt) ? k : -1;
+    L.inv = 65535u / (uint32_t)L.S + 1u;
     return L;
 }
 
-// Member x candidate filter of one tile.  Phase A: for every chunk of 32 of the lane's
-// slice, a bit mask of the candidates inside the member's FP32 threshold, tested in
-// dot-product form |p|^2 - 2 p.m < h^2 - |m|^2 (three FMAs; its rounding stays inside
-// the FP64 decision band).  Phase B: every lane walks its own set bits across all chunks
-// (no per-chunk wait for the slowest lane) for the exact decision and the pair terms;
-// forward partial sums are folded into the compensated totals after the tile.
+// sum over the slices, ending in slice 0: halves folded onto each other
+template <class Mem>
+__device__ __forceinline__ void slice_sum(Mem& M, const Layout& L) {
+    for (int n = L.S; n > 1;) {
+        const int half = (n + 1) >> 1;
+        slice_add(M, SliceStep{half * L.gw, L.slice + half < n});
+        n = half;
+    }
+}
+
+// Phase A of one mask word: the lane's next 2 * rows candidates (rows a multiple of 4, at
+// most 16; pairs first, first + S, ...) against the member's FP32 threshold, the first
+// candidate in the top bit of the 2 * rows lowest ones.  Dot form, packed: per pair of
+// candidates two shared-memory loads, three packed FMAs, one packed add and two shifts
+// that collect the signs; its rounding stays inside the FP64 decision band.
+template <class K, bool WRAP>
+__device__ __forceinline__ uint32_t test_word(const typename K::Tile& T, const typename K::Member& Mb, int first,
+                                              int S, int rows) {
+    uint32_t mask = 0u;
+    if constexpr (!WRAP) {
+        const unsigned long long ax = pair_of(-2.0f * Mb.mx, -2.0f * Mb.mx), ay = pair_of(-2.0f * Mb.my, -2.0f * Mb.my),
+                                 az = pair_of(-2.0f * Mb.mz, -2.0f * Mb.mz),
+                                 at = pair_of(-thr_dot(Mb), -thr_dot(Mb));
+        for (int r = 0; r < rows; r += 4) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = first + (r + q) * S;
+                const ulonglong2 pa = *reinterpret_cast<const ulonglong2*>(&T.a[i]);
+                const ulonglong2 pb = *reinterpret_cast<const ulonglong2*>(&T.b[i]);
+                unsigned long long w = add_pair(pb.y, at);
+                if constexpr (K::sym) {
+                    const float2 hj2 = *reinterpret_cast<const float2*>(&T.h2[2 * i]);
+                    constexpr float kk = -(1.0f + 3.0f * kBandRel);
+                    w = fma_pair(pair_of(fmaxf(Mb.h2, hj2.x), fmaxf(Mb.h2, hj2.y)), pair_of(kk, kk), w);
+                }
+                const unsigned long long t = fma_pair(pa.x, ax, fma_pair(pa.y, ay, fma_pair(pb.x, az, w)));
+                mask = push_sign(mask, (uint32_t)t);
+                mask = push_sign(mask, (uint32_t)(t >> 32));
+            }
+        }
+    } else {
+        for (int r = 0; r < 2 * rows; ++r) {
+            const int t = 2 * (first + (r >> 1) * S) + (r & 1);
+            const float3 p = T.pos(t);
+            float hj2 = 0.0f;
+            if constexpr (K::sym) hj2 = T.h2[t];
+            const float dx = rel_diff<true>(p.x, Mb.mx), dy = rel_diff<true>(p.y, Mb.my), dz = rel_diff<true>(p.z, Mb.mz);
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            mask = (mask << 1) | (r2 < thr_diff(Mb, hj2) ? 1u : 0u);
+        }
+    }
+    return mask;
+}
+
+// Member x candidate filter of the nt candidates in the tile.  Phase A: bit masks of the
+// lane's slice, a word per 32 candidates.  Phase B: every lane walks its own set bits
+// across all words (no per-word wait for the slowest lane) for the exact decision and the
+// pair terms; forward partial sums are folded into the compensated totals after the
+// tile.
 template <class K, int MODE, bool WRAP>
 __device__ __forceinline__ void filter_tile(typename K::Tile& T, const Layout& L, typename K::Member& Mb, int nt,
                                             const SearchArgs& a, LocalCounters& lc, int lane) {
     const int S = L.S;
-    if (L.slice >= S) return;
-    const int cnt_slice = (nt > L.slice) ? (nt - L.slice + S - 1) / S : 0;
-    const int nch = ((nt + S - 1) / S + 31) >> 5;
-    const float mx = Mb.mx, my = Mb.my, mz = Mb.mz;
-    const float ax = -2.0f * mx, ay = -2.0f * my, az = -2.0f * mz;
-    for (int c = 0; c < nch; ++c) {
-        uint32_t mask = 0u;
-        const int j0 = L.slice + S * (c << 5);
-#pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            const int j = j0 + q * S;
-            const float4 cp = T.p[j];
-            float hj2 = 0.0f;
-            if constexpr (K::sym) hj2 = T.q[j].x;
-            bool pass;
-            if constexpr (!WRAP) {
-                float t = fmaf(cp.x, ax, fmaf(cp.y, ay, fmaf(cp.z, az, cp.w)));
-                pass = t < thr_dot(Mb, hj2);
-            } else {
-                float dx = rel_diff<true>(cp.x, mx), dy = rel_diff<true>(cp.y, my), dz = rel_diff<true>(cp.z, mz);
-                float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                pass = r2 < thr_diff(Mb, hj2);
-            }
-            mask |= (pass ? 1u : 0u) << q;
-        }
-        T.masks[(c << 5) + lane] = mask;
+    const int npair = (nt + 1) >> 1;
+    const int rows = (int)(((npair + S - 1) * L.inv) >> 16);   // of slice 0, the longest
+    // the lane's own candidates: whole pairs, and the last half pair if it is its
+    int mine = 0;
+    if (Mb.rank >= 0)
+        mine = (int)((((nt >> 1) + S - 1 - L.slice) * L.inv) >> 16) +
+               (int)(((npair + S - 1 - L.slice) * L.inv) >> 16);
+    lc.tests += mine;
+    const int nw = (rows + 15) >> 4;
+    const int sl = L.slice < S ? L.slice : 0;   // lanes without a member test slice 0's and drop it
+    for (int c = 0; c < nw; ++c) {
+        const int rw = min(16, (rows - 16 * c + 3) & ~3);
+        const uint32_t mask = test_word<K, WRAP>(T, Mb, sl + 16 * c * S, S, rw) << (32 - 2 * rw);
+        const int own = min(max(mine - 32 * c, 0), 32);
+        T.masks[(c << 5) + lane] = mask & (uint32_t)(0xffffffff00000000ull >> own);
     }
-    if (Mb.rank >= 0) lc.tests += cnt_slice;
     int c = 0;
-    uint32_t cur = T.masks[lane];
+    uint32_t cur = nw > 0 ? T.masks[lane] : 0u;
     for (;;) {
         while (cur == 0u) {
-            if (++c >= nch) break;
+            if (++c >= nw) break;
             cur = T.masks[(c << 5) + lane];
         }
         if (cur == 0u) break;
-        const int q = __ffs(cur) - 1;
-        cur &= cur - 1u;
-        tile_pair<MODE, WRAP>(Mb, a, T, L.slice + S * ((c << 5) + q), lc);
+        const int q = __clz(cur);
+        cur &= ~(0x80000000u >> q);
+        const int l = (c << 5) + q;
+        tile_pair<MODE, WRAP>(Mb, a, T, 2 * ((l >> 1) * S + sl) + (l & 1), lc);
     }
     if (MODE == kAcc) flush(Mb);
-}
-
-// Filter of the nt candidates in the tile: NaN dummies up to whole chunks of 32 in every
-// slice, then the member x candidate filter (dot form unless the group wraps).
-template <class K, int MODE>
-__device__ __forceinline__ void filter_staged(typename K::Tile& T, const Layout& L, typename K::Member& mem, int nt,
-                                              const SearchArgs& a, LocalCounters& lc, int lane, bool wrap_safe) {
-    const int padded = L.S * ((((nt + L.S - 1) / L.S) + 31) >> 5) * 32;
-    const float nanv = __int_as_float(0x7fffffff);
-    for (int t = nt + lane; t < padded; t += 32) T.p[t] = make_float4(nanv, nanv, nanv, nanv);
-    copies_wait();
-    __syncwarp();
-    if (wrap_safe) filter_tile<K, MODE, false>(T, L, mem, nt, a, lc, lane);
-    else filter_tile<K, MODE, true>(T, L, mem, nt, a, lc, lane);
-    __syncwarp();
 }
 
 // Work item of the grouped kernels: members U[base, base + cnt), the walk's start node
@@ -1173,13 +1269,14 @@ struct GroupDesc {
 __device__ __forceinline__ GroupDesc group_desc(const SearchArgs& a, int gid) {
     GroupDesc d;
     d.root = 0;
-    d.smax = 4;
+    d.smax = 32;
     if (a.groups4) {
         const int4 G = a.groups4[gid];
         d.base = G.x;
         d.cnt = G.y;
         d.root = G.z;
         d.smax = (G.w >> 8) & 0xff;   // bits 16.. carry the box's leaf size
+        if (d.smax >= 4) d.smax = 32;   // 4, the largest limit that can be set: all lanes
     } else if (a.groups) {
         const int2 G = a.groups[gid];
         d.base = G.x;
@@ -1482,9 +1579,9 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
             const unsigned im = __ballot_sync(0xffffffffu, in);
             if (in) {
                 const int t = ns + __popc(im & lt);
-                T.p[t] = make_float4(px, py, pz, fmaf(px, px, fmaf(py, py, pz * pz)));
-                if constexpr (K::sym) T.q[t] = make_float2(hj2, mj);
-                else T.m[t] = mj;
+                T.put(t, px, py, pz);
+                T.m[t] = mj;
+                if constexpr (K::sym) T.h2[t] = hj2;
                 T.r[t] = rank;
                 stage_records(T, a, t, rank);
             }
@@ -1492,7 +1589,13 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
         }
         const bool last = walked && w.total == w.done;
         if (ns > kTile - 32 || last) {
-            if (ns > 0) filter_staged<K, MODE>(T, L, mem, ns, a, lc, lane, wrap_safe);
+            if (ns > 0) {
+                copies_wait();
+                __syncwarp();
+                if (wrap_safe) filter_tile<K, MODE, false>(T, L, mem, ns, a, lc, lane);
+                else filter_tile<K, MODE, true>(T, L, mem, ns, a, lc, lane);
+                __syncwarp();
+            }
             ns = 0;
             if (last) break;
         }
@@ -1503,7 +1606,8 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
 template <class K, int MODE>
 __device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, int base, int cnt,
                                              int root, int smax, LocalCounters& lc, int lane) {
-    const Layout L = make_layout(cnt, lane, MODE == kAcc, min(kTile / 32, smax));
+    constexpr bool kLists = K::id == kKindDensityList;
+    const Layout L = make_layout(cnt, lane, MODE == kAcc, kLists ? min(4, smax) : smax, kLists);
     const MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[base + L.k] : -1)};
     uint32_t cx = 0, cy = 0, cz = 0;
     if (!group_centre<1>(a, rec, cx, cy, cz)) return;
@@ -1541,7 +1645,7 @@ __device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, t
             a.o_lslot[mem.rank] = slot;
         }
     }
-    for (int o = L.gw; o < L.gw * L.S; o <<= 1) slice_add(mem, o);
+    slice_sum(mem, L);
     if (L.slice == 0 && mem.rank >= 0) write_result<MODE>(mem, a);
 }
 
@@ -1736,7 +1840,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
         if (gid >= ng) break;
         const GroupDesc d = group_desc(a, gid);
         for (int b = 0; b < d.cnt; b += kPartMax) {
-            const Layout L = make_layout(min(kPartMax, d.cnt - b), lane, true, min(kTile / 32, d.smax));
+            const Layout L = make_layout(min(kPartMax, d.cnt - b), lane, true, d.smax, false);
             MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[d.base + b + L.k] : -1)};
             double lo = 0.0, hi = __longlong_as_double(0x7ff0000000000000ll);
             for (int pass = 1;; ++pass) {
@@ -1746,9 +1850,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
                 member_init(mem, a, rec[0], cx, cy, cz);
                 group_search<KDens, kAcc>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
                 lc.pairs += mem.n;
-                for (int o = L.gw; o < L.gw * L.S; o <<= 1) slice_add(mem, o);
-                if (rec[0].rank >= 0 && hsml_step(a, it, rec[0].rank, rec[0].h, lo, hi, mem.s0 - mem.c0,
-                                                  mem.s1 - mem.c1, mem.n, pass, L.slice == 0))
+                slice_sum(mem, L);
+                // every slice takes the step, from the sums of its member in slice 0
+                const int src = L.k >= 0 ? L.k : 0;
+                const float s0 = __shfl_sync(0xffffffffu, mem.s0 - mem.c0, src);
+                const float s1 = __shfl_sync(0xffffffffu, mem.s1 - mem.c1, src);
+                const int nn = __shfl_sync(0xffffffffu, mem.n, src);
+                if (rec[0].rank >= 0 &&
+                    hsml_step(a, it, rec[0].rank, rec[0].h, lo, hi, s0, s1, nn, pass, L.slice == 0))
                     rec[0].rank = -1;
                 // the new h (global memory) is read by the next pass's FP64 re-tests
                 __syncwarp();
@@ -1799,8 +1908,8 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                     for (int q = lk.x; q < lk.x + lk.y; ++q) {
                         uint4 Q = a.pfix[q];
                         float4 O = a.poff[q];
-                        float4 rel = make_float4(rel_coord(Q.x, O.x, cx), rel_coord(Q.y, O.y, cy),
-                                                 rel_coord(Q.z, O.z, cz), O.w);
+                        const float3 rel = make_float3(rel_coord(Q.x, O.x, cx), rel_coord(Q.y, O.y, cy),
+                                                       rel_coord(Q.z, O.z, cz));
                         if (KIND == 0) {
                             density_pair<MODE>(dm, a, rel, O.w, q, lc);
                         } else {
