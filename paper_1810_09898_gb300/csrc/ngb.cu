@@ -677,61 +677,72 @@ __device__ __forceinline__ void density_terms(D2Member& M, float mj, float q) {
     M.p2 = fmaf(mj, fmaf(q * q, d2w, fmaf(8.0f * q, dw, 12.0f * w)), M.p2);
 }
 
-// density pair: p = candidate's coordinates relative to the member's centre, m_j its mass
+// Decision of the density criterion |r| < h_i, and the pair's difference.  Only the rare
+// slow path branches: the FP64 re-test inside the band, and the exact differences of
+// members far from the centre.
+template <bool WRAP, class Mem>
+__device__ __forceinline__ bool dens_decide(const Mem& M, const SearchArgs& a, float3 p, int crank, LocalCounters& lc,
+                                            float& dx, float& dy, float& dz, float& r2) {
+    dx = rel_diff<WRAP>(p.x, M.mx);
+    dy = rel_diff<WRAP>(p.y, M.my);
+    dz = rel_diff<WRAP>(p.z, M.mz);
+    r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    bool in = r2 < M.h2lo;
+    if (M.precise || (!in && r2 < M.h2hi)) {
+        if (!in && r2 < M.h2hi) {
+            const double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
+            const double h = a.h64[M.rank];
+            in = e < __dmul_rn(h, h);
+            lc.retests++;
+        }
+        if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
+    }
+    return in;
+}
+
+// export of a pair: the next entry of the member's list
+__device__ __forceinline__ void export_pair(MemberPos& M, const SearchArgs& a, int crank) {
+    const int64_t q = M.xpos++;
+    if (q < a.x_cap) a.x_idx[q] = a.perm[crank];
+    else atomicOr(a.err, kErrCap);
+}
+
+// density pair: p = candidate's coordinates relative to the member's centre, m_j its mass.
+// A candidate outside enters the sums with mass 0 (phase A leaves few of them).
 template <int MODE, bool WRAP = false, class Mem>
 __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float3 p, float mj, int crank,
                                              LocalCounters& lc) {
-    float dx = rel_diff<WRAP>(p.x, M.mx), dy = rel_diff<WRAP>(p.y, M.my), dz = rel_diff<WRAP>(p.z, M.mz);
-    float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    bool in = r2 < M.h2lo;
-    if (!in) {
-        if (!(r2 < M.h2hi)) return;
-        double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
-        double h = a.h64[M.rank];
-        in = e < __dmul_rn(h, h);
-        lc.retests++;
-    }
-    if (!in) return;
-    M.n++;
-    if (MODE == kAcc) {
-        if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
-        float q = r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)) * M.hinv;
-        density_terms(M, mj, q);
-    } else if (MODE == kFill) {
-        int64_t q = M.xpos++;
-        if (q < a.x_cap) a.x_idx[q] = a.perm[crank];
-        else atomicOr(a.err, kErrCap);
-    }
+    float dx, dy, dz, r2;
+    const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
+    M.n += in ? 1 : 0;
+    if (MODE == kAcc) density_terms(M, in ? mj : 0.0f, r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)) * M.hinv);
+    else if (MODE == kFill && in) export_pair(M, a, crank);
 }
 
-// density pair with the velocity derivatives: the density decision and sums of
-// density_pair, then (for pairs at r > 0) the divergence and curl terms with
-// grad_i W = W'(r, h_i) (x_i - x_j) / r and v_ij = v_i - v_j
-template <int MODE, bool WRAP = false>
-__device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, float3 p, float mj, float4 vj,
-                                             int crank, LocalCounters& lc) {
-    const int n0 = M.n;
-    density_pair<MODE, WRAP>(static_cast<DMember&>(M), a, p, mj, crank, lc);
-    if (MODE != kAcc || M.n == n0) return;
-    float dx, dy, dz, r2;
-    if (M.precise) {
-        precise_diff(M, a, crank, dx, dy, dz, r2);
-    } else {
-        dx = rel_diff<WRAP>(p.x, M.mx);
-        dy = rel_diff<WRAP>(p.y, M.my);
-        dz = rel_diff<WRAP>(p.z, M.mz);
-        r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    }
-    if (r2 == 0.0f) return;
+// divergence and curl terms of a neighbour at x_j - x_i = d: grad_i W = W'(r, h_i) (x_i -
+// x_j) / r, v_ij = v_i - v_j; r > 0 (at r = 0 grad W = 0)
+template <class Mem>
+__device__ __forceinline__ void velocity_terms(Mem& M, float mj, float4 vj, float dx, float dy, float dz, float r2) {
     const float rinv = rsqrt_fast(r2);
-    const float dw = m4_slope(r2 * rinv * M.hinv);
-    const float c = -M.sk * dw * rinv;   // x_i - x_j = -d
+    const float c = -M.sk * m4_slope(r2 * rinv * M.hinv) * rinv;   // x_i - x_j = -d
     const float gx = c * dx, gy = c * dy, gz = c * dz;
     const float vx = M.vx - vj.x, vy = M.vy - vj.y, vz = M.vz - vj.z;
     M.pd = fmaf(-mj, fmaf(vx, gx, fmaf(vy, gy, vz * gz)), M.pd);
     M.px_ = fmaf(mj, fmaf(vy, gz, -vz * gy), M.px_);
     M.py_ = fmaf(mj, fmaf(vz, gx, -vx * gz), M.py_);
     M.pz_ = fmaf(mj, fmaf(vx, gy, -vy * gx), M.pz_);
+}
+
+// density pair with the velocity derivatives over the same decision
+template <int MODE, bool WRAP = false>
+__device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, float3 p, float mj, float4 vj,
+                                             int crank, LocalCounters& lc) {
+    float dx, dy, dz, r2;
+    const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
+    M.n += in ? 1 : 0;
+    if (MODE != kAcc) return;
+    density_terms(M, in ? mj : 0.0f, r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)) * M.hinv);
+    if (in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
 // density pair of the recycled iteration: a candidate inside the widened threshold joins
@@ -753,33 +764,13 @@ __device__ __forceinline__ void density_list_pair(DLMember& M, const SearchArgs&
 template <int MODE, bool WRAP = false>
 __device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float3 p, float mj, float4 vj, int crank,
                                          LocalCounters& lc) {
-    float dx = rel_diff<WRAP>(p.x, M.mx), dy = rel_diff<WRAP>(p.y, M.my), dz = rel_diff<WRAP>(p.z, M.mz);
-    float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    bool in = r2 < M.h2lo;
-    if (!in) {
-        if (!(r2 < M.h2hi)) return;
-        double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
-        double h = a.h64[M.rank];
-        in = e < __dmul_rn(h, h);
-        lc.retests++;
-    }
-    if (!in) return;
-    M.n++;
-    if (MODE != kAcc) return;
-    if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
-    if (r2 == 0.0f) return;   // the particle itself (and coincident ones): grad W = 0
-    const float rinv = rsqrt_fast(r2);
-    const float dw = m4_slope(r2 * rinv * M.hinv);
-    const float c = -M.sk * dw * rinv;   // grad_i W = W' (x_i - x_j) / r, x_i - x_j = -d
-    const float gx = c * dx, gy = c * dy, gz = c * dz;
-    const float vx = M.vx - vj.x, vy = M.vy - vj.y, vz = M.vz - vj.z;
-    M.pd = fmaf(-mj, fmaf(vx, gx, fmaf(vy, gy, vz * gz)), M.pd);
-    M.px_ = fmaf(mj, fmaf(vy, gz, -vz * gy), M.px_);
-    M.py_ = fmaf(mj, fmaf(vz, gx, -vx * gz), M.py_);
-    M.pz_ = fmaf(mj, fmaf(vx, gy, -vy * gx), M.pz_);
+    float dx, dy, dz, r2;
+    const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
+    M.n += in ? 1 : 0;
+    if (MODE == kAcc && in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
-// decision of the symmetric criterion |r| < max(h_i, h_j) with the FP64 band re-test
+// decision of the symmetric criterion |r| < max(h_i, h_j), as dens_decide
 template <bool WRAP, class Mem>
 __device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, float3 p, float hj2, int crank,
                                            LocalCounters& lc, float& dx, float& dy, float& dz, float& r2) {
@@ -787,62 +778,56 @@ __device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, fl
     dy = rel_diff<WRAP>(p.y, M.my);
     dz = rel_diff<WRAP>(p.z, M.mz);
     r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    float H2 = fmaxf(M.h2, hj2);
+    const float H2 = fmaxf(M.h2, hj2);
     bool in = r2 < fmaf(H2, 1.0f - 3.0f * kBandRel, -M.bk);
-    if (!in) {
-        if (!(r2 < fmaf(H2, 1.0f + 3.0f * kBandRel, M.bk))) return false;
-        double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
-        double hi = a.h64[M.rank], hj = a.h64[crank];
-        in = e < fmax(__dmul_rn(hi, hi), __dmul_rn(hj, hj));
-        lc.retests++;
+    const bool band = !in && r2 < fmaf(H2, 1.0f + 3.0f * kBandRel, M.bk);
+    if (M.precise || band) {
+        if (band) {
+            const double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
+            const double hi = a.h64[M.rank], hj = a.h64[crank];
+            in = e < fmax(__dmul_rn(hi, hi), __dmul_rn(hj, hj));
+            lc.retests++;
+        }
+        if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
     }
     return in;
 }
 
 // hydro pair: p = relative coordinates, q = {h_j^2, m_j}, v = {vx, vy, vz, c_j},
-// hh = {A_j, rho_j, 1/h_j, limiter_j}
+// hh = {A_j, rho_j, 1/h_j, limiter_j}.  A pair at r = 0 (coincident, or the member itself)
+// has no kernel gradient.
 template <int MODE, bool WRAP = false>
 __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float3 p, float2 q,
                                            float4 v, float4 hh, int crank, LocalCounters& lc) {
-    // The member itself is a candidate: the exports skip it by rank; the sums skip it
-    // as a pair at r = 0 (counted, then taken off the neighbour count at the end).
+    // The member itself is a candidate: the exports skip it by rank; the sums count it
+    // as a pair at r = 0, taken off the neighbour count at the end.
     if (MODE != kAcc && crank == M.rank) return;
     float dx, dy, dz, r2;
-    if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
-    M.n++;
-    if (MODE == kFill) {
-        int64_t k = M.xpos++;
-        if (k < a.x_cap) a.x_idx[k] = a.perm[crank];
-        else atomicOr(a.err, kErrCap);
-        return;
-    }
-    if (MODE != kAcc) return;
-    if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
-    if (r2 == 0.0f) return;  // coincident: the kernel gradient vanishes
-    float rinv = rsqrt_fast(r2);
-    float r = r2 * rinv;
-    const float dwi = m4_slope(r * M.hinv), dwj = m4_slope(r * hh.z);
-    float dWi = M.sk * dwi;
-    float dWj = kSkernel * (hh.z * hh.z) * (hh.z * hh.z) * dwj;
-    float rx = -dx, ry = -dy, rz = -dz;  // r_ij = x_i - x_j
-    float vx = M.vx - v.x, vy = M.vy - v.y, vz = M.vz - v.z;
-    float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
-    float visc = 0.0f;
-    if (vr < 0.0f) {
-        float hb = 0.5f * fmaf(q.x, hh.z, M.h);
-        float mu = hb * vr * rcp_fast(fmaf(a.eps * hb, hb, r2));
-        float cb = 0.5f * (M.cs + v.w);
-        // Pi = (-alpha cbar mu + beta mu^2) / rhobar, rhobar = (rho_i + rho_j) / 2, scaled by
-        // the pair mean of the limiter (1 for the plain viscosity)
-        visc = 2.0f * fmaf(-a.alpha * cb, mu, a.beta * mu * mu) * rcp_fast(M.rho + hh.y);
-        visc *= 0.5f * (M.fb + hh.w);
-    }
-    float gbar = 0.5f * (dWi + dWj);
-    float coef = q.y * fmaf(M.A, dWi, fmaf(hh.x, dWj, visc * gbar)) * rinv;
+    const bool in = sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2);
+    M.n += in ? 1 : 0;
+    if (MODE == kFill && in) export_pair(M, a, crank);
+    if (MODE != kAcc || !(in && r2 > 0.0f)) return;
+    const float rinv = rsqrt_fast(r2);
+    const float r = r2 * rinv;
+    const float dWi = M.sk * m4_slope(r * M.hinv);
+    const float dWj = kSkernel * (hh.z * hh.z) * (hh.z * hh.z) * m4_slope(r * hh.z);
+    const float rx = -dx, ry = -dy, rz = -dz;  // r_ij = x_i - x_j
+    const float vx = M.vx - v.x, vy = M.vy - v.y, vz = M.vz - v.z;
+    const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
+    // Pi = (-alpha cbar mu + beta mu^2) / rhobar for approaching pairs, rhobar = (rho_i +
+    // rho_j) / 2, scaled by the pair mean of the limiter (1 for the plain viscosity)
+    const float hb = 0.5f * fmaf(q.x, hh.z, M.h);
+    const float mu = hb * vr * rcp_fast(fmaf(a.eps * hb, hb, r2));
+    const float cb = 0.5f * (M.cs + v.w);
+    const float pi_ij = fmaf(-a.alpha * cb, mu, a.beta * mu * mu) * rcp_fast(M.rho + hh.y) * (M.fb + hh.w);
+    const float visc = vr < 0.0f ? pi_ij : 0.0f;
+    const float gbar = 0.5f * (dWi + dWj);
+    const float mr = q.y * rinv;
+    const float coef = mr * fmaf(M.A, dWi, fmaf(hh.x, dWj, visc * gbar));
     M.px_ = fmaf(coef, dx, M.px_);
     M.py_ = fmaf(coef, dy, M.py_);
     M.pz_ = fmaf(coef, dz, M.pz_);
-    M.pu = fmaf(q.y * fmaf(M.A, dWi, 0.5f * visc * gbar) * rinv, vr, M.pu);
+    M.pu = fmaf(mr * fmaf(M.A, dWi, 0.5f * visc * gbar), vr, M.pu);
 }
 
 // Adjoint of sum_i w_i . a_i over one pair, gathered at member k.  The pair enters
@@ -858,7 +843,6 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
     M.n++;
     if (MODE != kAcc) return;
-    if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
     if (r2 == 0.0f) return;
     const float rinv = rsqrt_fast(r2);
     const float r = r2 * rinv;
@@ -934,7 +918,6 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
     if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
     M.n++;
     if (MODE != kAcc) return;
-    if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
     const float rinv = r2 > 0.0f ? rsqrt_fast(r2) : 0.0f;
     const float r = r2 * rinv;
     float wk_, dwk, d2wk, wj_, dwj, d2wj;
@@ -1244,18 +1227,21 @@ __device__ __forceinline__ void filter_tile(typename K::Tile& T, const Layout& L
         const int own = min(max(mine - 32 * c, 0), 32);
         T.masks[(c << 5) + lane] = mask & (uint32_t)(0xffffffff00000000ull >> own);
     }
-    int c = 0;
-    uint32_t cur = nw > 0 ? T.masks[lane] : 0u;
-    for (;;) {
-        while (cur == 0u) {
-            if (++c >= nw) break;
-            cur = T.masks[(c << 5) + lane];
+    // two words at a time in registers, the second following the first without a branch
+    for (int c = 0; c < nw; c += 2) {
+        uint32_t cur = T.masks[(c << 5) + lane], nxt = c + 1 < nw ? T.masks[(c << 5) + 32 + lane] : 0u;
+        int l0 = c << 5;
+        while (cur | nxt) {
+            if (cur == 0u) {
+                cur = nxt;
+                nxt = 0u;
+                l0 += 32;
+            }
+            const int q = __clz(cur);
+            cur ^= 0x80000000u >> q;
+            const int l = l0 + q;
+            tile_pair<MODE, WRAP>(Mb, a, T, 2 * ((l >> 1) * S + sl) + (l & 1), lc);
         }
-        if (cur == 0u) break;
-        const int q = __clz(cur);
-        cur &= ~(0x80000000u >> q);
-        const int l = (c << 5) + q;
-        tile_pair<MODE, WRAP>(Mb, a, T, 2 * ((l >> 1) * S + sl) + (l & 1), lc);
     }
     if (MODE == kAcc) flush(Mb);
 }
@@ -1329,40 +1315,48 @@ __device__ __forceinline__ bool group_centre(const SearchArgs& a, const MemberRe
     return true;
 }
 
-// Morton index of a cell of level l (l bits per axis, axis 0 most significant).
-__device__ __forceinline__ uint32_t cell_morton(uint32_t x, uint32_t y, uint32_t z, int l) {
-    uint32_t m = 0;
-    for (int b = l - 1; b >= 0; --b) m = (m << 3) | (((x >> b) & 1u) << 2) | (((y >> b) & 1u) << 1) | ((z >> b) & 1u);
-    return m;
+// 6-bit v spread so that bit b lands on bit 3b
+__device__ __forceinline__ uint32_t spread6(uint32_t v) {
+    v = (v | (v << 8)) & 0x300fu;
+    v = (v | (v << 4)) & 0x30c3u;
+    return (v | (v << 2)) & 0x9249u;
 }
 
-// First node of the walk: the node of the deepest cell (level <= kStartLevels) of the
-// tree rooted at `root` (tab: that tree's start table) that holds the cube of half width
-// Rb (box units) around C, which covers the whole search region.  Every particle
-// within the region lies in that cell and hence in that node's subtree (a node is the
-// set of particles whose keys share its cell's prefix).  Cells the tree did not reach
-// fall back to the nearest ancestor cell with a node.
-__device__ __forceinline__ int walk_start(const int32_t* __restrict__ tab, int root, uint32_t cx, uint32_t cy,
-                                          uint32_t cz, float Rb) {
+// First nodes of the walk, one per lane (-1: none): the nodes of the up to eight cells of
+// one octree level (<= kStartLevels) that the cube of half width Rb (box units) around C,
+// which covers the whole search region, can meet (tab: the start table of the tree rooted
+// at `root`).  The level is the deepest whose cells are at least as wide as the cube, so
+// it meets at most two per axis; every particle within the region lies in one of
+// those cells and hence in its node's subtree.  A cell without a node of its own is
+// empty, unless an ancestor is a leaf: then that leaf, once.
+__device__ __forceinline__ int walk_start(const SearchArgs& a, int root, uint32_t cx, uint32_t cy, uint32_t cz,
+                                          float Rb, int lane) {
+    static_assert(kStartLevels <= 6, "spread6 takes 6 bits per axis");
     // half width in fixed-point units, rounded up, plus the sub-unit offsets of the positions
     const float Ru = __fmul_ru(__fmul_ru(Rb, 1.000002f), 4294967296.0f);
-    if (!(Ru < 2147483648.0f)) return root;
-    const int64_t r = (int64_t)Ru + 3;
-    int lvl = kStartLevels;
-    const uint32_t c3[3] = {cx, cy, cz};
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-        const int64_t lo = (int64_t)c3[ax] - r, hi = (int64_t)c3[ax] + r;
-        if (lo < 0 || hi > 0xffffffffll) lvl = 0;   // the region wraps around the box
-        else lvl = min(lvl, __clz((uint32_t)lo ^ (uint32_t)hi));
+    int node = lane == 0 ? root : -1;
+    if (!a.start_tab || !(Ru < 1.07e9f)) return node;   // below a quarter of the box (2^30): level >= 1
+    const uint32_t r = (uint32_t)Ru + 3u;
+    int lvl = min(kStartLevels, __clz(2u * r));
+    const int sh = 32 - lvl;
+    const uint32_t x0 = (cx - r) >> sh, y0 = (cy - r) >> sh, z0 = (cz - r) >> sh;
+    const uint32_t x1 = (cx + r) >> sh, y1 = (cy + r) >> sh, z1 = (cz + r) >> sh;
+    const bool bx = lane & 4, by = lane & 2, bz = lane & 1;
+    node = -1;
+    if (lane < 8 && !(bx && x0 == x1) && !(by && y0 == y1) && !(bz && z0 == z1)) {
+        const int32_t* tab = a.start_tab + (size_t)root * kStartTableSize;
+        uint32_t m = (spread6(bx ? x1 : x0) << 2) | (spread6(by ? y1 : y0) << 1) | spread6(bz ? z1 : z0);
+        node = tab[start_table_offset(lvl) + m];
+        const bool own = node >= 0;
+        while (node < 0) {
+            m >>= 3;
+            --lvl;
+            node = lvl >= 1 ? tab[start_table_offset(lvl) + m] : root;
+        }
+        if (!own && a.nlink[node].z >= 0) node = -1;
     }
-    if (lvl < 1) return root;
-    uint32_t m = cell_morton(cx >> (32 - lvl), cy >> (32 - lvl), cz >> (32 - lvl), lvl);
-    for (; lvl >= 1; --lvl, m >>= 3) {
-        const int nd = tab[start_table_offset(lvl) + m];
-        if (nd >= 0) return nd;
-    }
-    return root;
+    const unsigned same = __match_any_sync(0xffffffffu, node);
+    return (node >= 0 && lane == __ffs(same) - 1) ? node : -1;
 }
 
 // The walk's stack and the ring of particle ranges it emits.  The stack lives in shared
@@ -1378,14 +1372,11 @@ struct Walk {
     __device__ __forceinline__ bool empty() const { return sp == 0 && gsp == 0; }
 };
 
-__device__ __forceinline__ Walk walk_begin(const SearchArgs& a, WalkSmem& W, int start, int lane) {
+__device__ __forceinline__ Walk walk_begin(const SearchArgs& a) {
     Walk w;
     w.spill = a.stack_spill + (size_t)(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * kSpillCap;
-    w.sp = 1;
-    w.gsp = 0;
+    w.sp = w.gsp = 0;
     w.e0 = w.e1 = w.done = w.total = 0;
-    if (lane == 0) W.stack[0] = (uint32_t)start << 3;   // one node
-    __syncwarp();
     return w;
 }
 
@@ -1394,40 +1385,13 @@ __device__ __forceinline__ bool walk_can_step(const SearchArgs& a, const Walk& w
     return !w.empty() && w.sp <= a.stack_cap - 32 && w.e1 - w.e0 <= kRangeCap - 32;
 }
 
-// One step: up to 32 nodes from the top of the stack are tested (open(cen, ext)); of the
-// open ones, leaves and nodes of at most `whole` particles emit their range, the
-// others push their children.
+// One node per lane (-1: none) is tested (open(cen, ext)); of the open ones, leaves and
+// nodes of at most `whole` particles emit their range, the others push their children.
 template <class Open>
-__device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk& w, int whole, LocalCounters& lc,
-                                          int lane, Open open_node) {
+__device__ __forceinline__ void walk_visit(const SearchArgs& a, WalkSmem& W, Walk& w, int node, int whole,
+                                           LocalCounters& lc, int lane, Open open_node) {
     const uint32_t lt = (1u << lane) - 1u;
-    if (w.sp == 0) {
-        const int m = min(w.gsp, 32);
-        if (lane < m) W.stack[lane] = w.spill[w.gsp - m + lane];
-        w.gsp -= m;
-        w.sp = m;
-        __syncwarp();
-    }
-    // take range entries from the top of the stack, up to 32 nodes
-    uint32_t ent = 0;
-    int ecnt = 0;
-    if (lane < w.sp) {
-        ent = W.stack[w.sp - 1 - lane];
-        ecnt = (int)(ent & 7u) + 1;
-    }
-    const int incl = warp_incl_scan(ecnt, lane);
-    const bool take = (lane < w.sp) && (incl <= 32);
-    const unsigned tm = __ballot_sync(0xffffffffu, take);
-    const int nent = __popc(tm);
-    const int nnodes = __shfl_sync(0xffffffffu, incl, nent - 1);
-    // node slot l belongs to the taken entry whose first slot is the highest entry
-    // start <= l (the starts as a bit mask; entries sit on lanes 0 .. nent-1)
-    const unsigned starts = __reduce_or_sync(0xffffffffu, take ? 1u << (incl - ecnt) : 0u);
-    const unsigned below = starts & ((2u << lane) - 1u);
-    const uint32_t my_ent = __shfl_sync(0xffffffffu, ent, max(__popc(below) - 1, 0));
-    w.sp -= nent;
-    const int node = lane < nnodes ? (int)(my_ent >> 3) + (lane - (31 - __clz(below))) : -1;
-    bool open = false, emit = false;
+    bool emit = false, push = false;
     int4 lk = make_int4(0, 0, -1, 0);
     int nch = 0;
     if (node >= 0) {
@@ -1435,10 +1399,12 @@ __device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk
         const float4 ext = a.next[node];
         lk = a.nlink[node];
         nch = __float_as_int(ext.w);
-        open = open_node(cen, ext);
+        const bool open = open_node(cen, ext);
         emit = open && lk.y > 0 && (lk.z < 0 || lk.y <= whole);
+        push = open && lk.z >= 0 && !emit;
     }
-    lc.nodes += (lane == 0) ? nnodes : 0;
+    const int nn = __popc(__ballot_sync(0xffffffffu, node >= 0));
+    lc.nodes += (lane == 0) ? nn : 0;
     const unsigned em = __ballot_sync(0xffffffffu, emit);
     if (em) {
         const int add = emit ? lk.y : 0;
@@ -1450,12 +1416,34 @@ __device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk
         w.e1 += __popc(em);
         w.total += __shfl_sync(0xffffffffu, pre, 31);
     }
-    const bool push = open && lk.z >= 0 && !emit;
     const unsigned pm = __ballot_sync(0xffffffffu, push);
     if (push) W.stack[w.sp + __popc(pm & lt)] = ((uint32_t)lk.z << 3) | (uint32_t)(nch - 1);
     w.sp += __popc(pm);
     lc.max_stack = max(lc.max_stack, w.sp + w.gsp);
     __syncwarp();
+}
+
+// One step: the children of up to four entries from the top of the stack, eight lanes to
+// an entry.
+template <class Open>
+__device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk& w, int whole, LocalCounters& lc,
+                                          int lane, Open open_node) {
+    if (w.sp == 0) {
+        const int m = min(w.gsp, 32);
+        if (lane < m) W.stack[lane] = w.spill[w.gsp - m + lane];
+        w.gsp -= m;
+        w.sp = m;
+        __syncwarp();
+    }
+    const int e = w.sp - 1 - (lane >> 3);
+    int node = -1;
+    if (e >= 0) {
+        const uint32_t ent = W.stack[e];
+        if ((uint32_t)(lane & 7) <= (ent & 7u)) node = (int)(ent >> 3) + (lane & 7);
+    }
+    w.sp = max(w.sp - 4, 0);
+    __syncwarp();
+    walk_visit(a, W, w, node, whole, lc, lane, open_node);
 }
 
 // When the next step could push more entries than the shared part holds, the oldest (up
@@ -1535,17 +1523,14 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
     const float emax = fmaxf(ex, fmaxf(ey, ez));
     const float reach = emax + (K::sym ? fmaxf(H, __uint_as_float(a.ncen[root].w)) : H);
     const bool wrap_safe = reach < 0.49f;
-    // the start table of the walk's tree (one per box of a forest, whose roots are the
-    // first nodes)
-    const int start = a.start_tab ? walk_start(a.start_tab + (size_t)root * kStartTableSize, root, cx, cy, cz, reach)
-                                  : root;
     auto open_node = [&](const uint4& cen, const float4& ext) {
         const float gap2 = node_gap2(cen, make_float4(__fadd_ru(ext.x, nx), __fadd_ru(ext.y, ny),
                                                       __fadd_ru(ext.z, nz), 0.0f), cx, cy, cz);
         if constexpr (K::sym) return gap2 <= radius2_units(fmaxf(H, __uint_as_float(cen.w)));
         else return gap2 <= H2u;
     };
-    Walk w = walk_begin(a, W, start, lane);
+    Walk w = walk_begin(a);
+    walk_visit(a, W, w, walk_start(a, root, cx, cy, cz, reach, lane), kWalkWhole, lc, lane, open_node);
     int ns = 0;   // candidates in the tile
     for (;;) {
         while (walk_can_step(a, w) && w.total - w.done < 64) walk_step(a, W, w, kWalkWhole, lc, lane, open_node);
@@ -1750,14 +1735,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_superset(SearchArgs a) 
         const float R = warp_max(rlane), hmax_g = warp_max(hlane);
         const float R2d = radius2_units(R);
         const float reach = SYM ? R + fmaxf(hmax_g, __uint_as_float(a.ncen[d.root].w)) : R;
-        const int start = a.start_tab ? walk_start(a.start_tab + (size_t)d.root * kStartTableSize, d.root, cx, cy, cz,
-                                                   reach)
-                                      : d.root;
         auto open_node = [&](const uint4& cen, const float4& ext) {
             const float R2 = SYM ? radius2_units(R + fmaxf(hmax_g, __uint_as_float(cen.w))) : R2d;
             return node_gap2(cen, ext, cx, cy, cz) <= R2;
         };
-        Walk w = walk_begin(a, W, start, lane);
+        Walk w = walk_begin(a);
+        walk_visit(a, W, w, walk_start(a, d.root, cx, cy, cz, reach, lane), 0, lc, lane, open_node);
         const int64_t pos = FILL ? a.x_off[gid] : 0;
         while (!w.empty() || w.total > w.done) {
             while (walk_can_step(a, w)) walk_step(a, W, w, 0, lc, lane, open_node);
