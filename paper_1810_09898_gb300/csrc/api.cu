@@ -285,6 +285,7 @@ int finish(Ctx* c, cudaStream_t s, int rc) {
     if (rc) return rc;
     err = (unsigned)c->host_small[1];
     std::memcpy(&dc, c->host_small + 8, sizeof(dc));
+    c->dev_walks = (int64_t)dc.walks;
     c->last.nodes_tested = (int64_t)dc.nodes;
     c->last.candidates = (int64_t)dc.cands;
     c->last.pair_tests = (int64_t)dc.tests;
@@ -466,6 +467,37 @@ int make_groups(Ctx* c, SearchArgs* a, const int32_t* U, int nu, int g, cudaStre
     a->groups = c->groups;
     a->ngroups = c->host_small[40];
     return SPHGRP_OK;
+}
+
+// A small work list is cut into smaller chunks while it would make fewer pieces than this
+// many per SM: below that the launch lasts as long as its slowest piece.
+constexpr int kSmallPieces = 16;
+
+// Work items of a search that computes: in count mode the pieces of the chunks (their number
+// stays on the device; a->ngroups bounds it), else the listed groups.
+int make_pieces(Ctx* c, SearchArgs* a, const int32_t* U, int nu, int g, cudaStream_t s) {
+    if (c->p.group_mode != SPHGRP_GROUP_COUNT) return make_groups(c, a, U, nu, g, s);
+    a->groups = nullptr;
+    a->ngroups = nu <= 0 ? 0 : (nu + g - 1) / g;
+    if (nu <= 0 || g <= 1) return SPHGRP_OK;
+    CutArgs ca;
+    std::memset(&ca, 0, sizeof(ca));
+    ca.U = U;
+    ca.pfix = c->pfix;
+    ca.h64 = c->h64;
+    ca.nu = nu;
+    ca.g = std::min(g, 32);
+    while (ca.g > 4 && nu < kSmallPieces * (int64_t)c->sm_count * ca.g) ca.g = (ca.g + 1) / 2;
+    ca.width = 32 / ca.g * ca.g;
+    ca.nwindows = (nu + ca.width - 1) / ca.width;
+    ca.split = (float)c->p.group_split;
+    ca.pieces = c->groups;
+    ca.cap = c->n_max + 1;
+    ca.npieces = c->work + 16;
+    a->pieces = c->groups;
+    a->pieces_cap = ca.cap;
+    a->npieces = c->work + 16;
+    return launch_cut_pieces(ca, c->sm_count, s);
 }
 
 SearchArgs base_args(Ctx* c) {
@@ -834,7 +866,7 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
         a.nu = nu;
         a.g = group_size;
         a.ngroups = (nu + group_size - 1) / group_size;
-        if (nu > 0 && (rc = make_groups(c, &a, U, nu, group_size, s))) return rc;
+        if (nu > 0 && (rc = make_pieces(c, &a, U, nu, group_size, s))) return rc;
         int* max_pass = c->work + 10;
         cudaMemsetAsync(max_pass, 0, sizeof(int), s);
         IterArgs it;
@@ -861,7 +893,7 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
         cudaMemcpyAsync(c->host_small + 2, nfail, sizeof(int), cudaMemcpyDeviceToHost, s);
         cudaMemcpyAsync(c->host_small + 3, max_pass, sizeof(int), cudaMemcpyDeviceToHost, s);
         rc = finish(c, s, 0);
-        c->last.walks = a.ngroups;
+        c->last.walks = c->dev_walks;
         c->last.members = nu;
         c->last.iterations = c->host_small[3];
         if (rc) return rc;
@@ -894,8 +926,8 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
         a.nu = nu;
         a.g = grouped ? group_size : 1;
         a.ngroups = grouped ? (nu + group_size - 1) / group_size : nu;
-        if (grouped && (rc = make_groups(c, &a, U, nu, group_size, s))) return rc;
-        walks += a.ngroups;
+        if (grouped && (rc = make_pieces(c, &a, U, nu, group_size, s))) return rc;
+        walks += grouped ? 0 : nu;
         members += nu;
         UpdateArgs ua;
         std::memset(&ua, 0, sizeof(ua));
@@ -1003,7 +1035,7 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
     }
     cudaMemcpyAsync(c->host_small + 2, nfail, sizeof(int), cudaMemcpyDeviceToHost, s);
     rc = finish(c, s, 0);
-    c->last.walks = walks;
+    c->last.walks = walks + c->dev_walks;
     c->last.members = members;
     c->last.iterations = std::min(std::max(it, list_passes), max_iter);
     if (rc) return rc;
@@ -1031,7 +1063,7 @@ int hydro_force(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, const dou
     a.nu = nu;
     a.g = grouped ? group_size : 1;
     a.ngroups = grouped ? (nu + group_size - 1) / group_size : nu;
-    if (grouped && (rc = make_groups(c, &a, c->act, nu, group_size, s))) return rc;
+    if (grouped && (rc = make_pieces(c, &a, c->act, nu, group_size, s))) return rc;
     a.o_res4 = c->res4;
     a.o_rcnt = c->acc_n;
     timer_begin(c, s);
@@ -1043,9 +1075,10 @@ int hydro_force(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, const dou
                                                           nngb);
         note_launch();
     }
-    c->last.walks = a.ngroups;
+    rc = finish(c, s, 0);
+    c->last.walks = grouped ? c->dev_walks : nu;
     c->last.members = nu;
-    return finish(c, s, 0);
+    return rc;
 }
 
 }  // namespace sphgrp
@@ -1103,7 +1136,7 @@ int sphgrp_velocity_derivs(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active
     a.nu = nu;
     a.g = group_size;
     a.ngroups = (nu + group_size - 1) / group_size;
-    if ((rc = make_groups(c, &a, c->act, nu, group_size, s))) return rc;
+    if ((rc = make_pieces(c, &a, c->act, nu, group_size, s))) return rc;
     a.o_res4 = c->res4;
     timer_begin(c, s);
     rc = launch_search(a, kKindVelocity, kAcc, true, c->sm_count, s);
@@ -1113,9 +1146,10 @@ int sphgrp_velocity_derivs(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active
         k_out_vel<<<blocks_for(n_act, 256), 256, 0, s>>>(n_act, active, c->n, c->rank_of, c->res4, divv, curlv);
         note_launch();
     }
-    c->last.walks = a.ngroups;
+    rc = finish(c, s, 0);
+    c->last.walks = c->dev_walks;
     c->last.members = nu;
-    return finish(c, s, 0);
+    return rc;
 }
 
 int sphgrp_get_launch_log(sphgrp_ctx* ctx, int cap, int64_t* members, int64_t* candidates,

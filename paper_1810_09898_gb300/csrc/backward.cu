@@ -189,7 +189,7 @@ extern "C" int sphgrp_backward(sphgrp_ctx* ctx, const double* h, const float* ve
     a.nu = nu;
     a.g = group_size;
     a.ngroups = (nu + group_size - 1) / group_size;
-    if ((rc = make_groups(c, &a, c->act, nu, group_size, s))) return rc;
+    if ((rc = make_pieces(c, &a, c->act, nu, group_size, s))) return rc;
 
     // 1. density sums at the given h: rho, rho', rho''
     SearchArgs ad = a;
@@ -229,7 +229,8 @@ extern "C" int sphgrp_backward(sphgrp_ctx* ctx, const double* h, const float* ve
     if (rc) return rc;
     if ((rc = launch_bwd_combine(c, g_pos, g_vel, g_m, s))) return rc;
     rc = check_cuda(cudaGetLastError(), "backward kernels");
-    c->last.walks = (with_acc ? 3 : 2) * (int64_t)a.ngroups;
+    rc = finish(c, s, rc);
+    c->last.walks = c->dev_walks;
     c->last.members = (with_acc ? 3 : 2) * (int64_t)nu;
-    return finish(c, s, rc);
+    return rc;
 }

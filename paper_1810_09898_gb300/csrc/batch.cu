@@ -32,10 +32,9 @@ constexpr int kMinBatchLeaf = 8;      // smallest per-class leaf size: the fores
 // device scalars of a batch call
 enum Scalar {
     kNu = 0,         // active particles
-    kNChunk = 1,     // chunks of the active list
-    kNGroups = 2,    // groups of the active list
-    kNChunkAll = 3,  // chunks of the all-particle list (backward)
-    kNGroupsAll = 4, // groups of the all-particle list
+    kNWindows = 1,   // windows of the list being cut
+    kNPieces = 8,    // pieces of the active list: small, large
+    kNPiecesAll = 10,  // pieces of the all-particle list (backward)
     kNFail = 5,      // particles that did not converge
     kTot = 6,        // scan total scratch
     kNScalars = 16
@@ -74,13 +73,10 @@ struct Batch {
     int32_t* U_all = nullptr;       // identity work list
     int32_t* dsc = nullptr;         // device scalars
     int32_t* box_act = nullptr;     // nbox + 1: first entry of the box in the work list
-    int32_t* box_chunk = nullptr;   // nbox + 1: first chunk of the box
-    int4* chunks = nullptr;         // (first entry, count, box, -)
-    int32_t* ccnt = nullptr;        // groups per chunk
-    int32_t* coff = nullptr;
-    int2* gtmp = nullptr;           // split output
-    int4* groups = nullptr;         // active groups
-    int4* groups_all = nullptr;     // all-particle groups (backward)
+    int32_t* box_chunk = nullptr;   // nbox + 1: first window of the box
+    int4* chunks = nullptr;         // windows: (first entry, count, box, configuration)
+    int4* groups = nullptr;         // active pieces
+    int4* groups_all = nullptr;     // all-particle pieces (backward)
     float4* hyd0b = nullptr;        // hydro inputs of the backward (all particles at h)
     float4* hyd1b = nullptr;
     int32_t* start_tabs = nullptr;  // walk start tables, one per box
@@ -129,8 +125,14 @@ __global__ void k_batch_compact(int64_t n, const int32_t* __restrict__ flag, con
         if (flag[r]) U[pos[r]] = (int32_t)r;
 }
 
+// entries of a box's window: whole chunks of its group size, at most 32
+__device__ __forceinline__ int window_width(int cfg) {
+    const int g = min(cfg & 0xff, 32);
+    return 32 / g * g;
+}
+
 // One warp: per box, the first entry of the work list (from the flag scan, or the box
-// offsets for the all-particle list) and the chunk offsets (chunks of g entries).
+// offsets for the all-particle list) and the offsets of its windows.
 __global__ void k_box_chunks(int nbox, const int64_t* __restrict__ box_off, const int32_t* __restrict__ scan,
                              const int32_t* __restrict__ nu_dev, int all, int64_t n,
                              const int32_t* __restrict__ box_g, int32_t* __restrict__ box_act,
@@ -144,8 +146,8 @@ __global__ void k_box_chunks(int nbox, const int64_t* __restrict__ box_off, cons
         if (b < nbox) {
             const int a0 = all ? (int)box_off[b] : scan[box_off[b]];
             const int a1 = (b + 1 < nbox) ? (all ? (int)box_off[b + 1] : scan[box_off[b + 1]]) : nu;
-            const int g = box_g[b] & 0xff;
-            ch = (a1 - a0 + g - 1) / g;
+            const int wd = window_width(box_g[b]);
+            ch = (a1 - a0 + wd - 1) / wd;
             box_act[b] = a0;
         }
         const int inc = warp_scan_incl(ch, lane);
@@ -169,75 +171,9 @@ __global__ void k_chunk_desc(int nbox, const int32_t* __restrict__ box_act, cons
             const int mid = (lo + hi) >> 1;
             if (box_chunk[mid] <= c) lo = mid; else hi = mid;
         }
-        const int g = box_g[lo] & 0xff;
-        const int start = box_act[lo] + (c - box_chunk[lo]) * g;
-        chunks[c] = make_int4(start, min(g, box_act[lo + 1] - start), lo, 0);
-    }
-}
-
-// The chunk cut in halves (recursively) while the group's search sphere exceeds split
-// times its members' spheres in volume (as k_split_groups); output at the chunk's
-// first entry (a chunk of c entries gives at most c groups).
-__global__ void k_split_chunks(const int32_t* __restrict__ U, const int4* __restrict__ chunks,
-                               const int32_t* __restrict__ nchunk, const uint4* __restrict__ pfix,
-                               const double* __restrict__ h64, const float* __restrict__ box_split,
-                               int2* __restrict__ tmp, int32_t* __restrict__ cnt) {
-    const int nc = *nchunk;
-    for (int ch = blockIdx.x * blockDim.x + threadIdx.x; ch < nc; ch += gridDim.x * blockDim.x) {
-        const int4 C = chunks[ch];
-        const float split = box_split[C.z];
-        int2 st[16];
-        int sp = 0, ng = 0;
-        st[sp++] = make_int2(C.x, C.x + C.y);
-        while (sp > 0) {
-            const int2 r = st[--sp];
-            const int s = r.x, e = r.y;
-            bool keep = (e - s == 1) || split <= 0.0f;
-            if (!keep) {
-                const uint4 P0 = pfix[U[s]];
-                int lox = 0, loy = 0, loz = 0, hix = 0, hiy = 0, hiz = 0;
-                float hmin = (float)h64[U[s]];
-                for (int k = s + 1; k < e; ++k) {
-                    const int rk = U[k];
-                    const uint4 P = pfix[rk];
-                    const int dx = (int32_t)(P.x - P0.x), dy = (int32_t)(P.y - P0.y), dz = (int32_t)(P.z - P0.z);
-                    lox = min(lox, dx); hix = max(hix, dx);
-                    loy = min(loy, dy); hiy = max(hiy, dy);
-                    loz = min(loz, dz); hiz = max(hiz, dz);
-                    hmin = fminf(hmin, (float)h64[rk]);
-                }
-                const float ext = fmaxf(fmaxf((float)((int64_t)hix - lox), (float)((int64_t)hiy - loy)),
-                                        (float)((int64_t)hiz - loz)) * kUnitToBox;
-                const float rel = fmaf(0.8660254f, ext / hmin, 1.0f);
-                keep = rel * rel * rel <= split * (float)(e - s);
-            }
-            if (keep) {
-                tmp[C.x + ng++] = make_int2(s, e - s);
-            } else if (sp + 2 <= 16) {
-                const int mid = s + (e - s + 1) / 2;
-                st[sp++] = make_int2(mid, e);
-                st[sp++] = make_int2(s, mid);
-            } else {
-                tmp[C.x + ng++] = make_int2(s, e - s);
-            }
-        }
-        cnt[ch] = ng;
-    }
-}
-
-__global__ void k_gather_chunk_groups(const int4* __restrict__ chunks, const int32_t* __restrict__ nchunk,
-                                      const int32_t* __restrict__ cnt, const int32_t* __restrict__ off,
-                                      const int2* __restrict__ tmp, const int32_t* __restrict__ box_g,
-                                      int4* __restrict__ groups) {
-    const int nc = *nchunk;
-    for (int ch = blockIdx.x * blockDim.x + threadIdx.x; ch < nc; ch += gridDim.x * blockDim.x) {
-        const int4 C = chunks[ch];
-        const int o = off[ch];
-        const int gw = box_g[C.z];
-        for (int k = 0; k < cnt[ch]; ++k) {
-            const int2 t = tmp[C.x + k];
-            groups[o + k] = make_int4(t.x, t.y, C.z, gw);
-        }
+        const int wd = window_width(box_g[lo]);
+        const int start = box_act[lo] + (c - box_chunk[lo]) * wd;
+        chunks[c] = make_int4(start, min(wd, box_act[lo + 1] - start), lo, box_g[lo]);
     }
 }
 
@@ -271,45 +207,47 @@ void drop_graph(Batch* b) {
     b->cap_flags = -1;
 }
 
-// Work list U (active ranks, or all ranks), its chunks, split groups and the group
-// count on the device.
+// Work list (active ranks, or all ranks), its windows and their pieces, counted on the device.
 int make_batch_groups(Batch* b, bool all, int only_cls, const uint8_t* active, cudaStream_t s) {
     Ctx* c = b->c;
     const int64_t n = b->n;
     int rc = SPHGRP_OK;
-    const int32_t* U = b->U_all;
-    int32_t* nchunk = b->dsc + (all ? kNChunkAll : kNChunk);
-    int32_t* ngroups = b->dsc + (all ? kNGroupsAll : kNGroups);
-    int4* groups = all ? b->groups_all : b->groups;
     if (!all) {
         k_batch_flags<<<kGrid, 256, 0, s>>>(n, c->perm, active, b->box_of_rank, b->box_cls, only_cls, c->flag);
         note_launch();
         if ((rc = exclusive_scan_i32(c, c->flag, c->scan, n, b->dsc + kNu, s))) return rc;
         k_batch_compact<<<kGrid, 256, 0, s>>>(n, c->flag, c->scan, c->act);
         note_launch();
-        U = c->act;
     }
     k_box_chunks<<<1, 32, 0, s>>>(b->nbox, b->box_off, c->scan, b->dsc + kNu, all ? 1 : 0, n, b->box_g, b->box_act,
-                                  b->box_chunk, nchunk);
+                                  b->box_chunk, b->dsc + kNWindows);
     note_launch();
-    k_chunk_desc<<<kGrid, 256, 0, s>>>(b->nbox, b->box_act, b->box_chunk, b->box_g, nchunk, b->chunks);
+    k_chunk_desc<<<kGrid, 256, 0, s>>>(b->nbox, b->box_act, b->box_chunk, b->box_g, b->dsc + kNWindows, b->chunks);
     note_launch();
-    k_split_chunks<<<kGrid, 128, 0, s>>>(U, b->chunks, nchunk, c->pfix, c->h64, b->box_split, b->gtmp, b->ccnt);
-    note_launch();
-    if ((rc = exclusive_scan_i32_dev(c, b->ccnt, b->coff, nchunk, nullptr, n, ngroups, s))) return rc;
-    k_gather_chunk_groups<<<kGrid, 256, 0, s>>>(b->chunks, nchunk, b->ccnt, b->coff, b->gtmp, b->box_g, groups);
-    note_launch();
+    CutArgs ca;
+    std::memset(&ca, 0, sizeof(ca));
+    ca.U = all ? b->U_all : c->act;
+    ca.pfix = c->pfix;
+    ca.h64 = c->h64;
+    ca.windows = b->chunks;
+    ca.nwindows_dev = b->dsc + kNWindows;
+    ca.box_split = b->box_split;
+    ca.pieces4 = all ? b->groups_all : b->groups;
+    ca.cap = n;
+    ca.npieces = b->dsc + (all ? kNPiecesAll : kNPieces);
+    if ((rc = launch_cut_pieces(ca, c->sm_count, s))) return rc;
     return check_cuda(cudaGetLastError(), "batch groups");
 }
 
 SearchArgs batch_args(Batch* b, bool all) {
     SearchArgs a = base_args(b->c);
     a.U = all ? b->U_all : b->c->act;
-    a.nu = (int)b->n;   // bound only; groups4 carries the ranges
+    a.nu = (int)b->n;   // bound only; the pieces carry the ranges
     a.g = b->max_g;
-    a.groups4 = all ? b->groups_all : b->groups;
+    a.pieces4 = all ? b->groups_all : b->groups;
+    a.pieces_cap = b->n;
+    a.npieces = b->dsc + (all ? kNPiecesAll : kNPieces);
     a.start_tab = b->start_tabs;   // one start table per box, indexed by the box's root
-    a.ngroups_dev = b->dsc + (all ? kNGroupsAll : kNGroups);
     return a;
 }
 
@@ -401,7 +339,7 @@ int read_status(Batch* b, int flags) {
     c->last.fp64_retests = (int64_t)dc.retests;
     c->last.max_stack = (int64_t)dc.max_stack;
     const bool bwd = (flags & SPHGRP_BATCH_BACKWARD) != 0;
-    c->last.walks = 2 * (int64_t)sc[kNGroups] + (bwd ? 3 * (int64_t)sc[kNGroupsAll] : 0);
+    c->last.walks = (int64_t)dc.walks;
     c->last.members = 2 * (int64_t)sc[kNu] + (bwd ? 3 * b->n : 0);
     c->last.iterations = b->replayed ? 1 : 0;
     c->last.search_launches = b->step_kernels;
@@ -501,9 +439,6 @@ int sphgrp_batch_create(sphgrp_batch** out, const sphgrp_params* params, int nbo
     rc = rc ? rc : dalloc(&b->box_act, nbox + 1);
     rc = rc ? rc : dalloc(&b->box_chunk, nbox + 1);
     rc = rc ? rc : dalloc(&b->chunks, n);
-    rc = rc ? rc : dalloc(&b->ccnt, n + 1);
-    rc = rc ? rc : dalloc(&b->coff, n + 1);
-    rc = rc ? rc : dalloc(&b->gtmp, n);
     rc = rc ? rc : dalloc(&b->groups, n);
     rc = rc ? rc : dalloc(&b->groups_all, n);
     rc = rc ? rc : dalloc(&b->hyd0b, n);
@@ -543,7 +478,7 @@ int sphgrp_batch_destroy(sphgrp_batch* w) {
     drop_graph(b);
     void* ptrs[] = {b->box_off, b->box_g, b->box_split, b->box_cls, b->box_of_rank, b->tmp64a, b->tmp64b,
                     b->tmp32a, b->tmp32b, b->lvl, b->blo, b->bhi, b->U_all, b->dsc, b->box_act, b->box_chunk,
-                    b->chunks, b->ccnt, b->coff, b->gtmp, b->groups, b->groups_all, b->hyd0b, b->hyd1b,
+                    b->chunks, b->groups, b->groups_all, b->hyd0b, b->hyd1b,
                     b->start_tabs};
     for (void* p : ptrs)
         if (p) cudaFree(p);

@@ -35,10 +35,14 @@ constexpr int kPartMax = 32;                   // members searched at once (one 
 constexpr int kWalkWhole = 32;
 
 
-// per-lane counts of one launch (nodes and cands on lane 0 only); summed in 64 bits
+// per-lane counts of one launch, summed in 64 bits
 struct LocalCounters {
-    unsigned nodes = 0, cands = 0, tests = 0, pairs = 0, retests = 0;
-    int max_stack = 0;
+    unsigned tests = 0, pairs = 0, retests = 0;
+};
+// counts of a warp's walks, in its shared memory (they would hold registers through every
+// search)
+struct WalkCounters {
+    unsigned walks, nodes, cands, deep;
 };
 
 __device__ __forceinline__ unsigned long long warp_sum(unsigned v) {
@@ -48,18 +52,18 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned v) {
     return t;
 }
 
-__device__ __forceinline__ void flush_counters(const SearchArgs& a, const LocalCounters& lc, int lane) {
+__device__ __forceinline__ void flush_counters(const SearchArgs& a, const LocalCounters& lc, const WalkCounters& wc,
+                                               int lane) {
     // warp-reduce then one atomic per warp
-    const unsigned long long nodes = warp_sum(lc.nodes), cands = warp_sum(lc.cands), tests = warp_sum(lc.tests),
-                             pairs = warp_sum(lc.pairs), retests = warp_sum(lc.retests);
-    const int deep = __reduce_max_sync(0xffffffffu, lc.max_stack);
+    const unsigned long long tests = warp_sum(lc.tests), pairs = warp_sum(lc.pairs), retests = warp_sum(lc.retests);
     if (lane == 0) {
-        if (nodes) atomicAdd(&a.ctr->nodes, nodes);
-        if (cands) atomicAdd(&a.ctr->cands, cands);
+        if (wc.walks) atomicAdd(&a.ctr->walks, (unsigned long long)wc.walks);
+        if (wc.nodes) atomicAdd(&a.ctr->nodes, (unsigned long long)wc.nodes);
+        if (wc.cands) atomicAdd(&a.ctr->cands, (unsigned long long)wc.cands);
         if (tests) atomicAdd(&a.ctr->tests, tests);
         if (pairs) atomicAdd(&a.ctr->pairs, pairs);
         if (retests) atomicAdd(&a.ctr->retests, retests);
-        atomicMax(&a.ctr->max_stack, (unsigned long long)deep);
+        atomicMax(&a.ctr->max_stack, (unsigned long long)wc.deep);
     }
 }
 
@@ -125,6 +129,10 @@ __device__ __forceinline__ float rcp_fast(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+
+// q = r / h rounded on its own: fused into the 1 - q of the splines it would differ by an
+// ulp between kernels that inline the same pair terms
+__device__ __forceinline__ float q_of(float r, float hinv) { return __fmul_rn(r, hinv); }
 
 // M4 slope w'(q) (zero for q >= 1; q >= 0)
 __device__ __forceinline__ float m4_slope(float q) {
@@ -528,7 +536,7 @@ struct DAdjTile : SymTile {
 
 // kind policies; min_blocks: resident blocks per SM (register budget; 0: compiler's choice)
 struct KDens {
-    static constexpr int min_blocks = 8;
+    static constexpr int min_blocks = 7;
     static constexpr int id = 0;
     static constexpr bool sym = false;
     using Member = DMember;
@@ -542,7 +550,7 @@ struct KDens2 {
     using Tile = PlainTile;
 };
 struct KDensVel {
-    static constexpr int min_blocks = 6;
+    static constexpr int min_blocks = 5;
     static constexpr int id = kKindDensityVel;
     static constexpr bool sym = false;
     using Member = DVMember;
@@ -563,7 +571,7 @@ struct KHydro {
     using Tile = HydroTile;
 };
 struct KHAdj {
-    static constexpr int min_blocks = 0;
+    static constexpr int min_blocks = 4;
     static constexpr int id = 2;
     static constexpr bool sym = true;
     using Member = HAMember;
@@ -715,7 +723,7 @@ __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float3
     float dx, dy, dz, r2;
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
     M.n += in ? 1 : 0;
-    if (MODE == kAcc) density_terms(M, in ? mj : 0.0f, r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)) * M.hinv);
+    if (MODE == kAcc) density_terms(M, in ? mj : 0.0f, q_of(r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)), M.hinv));
     else if (MODE == kFill && in) export_pair(M, a, crank);
 }
 
@@ -724,7 +732,7 @@ __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float3
 template <class Mem>
 __device__ __forceinline__ void velocity_terms(Mem& M, float mj, float4 vj, float dx, float dy, float dz, float r2) {
     const float rinv = rsqrt_fast(r2);
-    const float c = -M.sk * m4_slope(r2 * rinv * M.hinv) * rinv;   // x_i - x_j = -d
+    const float c = -M.sk * m4_slope(q_of(r2 * rinv, M.hinv)) * rinv;   // x_i - x_j = -d
     const float gx = c * dx, gy = c * dy, gz = c * dz;
     const float vx = M.vx - vj.x, vy = M.vy - vj.y, vz = M.vz - vj.z;
     M.pd = fmaf(-mj, fmaf(vx, gx, fmaf(vy, gy, vz * gz)), M.pd);
@@ -741,7 +749,7 @@ __device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, f
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
     M.n += in ? 1 : 0;
     if (MODE != kAcc) return;
-    density_terms(M, in ? mj : 0.0f, r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)) * M.hinv);
+    density_terms(M, in ? mj : 0.0f, q_of(r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)), M.hinv));
     if (in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
@@ -809,8 +817,8 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
     if (MODE != kAcc || !(in && r2 > 0.0f)) return;
     const float rinv = rsqrt_fast(r2);
     const float r = r2 * rinv;
-    const float dWi = M.sk * m4_slope(r * M.hinv);
-    const float dWj = kSkernel * (hh.z * hh.z) * (hh.z * hh.z) * m4_slope(r * hh.z);
+    const float dWi = M.sk * m4_slope(q_of(r, M.hinv));
+    const float dWj = kSkernel * (hh.z * hh.z) * (hh.z * hh.z) * m4_slope(q_of(r, hh.z));
     const float rx = -dx, ry = -dy, rz = -dz;  // r_ij = x_i - x_j
     const float vx = M.vx - v.x, vy = M.vy - v.y, vz = M.vz - v.z;
     const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
@@ -849,7 +857,7 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     const float D0 = -dx, D1 = -dy, D2 = -dz;   // x_k - x_j
     const float e0 = D0 * rinv, e1 = D1 * rinv, e2 = D2 * rinv;
     float wk_, dwk, d2wk, wj_, dwj, d2wj;
-    const float qk = r * M.hinv, qj = r * hh.z;
+    const float qk = q_of(r, M.hinv), qj = q_of(r, hh.z);
     m4_shape2(qk, wk_, dwk, d2wk);
     m4_shape2(qj, wj_, dwj, d2wj);
     const float Wr_k = M.sk * dwk, Wr_j = hh.w * dwj;
@@ -921,7 +929,7 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
     const float rinv = r2 > 0.0f ? rsqrt_fast(r2) : 0.0f;
     const float r = r2 * rinv;
     float wk_, dwk, d2wk, wj_, dwj, d2wj;
-    const float qk = r * M.hinv, qj = r * d.z;
+    const float qk = q_of(r, M.hinv), qj = q_of(r, d.z);
     m4_shape2(qk, wk_, dwk, d2wk);
     m4_shape2(qj, wj_, dwj, d2wj);
     // k as a neighbour of j: rho_j gains m_k W(r, h_j), dRho_j/dh_j gains m_k W_h(r, h_j)
@@ -1116,7 +1124,12 @@ __device__ __forceinline__ void write_result(const DAMember& D, const SearchArgs
 struct alignas(16) WalkSmem {
     uint32_t stack[kStackCap];   // node ranges: (first child << 3) | (count - 1)
     int2 ranges[kRangeCap];      // ring of pending particle ranges {first rank - flat start, flat start}
+    WalkCounters ctr;            // written by lane 0
 };
+
+__device__ __forceinline__ void clear_counters(WalkSmem& W, int lane) {
+    if (lane == 0) W.ctr = WalkCounters{0u, 0u, 0u, 0u};
+}
 
 __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 #pragma unroll
@@ -1246,36 +1259,64 @@ __device__ __forceinline__ void filter_tile(typename K::Tile& T, const Layout& L
     if (MODE == kAcc) flush(Mb);
 }
 
-// Work item of the grouped kernels: members U[base, base + cnt), the walk's start node
-// (a root of the forest) and the slice limit.
+// Work item of the grouped kernels: members U[base, base + cnt), or the set bits of `mask`
+// as offsets from base (pieces of at most 32 entries; mask 0: the range), the walk's
+// start node (a root of the forest) and the slice limit.
 struct GroupDesc {
-    int base, cnt, root, smax;
+    int base, cnt;
+    uint32_t mask;
+    int root, smax;
 };
 
-__device__ __forceinline__ GroupDesc group_desc(const SearchArgs& a, int gid) {
+// entry of the piece list for item gid: the large pieces, listed from the end, go first
+__device__ __forceinline__ int64_t piece_index(const SearchArgs& a, int gid, int nlarge) {
+    return gid < nlarge ? a.pieces_cap - 1 - gid : gid - nlarge;
+}
+
+__device__ __forceinline__ GroupDesc group_desc(const SearchArgs& a, int gid, int nlarge) {
     GroupDesc d;
     d.root = 0;
     d.smax = 32;
-    if (a.groups4) {
-        const int4 G = a.groups4[gid];
+    d.mask = 0u;
+    if (a.pieces4) {
+        const int4 G = a.pieces4[piece_index(a, gid, nlarge)];
         d.base = G.x;
-        d.cnt = G.y;
+        d.mask = (uint32_t)G.y;
+        d.cnt = __popc(d.mask);
         d.root = G.z;
-        d.smax = (G.w >> 8) & 0xff;   // bits 16.. carry the box's leaf size
-        if (d.smax >= 4) d.smax = 32;   // 4, the largest limit that can be set: all lanes
-    } else if (a.groups) {
-        const int2 G = a.groups[gid];
+        const int s = (G.w >> 8) & 0xff;   // bits 16.. carry the box's leaf size
+        d.smax = s >= 4 ? 32 : s;          // 4, the largest limit that can be set: all lanes
+    } else if (a.pieces) {
+        const int2 G = a.pieces[piece_index(a, gid, nlarge)];
         d.base = G.x;
-        d.cnt = G.y;
+        d.mask = (uint32_t)G.y;
+        d.cnt = __popc(d.mask);
     } else {
-        d.base = gid * a.g;
-        d.cnt = min(a.g, a.nu - d.base);
+        // a group of more than 32 members is `parts` items of 32
+        const int k = a.parts > 1 ? gid / a.parts : gid;
+        if (a.groups) {
+            const int2 G = a.groups[k];
+            d.base = G.x;
+            d.cnt = G.y;
+        } else {
+            d.base = k * a.g;
+            d.cnt = min(a.g, a.nu - d.base);
+        }
+        if (a.parts > 1) {
+            const int b = (gid - k * a.parts) * kPartMax;
+            d.base += b;
+            d.cnt = min(d.cnt - b, kPartMax);
+        }
     }
     return d;
 }
 
-__device__ __forceinline__ int group_count(const SearchArgs& a) {
-    return a.ngroups_dev ? *a.ngroups_dev : a.ngroups;
+// items of the launch, and how many of them are large pieces
+__device__ __forceinline__ int group_count(const SearchArgs& a, int& nlarge) {
+    nlarge = 0;
+    if (!a.npieces) return a.ngroups * max(a.parts, 1);
+    nlarge = a.npieces[1];
+    return a.npieces[0] + nlarge;
 }
 
 // Group centre: the fixed-point position of the lowest lane that holds a member, or the
@@ -1365,16 +1406,18 @@ __device__ __forceinline__ int walk_start(const SearchArgs& a, int root, uint32_
 // the shared part when that runs empty.  The ranges, laid end to end in walk order, number
 // the candidates flat: [done, total) are pending, in ring entries [e0, e1).
 struct Walk {
-    uint32_t* spill;
     int sp, gsp;
     int e0, e1, done, total;
 
     __device__ __forceinline__ bool empty() const { return sp == 0 && gsp == 0; }
 };
 
-__device__ __forceinline__ Walk walk_begin(const SearchArgs& a) {
+__device__ __forceinline__ uint32_t* walk_overflow(const SearchArgs& a) {
+    return a.stack_spill + (size_t)(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * kSpillCap;
+}
+
+__device__ __forceinline__ Walk walk_begin() {
     Walk w;
-    w.spill = a.stack_spill + (size_t)(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * kSpillCap;
     w.sp = w.gsp = 0;
     w.e0 = w.e1 = w.done = w.total = 0;
     return w;
@@ -1385,26 +1428,29 @@ __device__ __forceinline__ bool walk_can_step(const SearchArgs& a, const Walk& w
     return !w.empty() && w.sp <= a.stack_cap - 32 && w.e1 - w.e0 <= kRangeCap - 32;
 }
 
-// One node per lane (-1: none) is tested (open(cen, ext)); of the open ones, leaves and
-// nodes of at most `whole` particles emit their range, the others push their children.
+// One node per lane (-1: none) is tested (open_node(have, cen, ext, candidates so far),
+// called by all lanes); of the open ones, leaves and nodes of at most `whole` particles emit
+// their range, the others push their children.
 template <class Open>
 __device__ __forceinline__ void walk_visit(const SearchArgs& a, WalkSmem& W, Walk& w, int node, int whole,
-                                           LocalCounters& lc, int lane, Open open_node) {
+                                           int lane, Open open_node) {
     const uint32_t lt = (1u << lane) - 1u;
     bool emit = false, push = false;
     int4 lk = make_int4(0, 0, -1, 0);
     int nch = 0;
+    uint4 cen = make_uint4(0u, 0u, 0u, 0u);
+    float4 ext = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (node >= 0) {
-        const uint4 cen = a.ncen[node];
-        const float4 ext = a.next[node];
+        cen = a.ncen[node];
+        ext = a.next[node];
         lk = a.nlink[node];
         nch = __float_as_int(ext.w);
-        const bool open = open_node(cen, ext);
-        emit = open && lk.y > 0 && (lk.z < 0 || lk.y <= whole);
-        push = open && lk.z >= 0 && !emit;
     }
+    const bool open = open_node(node >= 0, cen, ext, w.total);
+    emit = open && lk.y > 0 && (lk.z < 0 || lk.y <= whole);
+    push = open && lk.z >= 0 && !emit;
     const int nn = __popc(__ballot_sync(0xffffffffu, node >= 0));
-    lc.nodes += (lane == 0) ? nn : 0;
+    if (lane == 0) W.ctr.nodes += nn;
     const unsigned em = __ballot_sync(0xffffffffu, emit);
     if (em) {
         const int add = emit ? lk.y : 0;
@@ -1419,18 +1465,18 @@ __device__ __forceinline__ void walk_visit(const SearchArgs& a, WalkSmem& W, Wal
     const unsigned pm = __ballot_sync(0xffffffffu, push);
     if (push) W.stack[w.sp + __popc(pm & lt)] = ((uint32_t)lk.z << 3) | (uint32_t)(nch - 1);
     w.sp += __popc(pm);
-    lc.max_stack = max(lc.max_stack, w.sp + w.gsp);
+    if (lane == 0) W.ctr.deep = max(W.ctr.deep, (unsigned)(w.sp + w.gsp));
     __syncwarp();
 }
 
 // One step: the children of up to four entries from the top of the stack, eight lanes to
 // an entry.
 template <class Open>
-__device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk& w, int whole, LocalCounters& lc,
-                                          int lane, Open open_node) {
+__device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk& w, int whole, int lane,
+                                          Open open_node) {
     if (w.sp == 0) {
         const int m = min(w.gsp, 32);
-        if (lane < m) W.stack[lane] = w.spill[w.gsp - m + lane];
+        if (lane < m) W.stack[lane] = walk_overflow(a)[w.gsp - m + lane];
         w.gsp -= m;
         w.sp = m;
         __syncwarp();
@@ -1443,7 +1489,7 @@ __device__ __forceinline__ void walk_step(const SearchArgs& a, WalkSmem& W, Walk
     }
     w.sp = max(w.sp - 4, 0);
     __syncwarp();
-    walk_visit(a, W, w, node, whole, lc, lane, open_node);
+    walk_visit(a, W, w, node, whole, lane, open_node);
 }
 
 // When the next step could push more entries than the shared part holds, the oldest (up
@@ -1453,7 +1499,7 @@ __device__ __forceinline__ void walk_spill(const SearchArgs& a, WalkSmem& W, Wal
     if (w.sp <= a.stack_cap - 32) return;
     const int ev = min(32, w.sp);
     if (w.gsp + ev > kSpillCap) atomicOr(a.err, kErrStack);
-    else if (lane < ev) w.spill[w.gsp + lane] = W.stack[lane];
+    else if (lane < ev) walk_overflow(a)[w.gsp + lane] = W.stack[lane];
     __syncwarp();
     for (int b = 0; b < w.sp - ev; b += 32) {
         const uint32_t v = (b + lane < w.sp - ev) ? W.stack[ev + b + lane] : 0u;
@@ -1484,6 +1530,38 @@ __device__ __forceinline__ int walk_take(WalkSmem& W, Walk& w, int lane, int& ra
     w.done += take;
     __syncwarp();
     return take;
+}
+
+// A group beside a dense clump can have the clump within H of its box, and thousands of
+// candidates, though no member's own sphere meets it.  Testing every node against every
+// member costs about as much as the rest of a step per 8 members, so it starts when a walk
+// has found kRefineBase + kRefinePerMember * members candidates (three times what an even
+// density gives).  A density pass of 414k actives in runs among 2.1M clustered particles
+// had groups of up to 10^4 candidates for 345 pairs, which ran for 0.4 ms of its 0.7 ms.
+constexpr int kRefineBase = 256;
+constexpr int kRefinePerMember = 48;
+
+// Whether every lane's node (centre d relative to the group's, half extents in units, largest
+// h) meets a member's sphere (lane k < gw: {m, radius}, radius 0: none).  Called by all
+// lanes; not inlined, so that its registers are not held by the walk, which rarely comes
+// here.  Margins of 1e-6 cover the FP32 errors of the coordinates.
+__device__ __noinline__ bool meets_members(float3 d, float4 ext, float hnode, float4 mine, int gw) {
+    const float slack = 1.0e-6f * (warp_max(fmaxf(fabsf(mine.x), fmaxf(fabsf(mine.y), fabsf(mine.z)))) + warp_max(mine.w));
+    constexpr float kUp = 1.000001f * kUnitToBox;
+    const float wx = fmaf(ext.x, kUp, slack), wy = fmaf(ext.y, kUp, slack), wz = fmaf(ext.z, kUp, slack);
+    bool any = false;
+    for (int k = 0; k < gw; ++k) {
+        // nearest image of the node's centre, less the half extent
+        const float ax = fabsf(d.x - __shfl_sync(0xffffffffu, mine.x, k)),
+                    ay = fabsf(d.y - __shfl_sync(0xffffffffu, mine.y, k)),
+                    az = fabsf(d.z - __shfl_sync(0xffffffffu, mine.z, k));
+        const float gx = fmaxf(fminf(ax, 1.0f - ax) - wx, 0.0f), gy = fmaxf(fminf(ay, 1.0f - ay) - wy, 0.0f),
+                    gz = fmaxf(fminf(az, 1.0f - az) - wz, 0.0f);
+        float r = __shfl_sync(0xffffffffu, mine.w, k);
+        r = r > 0.0f ? fmaxf(r, hnode) : 0.0f;
+        any = any || fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < 1.000004f * r * r;
+    }
+    return any;
 }
 
 // One search's walk from the tree rooted at `root` and the member x candidate filter of
@@ -1523,24 +1601,34 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
     const float emax = fmaxf(ex, fmaxf(ey, ez));
     const float reach = emax + (K::sym ? fmaxf(H, __uint_as_float(a.ncen[root].w)) : H);
     const bool wrap_safe = reach < 0.49f;
-    auto open_node = [&](const uint4& cen, const float4& ext) {
+    auto open_box = [&](const uint4& cen, const float4& ext) {
         const float gap2 = node_gap2(cen, make_float4(__fadd_ru(ext.x, nx), __fadd_ru(ext.y, ny),
                                                       __fadd_ru(ext.z, nz), 0.0f), cx, cy, cz);
         if constexpr (K::sym) return gap2 <= radius2_units(fmaxf(H, __uint_as_float(cen.w)));
         else return gap2 <= H2u;
     };
-    Walk w = walk_begin(a);
-    walk_visit(a, W, w, walk_start(a, root, cx, cy, cz, reach, lane), kWalkWhole, lc, lane, open_node);
+    // candidates after which the walk also tests nodes against the members' own spheres
+    const int refine_after = kRefineBase + kRefinePerMember * L.gw;
+    auto open_node = [&](bool have, const uint4& cen, const float4& ext, int found) {
+        bool open = have && open_box(cen, ext);
+        if (found > refine_after)
+            open = meets_members(make_float3(rel_coord(cen.x, 0.0f, cx), rel_coord(cen.y, 0.0f, cy),
+                                             rel_coord(cen.z, 0.0f, cz)),
+                                 ext, K::sym ? __uint_as_float(cen.w) : 0.0f,
+                                 make_float4(mem.mx, mem.my, mem.mz, member_radius(mem)), L.gw) && open;
+        return open;
+    };
+    Walk w = walk_begin();
+    walk_visit(a, W, w, walk_start(a, root, cx, cy, cz, reach, lane), kWalkWhole, lane, open_node);
     int ns = 0;   // candidates in the tile
     for (;;) {
-        while (walk_can_step(a, w) && w.total - w.done < 64) walk_step(a, W, w, kWalkWhole, lc, lane, open_node);
+        while (walk_can_step(a, w) && w.total - w.done < 64) walk_step(a, W, w, kWalkWhole, lane, open_node);
         walk_spill(a, W, w, lane);
         const bool walked = w.empty();
         // candidates by whole windows of 32 while the walk goes on
         while (ns <= kTile - 32 && (w.total - w.done >= 32 || (walked && w.total > w.done))) {
             int rank;
             const int nt = walk_take(W, w, lane, rank);
-            lc.cands += (lane == 0) ? nt : 0;
             bool in = false;
             float px = 0.0f, py = 0.0f, pz = 0.0f, mj = 0.0f, hj2 = 0.0f;
             if (lane < nt) {
@@ -1573,6 +1661,7 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
             ns += __popc(im);
         }
         const bool last = walked && w.total == w.done;
+        if (last && lane == 0) W.ctr.cands += w.total;
         if (ns > kTile - 32 || last) {
             if (ns > 0) {
                 copies_wait();
@@ -1587,31 +1676,44 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
     }
 }
 
-// One part of a work item: up to 32 members U[base, base + cnt), one per lane and slice.
+// work-list entry of the lane's member
+__device__ __forceinline__ int member_entry(const GroupDesc& d, const Layout& L, WalkSmem& W, int lane) {
+    if (d.mask == 0u) return d.base + L.k;
+    // member index -> offset, through the walk stack (free between searches)
+    if (d.mask >> lane & 1u) W.stack[__popc(d.mask & ((1u << lane) - 1u))] = (uint32_t)lane;
+    __syncwarp();
+    const int off = (int)W.stack[max(L.k, 0)];
+    __syncwarp();
+    return d.base + off;
+}
+
+// The search of up to 32 members, one per lane and slice.
 template <class K, int MODE>
-__device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, int base, int cnt,
-                                             int root, int smax, LocalCounters& lc, int lane) {
+__device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, const GroupDesc& d,
+                                             LocalCounters& lc, int lane) {
     constexpr bool kLists = K::id == kKindDensityList;
-    const Layout L = make_layout(cnt, lane, MODE == kAcc, kLists ? min(4, smax) : smax, kLists);
-    const MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[base + L.k] : -1)};
+    const Layout L = make_layout(d.cnt, lane, MODE == kAcc, kLists ? min(4, d.smax) : d.smax, kLists);
+    const int entry = member_entry(d, L, W, lane);
+    const MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[entry] : -1)};
     uint32_t cx = 0, cy = 0, cz = 0;
     if (!group_centre<1>(a, rec, cx, cy, cz)) return;
     typename K::Member mem;
     member_init(mem, a, rec[0], cx, cy, cz);
-    if constexpr (K::id == kKindDensityList) {
+    if constexpr (kLists) {
         // list slot = the member's index in the work list; sub-list of this lane's slice
         if (mem.rank >= 0) {
             mem.lsub = kListCap / L.S;
-            mem.lptr = a.o_list + (int64_t)(base + L.k) * kListCap + L.slice * mem.lsub;
+            mem.lptr = a.o_list + (int64_t)entry * kListCap + L.slice * mem.lsub;
         }
     }
     // export: write position of the member's neighbours
     if (MODE == kFill && mem.rank >= 0) mem.xpos = a.x_off[a.perm[mem.rank]];
-    group_search<K, MODE>(a, W, T, L, mem, cx, cy, cz, root, lc, lane);
+    if (lane == 0) W.ctr.walks++;
+    group_search<K, MODE>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
     // the symmetric sums count the member itself as a pair at r = 0 (once, in slice 0)
     constexpr bool kSelfPair = MODE == kAcc && (K::id == kKindHydro || K::id == kKindHydroAdj);
     lc.pairs += mem.n - ((kSelfPair && L.slice == 0 && mem.rank >= 0) ? 1 : 0);
-    if constexpr (K::id == kKindDensityList) {
+    if constexpr (kLists) {
         // the member's slice-0 lane records its sub-list lengths, S and whether all fit
         int cnt4[4];
 #pragma unroll
@@ -1623,11 +1725,10 @@ __device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, t
         if (L.slice == 0 && mem.rank >= 0) {
             const int lsub = kListCap / L.S;
             const bool ok = cnt4[0] <= lsub && cnt4[1] <= lsub && cnt4[2] <= lsub && cnt4[3] <= lsub;
-            const int slot = base + L.k;
-            a.o_lrec[slot] = make_int4(ok ? cnt4[0] | (cnt4[1] << 16) : 0, ok ? cnt4[2] | (cnt4[3] << 16) : 0, L.S,
-                                       ok ? 1 : 0);
-            a.o_lhw[slot] = rec[0].h * a.list_widen;
-            a.o_lslot[mem.rank] = slot;
+            a.o_lrec[entry] = make_int4(ok ? cnt4[0] | (cnt4[1] << 16) : 0, ok ? cnt4[2] | (cnt4[3] << 16) : 0, L.S,
+                                        ok ? 1 : 0);
+            a.o_lhw[entry] = rec[0].h * a.list_widen;
+            a.o_lslot[mem.rank] = entry;
         }
     }
     slice_sum(mem, L);
@@ -1640,10 +1741,9 @@ __device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, t
 // in parts of 32 9.7 ms, all with the walk and staging before culling).
 template <class K, int MODE>
 __device__ __forceinline__ void process_group(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, int gid,
-                                              LocalCounters& lc, int lane) {
-    const GroupDesc d = group_desc(a, gid);
-    for (int b = 0; b < d.cnt; b += kPartMax)
-        process_part<K, MODE>(a, W, T, d.base + b, min(kPartMax, d.cnt - b), d.root, d.smax, lc, lane);
+                                              int nlarge, LocalCounters& lc, int lane) {
+    const GroupDesc d = group_desc(a, gid, nlarge);
+    if (d.cnt > 0) process_part<K, MODE>(a, W, T, d, lc, lane);
 }
 
 __device__ __forceinline__ int next_item(const SearchArgs& a, int lane) {
@@ -1658,15 +1758,17 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, K::min_blocks) k_group(Se
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[wib];
+    clear_counters(W, lane);
     auto& T = reinterpret_cast<typename K::Tile*>(smem_raw + kWarpsPerBlock * sizeof(WalkSmem))[wib];
     LocalCounters lc;
-    const int ng = group_count(a);
+    int nlarge;
+    const int ng = group_count(a, nlarge);
     for (;;) {
         const int gid = next_item(a, lane);
         if (gid >= ng) break;
-        process_group<K, MODE>(a, W, T, gid, lc, lane);
+        process_group<K, MODE>(a, W, T, gid, nlarge, lc, lane);
     }
-    flush_counters(a, lc, lane);
+    flush_counters(a, lc, W.ctr, lane);
 }
 
 // Two kinds of work item in one persistent queue: the groups of a0 (kind K0) first,
@@ -1681,18 +1783,21 @@ k_group_pair(SearchArgs a0, SearchArgs a1) {
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[wib];
+    clear_counters(W, lane);
     unsigned char* tile = smem_raw + kWarpsPerBlock * sizeof(WalkSmem) + wib * kTileBytes;
     LocalCounters lc;
-    const int n0 = group_count(a0), n1 = group_count(a1);
+    int large0, large1;
+    const int n0 = group_count(a0, large0), n1 = group_count(a1, large1);
     for (;;) {
         const int gid = next_item(a0, lane);
         if (gid >= n0 + n1) break;
         if (gid < n0)
-            process_group<K0, kAcc>(a0, W, *reinterpret_cast<typename K0::Tile*>(tile), gid, lc, lane);
+            process_group<K0, kAcc>(a0, W, *reinterpret_cast<typename K0::Tile*>(tile), gid, large0, lc,
+                                    lane);
         else
-            process_group<K1, kAcc>(a1, W, *reinterpret_cast<typename K1::Tile*>(tile), gid - n0, lc, lane);
+            process_group<K1, kAcc>(a1, W, *reinterpret_cast<typename K1::Tile*>(tile), gid - n0, large1, lc, lane);
     }
-    flush_counters(a0, lc, lane);
+    flush_counters(a0, lc, W.ctr, lane);
 }
 
 // The candidate superset of every group (inspection): the particles of the leaves that
@@ -1706,12 +1811,14 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_superset(SearchArgs a) 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[threadIdx.x >> 5];
+    clear_counters(W, lane);
     LocalCounters lc;
-    const int ng = group_count(a);
+    int nlarge;
+    const int ng = group_count(a, nlarge);
     for (;;) {
         const int gid = next_item(a, lane);
         if (gid >= ng) break;
-        const GroupDesc d = group_desc(a, gid);
+        const GroupDesc d = group_desc(a, gid, 0);
         MemberRec rec[kSupSlots];
 #pragma unroll
         for (int mm = 0; mm < kSupSlots; ++mm) {
@@ -1735,15 +1842,15 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_superset(SearchArgs a) 
         const float R = warp_max(rlane), hmax_g = warp_max(hlane);
         const float R2d = radius2_units(R);
         const float reach = SYM ? R + fmaxf(hmax_g, __uint_as_float(a.ncen[d.root].w)) : R;
-        auto open_node = [&](const uint4& cen, const float4& ext) {
+        auto open_node = [&](bool have, const uint4& cen, const float4& ext, int) {
             const float R2 = SYM ? radius2_units(R + fmaxf(hmax_g, __uint_as_float(cen.w))) : R2d;
-            return node_gap2(cen, ext, cx, cy, cz) <= R2;
+            return have && node_gap2(cen, ext, cx, cy, cz) <= R2;
         };
-        Walk w = walk_begin(a);
-        walk_visit(a, W, w, walk_start(a, d.root, cx, cy, cz, reach, lane), 0, lc, lane, open_node);
+        Walk w = walk_begin();
+        walk_visit(a, W, w, walk_start(a, d.root, cx, cy, cz, reach, lane), 0, lane, open_node);
         const int64_t pos = FILL ? a.x_off[gid] : 0;
         while (!w.empty() || w.total > w.done) {
-            while (walk_can_step(a, w)) walk_step(a, W, w, 0, lc, lane, open_node);
+            while (walk_can_step(a, w)) walk_step(a, W, w, 0, lane, open_node);
             walk_spill(a, W, w, lane);
             while (w.total > w.done) {
                 const int64_t at = pos + w.done;
@@ -1755,10 +1862,10 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_superset(SearchArgs a) 
                 }
             }
         }
-        lc.cands += (lane == 0) ? w.total : 0;
+        if (lane == 0) W.ctr.cands += w.total;
         if (!FILL && lane == 0) a.x_cnt[gid] = w.total;
     }
-    flush_counters(a, lc, lane);
+    flush_counters(a, lc, W.ctr, lane);
 }
 
 // Density with the smoothing-length iteration inside the group (no host loop, no
@@ -1815,39 +1922,42 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     WalkSmem& W = reinterpret_cast<WalkSmem*>(smem_raw)[wib];
+    clear_counters(W, lane);
     PlainTile& T = reinterpret_cast<PlainTile*>(smem_raw + kWarpsPerBlock * sizeof(WalkSmem))[wib];
     LocalCounters lc;
-    const int ng = group_count(a);
+    int nlarge;
+    const int ng = group_count(a, nlarge);
     for (;;) {
         const int gid = next_item(a, lane);
         if (gid >= ng) break;
-        const GroupDesc d = group_desc(a, gid);
-        for (int b = 0; b < d.cnt; b += kPartMax) {
-            const Layout L = make_layout(min(kPartMax, d.cnt - b), lane, true, d.smax, false);
-            MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[d.base + b + L.k] : -1)};
-            double lo = 0.0, hi = __longlong_as_double(0x7ff0000000000000ll);
-            for (int pass = 1;; ++pass) {
-                uint32_t cx = 0, cy = 0, cz = 0;
-                if (!group_centre<1>(a, rec, cx, cy, cz)) break;
-                DMember mem;
-                member_init(mem, a, rec[0], cx, cy, cz);
-                group_search<KDens, kAcc>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
-                lc.pairs += mem.n;
-                slice_sum(mem, L);
-                // every slice takes the step, from the sums of its member in slice 0
-                const int src = L.k >= 0 ? L.k : 0;
-                const float s0 = __shfl_sync(0xffffffffu, mem.s0 - mem.c0, src);
-                const float s1 = __shfl_sync(0xffffffffu, mem.s1 - mem.c1, src);
-                const int nn = __shfl_sync(0xffffffffu, mem.n, src);
-                if (rec[0].rank >= 0 &&
-                    hsml_step(a, it, rec[0].rank, rec[0].h, lo, hi, s0, s1, nn, pass, L.slice == 0))
-                    rec[0].rank = -1;
-                // the new h (global memory) is read by the next pass's FP64 re-tests
-                __syncwarp();
-            }
+        const GroupDesc d = group_desc(a, gid, nlarge);
+        if (d.cnt <= 0) continue;
+        const Layout L = make_layout(d.cnt, lane, true, d.smax, false);
+        const int entry = member_entry(d, L, W, lane);
+        MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[entry] : -1)};
+        double lo = 0.0, hi = __longlong_as_double(0x7ff0000000000000ll);
+        for (int pass = 1;; ++pass) {
+            uint32_t cx = 0, cy = 0, cz = 0;
+            if (!group_centre<1>(a, rec, cx, cy, cz)) break;
+            DMember mem;
+            member_init(mem, a, rec[0], cx, cy, cz);
+            if (lane == 0) W.ctr.walks++;
+            group_search<KDens, kAcc>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
+            lc.pairs += mem.n;
+            slice_sum(mem, L);
+            // every slice takes the step, from the sums of its member in slice 0
+            const int src = max(L.k, 0);
+            const float s0 = __shfl_sync(0xffffffffu, mem.s0 - mem.c0, src);
+            const float s1 = __shfl_sync(0xffffffffu, mem.s1 - mem.c1, src);
+            const int nn = __shfl_sync(0xffffffffu, mem.n, src);
+            if (rec[0].rank >= 0 &&
+                hsml_step(a, it, rec[0].rank, rec[0].h, lo, hi, s0, s1, nn, pass, L.slice == 0))
+                rec[0].rank = -1;
+            // the new h (global memory) is read by the next pass's FP64 re-tests
+            __syncwarp();
         }
     }
-    flush_counters(a, lc, lane);
+    flush_counters(a, lc, W.ctr, lane);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1858,6 +1968,7 @@ template <int KIND, int MODE>
 __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
     const int lane = threadIdx.x & 31;
     LocalCounters lc;
+    unsigned nodes = 0, cands = 0;
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u < a.nu) {
         const int rank = a.U[u];
@@ -1881,12 +1992,12 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
             uint4 cen = a.ncen[node];
             float4 ext = a.next[node];
             int4 lk = a.nlink[node];
-            lc.nodes++;
+            nodes++;
             float gap2 = node_gap2(cen, ext, cx, cy, cz);
             float R2 = KIND == 0 ? R2d : radius2_units(fmaxf(Rbox, __uint_as_float(cen.w)));
             if (gap2 <= R2) {
                 if (lk.z < 0) {
-                    lc.cands += lk.y;
+                    cands += lk.y;
                     lc.tests += lk.y;
                     for (int q = lk.x; q < lk.x + lk.y; ++q) {
                         uint4 Q = a.pfix[q];
@@ -1922,7 +2033,149 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
         if (KIND == 0) write_result<MODE>(dm, a);
         else write_result<MODE>(hm, a);
     }
-    flush_counters(a, lc, lane);
+    const unsigned long long tn = warp_sum(nodes), tc = warp_sum(cands);
+    if (lane == 0) {
+        atomicAdd(&a.ctr->nodes, tn);
+        atomicAdd(&a.ctr->cands, tc);
+    }
+    flush_counters(a, lc, WalkCounters{0u, 0u, 0u, 0u}, lane);
+}
+
+// ---------------------------------------------------------------------------------
+// Pieces of the searches that compute (count mode): one warp per window of up to 32
+// consecutive work-list entries, whole chunks of g (g > 32: chunks of 32).  Every chunk is
+// cut as k_split_groups cuts the exported groups: (recursively) while its members' search
+// sphere, ((sqrt(3)/2) box width + h_min)^3, exceeds split * (members) member spheres
+// h_min^3, at the largest gap in key order between consecutive members (ties: nearest the
+// middle; the middle when they are contiguous); in a batch, whose active particles are
+// not runs, in the middle (gap cuts peel off single members there: a 16-box step 22.7 ->
+// 23.5 ms).
+//
+// Pieces that reach far beyond their smallest h have the most candidates; they are listed
+// from the end of the list, which the search kernels take first.
+//
+// The pieces go straight to the list, a block's together, with one atomic each for the
+// large ones and the others: no scan of counts, and their number stays on the device.
+// The list's order varies from run to run; every piece's sums are its own.
+// ---------------------------------------------------------------------------------
+
+constexpr int kCutWarps = 8;
+constexpr float kLargeReach = 2.5f;  // 0.5 width + h_max above this many h_min: goes first
+
+template <bool BATCH>
+__global__ void __launch_bounds__(kCutWarps * 32) k_cut_pieces(CutArgs a) {
+    __shared__ int cnt[2][kCutWarps];
+    __shared__ int at[2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nwin = BATCH ? *a.nwindows_dev : a.nwindows;
+    for (int w0 = blockIdx.x * kCutWarps; w0 < nwin; w0 += gridDim.x * kCutWarps) {   // block-uniform
+        const int win = w0 + w;
+        int base = 0, n = 0, g = a.g, root = 0, cfg = 0;
+        float split = a.split;
+        if (win < nwin) {
+            if (BATCH) {
+                const int4 C = a.windows[win];
+                base = C.x;
+                n = C.y;
+                root = C.z;
+                cfg = C.w;
+                g = min(cfg & 0xff, 32);
+                split = a.box_split[root];
+            } else {
+                base = win * a.width;
+                n = min(a.width, a.nu - base);
+            }
+        }
+        const int rank = lane < n ? a.U[base + lane] : -1;
+        uint4 P = make_uint4(0u, 0u, 0u, 0u);
+        float hf = 0.0f;
+        if (rank >= 0) {
+            P = a.pfix[rank];
+            hf = (float)a.h64[rank];
+        }
+        const int up = __shfl_up_sync(0xffffffffu, rank, 1);
+        uint32_t starts = __ballot_sync(0xffffffffu, lane % g == 0);
+        uint32_t small = 0u, large = 0u;   // lane k: the mask of the k-th small / large piece
+        int ns = 0, nl = 0;
+        for (int s = 0; s < n;) {
+            const uint32_t later = starts & ~((2u << s) - 1u);
+            const int e = later ? min(__ffs(later) - 1, n) : n;
+            const bool in = lane >= s && lane < e;
+            float ext = 0.0f, hmin = 0.0f, hmax = 0.0f;
+            if (e - s > 1) {
+                const uint32_t x0 = __shfl_sync(0xffffffffu, P.x, s), y0 = __shfl_sync(0xffffffffu, P.y, s),
+                               z0 = __shfl_sync(0xffffffffu, P.z, s);
+                const int dx = in ? (int32_t)(P.x - x0) : 0, dy = in ? (int32_t)(P.y - y0) : 0,
+                          dz = in ? (int32_t)(P.z - z0) : 0;
+                const float wx = (float)((int64_t)__reduce_max_sync(0xffffffffu, dx) - __reduce_min_sync(0xffffffffu, dx)),
+                            wy = (float)((int64_t)__reduce_max_sync(0xffffffffu, dy) - __reduce_min_sync(0xffffffffu, dy)),
+                            wz = (float)((int64_t)__reduce_max_sync(0xffffffffu, dz) - __reduce_min_sync(0xffffffffu, dz));
+                ext = fmaxf(wx, fmaxf(wy, wz)) * kUnitToBox;
+                hmin = __uint_as_float(__reduce_min_sync(0xffffffffu, in ? __float_as_uint(hf) : 0x7f800000u));
+                const float rel = fmaf(0.8660254f, ext / hmin, 1.0f);
+                if (split > 0.0f && !(rel * rel * rel <= split * (float)(e - s))) {
+                    const int mid = s + (e - s + 1) / 2;
+                    const int gap = (in && lane > s) ? rank - up : 0;
+                    const int best = BATCH ? 0 : __reduce_max_sync(0xffffffffu, gap);
+                    int c = mid;
+                    if (best > 1)
+                        c = (int)(__reduce_min_sync(0xffffffffu, gap == best ? (unsigned)(abs(lane - mid) * 64 + lane)
+                                                                             : 0xffffu) & 63u);
+                    starts |= 1u << c;
+                    continue;
+                }
+                hmax = warp_max(in ? hf : 0.0f);
+            }
+            const uint32_t piece = __ballot_sync(0xffffffffu, in);
+            if (fmaf(0.5f, ext, hmax) > kLargeReach * hmin) {
+                if (lane == nl) large = piece;
+                ++nl;
+            } else {
+                if (lane == ns) small = piece;
+                ++ns;
+            }
+            s = e;
+        }
+        if (lane == 0) {
+            cnt[0][w] = ns;
+            cnt[1][w] = nl;
+        }
+        __syncthreads();
+        int pre[2] = {0, 0}, tot[2] = {0, 0};
+        for (int k = 0; k < kCutWarps; ++k) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int v = cnt[q][k];
+                if (k < w) pre[q] += v;
+                tot[q] += v;
+            }
+        }
+        if (threadIdx.x < 2 && tot[threadIdx.x] > 0) at[threadIdx.x] = atomicAdd(&a.npieces[threadIdx.x], tot[threadIdx.x]);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (lane >= (q ? nl : ns)) continue;
+            const int64_t k = at[q] + pre[q] + lane;
+            const int64_t slot = q ? a.cap - 1 - k : k;
+            const uint32_t mask = q ? large : small;
+            if (BATCH) a.pieces4[slot] = make_int4(base, (int)mask, root, cfg);
+            else a.pieces[slot] = make_int2(base, (int)mask);
+        }
+        __syncthreads();   // cnt and at are rewritten by the next round
+    }
+}
+
+int launch_cut_pieces(const CutArgs& a, int sm_count, cudaStream_t s) {
+    cudaMemsetAsync(a.npieces, 0, 2 * sizeof(int), s);
+    if (a.windows) {
+        k_cut_pieces<true><<<8 * sm_count, kCutWarps * 32, 0, s>>>(a);
+    } else {
+        const int64_t blocks = std::min<int64_t>((a.nwindows + kCutWarps - 1) / kCutWarps, 32 * (int64_t)sm_count);
+        if (blocks < 1) return SPHGRP_OK;
+        k_cut_pieces<false><<<(unsigned)blocks, kCutWarps * 32, 0, s>>>(a);
+    }
+    note_launch();
+    return check_cuda(cudaGetLastError(), "group pieces");
 }
 
 // ---------------------------------------------------------------------------------
@@ -2073,8 +2326,8 @@ static size_t group_smem() {
     return kWarpsPerBlock * (sizeof(WalkSmem) + sizeof(typename K::Tile));
 }
 
-// Persistent grid: every resident block slot of the GPU (at most one block per four
-// groups when the group count is known on the host).
+// Persistent grid: every resident block slot of the GPU, but at most one block per four
+// groups (ngroups_host: their number, or a bound on it; -1: unknown).
 template <typename Kern, typename... Args>
 static int launch_persistent(Kern kern, bool& configured, size_t sh, int64_t ngroups_host, int sm_count,
                              cudaStream_t s, const char* what, Args... args) {
@@ -2097,8 +2350,10 @@ template <class K, int MODE>
 static int launch_group(const SearchArgs& a, int sm_count, cudaStream_t s) {
     static bool configured = false;
     if (a.g > 128) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
-    return launch_persistent(k_group<K, MODE>, configured, group_smem<K>(), a.ngroups_dev ? -1 : a.ngroups, sm_count,
-                             s, "grouped search kernel", a);
+    SearchArgs b = a;
+    b.parts = (a.g + kPartMax - 1) / kPartMax;
+    return launch_persistent(k_group<K, MODE>, configured, group_smem<K>(),
+                             a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s, "grouped search kernel", b);
 }
 
 template <bool SYM, bool FILL>
@@ -2125,7 +2380,7 @@ int launch_search_dev(const SearchArgs& a, int kind, int max_g, int sm_count, cu
     if (max_g < 1 || max_g > 128) return set_error(SPHGRP_EINVAL, "group size outside [1, 128]");
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     SearchArgs b = a;
-    b.g = max_g;   // bound only; groups4 carries every group's size
+    b.g = max_g;   // bound only; the pieces carry their members
     switch (kind) {
         case kKindDensity:
             return b.o_s2 ? launch_group<KDens2, kAcc>(b, sm_count, s) : launch_group<KDens, kAcc>(b, sm_count, s);
@@ -2140,8 +2395,11 @@ int launch_density_iter(const SearchArgs& a, const IterArgs& it, int max_g, int 
     if (max_g < 1 || max_g > 128) return set_error(SPHGRP_EINVAL, "group size outside [1, 128]");
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     static bool configured = false;
-    return launch_persistent(k_group_dens_iter, configured, group_smem<KDens>(), a.ngroups_dev ? -1 : a.ngroups,
-                             sm_count, s, "grouped density iteration kernel", a, it);
+    SearchArgs b = a;
+    b.parts = (a.g + kPartMax - 1) / kPartMax;
+    return launch_persistent(k_group_dens_iter, configured, group_smem<KDens>(),
+                             a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s,
+                             "grouped density iteration kernel", b, it);
 }
 
 template <class K0, class K1>

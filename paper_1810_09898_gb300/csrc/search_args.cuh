@@ -107,10 +107,16 @@ struct SearchArgs {
     int nu;
     int g;          // group size (grouped form)
     int ngroups;
+    int parts;      // items per group (of up to 32 members each; set by the launcher)
     bool centre_box; // group sphere centred on the members' box (else on the first member)
     const int2* groups; // (first entry of U, count) per group; null: chunks of g
-    const int4* groups4; // batch groups: (first entry of U, count, root node, g | max_slices << 8)
-    const int* ngroups_dev; // device group count (graph-capturable launches); null: ngroups
+    // pieces cut by k_cut_pieces (null: groups): (first entry of U, mask of the members as
+    // offsets from it), the large ones from the end of the list; batch: {first, mask, root
+    // node, g | max_slices << 8}; npieces: device counts of the others and the large ones
+    const int2* pieces;
+    const int4* pieces4;
+    const int* npieces;
+    int64_t pieces_cap;  // entries of the list
     // density pass results (rank space)
     float* o_s0;
     float* o_s1;
@@ -157,6 +163,26 @@ struct SearchArgs {
 };
 
 
+// windows of the work list to be cut into pieces
+struct CutArgs {
+    const int32_t* U;
+    const uint4* pfix;
+    const double* h64;
+    // one box: windows of `width` entries (a multiple of g), g and split for all
+    int nu, nwindows, width, g;
+    float split;
+    // batch: (first entry, count, box, g | max_slices << 8) per window, their count on the
+    // device, the split factor per box
+    const int4* windows;
+    const int* nwindows_dev;
+    const float* box_split;
+    // output
+    int2* pieces;
+    int4* pieces4;
+    int64_t cap;
+    int* npieces;
+};
+
 // smoothing-length iteration inside the grouped density kernel (batch path)
 struct IterArgs {
     double nngb, tol;
@@ -182,6 +208,7 @@ int launch_search_dev(const SearchArgs& a, int kind, int max_g, int sm_count, cu
 int launch_density_iter(const SearchArgs& a, const IterArgs& it, int max_g, int sm_count, cudaStream_t s);
 int launch_search_pair(const SearchArgs& a0, int kind0, const SearchArgs& a1, int kind1, int max_g, int sm_count,
                        cudaStream_t s);
+int launch_cut_pieces(const CutArgs& a, int sm_count, cudaStream_t s);
 int launch_split_groups(const int32_t* U, int nu, int g, float split, const uint4* pfix, const double* h64,
                         int2* tmp, int32_t* cnt, cudaStream_t s);
 // radius grouping: the greedy scan restarts at the start of every run of this many
@@ -210,6 +237,7 @@ int finish(Ctx* c, cudaStream_t s, int rc);
 void reset_flags(Ctx* c, cudaStream_t s);
 int prepare_active(Ctx* c, int64_t n_act, const int32_t* active, cudaStream_t s, int* nu);
 int make_groups(Ctx* c, SearchArgs* a, const int32_t* U, int nu, int g, cudaStream_t s);
+int make_pieces(Ctx* c, SearchArgs* a, const int32_t* U, int nu, int g, cudaStream_t s);
 SearchArgs base_args(Ctx* c);
 int check_common(Ctx* c, int64_t n_act, const int32_t* active, int mode, int group_size);
 

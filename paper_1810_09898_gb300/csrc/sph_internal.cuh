@@ -157,6 +157,7 @@ struct Ctx {
     int* work = nullptr;           // dynamic work counters for persistent kernels
     int* host_small = nullptr;     // pinned host scratch
     sphgrp_stats last{};
+    int64_t dev_walks = 0;         // walks counted by the kernels of the last call
     // device timing of the search kernels of the current call
     static constexpr int kMaxTimed = 128;
     cudaEvent_t tev[2 * kMaxTimed] = {};
