@@ -1746,9 +1746,9 @@ __device__ __forceinline__ void process_group(const SearchArgs& a, WalkSmem& W, 
     if (d.cnt > 0) process_part<K, MODE>(a, W, T, d, lc, lane);
 }
 
-__device__ __forceinline__ int next_item(const SearchArgs& a, int lane) {
+__device__ __forceinline__ int next_item(const SearchArgs& a, int lane, int take = 1) {
     int gid = 0;
-    if (lane == 0) gid = atomicAdd(a.work, 1);
+    if (lane == 0) gid = atomicAdd(a.work, take);
     return __shfl_sync(0xffffffffu, gid, 0);
 }
 
@@ -1763,10 +1763,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, K::min_blocks) k_group(Se
     LocalCounters lc;
     int nlarge;
     const int ng = group_count(a, nlarge);
+    const int take = a.take;
     for (;;) {
-        const int gid = next_item(a, lane);
-        if (gid >= ng) break;
-        process_group<K, MODE>(a, W, T, gid, nlarge, lc, lane);
+        const int first = next_item(a, lane, take);
+        if (first >= ng) break;
+        for (int gid = first; gid < min(first + take, ng); ++gid)
+            process_group<K, MODE>(a, W, T, gid, nlarge, lc, lane);
     }
     flush_counters(a, lc, W.ctr, lane);
 }
@@ -1961,7 +1963,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
 }
 
 // ---------------------------------------------------------------------------------
-// Individual form: one thread per particle, depth-first walk with skip pointers
+// Individual form: one walk per particle.  The density and hydro loops take groups of one
+// member in the kernel above: a warp walks for one particle, the box of its one member is
+// a point, so the candidates kept are its neighbours, and its 32 lanes share them.
+// One thread per particle with a depth-first walk (kept for the exports, which one lane
+// writes) diverges at every node: 1.0M clustered particles, density + hydro 12.2 ms
+// against 9.7 ms.
 // ---------------------------------------------------------------------------------
 
 template <int KIND, int MODE>
@@ -2017,10 +2024,6 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                             }
                         }
                     }
-                    if (MODE == kAcc) {
-                        if (KIND == 0) flush(dm);
-                        else flush(hm);
-                    }
                     node = lk.w;
                 } else {
                     node = lk.z;
@@ -2029,7 +2032,7 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                 node = lk.w;
             }
         }
-        lc.pairs += (KIND == 0) ? dm.n : hm.n - (MODE == kAcc ? 1 : 0);
+        lc.pairs += (KIND == 0) ? dm.n : hm.n;
         if (KIND == 0) write_result<MODE>(dm, a);
         else write_result<MODE>(hm, a);
     }
@@ -2352,6 +2355,8 @@ static int launch_group(const SearchArgs& a, int sm_count, cudaStream_t s) {
     if (a.g > 128) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
     SearchArgs b = a;
     b.parts = (a.g + kPartMax - 1) / kPartMax;
+    // many single members: several items per counter access (one address serves all warps)
+    b.take = a.g == 1 && a.ngroups >= 1 << 16 ? 4 : 1;
     return launch_persistent(k_group<K, MODE>, configured, group_smem<K>(),
                              a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s, "grouped search kernel", b);
 }
@@ -2447,20 +2452,22 @@ int launch_search(const SearchArgs& a, int kind, int mode, bool grouped, int sm_
         }
         return set_error(SPHGRP_EINVAL, "bad kind");
     }
-    int blocks = blocks_for(a.nu, 128);
-    if (kind == 0) {
-        if (mode == kAcc) k_indiv<0, kAcc><<<blocks, 128, 0, s>>>(a);
-        else if (mode == kCount) k_indiv<0, kCount><<<blocks, 128, 0, s>>>(a);
-        else if (mode == kFill) k_indiv<0, kFill><<<blocks, 128, 0, s>>>(a);
-        else return set_error(SPHGRP_EINVAL, "bad search mode");
-    } else if (kind == 1) {
-        if (mode == kAcc) k_indiv<1, kAcc><<<blocks, 128, 0, s>>>(a);
-        else if (mode == kCount) k_indiv<1, kCount><<<blocks, 128, 0, s>>>(a);
-        else if (mode == kFill) k_indiv<1, kFill><<<blocks, 128, 0, s>>>(a);
-        else return set_error(SPHGRP_EINVAL, "bad search mode");
-    } else {
+    if (kind != 0 && kind != 1)
         return set_error(SPHGRP_EINVAL, "the adjoint kernels exist in the grouped form only");
+    if (mode == kAcc) {
+        // one walk per particle, a warp to a particle: groups of one member
+        cudaMemsetAsync(a.work, 0, sizeof(int), s);
+        SearchArgs b = a;
+        b.g = 1;
+        b.ngroups = a.nu;
+        return kind == 0 ? launch_group<KDens, kAcc>(b, sm_count, s) : launch_group<KHydro, kAcc>(b, sm_count, s);
     }
+    const int blocks = blocks_for(a.nu, 128);
+    if (kind == 0 && mode == kCount) k_indiv<0, kCount><<<blocks, 128, 0, s>>>(a);
+    else if (kind == 0 && mode == kFill) k_indiv<0, kFill><<<blocks, 128, 0, s>>>(a);
+    else if (kind == 1 && mode == kCount) k_indiv<1, kCount><<<blocks, 128, 0, s>>>(a);
+    else if (kind == 1 && mode == kFill) k_indiv<1, kFill><<<blocks, 128, 0, s>>>(a);
+    else return set_error(SPHGRP_EINVAL, "bad search mode");
     note_launch();
     return check_cuda(cudaGetLastError(), "individual search kernel");
 }

@@ -107,6 +107,7 @@ struct SearchArgs {
     int nu;
     int g;          // group size (grouped form)
     int ngroups;
+    int take;       // items a warp takes at once (set by the launcher)
     int parts;      // items per group (of up to 32 members each; set by the launcher)
     bool centre_box; // group sphere centred on the members' box (else on the first member)
     const int2* groups; // (first entry of U, count) per group; null: chunks of g
