@@ -459,7 +459,7 @@ int sphgrp_mask_compact(sphgrp_ctx* ctx, int64_t n, const uint64_t* mask, int bi
  * take the implicit device synchronisation of an allocation.  The paper has no
  * counterpart; this is a deployment variant of the a1 + a2 step.
  * The sort's scratch lives in one fixed-size __device__ array inside the library
- * (about 6.3 MB, held on every GPU that loads the library until the process exits),
+ * (about 7.4 MB, held on every GPU that loads the library until the process exits),
  * so n may not exceed SPHGRP_STATIC_SORT_MAX_N (EINVAL otherwise).
  * pos:      device, n x 3 FP64 in [0,1).
  * keys_out: device, n uint64, receives the sorted keys (also used as sort scratch).

@@ -308,7 +308,7 @@ int finish(Ctx* c, cudaStream_t s, int rc) {
     if (err & kErrStack) return set_error(SPHGRP_EOVERFLOW, "walk stack overflow");
     if (err & kErrNodes) return set_error(SPHGRP_EOVERFLOW, "octree capacity exceeded");
     if (err & kErrCap) return set_error(SPHGRP_EOVERFLOW, "export capacity exceeded");
-    if (err & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait (tile copy) gave up");
+    if (err & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait gave up");
     return SPHGRP_OK;
 }
 
@@ -604,7 +604,7 @@ int sphgrp_ctx_create(sphgrp_ctx** out, const sphgrp_params* p, int64_t n_max) {
     rc |= dalloc(&c->perm, n);
     rc |= dalloc(&c->perm_alt, n);
     rc |= dalloc(&c->rank_of, n);
-    c->hist_cap = 256 * ((n + 2047) / 2048) + 256;
+    c->hist_cap = sort_scratch_cap(n);
     rc |= dalloc(&c->hist, c->hist_cap);
     rc |= dalloc(&c->xd, n);
     rc |= dalloc(&c->yd, n);
@@ -659,7 +659,8 @@ int sphgrp_ctx_destroy(sphgrp_ctx* ctx) {
                     c->cnt64, c->groups, c->groups_tmp, c->grp_cnt, c->grp_off,
                     c->acc_s2, c->wadj, c->dadj, c->adj0, c->adj1, c->adj2, c->adj3,
                     c->stack_spill, c->start_tab, c->ctr, c->err, c->work, c->ctr_log, c->tree.ncen, c->tree.next, c->tree.nlink,
-                    c->tree.nlevel, c->tree.box_lo, c->tree.box_hi, c->tree.top_cells, c->lst, c->lrec, c->lhw,
+                    c->tree.nlevel, c->tree.nparent, c->tree.narrive, c->tree.level_cnt, c->tree.box_lo, c->tree.box_hi,
+                    c->tree.top_cells, c->lst, c->lrec, c->lhw,
                     c->lslot, c->npass};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -681,9 +682,7 @@ int sphgrp_sfc_keys_sort(sphgrp_ctx* ctx, int64_t n, const double* pos, uint64_t
     c->built = false;
     c->n = n;
     reset_flags(c, s);
-    int rc = sort_keys(c, n, pos, s);
-    if (!rc && keys_out) rc = check_cuda(cudaMemcpyAsync(keys_out, c->keys, n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s), "keys copy");
-    if (!rc && perm_out) rc = check_cuda(cudaMemcpyAsync(perm_out, c->perm, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s), "perm copy");
+    int rc = sort_keys(c, n, pos, s, keys_out, perm_out);
     rc = finish(c, s, rc);
     if (!rc) c->sorted = true;
     return rc;

@@ -24,7 +24,6 @@ namespace sphgrp {
 namespace {
 
 constexpr int kGrid = 1024;   // blocks of the grid-stride kernels
-constexpr int kLevels = kKeyLevels + 3;
 constexpr int kMaxTableBoxes = 256;   // boxes that get a walk start table
 constexpr int kMinBatchLeaf = 8;      // smallest per-class leaf size: the forest's node
                                       // capacity (n/2 + 64 per box) holds trees of leaves >= 8
@@ -36,7 +35,6 @@ enum Scalar {
     kNPieces = 8,    // pieces of the active list: small, large
     kNPiecesAll = 10,  // pieces of the all-particle list (backward)
     kNFail = 5,      // particles that did not converge
-    kTot = 6,        // scan total scratch
     kNScalars = 16
 };
 
@@ -67,9 +65,6 @@ struct Batch {
     uint64_t* tmp64b = nullptr;
     int32_t* tmp32a = nullptr;
     int32_t* tmp32b = nullptr;
-    int32_t* lvl = nullptr;         // forest level table
-    uint4* blo = nullptr;
-    uint4* bhi = nullptr;
     int32_t* U_all = nullptr;       // identity work list
     int32_t* dsc = nullptr;         // device scalars
     int32_t* box_act = nullptr;     // nbox + 1: first entry of the box in the work list
@@ -266,8 +261,7 @@ int issue_step(Batch* b, const sphgrp_batch_io* io, int flags, cudaStream_t s) {
         return rc;
     if ((rc = gather_particles(c, io->pos, io->m, s))) return rc;
     if ((rc = launch_gather_h(c, io->h, s))) return rc;
-    if ((rc = build_forest(c, b->nbox, b->box_off, b->lvl, b->blo, b->bhi, b->dsc + kTot, b->box_of_rank,
-                           b->start_tabs, s, b->box_g)))
+    if ((rc = build_forest(c, b->nbox, b->box_off, b->box_of_rank, b->start_tabs, s, b->box_g)))
         return rc;
     // density with the smoothing-length iteration over the active groups
     if ((rc = make_batch_groups(b, false, -1, io->active, s))) return rc;
@@ -290,7 +284,7 @@ int issue_step(Batch* b, const sphgrp_batch_io* io, int flags, cudaStream_t s) {
     }
     // hydro inputs of every particle, node hmax at the new h
     if ((rc = launch_hydro_prep(c, io->h, io->rho, io->fgrad, io->vel, io->u, s))) return rc;
-    if ((rc = refresh_hmax_forest(c, b->lvl, s))) return rc;
+    if ((rc = refresh_hmax(c, s))) return rc;
     SearchArgs ah = batch_args(b, false);
     ah.o_acc = io->acc;
     ah.o_dudt = io->dudt;
@@ -347,7 +341,7 @@ int read_status(Batch* b, int flags) {
     if (err & kErrH) return set_error(SPHGRP_EINVAL, "a smoothing length is outside (0, 0.5)");
     if (err & kErrStack) return set_error(SPHGRP_EOVERFLOW, "walk stack overflow");
     if (err & kErrNodes) return set_error(SPHGRP_EOVERFLOW, "forest capacity exceeded");
-    if (err & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait (tile copy) gave up");
+    if (err & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait gave up");
     if (sc[kNFail] > 0) return set_error(SPHGRP_ENOCONV, std::to_string(sc[kNFail]) + " particles did not converge");
     return SPHGRP_OK;
 }
@@ -431,9 +425,6 @@ int sphgrp_batch_create(sphgrp_batch** out, const sphgrp_params* params, int nbo
     rc = rc ? rc : dalloc(&b->tmp64b, n);
     rc = rc ? rc : dalloc(&b->tmp32a, n);
     rc = rc ? rc : dalloc(&b->tmp32b, n);
-    rc = rc ? rc : dalloc(&b->lvl, kLevels);
-    rc = rc ? rc : dalloc(&b->blo, node_cap);
-    rc = rc ? rc : dalloc(&b->bhi, node_cap);
     rc = rc ? rc : dalloc(&b->U_all, n);
     rc = rc ? rc : dalloc(&b->dsc, kNScalars);
     rc = rc ? rc : dalloc(&b->box_act, nbox + 1);
@@ -446,7 +437,7 @@ int sphgrp_batch_create(sphgrp_batch** out, const sphgrp_params* params, int nbo
     // walk start tables: 1.2 MB per box, so only for batches of up to kMaxTableBoxes
     // boxes (larger batches walk from their boxes' roots)
     if (nbox <= kMaxTableBoxes) rc = rc ? rc : dalloc(&b->start_tabs, (int64_t)nbox * kStartTableSize);
-    rc = rc ? rc : alloc_forest(b->c, node_cap);
+    rc = rc ? rc : alloc_tree(b->c, node_cap);
     rc = rc ? rc : backward_buffers(b->c);
     if (!rc && cudaMallocHost(&b->host, (2 + kNScalars) * sizeof(int32_t)) != cudaSuccess) rc = SPHGRP_ENOMEM;
     if (!rc && cudaMallocHost(&b->host_ctr, sizeof(DevCounters)) != cudaSuccess) rc = SPHGRP_ENOMEM;
@@ -477,7 +468,7 @@ int sphgrp_batch_destroy(sphgrp_batch* w) {
     Batch* b = &w->b;
     drop_graph(b);
     void* ptrs[] = {b->box_off, b->box_g, b->box_split, b->box_cls, b->box_of_rank, b->tmp64a, b->tmp64b,
-                    b->tmp32a, b->tmp32b, b->lvl, b->blo, b->bhi, b->U_all, b->dsc, b->box_act, b->box_chunk,
+                    b->tmp32a, b->tmp32b, b->U_all, b->dsc, b->box_act, b->box_chunk,
                     b->chunks, b->groups, b->groups_all, b->hyd0b, b->hyd1b,
                     b->start_tabs};
     for (void* p : ptrs)
@@ -617,9 +608,8 @@ int sphgrp_batch_tune(sphgrp_batch* w, const sphgrp_batch_io* io, cudaStream_t s
     // the forest again (the order is unchanged) with the classes' current leaf sizes,
     // and its node hmax at the converged h; reports whether it fit the node capacity
     auto rebuild = [&](bool* fits) -> int {
-        int r = build_forest(c, b->nbox, b->box_off, b->lvl, b->blo, b->bhi, b->dsc + kTot, b->box_of_rank,
-                             b->start_tabs, s, b->box_g);
-        if (!r) r = refresh_hmax_forest(c, b->lvl, s);
+        int r = build_forest(c, b->nbox, b->box_off, b->box_of_rank, b->start_tabs, s, b->box_g);
+        if (!r) r = refresh_hmax(c, s);
         unsigned err = 0;
         if (!r) r = check_cuda(cudaMemcpyAsync(b->host, c->err, sizeof(unsigned), cudaMemcpyDeviceToHost, s),
                                "forest status");

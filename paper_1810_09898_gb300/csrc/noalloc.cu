@@ -5,8 +5,7 @@
 // budget, and latency-critical paths where the implicit device-wide synchronisation
 // of cudaMalloc / cudaFree is not acceptable.  For them sphgrp_sfc_keys_sort_static
 // runs the same key and radix-sort kernels as sphgrp_sfc_keys_sort, with the sort's
-// scratch (the second ping-pong buffer pair, the digit histograms, the scan's block
-// sums and the error flag) in one file-scope __device__ array of fixed size instead of
+// scratch (the second ping-pong buffer pair, the digit counts and the error flag) in one file-scope __device__ array of fixed size instead of
 // a context's workspace.  Every GPU that loads the library holds that array until the
 // process exits.
 #include <mutex>
@@ -15,8 +14,8 @@
 
 namespace sphgrp {
 int sort_keys_scratch(int64_t n, const double* pos, uint64_t* keys_out, int32_t* perm_out,
-                      uint64_t* keys_alt, int32_t* perm_alt, uint32_t* hist, int64_t hist_words,
-                      int32_t* scan_aux, int64_t scan_aux_words, unsigned* err, cudaStream_t s);
+                      uint64_t* keys_alt, int32_t* perm_alt, uint32_t* scratch, int64_t scratch_words,
+                      unsigned* err, cudaStream_t s);
 }
 
 using namespace sphgrp;
@@ -26,14 +25,13 @@ namespace {
 constexpr int64_t kMaxN = SPHGRP_STATIC_SORT_MAX_N;
 constexpr size_t kAlign = 256;
 constexpr size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
-constexpr size_t kHistWords = 256 * ((kMaxN + kSortTile - 1) / kSortTile);   // one row per sort tile
-constexpr size_t kAuxWords = 4096;
+// two sets of 512 words per tile of 2048 keys (checked against the sort's need on every call)
+constexpr size_t kHistWords = kSortHeadWords + 2 * 512 * (kMaxN / 2048);
 constexpr size_t kOffErr = 0;
 constexpr size_t kOffKeys = round_up(kOffErr + sizeof(unsigned));
 constexpr size_t kOffPerm = round_up(kOffKeys + sizeof(uint64_t) * kMaxN);
 constexpr size_t kOffHist = round_up(kOffPerm + sizeof(int32_t) * kMaxN);
-constexpr size_t kOffAux = round_up(kOffHist + sizeof(uint32_t) * kHistWords);
-constexpr size_t kBytes = round_up(kOffAux + sizeof(int32_t) * kAuxWords);
+constexpr size_t kBytes = round_up(kOffHist + sizeof(uint32_t) * kHistWords);
 
 // The scratch itself.  Host code must not use its name as a device address (on the
 // host it names a stand-in); the device address comes from cudaGetSymbolAddress.
@@ -78,14 +76,14 @@ extern "C" int sphgrp_sfc_keys_sort_static(int64_t n, const double* pos, uint64_
     if (rc) return rc;
     rc = sort_keys_scratch(n, pos, keys_out, perm_out, reinterpret_cast<uint64_t*>(base + kOffKeys),
                            reinterpret_cast<int32_t*>(base + kOffPerm), reinterpret_cast<uint32_t*>(base + kOffHist),
-                           (int64_t)kHistWords, reinterpret_cast<int32_t*>(base + kOffAux), (int64_t)kAuxWords,
-                           err, stream);
+                           (int64_t)kHistWords, err, stream);
     if (rc) return rc;
     unsigned flag = 0;
     rc = check_cuda(cudaMemcpyAsync(&flag, err, sizeof(unsigned), cudaMemcpyDeviceToHost, stream), "read error flag");
     if (rc) return rc;
     rc = check_cuda(cudaStreamSynchronize(stream), "stream");
     if (rc) return rc;
+    if (flag & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait (radix pass) gave up");
     if (flag & kErrRange) return set_error(SPHGRP_EINVAL, "a position is outside [0,1) or not finite");
     return SPHGRP_OK;
 }

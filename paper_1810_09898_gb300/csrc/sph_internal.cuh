@@ -56,21 +56,22 @@ constexpr int kStartTableSize = start_table_offset(kStartLevels + 1);
 //                                          to cover the sub-unit offsets
 //   nlink int4   {first, count, child_first (-1 = leaf), skip}
 // skip = the node visited after this one's subtree in a depth-first walk (-1 = end).
+constexpr int kTreeLevels = kKeyLevels + 1;   // levels 0 .. 21
 struct Tree {
     uint4* ncen = nullptr;
     float4* next = nullptr;
     int4* nlink = nullptr;
     int32_t* nlevel = nullptr;     // level of every node
-    int64_t cap = 0;               // allocated nodes
-    int64_t count = 0;             // nodes in the current tree
-    int level_begin[kKeyLevels + 3] = {0};  // node ranges per level (host copy)
-    int nlevels = 0;
-    // build scratch kept between builds (no allocation per call): fixed-point node
-    // boxes of the bottom-up pass (box_cap nodes) and the top levels' cell table
-    uint4* box_lo = nullptr;
+    int32_t* nparent = nullptr;    // parent of every node (-1: a root)
+    uint32_t* narrive = nullptr;   // children that arrived in the running bottom-up pass
+    uint4* box_lo = nullptr;       // fixed-point boxes (scratch of the bottom-up pass)
     uint4* box_hi = nullptr;
-    int64_t box_cap = 0;
-    int32_t* top_cells = nullptr;
+    int32_t* level_cnt = nullptr;  // nodes per level (device, kTreeLevels)
+    int64_t cap = 0;               // allocated nodes
+    int64_t count = 0;             // nodes in the current tree (a forest: a bound)
+    int nlevels = 10;              // deepest level of the last build (first: a guess)
+    int nroots = 1;
+    int32_t* top_cells = nullptr;  // the top levels' cell table (single-box build)
 };
 
 struct DevCounters {
@@ -102,7 +103,7 @@ struct Ctx {
     // sort scratch
     uint64_t* keys_alt = nullptr;
     int32_t* perm_alt = nullptr;
-    uint32_t* hist = nullptr;      // radix histograms
+    uint32_t* hist = nullptr;      // radix sort scratch
     int64_t hist_cap = 0;
     // particle copies
     double *xd = nullptr, *yd = nullptr, *zd = nullptr;
@@ -247,11 +248,7 @@ __device__ __forceinline__ double exact_r2(const double* xd, const double* yd, c
 // differences; nearer ones lose at most about 8 ulps of r in the FP32 difference.
 constexpr float kBandRel = 3.814697265625e-06f;  // 2^-18
 
-// Radix sort tile (sort.cu): 256 threads x 8 keys; the digit histograms take 256
-// counters per tile.
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kSortHeadWords = 3840;   // fixed part of the radix sort's scratch (sort.cu)
 
 // launch helpers
 // at least one block: kernels bound-check their index, and an empty grid is a launch error
@@ -261,21 +258,19 @@ inline int blocks_for(int64_t n, int threads) {
 }
 
 // kernels' host launchers (defined in the .cu files)
-int sort_keys(Ctx* c, int64_t n, const double* pos, cudaStream_t s);              // sort.cu
+int sort_keys(Ctx* c, int64_t n, const double* pos, cudaStream_t s, uint64_t* keys_copy,
+              int32_t* perm_copy);                                                 // sort.cu
+int64_t sort_scratch_cap(int64_t n_max);                                           // sort.cu
 int exclusive_scan_i32(Ctx* c, const int32_t* in, int32_t* out, int64_t n,
                        int32_t* total_dev, cudaStream_t s);                        // sort.cu
 int build_tree(Ctx* c, cudaStream_t s);                                            // tree.cu
 int refresh_hmax(Ctx* c, cudaStream_t s);                                          // tree.cu
-int exclusive_scan_i32_dev(Ctx* c, const int32_t* in, int32_t* out, const int32_t* n_hi, const int32_t* n_lo,
-                           int64_t n_bound, int32_t* total_dev, cudaStream_t s);            // sort.cu
 int sort_keys_boxed(Ctx* c, int64_t n, const double* pos, const int64_t* box_off_dev, int nbox, uint64_t* tmp64a,
                     uint64_t* tmp64b, int32_t* tmp32a, int32_t* tmp32b, int32_t* box_of_rank,
                     cudaStream_t s);                                                        // sort.cu
-int alloc_forest(Ctx* c, int64_t cap);                                                     // tree.cu
-int build_forest(Ctx* c, int nbox, const int64_t* box_off_dev, int32_t* lvl, uint4* blo, uint4* bhi,
-                 int32_t* tot, const int32_t* box_of_rank, int32_t* start_tabs, cudaStream_t s,
-                 const int32_t* box_cfg = nullptr);                                         // tree.cu
-int refresh_hmax_forest(Ctx* c, const int32_t* lvl, cudaStream_t s);                       // tree.cu
+int alloc_tree(Ctx* c, int64_t cap);                                                       // tree.cu
+int build_forest(Ctx* c, int nbox, const int64_t* box_off_dev, const int32_t* box_of_rank, int32_t* start_tabs,
+                 cudaStream_t s, const int32_t* box_cfg = nullptr);                         // tree.cu
 void note_launches(long long k);                                                           // api.cu
 
 // results of a finished particle (caller's order; rho, dRho/dh and f are FP32 outputs)

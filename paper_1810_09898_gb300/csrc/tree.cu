@@ -123,432 +123,262 @@ __device__ __forceinline__ void node_bounds(const uint64_t* __restrict__ keys, c
     octant_bounds(keys, lo, hi, 3 * (kKeyLevels - 1 - level), b);
 }
 
-// Number of non-empty octants of every node of one level that must split.
-__global__ void k_split_count(const uint64_t* __restrict__ keys, const int4* __restrict__ nlink,
-                              int a, int nf, int level, int leaf_size, int32_t* __restrict__ nchild,
-                              const int32_t* __restrict__ tab) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nf) return;
-    int4 L = nlink[a + k];
-    int cnt = 0;
-    if (L.y > leaf_size && level < kKeyLevels) {
-        int b[9];
-        node_bounds(keys, tab, level, L.x, L.x + L.y, b);
-#pragma unroll
-        for (int d = 0; d < 8; ++d) cnt += b[d + 1] > b[d] ? 1 : 0;
-    }
-    nchild[k] = cnt;
+// Octrees are built level by level over one or many boxes (a forest): the roots are nodes
+// 0 .. nbox - 1, the nodes of a level are contiguous and so are a node's children, and the
+// number of nodes of every level stays on the device (lcnt), so that the levels follow each
+// other without a read-back.  Within a level the nodes' order varies from run to run (a
+// block takes the ids of its nodes' children with one atomic); walks and results do not
+// depend on it.
+
+// first node and number of nodes of a level
+__device__ __forceinline__ void level_range(const int32_t* __restrict__ lcnt, int level, int64_t cap, int& a, int& nf) {
+    int64_t first = 0;
+    for (int l = 0; l < level; ++l) first += lcnt[l];
+    a = (int)min(first, cap);
+    nf = (int)max((int64_t)0, min((int64_t)lcnt[level], cap - first));
 }
 
-// Writes the children of every splitting node of one level.
-__global__ void k_split_write(const uint64_t* __restrict__ keys, int4* __restrict__ nlink,
-                              float4* __restrict__ next, int32_t* __restrict__ nlevel, int a,
-                              int nf, int level, const int32_t* __restrict__ nchild,
-                              const int32_t* __restrict__ coff, int b, const int32_t* __restrict__ tab) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nf) return;
-    int nc = nchild[k];
-    int4 L = nlink[a + k];
-    next[a + k].w = __int_as_float(nc);
-    if (nc == 0) return;
-    int child0 = b + coff[k];
-    int bd[9];
-    node_bounds(keys, tab, level, L.x, L.x + L.y, bd);
-    int c = 0;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) {
-        if (bd[d + 1] > bd[d]) {
-            int id = child0 + c;
-            int skip = (c + 1 < nc) ? id + 1 : L.w;
-            nlink[id] = make_int4(bd[d], bd[d + 1] - bd[d], -1, skip);
-            nlevel[id] = level + 1;
-            ++c;
-        }
+__global__ void k_tree_roots(int nbox, const int64_t* __restrict__ box_off, int64_t n, int4* __restrict__ nlink,
+                             float4* __restrict__ next, int32_t* __restrict__ nlevel, int32_t* __restrict__ nparent,
+                             uint32_t* __restrict__ narrive, int32_t* __restrict__ lcnt) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < nbox) {
+        const int64_t lo = box_off ? box_off[k] : 0, hi = box_off ? box_off[k + 1] : n;
+        nlink[k] = make_int4((int)lo, (int)(hi - lo), -1, -1);
+        next[k] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0));
+        nlevel[k] = 0;
+        nparent[k] = -1;
+        narrive[k] = 0u;
     }
-    L.z = child0;
-    nlink[a + k] = L;
+    if (k < kTreeLevels) lcnt[k] = k == 0 ? nbox : 0;
 }
 
-// Tight boxes (fixed point) and hmax of one level, leaves from their particles,
-// internal nodes from their children.
-__global__ void k_box_level(int a, int nf, const int4* __restrict__ nlink, const float4* __restrict__ next,
-                            const uint4* __restrict__ pfix, uint4* __restrict__ blo, uint4* __restrict__ bhi,
-                            uint4* __restrict__ ncen) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nf) return;
-    int id = a + k;
-    int4 L = nlink[id];
-    uint32_t lx = 0xffffffffu, ly = 0xffffffffu, lz = 0xffffffffu, hx = 0, hy = 0, hz = 0;
-    float hm = 0.0f;
-    if (L.z < 0) {
-        for (int q = L.x; q < L.x + L.y; ++q) {
-            uint4 P = pfix[q];
-            lx = min(lx, P.x); ly = min(ly, P.y); lz = min(lz, P.z);
-            hx = max(hx, P.x); hy = max(hy, P.y); hz = max(hz, P.z);
-            hm = fmaxf(hm, __uint_as_float(P.w));
+// The nodes of one level with more than leaf_size particles get their children, one per
+// non-empty octant.  box_cfg (optional): per box, bits 16..23 = that box's leaf size (0:
+// leaf_size); the node's box is the box of its first particle.  Children beyond the
+// capacity are not created: their parent stays a leaf, the ids it was given below the
+// capacity become empty leaves that nothing links to, and the error flag is set.
+__global__ void __launch_bounds__(256) k_split_level(const uint64_t* __restrict__ keys, int4* __restrict__ nlink,
+                                                     float4* __restrict__ next, int32_t* __restrict__ nlevel,
+                                                     int32_t* __restrict__ nparent, uint32_t* __restrict__ narrive,
+                                                     int32_t* __restrict__ lcnt, int level, int leaf_size,
+                                                     const int32_t* __restrict__ tab,
+                                                     const int32_t* __restrict__ box_cfg,
+                                                     const int32_t* __restrict__ box_of_rank, int64_t cap,
+                                                     unsigned* err) {
+    __shared__ int wtot[8];
+    __shared__ int first;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int a, nf;
+    level_range(lcnt, level, cap, a, nf);
+    for (int k0 = blockIdx.x * 256; k0 < nf; k0 += gridDim.x * 256) {   // block-uniform
+        const int k = k0 + threadIdx.x;
+        int4 L = make_int4(0, 0, -1, -1);
+        int bd[9];
+        int nc = 0;
+        if (k < nf) {
+            L = nlink[a + k];
+            int leaf = leaf_size;
+            if (box_cfg && L.y > 0) {
+                const int lb = (box_cfg[box_of_rank[L.x]] >> 16) & 0xff;
+                if (lb > 0) leaf = lb;
+            }
+            if (L.y > leaf && level < kKeyLevels) {
+                node_bounds(keys, tab, level, L.x, L.x + L.y, bd);
+#pragma unroll
+                for (int d = 0; d < 8; ++d) nc += bd[d + 1] > bd[d] ? 1 : 0;
+            }
         }
-    } else {
-        int nc = __float_as_int(next[id].w);
-        for (int c = L.z; c < L.z + nc; ++c) {
-            uint4 l = blo[c], h = bhi[c];
-            lx = min(lx, l.x); ly = min(ly, l.y); lz = min(lz, l.z);
-            hx = max(hx, h.x); hy = max(hy, h.y); hz = max(hz, h.z);
-            hm = fmaxf(hm, __uint_as_float(ncen[c].w));
+        int inc = nc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
         }
+        if (lane == 31) wtot[w] = inc;
+        __syncthreads();
+        int pre = inc - nc, tot = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            if (q < w) pre += wtot[q];
+            tot += wtot[q];
+        }
+        if (threadIdx.x == 0 && tot > 0) first = atomicAdd(&lcnt[level + 1], tot);
+        __syncthreads();
+        if (nc > 0) {
+            const int64_t child0 = (int64_t)a + nf + first + pre;
+            if (child0 + nc > cap) {
+                atomicOr(err, kErrNodes);
+                for (int64_t id = child0; id < min(child0 + nc, cap); ++id) {   // counted: empty leaves
+                    nlink[id] = make_int4(0, 0, -1, -1);
+                    next[id] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0));
+                    nlevel[id] = level + 1;
+                    nparent[id] = -1;
+                    narrive[id] = 0u;
+                }
+            } else {
+                int c = 0;
+#pragma unroll
+                for (int d = 0; d < 8; ++d) {
+                    if (bd[d + 1] > bd[d]) {
+                        const int id = (int)child0 + c;
+                        nlink[id] = make_int4(bd[d], bd[d + 1] - bd[d], -1, c + 1 < nc ? id + 1 : L.w);
+                        next[id] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0));
+                        nlevel[id] = level + 1;
+                        nparent[id] = a + k;
+                        narrive[id] = 0u;
+                        ++c;
+                    }
+                }
+                next[a + k].w = __int_as_float(nc);
+                L.z = (int)child0;
+                nlink[a + k] = L;
+            }
+        }
+        __syncthreads();   // wtot and first are rewritten by the next round
     }
-    blo[id] = make_uint4(lx, ly, lz, 0u);
-    bhi[id] = make_uint4(hx, hy, hz, 0u);
-    ncen[id].w = __float_as_uint(hm);
 }
 
 // Box -> centre (fixed point) and padded half extents.  Particles of the node lie in
 // [lo, hi + 1) units; with the centre rounded down to a whole unit the half extent
 // (hi - lo + 2) / 2 covers that interval.  Extents are rounded up.
-__global__ void k_box_final(int64_t nn, const uint4* __restrict__ blo, const uint4* __restrict__ bhi,
-                            uint4* __restrict__ ncen, float4* __restrict__ next) {
-    int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (id >= nn) return;
-    uint4 l = blo[id], h = bhi[id];
-    uint4 C = ncen[id];
-    uint64_t wx = (uint64_t)h.x - l.x + 1, wy = (uint64_t)h.y - l.y + 1, wz = (uint64_t)h.z - l.z + 1;
-    C.x = l.x + (uint32_t)(wx >> 1);
-    C.y = l.y + (uint32_t)(wy >> 1);
-    C.z = l.z + (uint32_t)(wz >> 1);
-    ncen[id] = C;
-    float4 E = next[id];
-    E.x = __fmul_ru(__ull2float_ru(wx + 1), 0.5f);
-    E.y = __fmul_ru(__ull2float_ru(wy + 1), 0.5f);
-    E.z = __fmul_ru(__ull2float_ru(wz + 1), 0.5f);
-    next[id] = E;
+__device__ __forceinline__ void write_box(int id, uint4 l, uint4 h, float hmax, uint4* __restrict__ blo,
+                                          uint4* __restrict__ bhi, uint4* __restrict__ ncen,
+                                          float4* __restrict__ next) {
+    blo[id] = l;
+    bhi[id] = h;
+    const uint64_t wx = (uint64_t)h.x - l.x + 1, wy = (uint64_t)h.y - l.y + 1, wz = (uint64_t)h.z - l.z + 1;
+    ncen[id] = make_uint4(l.x + (uint32_t)(wx >> 1), l.y + (uint32_t)(wy >> 1), l.z + (uint32_t)(wz >> 1),
+                          __float_as_uint(hmax));
+    float* e = reinterpret_cast<float*>(next + id);   // .w (the child count) is read meanwhile
+    e[0] = __fmul_ru(__ull2float_ru(wx + 1), 0.5f);
+    e[1] = __fmul_ru(__ull2float_ru(wy + 1), 0.5f);
+    e[2] = __fmul_ru(__ull2float_ru(wz + 1), 0.5f);
 }
 
-// hmax only (after the smoothing lengths changed)
-__global__ void k_hmax_level(int a, int nf, const int4* __restrict__ nlink, const float4* __restrict__ next,
-                             const uint4* __restrict__ pfix, uint4* __restrict__ ncen) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nf) return;
-    int id = a + k;
-    int4 L = nlink[id];
-    float hm = 0.0f;
-    if (L.z < 0) {
-        for (int q = L.x; q < L.x + L.y; ++q) hm = fmaxf(hm, __uint_as_float(pfix[q].w));
-    } else {
-        int nc = __float_as_int(next[id].w);
-        for (int c = L.z; c < L.z + nc; ++c) hm = fmaxf(hm, __uint_as_float(ncen[c].w));
+// What a node takes from its particles (a leaf) or its children: tight box (BOXES) and hmax.
+struct NodeBox {
+    uint4 l, h;
+    float hm;
+};
+
+// children [c0, c0 + nc), read past the L1 cache (they may have been written by this launch)
+template <bool BOXES>
+__device__ __forceinline__ NodeBox box_of_children(int c0, int nc, const uint4* blo, const uint4* bhi,
+                                                   const uint4* ncen) {
+    NodeBox b{make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0u), make_uint4(0u, 0u, 0u, 0u), 0.0f};
+    for (int c = c0; c < c0 + nc; ++c) {
+        if (BOXES) {
+            const uint4 cl = __ldcg(blo + c), ch = __ldcg(bhi + c);
+            b.l.x = min(b.l.x, cl.x); b.l.y = min(b.l.y, cl.y); b.l.z = min(b.l.z, cl.z);
+            b.h.x = max(b.h.x, ch.x); b.h.y = max(b.h.y, ch.y); b.h.z = max(b.h.z, ch.z);
+        }
+        b.hm = fmaxf(b.hm, __ldcg(reinterpret_cast<const float*>(ncen + c) + 3));
     }
-    ncen[id].w = __float_as_uint(hm);
+    return b;
 }
 
-// Walk start table (see kStartLevels): every node of levels 1 .. kStartLevels enters
-// under its cell, found from any of its particles (the cell of level l is the top l
-// bits of the fixed-point coordinates).
-__global__ void k_start_table(int first, int count, const int4* __restrict__ nlink,
+template <bool BOXES>
+__device__ __forceinline__ void write_node(int id, const NodeBox& b, uint4* blo, uint4* bhi, uint4* ncen,
+                                           float4* next) {
+    if (BOXES) write_box(id, b.l, b.h, b.hm, blo, bhi, ncen, next);
+    else reinterpret_cast<float*>(ncen + id)[3] = b.hm;
+}
+
+// The leaves, eight lanes to one.  CLIMB: the first lane then goes up, the last child to
+// arrive at a node completing it and going on; the arrival counters wrap to zero by
+// themselves.  Maxima and minima do not depend on the order.
+//
+// Climbing takes one launch where a launch per level spends 6-10 us on each level of a few
+// nodes (hmax of a 131k tree 81 -> 32 us, boxes of a 30k one 100 -> 40 us), but its fences
+// make it slow on many nodes (16.8M particles: boxes 1.35 ms, hmax 0.70 ms): trees above
+// kClimbNodes nodes take a launch per level above the leaves (k_tree_level).
+template <bool BOXES, bool CLIMB>
+__global__ void __launch_bounds__(256) k_tree_leaves(const int32_t* __restrict__ lcnt, int64_t cap,
+                                                     const int4* __restrict__ nlink, float4* next,
+                                                     const uint4* __restrict__ pfix,
+                                                     const int32_t* __restrict__ nparent, uint32_t* narrive,
+                                                     uint4* blo, uint4* bhi, uint4* ncen) {
+    int a, nf;
+    level_range(lcnt, kTreeLevels - 1, cap, a, nf);
+    const int nn = a + nf;
+    const int sub = threadIdx.x & 7;
+    for (int64_t base = (blockIdx.x * 256ll + threadIdx.x) >> 5 << 2; base < nn; base += gridDim.x * 32ll) {   // warp-uniform
+        int id = (int)base + ((threadIdx.x & 31) >> 3);
+        int4 L = make_int4(0, 0, 0, -1);
+        if (id < nn) L = nlink[id];
+        const bool leaf = id < nn && L.z < 0;
+        NodeBox b{make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0u), make_uint4(0u, 0u, 0u, 0u), 0.0f};
+        if (leaf) {
+            for (int q = L.x + sub; q < L.x + L.y; q += 8) {
+                if (BOXES) {
+                    const uint4 P = pfix[q];
+                    b.l.x = min(b.l.x, P.x); b.l.y = min(b.l.y, P.y); b.l.z = min(b.l.z, P.z);
+                    b.h.x = max(b.h.x, P.x); b.h.y = max(b.h.y, P.y); b.h.z = max(b.h.z, P.z);
+                    b.hm = fmaxf(b.hm, __uint_as_float(P.w));
+                } else {
+                    b.hm = fmaxf(b.hm, __uint_as_float(pfix[q].w));
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            if (BOXES) {
+                b.l.x = min(b.l.x, __shfl_xor_sync(0xffffffffu, b.l.x, o));
+                b.l.y = min(b.l.y, __shfl_xor_sync(0xffffffffu, b.l.y, o));
+                b.l.z = min(b.l.z, __shfl_xor_sync(0xffffffffu, b.l.z, o));
+                b.h.x = max(b.h.x, __shfl_xor_sync(0xffffffffu, b.h.x, o));
+                b.h.y = max(b.h.y, __shfl_xor_sync(0xffffffffu, b.h.y, o));
+                b.h.z = max(b.h.z, __shfl_xor_sync(0xffffffffu, b.h.z, o));
+            }
+            b.hm = fmaxf(b.hm, __shfl_xor_sync(0xffffffffu, b.hm, o));
+        }
+        if (leaf && sub == 0) {
+            if (BOXES && L.y == 0) b.l = b.h = make_uint4(0u, 0u, 0u, 0u);
+            write_node<BOXES>(id, b, blo, bhi, ncen, next);
+            while (CLIMB) {
+                const int p = nparent[id];
+                if (p < 0) break;
+                const int nc = __float_as_int(reinterpret_cast<const float*>(next + p)[3]);
+                __threadfence();
+                if (atomicInc(&narrive[p], (unsigned)nc - 1u) != (unsigned)nc - 1u) break;
+                __threadfence();
+                id = p;
+                b = box_of_children<BOXES>(nlink[p].z, nc, blo, bhi, ncen);
+                write_node<BOXES>(id, b, blo, bhi, ncen, next);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// the internal nodes of one level, from their children
+template <bool BOXES>
+__global__ void __launch_bounds__(256) k_tree_level(const int32_t* __restrict__ lcnt, int level, int64_t cap,
+                                                    const int4* __restrict__ nlink, float4* next, uint4* blo,
+                                                    uint4* bhi, uint4* ncen) {
+    int a, nf;
+    level_range(lcnt, level, cap, a, nf);
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < nf; k += gridDim.x * 256) {
+        const int id = a + k;
+        const int c0 = nlink[id].z;
+        if (c0 < 0) continue;
+        const int nc = __float_as_int(reinterpret_cast<const float*>(next + id)[3]);
+        write_node<BOXES>(id, box_of_children<BOXES>(c0, nc, blo, bhi, ncen), blo, bhi, ncen, next);
+    }
+}
+
+// Walk start tables (see kStartLevels), one per box: every node of levels 1 .. kStartLevels
+// enters its box's table under its cell, found from any of its particles (the cell of
+// level l is the top l bits of the fixed-point coordinates).  box_of_rank null: one box.
+__global__ void k_start_table(const int32_t* __restrict__ lcnt, int64_t cap, const int4* __restrict__ nlink,
                               const int32_t* __restrict__ nlevel, const uint4* __restrict__ pfix,
-                              int32_t* __restrict__ tab) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    const int id = first + k;
-    const int l = nlevel[id];
-    const int4 L = nlink[id];
-    if (l < 1 || l > kStartLevels || L.y <= 0) return;
-    const uint4 P = pfix[L.x];
-    const uint32_t x = P.x >> (32 - l), y = P.y >> (32 - l), z = P.z >> (32 - l);
-    uint32_t m = 0;
-    for (int b = l - 1; b >= 0; --b) m = (m << 3) | (((x >> b) & 1u) << 2) | (((y >> b) & 1u) << 1) | ((z >> b) & 1u);
-    tab[start_table_offset(l) + m] = id;
-}
-
-static int grow_tree(Ctx* c, int64_t need, cudaStream_t s) {
-    Tree& t = c->tree;
-    if (need <= t.cap) return SPHGRP_OK;
-    int64_t cap = std::max<int64_t>(need + need / 2, 1024);
-    uint4* ncen;
-    float4* next;
-    int4* nlink;
-    int32_t* nlevel;
-    if (cudaMallocAsync(&ncen, cap * sizeof(uint4), s) != cudaSuccess ||
-        cudaMallocAsync(&next, cap * sizeof(float4), s) != cudaSuccess ||
-        cudaMallocAsync(&nlink, cap * sizeof(int4), s) != cudaSuccess ||
-        cudaMallocAsync(&nlevel, cap * sizeof(int32_t), s) != cudaSuccess)
-        return set_error(SPHGRP_ENOMEM, "octree allocation failed");
-    if (t.count > 0) {
-        cudaMemcpyAsync(ncen, t.ncen, t.count * sizeof(uint4), cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(next, t.next, t.count * sizeof(float4), cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(nlink, t.nlink, t.count * sizeof(int4), cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(nlevel, t.nlevel, t.count * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-    }
-    if (t.ncen) {
-        cudaFreeAsync(t.ncen, s);
-        cudaFreeAsync(t.next, s);
-        cudaFreeAsync(t.nlink, s);
-        cudaFreeAsync(t.nlevel, s);
-    }
-    t.ncen = ncen;
-    t.next = next;
-    t.nlink = nlink;
-    t.nlevel = nlevel;
-    t.cap = cap;
-    return check_cuda(cudaGetLastError(), "octree allocation");
-}
-
-int build_tree(Ctx* c, cudaStream_t s) {
-    Tree& t = c->tree;
-    const int64_t n = c->n;
-    int rc = grow_tree(c, std::max<int64_t>(1024, 2 * n / std::max(1, c->p.leaf_size) + 64), s);
-    if (rc) return rc;
-    int4 root = make_int4(0, (int)n, -1, -1);
-    cudaMemcpyAsync(t.nlink, &root, sizeof(int4), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(t.nlevel, 0, sizeof(int32_t), s);
-    cudaMemsetAsync(t.next, 0, sizeof(float4), s);
-    t.level_begin[0] = 0;
-    t.level_begin[1] = 1;
-    t.count = 1;
-    int level = 0;
-    int32_t* total_dev = reinterpret_cast<int32_t*>(c->work) + 12;
-    if (!t.top_cells && cudaMalloc(&t.top_cells, kTopTableSize * sizeof(int32_t)) != cudaSuccess) {
-        t.top_cells = nullptr;
-        return set_error(SPHGRP_ENOMEM, "octree top-cell table");
-    }
-    int32_t* top = t.top_cells;
-    cudaMemsetAsync(top, 0xff, kTopTableSize * sizeof(int32_t), s);
-    if (n > 0) {
-        k_top_cells<<<blocks_for(n, 256), 256, 0, s>>>(c->keys, n, top);
-        note_launch();
-    }
-    for (level = 0; level <= kKeyLevels; ++level) {
-        int a = t.level_begin[level], b = t.level_begin[level + 1];
-        int nf = b - a;
-        if (nf == 0) break;
-        k_split_count<<<blocks_for(nf, 256), 256, 0, s>>>(c->keys, t.nlink, a, nf, level,
-                                                          c->p.leaf_size, c->flag, top);
-        note_launch();
-        rc = exclusive_scan_i32(c, c->flag, c->scan, nf, total_dev, s);
-        if (rc) return rc;
-        cudaMemcpyAsync(c->host_small, total_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-        if ((rc = check_cuda(cudaStreamSynchronize(s), "octree level"))) return rc;
-        int total = c->host_small[0];
-        if (b + (int64_t)total > t.cap) {
-            if ((rc = grow_tree(c, b + (int64_t)total, s))) return rc;
-        }
-        k_split_write<<<blocks_for(nf, 256), 256, 0, s>>>(c->keys, t.nlink, t.next, t.nlevel, a, nf,
-                                                          level, c->flag, c->scan, b, top);
-        note_launch();
-        t.level_begin[level + 2] = b + total;
-        t.count = b + total;
-        if (total == 0) { ++level; break; }
-    }
-    t.nlevels = level;
-    // boxes bottom-up, in scratch kept by the tree (grown to the node count when needed)
-    if (t.box_cap < t.count) {
-        if (t.box_lo) cudaFree(t.box_lo);
-        if (t.box_hi) cudaFree(t.box_hi);
-        t.box_lo = t.box_hi = nullptr;
-        t.box_cap = 0;
-        const int64_t cap = t.count + t.count / 4 + 1024;
-        if (cudaMalloc(&t.box_lo, cap * sizeof(uint4)) != cudaSuccess ||
-            cudaMalloc(&t.box_hi, cap * sizeof(uint4)) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(SPHGRP_ENOMEM, "octree box scratch");
-        }
-        t.box_cap = cap;
-    }
-    uint4* blo = t.box_lo;
-    uint4* bhi = t.box_hi;
-    for (int lv = t.nlevels - 1; lv >= 0; --lv) {
-        int a = t.level_begin[lv], nf = t.level_begin[lv + 1] - a;
-        if (nf > 0) {
-            k_box_level<<<blocks_for(nf, 128), 128, 0, s>>>(a, nf, t.nlink, t.next, c->pfix, blo, bhi, t.ncen);
-            note_launch();
-        }
-    }
-    k_box_final<<<blocks_for(t.count, 256), 256, 0, s>>>(t.count, blo, bhi, t.ncen, t.next);
-    note_launch();
-    {
-        const int first = t.level_begin[1];
-        const int last = t.level_begin[std::min(t.nlevels, kStartLevels) + 1];
-        cudaMemsetAsync(c->start_tab, 0xff, kStartTableSize * sizeof(int32_t), s);
-        if (last > first) {
-            k_start_table<<<blocks_for(last - first, 256), 256, 0, s>>>(first, last - first, t.nlink, t.nlevel,
-                                                                        c->pfix, c->start_tab);
-            note_launch();
-        }
-        c->start_valid = true;
-    }
-    return check_cuda(cudaGetLastError(), "octree build");
-}
-
-int refresh_hmax(Ctx* c, cudaStream_t s) {
-    Tree& t = c->tree;
-    for (int lv = t.nlevels - 1; lv >= 0; --lv) {
-        int a = t.level_begin[lv], nf = t.level_begin[lv + 1] - a;
-        if (nf > 0) {
-            k_hmax_level<<<blocks_for(nf, 128), 128, 0, s>>>(a, nf, t.nlink, t.next, c->pfix, t.ncen);
-            note_launch();
-        }
-    }
-    return check_cuda(cudaGetLastError(), "hmax refresh");
-}
-
-// ---------------------------------------------------------------------------------
-// Forest of one octree per box (batch path).  Box k's particles are the ranks
-// [box_off[k], box_off[k+1]) (sorted by box, then key); node k < nbox is box k's
-// root.  Levels are built as above, but every count stays on the device (the level
-// table lvl, lvl[L] = first node of level L), so that the whole build can be captured
-// in a CUDA graph: the kernels of a level run over a grid-stride range read from lvl.
-// ---------------------------------------------------------------------------------
-
-constexpr int kForestGrid = 1024;   // blocks of the grid-stride kernels
-
-__global__ void k_forest_roots(int nbox, const int64_t* __restrict__ box_off, int4* __restrict__ nlink,
-                               float4* __restrict__ next, int32_t* __restrict__ nlevel, int32_t* __restrict__ lvl) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < nbox) {
-        nlink[k] = make_int4((int)box_off[k], (int)(box_off[k + 1] - box_off[k]), -1, -1);
-        next[k] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0));
-        nlevel[k] = 0;
-    }
-    if (k <= kKeyLevels + 2) lvl[k] = (k == 0) ? 0 : nbox;
-}
-
-// box_cfg (optional): per box, bits 16..23 = that box's leaf size (0: leaf_size); the
-// node's box is the box of its first particle
-__global__ void k_split_count_dev(const uint64_t* __restrict__ keys, const int4* __restrict__ nlink,
-                                  const int32_t* __restrict__ lvl, int level, int leaf_size,
-                                  int32_t* __restrict__ nchild, const int32_t* __restrict__ box_cfg,
-                                  const int32_t* __restrict__ box_of_rank) {
-    const int a = lvl[level], nf = lvl[level + 1] - a;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nf; k += gridDim.x * blockDim.x) {
-        int4 L = nlink[a + k];
-        int cnt = 0;
-        int leaf = leaf_size;
-        if (box_cfg && L.y > 0) {
-            const int lb = (box_cfg[box_of_rank[L.x]] >> 16) & 0xff;
-            if (lb > 0) leaf = lb;
-        }
-        if (L.y > leaf && level < kKeyLevels) {
-            int b[9];
-            octant_bounds(keys, L.x, L.x + L.y, 3 * (kKeyLevels - 1 - level), b);
-#pragma unroll
-            for (int d = 0; d < 8; ++d) cnt += b[d + 1] > b[d] ? 1 : 0;
-        }
-        nchild[k] = cnt;
-    }
-}
-
-// children of one level; nodes beyond the capacity are not created (their parent stays
-// a leaf, the error flag is set and the results of the call are invalid)
-__global__ void k_split_write_dev(const uint64_t* __restrict__ keys, int4* __restrict__ nlink,
-                                  float4* __restrict__ next, int32_t* __restrict__ nlevel, int32_t* lvl, int level,
-                                  const int32_t* __restrict__ nchild, const int32_t* __restrict__ coff,
-                                  const int32_t* __restrict__ total, int64_t cap, unsigned* err) {
-    const int a = lvl[level], b = lvl[level + 1], nf = b - a;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nf; k += gridDim.x * blockDim.x) {
-        const int nc = nchild[k];
-        int4 L = nlink[a + k];
-        const int child0 = b + coff[k];
-        if (nc == 0 || (int64_t)child0 + nc > cap) {
-            if (nc > 0) atomicOr(err, kErrNodes);
-            next[a + k].w = __int_as_float(0);
-            continue;
-        }
-        next[a + k].w = __int_as_float(nc);
-        int bd[9];
-        octant_bounds(keys, L.x, L.x + L.y, 3 * (kKeyLevels - 1 - level), bd);
-        int c = 0;
-#pragma unroll
-        for (int d = 0; d < 8; ++d) {
-            if (bd[d + 1] > bd[d]) {
-                const int id = child0 + c;
-                const int skip = (c + 1 < nc) ? id + 1 : L.w;
-                nlink[id] = make_int4(bd[d], bd[d + 1] - bd[d], -1, skip);
-                next[id] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0));
-                nlevel[id] = level + 1;
-                ++c;
-            }
-        }
-        L.z = child0;
-        nlink[a + k] = L;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) lvl[level + 2] = (int)min((int64_t)b + *total, cap);
-}
-
-__global__ void k_box_level_dev(const int32_t* __restrict__ lvl, int level, const int4* __restrict__ nlink,
-                                const float4* __restrict__ next, const uint4* __restrict__ pfix,
-                                uint4* __restrict__ blo, uint4* __restrict__ bhi, uint4* __restrict__ ncen) {
-    const int a = lvl[level], nf = lvl[level + 1] - a;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nf; k += gridDim.x * blockDim.x) {
-        const int id = a + k;
-        const int4 L = nlink[id];
-        uint32_t lx = 0xffffffffu, ly = 0xffffffffu, lz = 0xffffffffu, hx = 0, hy = 0, hz = 0;
-        float hm = 0.0f;
-        const int nc = __float_as_int(next[id].w);
-        if (nc == 0) {
-            for (int q = L.x; q < L.x + L.y; ++q) {
-                const uint4 P = pfix[q];
-                lx = min(lx, P.x); ly = min(ly, P.y); lz = min(lz, P.z);
-                hx = max(hx, P.x); hy = max(hy, P.y); hz = max(hz, P.z);
-                hm = fmaxf(hm, __uint_as_float(P.w));
-            }
-        } else {
-            for (int c = L.z; c < L.z + nc; ++c) {
-                const uint4 l = blo[c], h = bhi[c];
-                lx = min(lx, l.x); ly = min(ly, l.y); lz = min(lz, l.z);
-                hx = max(hx, h.x); hy = max(hy, h.y); hz = max(hz, h.z);
-                hm = fmaxf(hm, __uint_as_float(ncen[c].w));
-            }
-        }
-        if (L.y == 0) lx = ly = lz = hx = hy = hz = 0u;   // an empty box
-        blo[id] = make_uint4(lx, ly, lz, 0u);
-        bhi[id] = make_uint4(hx, hy, hz, 0u);
-        ncen[id].w = __float_as_uint(hm);
-    }
-}
-
-__global__ void k_box_final_dev(const int32_t* __restrict__ lvl, const uint4* __restrict__ blo,
-                                const uint4* __restrict__ bhi, uint4* __restrict__ ncen, float4* __restrict__ next) {
-    const int64_t nn = lvl[kKeyLevels + 1];
-    for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < nn; id += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 l = blo[id], h = bhi[id];
-        uint4 C = ncen[id];
-        const uint64_t wx = (uint64_t)h.x - l.x + 1, wy = (uint64_t)h.y - l.y + 1, wz = (uint64_t)h.z - l.z + 1;
-        C.x = l.x + (uint32_t)(wx >> 1);
-        C.y = l.y + (uint32_t)(wy >> 1);
-        C.z = l.z + (uint32_t)(wz >> 1);
-        ncen[id] = C;
-        float4 E = next[id];
-        E.x = __fmul_ru(__ull2float_ru(wx + 1), 0.5f);
-        E.y = __fmul_ru(__ull2float_ru(wy + 1), 0.5f);
-        E.z = __fmul_ru(__ull2float_ru(wz + 1), 0.5f);
-        next[id] = E;
-    }
-}
-
-__global__ void k_hmax_level_dev(const int32_t* __restrict__ lvl, int level, const int4* __restrict__ nlink,
-                                 const float4* __restrict__ next, const uint4* __restrict__ pfix,
-                                 uint4* __restrict__ ncen) {
-    const int a = lvl[level], nf = lvl[level + 1] - a;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nf; k += gridDim.x * blockDim.x) {
-        const int id = a + k;
-        const int4 L = nlink[id];
-        const int nc = __float_as_int(next[id].w);
-        float hm = 0.0f;
-        if (nc == 0) {
-            for (int q = L.x; q < L.x + L.y; ++q) hm = fmaxf(hm, __uint_as_float(pfix[q].w));
-        } else {
-            for (int c = L.z; c < L.z + nc; ++c) hm = fmaxf(hm, __uint_as_float(ncen[c].w));
-        }
-        ncen[id].w = __float_as_uint(hm);
-    }
-}
-
-// Start tables of a forest (one per box, see k_start_table): every node of levels
-// 1 .. kStartLevels enters its box's table under its cell.
-__global__ void k_start_table_forest(const int32_t* __restrict__ lvl, const int4* __restrict__ nlink,
-                                     const int32_t* __restrict__ nlevel, const uint4* __restrict__ pfix,
-                                     const int32_t* __restrict__ box_of_rank, int32_t* __restrict__ tab) {
-    const int first = lvl[1], count = lvl[kStartLevels + 1] - first;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
-        const int id = first + k;
+                              const int32_t* __restrict__ box_of_rank, int32_t* __restrict__ tab) {
+    int end, nf;
+    level_range(lcnt, kStartLevels, cap, end, nf);
+    end += nf;
+    for (int id = lcnt[0] + blockIdx.x * blockDim.x + threadIdx.x; id < end; id += gridDim.x * blockDim.x) {
         const int l = nlevel[id];
         const int4 L = nlink[id];
         if (l < 1 || l > kStartLevels || L.y <= 0) continue;
@@ -556,75 +386,155 @@ __global__ void k_start_table_forest(const int32_t* __restrict__ lvl, const int4
         const uint32_t x = P.x >> (32 - l), y = P.y >> (32 - l), z = P.z >> (32 - l);
         uint32_t m = 0;
         for (int b = l - 1; b >= 0; --b) m = (m << 3) | (((x >> b) & 1u) << 2) | (((y >> b) & 1u) << 1) | ((z >> b) & 1u);
-        tab[(size_t)box_of_rank[L.x] * kStartTableSize + start_table_offset(l) + m] = id;
+        tab[(size_t)(box_of_rank ? box_of_rank[L.x] : 0) * kStartTableSize + start_table_offset(l) + m] = id;
     }
 }
 
-int alloc_forest(Ctx* c, int64_t cap) {
+constexpr int kTreeGrid = 1024;   // most blocks of the grid-stride kernels
+
+// Node arrays for cap nodes (the old contents are dropped).
+int alloc_tree(Ctx* c, int64_t cap) {
     Tree& t = c->tree;
-    if (t.cap >= cap) return SPHGRP_OK;
-    if (t.ncen) {
-        cudaFree(t.ncen);
-        cudaFree(t.next);
-        cudaFree(t.nlink);
-        cudaFree(t.nlevel);
-        t.ncen = nullptr;
-        t.next = nullptr;
-        t.nlink = nullptr;
-        t.nlevel = nullptr;
-        t.cap = 0;
+    if (!t.level_cnt && cudaMalloc(&t.level_cnt, kTreeLevels * sizeof(int32_t)) != cudaSuccess) {
+        t.level_cnt = nullptr;
+        cudaGetLastError();
+        return set_error(SPHGRP_ENOMEM, "octree level counts");
     }
-    if (cudaMalloc(&t.ncen, cap * sizeof(uint4)) != cudaSuccess ||
-        cudaMalloc(&t.next, cap * sizeof(float4)) != cudaSuccess ||
-        cudaMalloc(&t.nlink, cap * sizeof(int4)) != cudaSuccess ||
-        cudaMalloc(&t.nlevel, cap * sizeof(int32_t)) != cudaSuccess)
-        return set_error(SPHGRP_ENOMEM, "forest allocation failed");
+    if (cap <= t.cap) return SPHGRP_OK;
+    void** ptrs[] = {(void**)&t.ncen, (void**)&t.next, (void**)&t.nlink, (void**)&t.nlevel, (void**)&t.nparent,
+                     (void**)&t.narrive, (void**)&t.box_lo, (void**)&t.box_hi};
+    const size_t bytes[] = {sizeof(uint4), sizeof(float4), sizeof(int4), sizeof(int32_t), sizeof(int32_t),
+                            sizeof(uint32_t), sizeof(uint4), sizeof(uint4)};
+    for (void** p : ptrs) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+    t.cap = 0;
+    for (int k = 0; k < 8; ++k) {
+        if (cudaMalloc(ptrs[k], (size_t)cap * bytes[k]) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(SPHGRP_ENOMEM, "octree allocation failed");
+        }
+    }
     t.cap = cap;
     return SPHGRP_OK;
 }
 
-// lvl: device, kKeyLevels + 3 entries; blo/bhi: device scratch of t.cap entries;
-// tot: one device int.  Uses c->flag and c->scan as per-level scratch.
-int build_forest(Ctx* c, int nbox, const int64_t* box_off_dev, int32_t* lvl, uint4* blo, uint4* bhi, int32_t* tot,
-                 const int32_t* box_of_rank, int32_t* start_tabs, cudaStream_t s, const int32_t* box_cfg) {
+static void launch_levels(Ctx* c, int from, int to, int nbox, const int32_t* tab, const int32_t* box_cfg,
+                          const int32_t* box_of_rank, cudaStream_t s) {
+    Tree& t = c->tree;
+    for (int level = from; level < to; ++level) {
+        // at most 8^level nodes per box
+        const int64_t bound = level < 7 ? std::min<int64_t>(t.cap, (int64_t)nbox << (3 * level)) : t.cap;
+        const int grid = (int)std::min<int64_t>((bound + 255) / 256, kTreeGrid);
+        k_split_level<<<grid, 256, 0, s>>>(c->keys, t.nlink, t.next, t.nlevel, t.nparent, t.narrive, t.level_cnt, level,
+                                           c->p.leaf_size, tab, box_cfg, box_of_rank, t.cap, c->err);
+        note_launch();
+    }
+}
+
+constexpr int64_t kClimbNodes = 1 << 17;
+
+// Boxes and hmax (BOXES) or hmax alone, of at most `bound` nodes in levels 0 .. deepest.
+template <bool BOXES>
+static void launch_up(Ctx* c, int64_t bound, int deepest, cudaStream_t s) {
+    Tree& t = c->tree;
+    const int grid = (int)std::min<int64_t>((bound + 31) / 32, 16 * kTreeGrid);
+    if (bound <= kClimbNodes) {
+        k_tree_leaves<BOXES, true><<<grid, 256, 0, s>>>(t.level_cnt, t.cap, t.nlink, t.next, c->pfix, t.nparent,
+                                                        t.narrive, t.box_lo, t.box_hi, t.ncen);
+        note_launch();
+        return;
+    }
+    k_tree_leaves<BOXES, false><<<grid, 256, 0, s>>>(t.level_cnt, t.cap, t.nlink, t.next, c->pfix, t.nparent,
+                                                     t.narrive, t.box_lo, t.box_hi, t.ncen);
+    note_launch();
+    for (int level = deepest - 1; level >= 0; --level) {
+        const int64_t most = level < 6 ? std::min<int64_t>(bound, (int64_t)t.nroots << (3 * level)) : bound;
+        k_tree_level<BOXES><<<(int)std::min<int64_t>((most + 255) / 256, 2 * kTreeGrid), 256, 0, s>>>(
+            t.level_cnt, level, t.cap, t.nlink, t.next, t.box_lo, t.box_hi, t.ncen);
+        note_launch();
+    }
+}
+
+int build_tree(Ctx* c, cudaStream_t s) {
+    Tree& t = c->tree;
+    const int64_t n = c->n;
+    int rc = alloc_tree(c, std::max<int64_t>(1024, 2 * n / std::max(1, c->p.leaf_size) + 64));
+    if (rc) return rc;
+    if (!t.top_cells && cudaMalloc(&t.top_cells, kTopTableSize * sizeof(int32_t)) != cudaSuccess) {
+        t.top_cells = nullptr;
+        return set_error(SPHGRP_ENOMEM, "octree top-cell table");
+    }
+    int32_t* top = t.top_cells;
+    cudaMemsetAsync(top, 0xff, kTopTableSize * sizeof(int32_t), s);
+    k_top_cells<<<blocks_for(n, 256), 256, 0, s>>>(c->keys, n, top);
+    note_launch();
+    int32_t* host = c->host_small + 8;   // kTreeLevels entries (the counters' place, unused here)
+    static_assert(8 + kTreeLevels <= 64, "pinned scratch");
+    for (;;) {
+        k_tree_roots<<<1, 256, 0, s>>>(1, nullptr, n, t.nlink, t.next, t.nlevel, t.nparent, t.narrive, t.level_cnt);
+        note_launch();
+        // as many levels as the last build had and two more; the rest if they were too few
+        int upto = std::min(kKeyLevels, t.nlevels + 2);
+        launch_levels(c, 0, upto, 1, top, nullptr, nullptr, s);
+        cudaMemcpyAsync(host, t.level_cnt, kTreeLevels * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+        if ((rc = check_cuda(cudaStreamSynchronize(s), "octree levels"))) return rc;
+        while (upto < kKeyLevels && host[upto] > 0) {
+            launch_levels(c, upto, kKeyLevels, 1, top, nullptr, nullptr, s);
+            upto = kKeyLevels;
+            cudaMemcpyAsync(host, t.level_cnt, kTreeLevels * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+            if ((rc = check_cuda(cudaStreamSynchronize(s), "octree levels"))) return rc;
+        }
+        int64_t total = 0;
+        t.nlevels = 0;
+        for (int l = 0; l < kTreeLevels; ++l) {
+            total += host[l];
+            if (host[l] > 0) t.nlevels = l;
+        }
+        t.count = total;
+        if (total <= t.cap) break;
+        // too few nodes: the counts of the deeper levels are those of the children that
+        // would have been made up to there
+        cudaMemsetAsync(c->err, 0, sizeof(unsigned), s);
+        if ((rc = alloc_tree(c, std::max(total + total / 2, 2 * t.cap)))) return rc;
+    }
+    t.nroots = 1;
+    launch_up<true>(c, t.count, t.nlevels, s);
+    cudaMemsetAsync(c->start_tab, 0xff, kStartTableSize * sizeof(int32_t), s);
+    k_start_table<<<(int)std::min<int64_t>((t.count + 255) / 256, kTreeGrid), 256, 0, s>>>(
+        t.level_cnt, t.cap, t.nlink, t.nlevel, c->pfix, nullptr, c->start_tab);
+    note_launch();
+    c->start_valid = true;
+    return check_cuda(cudaGetLastError(), "octree build");
+}
+
+int refresh_hmax(Ctx* c, cudaStream_t s) {
+    launch_up<false>(c, c->tree.count, c->tree.nlevels, s);
+    return check_cuda(cudaGetLastError(), "hmax refresh");
+}
+
+// Forest of one octree per box (batch path).  Box k's particles are the ranks
+// [box_off[k], box_off[k+1]) (sorted by box, then key); node k < nbox is box k's
+// root.  Nothing is read back, so that the build can be captured in a CUDA graph.
+int build_forest(Ctx* c, int nbox, const int64_t* box_off_dev, const int32_t* box_of_rank, int32_t* start_tabs,
+                 cudaStream_t s, const int32_t* box_cfg) {
     Tree& t = c->tree;
     c->start_valid = false;   // the single-box table does not describe a forest
-    const int64_t n = c->n;
-    k_forest_roots<<<blocks_for(std::max(nbox, kKeyLevels + 3), 256), 256, 0, s>>>(nbox, box_off_dev, t.nlink,
-                                                                                 t.next, t.nlevel, lvl);
+    t.count = t.cap;          // bounds
+    t.nlevels = kKeyLevels;
+    t.nroots = nbox;
+    k_tree_roots<<<blocks_for(std::max(nbox, kTreeLevels), 256), 256, 0, s>>>(
+        nbox, box_off_dev, c->n, t.nlink, t.next, t.nlevel, t.nparent, t.narrive, t.level_cnt);
     note_launch();
-    int rc = SPHGRP_OK;
-    for (int level = 0; level < kKeyLevels; ++level) {
-        k_split_count_dev<<<kForestGrid, 256, 0, s>>>(c->keys, t.nlink, lvl, level, c->p.leaf_size, c->flag,
-                                                      box_cfg, box_of_rank);
-        note_launch();
-        if ((rc = exclusive_scan_i32_dev(c, c->flag, c->scan, lvl + level + 1, lvl + level, n, tot, s))) return rc;
-        k_split_write_dev<<<kForestGrid, 256, 0, s>>>(c->keys, t.nlink, t.next, t.nlevel, lvl, level, c->flag,
-                                                      c->scan, tot, t.cap, c->err);
-        note_launch();
-    }
-    // lvl[kKeyLevels + 1] = node count
-    for (int level = kKeyLevels; level >= 0; --level) {
-        k_box_level_dev<<<kForestGrid, 128, 0, s>>>(lvl, level, t.nlink, t.next, c->pfix, blo, bhi, t.ncen);
-        note_launch();
-    }
-    k_box_final_dev<<<kForestGrid, 256, 0, s>>>(lvl, blo, bhi, t.ncen, t.next);
-    note_launch();
+    launch_levels(c, 0, kKeyLevels, nbox, nullptr, box_cfg, box_of_rank, s);
+    launch_up<true>(c, t.cap, kKeyLevels, s);
     if (start_tabs) {
         cudaMemsetAsync(start_tabs, 0xff, (size_t)nbox * kStartTableSize * sizeof(int32_t), s);
-        k_start_table_forest<<<kForestGrid, 256, 0, s>>>(lvl, t.nlink, t.nlevel, c->pfix, box_of_rank, start_tabs);
+        k_start_table<<<kTreeGrid, 256, 0, s>>>(t.level_cnt, t.cap, t.nlink, t.nlevel, c->pfix, box_of_rank, start_tabs);
         note_launch();
     }
     return check_cuda(cudaGetLastError(), "forest build");
-}
-
-int refresh_hmax_forest(Ctx* c, const int32_t* lvl, cudaStream_t s) {
-    Tree& t = c->tree;
-    for (int level = kKeyLevels; level >= 0; --level) {
-        k_hmax_level_dev<<<kForestGrid, 128, 0, s>>>(lvl, level, t.nlink, t.next, c->pfix, t.ncen);
-        note_launch();
-    }
-    return check_cuda(cudaGetLastError(), "forest hmax refresh");
 }
 
 int gather_particles(Ctx* c, const double* pos, const float* m, cudaStream_t s) {
