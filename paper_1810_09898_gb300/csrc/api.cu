@@ -281,6 +281,8 @@ int finish(Ctx* c, cudaStream_t s, int rc) {
                                     sizeof(DevCounters), cudaMemcpyDeviceToHost, s),
                     "counter copy");
     if (rc) return rc;
+    if (c->ntimed > 0)
+        cudaMemcpyAsync(c->ctr_log_host, c->ctr_log, c->ntimed * sizeof(DevCounters), cudaMemcpyDeviceToHost, s);
     rc = check_cuda(cudaStreamSynchronize(s), "stream");
     if (rc) return rc;
     err = (unsigned)c->host_small[1];
@@ -298,8 +300,6 @@ int finish(Ctx* c, cudaStream_t s, int rc) {
         if (cudaEventElapsedTime(&t, c->tev[2 * k], c->tev[2 * k + 1]) == cudaSuccess) ms += t;
         c->log_ms[k] = t;
     }
-    if (c->ntimed > 0)
-        cudaMemcpy(c->ctr_log_host, c->ctr_log, c->ntimed * sizeof(DevCounters), cudaMemcpyDeviceToHost);
     c->last.search_ms = ms;
     c->last.search_launches = c->ntimed;
     if (err & kErrRange) return set_error(SPHGRP_EINVAL, "a position is outside [0,1) or not finite");
@@ -831,6 +831,12 @@ int sphgrp_group_supersets(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active
 
 namespace sphgrp {
 
+// Work lists of at most this many particles per SM iterate inside their groups (one launch)
+// instead of by passes: there a pass costs its launches and its read-back, and the
+// regrouping gains little.  Passes / in groups, uniform sets from the uniform guess: 32k 600 /
+// 356 us, 131k 950 / 690, 524k 1950 / 1750, 1.0M 3530 / 3470, 4.2M 11.7 / 12.1 ms.
+constexpr int kInGroupPerSM = 4096;
+
 // The density with the smoothing-length iteration; with vel (not NULL) the same density
 // loop also sums the velocity divergence and curl (grouped form, walk passes), written to
 // divv / curlv at each particle's final h.
@@ -858,7 +864,9 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
     int* nfail = c->work + 8;
     cudaMemsetAsync(nfail, 0, sizeof(int), s);
     const int iteration = with_vel ? SPHGRP_ITER_PASSES : c->p.iteration;
-    if (grouped && iterate && iteration == SPHGRP_ITER_IN_GROUP) {
+    const bool small = iteration == SPHGRP_ITER_PASSES && !with_vel && c->p.group_mode == SPHGRP_GROUP_COUNT &&
+                       nu <= kInGroupPerSM * (int64_t)c->sm_count;
+    if (grouped && iterate && (iteration == SPHGRP_ITER_IN_GROUP || small)) {
         // one launch: every group iterates its members to convergence
         SearchArgs a = base_args(c);
         a.U = U;

@@ -1871,27 +1871,32 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) k_superset(SearchArgs a) 
 }
 
 // Density with the smoothing-length iteration inside the group (no host loop, no
-// regrouping): after every walk + filter the members update h in FP64 (the same
-// Newton / bisection step as k_hsml_update); converged members leave the group, the
-// centre and radius are recomputed over the remaining ones and the group walks again,
-// until every member has converged or reached max_iter passes.  A particle's density
-// at h depends only on the positions and its own h, so the iterates equal those of the
-// pass-by-pass iteration (up to the order of the FP32 sums).
-__device__ __forceinline__ bool hsml_step(const SearchArgs& a, const IterArgs& it, int r, double& h, double& lo,
-                                          double& hi, float s0, float s1, int nngb, int pass, bool writer) {
-    const double kPi = 3.14159265358979323846;
-    const double m = (double)a.poff[r].w;
-    const double sigma = 8.0 / (kPi * h * h * h);
-    const double rho = sigma * (double)s0;
-    const double drho = -sigma / h * (double)s1;
-    const double neff = 4.0 * kPi / 3.0 * h * h * h * rho / m;
-    const bool done = fabs(neff - it.nngb) <= it.tol;
+// regrouping): after every walk + filter the members take the Newton / bisection step (in
+// FP64); converged members leave the group, the centre and radius are recomputed over the
+// remaining ones and the group walks again, until every member has converged or reached
+// max_iter passes.  A particle's density at h depends only on the positions and its own
+// h, so the iterates equal those of the pass-by-pass iteration (up to the order of the
+// FP32 sums and the rounding of the step).
+//
+// Every lane takes its member's step, and an FP64 instruction of a warp takes 16 cycles of
+// an SM: written with rho, dRho/dh and their divisions the step took about as long as a
+// search.  In terms of the sums (see hsml_next) it has one division: N_eff = (32/3) S0 / m,
+// g / g' = h (32 S0 - 3 N_ngb m) / (32 (3 S0 - S1)); the results, once per particle, two.
+__device__ __forceinline__ bool hsml_step(const SearchArgs& a, const IterArgs& it, int r, float mf, double& h,
+                                          double& lo, double& hi, float s0, float s1, int nngb, int pass,
+                                          bool writer) {
+    const double m = (double)mf, a0 = (double)s0;
+    const double t = (32.0 / 3.0) * a0, nm = it.nngb * m;
+    const double den = 3.0 * a0 - (double)s1;
+    const bool done = fabs(t - nm) <= it.tol * m;
     if (done || pass >= it.max_iter) {
         if (writer) {
             const int orig = a.perm[r];
-            it.rho[orig] = (float)rho;
-            it.drhodh[orig] = (float)drho;
-            it.fgrad[orig] = (float)(1.0 / (1.0 + h / (3.0 * rho) * drho));
+            const double ih = 1.0 / h;
+            const double sigma = (8.0 / 3.14159265358979323846) * ih * ih * ih;
+            it.rho[orig] = (float)(sigma * a0);
+            it.drhodh[orig] = (float)(-sigma * ih * (double)s1);
+            it.fgrad[orig] = (float)(3.0 * a0 / den);   // 1 / (1 + h / (3 rho) dRho/dh)
             it.nngb_out[orig] = nngb;
             if (it.iters) it.iters[orig] = pass;
             it.h_out[orig] = h;
@@ -1900,21 +1905,18 @@ __device__ __forceinline__ bool hsml_step(const SearchArgs& a, const IterArgs& i
         }
         return true;
     }
-    if (neff < it.nngb) lo = h; else hi = h;
-    const double g = 4.0 * kPi / 3.0 * h * h * h * rho - it.nngb * m;
-    const double gp = 4.0 * kPi * h * h * rho + 4.0 * kPi / 3.0 * h * h * h * drho;
-    double hn = h - g / gp;
-    const double cbrt2 = 1.2599210498948731647672106;
+    if (t < nm) lo = h; else hi = h;
+    double hn = h - h * ((t - nm) * 3.0 / (32.0 * den));
     if (!(hn > lo && hn < hi) || !isfinite(hn)) {
+        const double cbrt2 = 1.2599210498948731647672106;
         if (isinf(hi)) hn = h * cbrt2;
         else if (lo == 0.0) hn = h / cbrt2;
         else hn = cbrt(0.5 * (lo * lo * lo + hi * hi * hi));
     }
-    hn = fmin(hn, 0.49);   // the minimum image needs h < 1/2 (such a particle cannot converge)
-    h = hn;
+    h = fmin(hn, 0.49);   // the minimum image needs h < 1/2 (such a particle cannot converge)
     if (writer) {
-        it.h64[r] = hn;
-        it.pfix[r].w = __float_as_uint((float)hn);
+        it.h64[r] = h;
+        it.pfix[r].w = __float_as_uint((float)h);
     }
     return false;
 }
@@ -1953,7 +1955,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
             const float s1 = __shfl_sync(0xffffffffu, mem.s1 - mem.c1, src);
             const int nn = __shfl_sync(0xffffffffu, mem.n, src);
             if (rec[0].rank >= 0 &&
-                hsml_step(a, it, rec[0].rank, rec[0].h, lo, hi, s0, s1, nn, pass, L.slice == 0))
+                hsml_step(a, it, rec[0].rank, rec[0].O.w, rec[0].h, lo, hi, s0, s1, nn, pass, L.slice == 0))
                 rec[0].rank = -1;
             // the new h (global memory) is read by the next pass's FP64 re-tests
             __syncwarp();
