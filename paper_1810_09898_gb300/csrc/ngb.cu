@@ -29,7 +29,10 @@ constexpr int kWarpsPerBlock = 4;
 constexpr int kStackCap = kStackSharedMax;     // walk stack entries in shared memory
 constexpr int kRangeCap = 64;                  // pending particle ranges (ring, power of two)
 constexpr int kSpillCap = kStackSpillPerWarp;  // overflow entries per warp (global memory)
-constexpr int kTile = 128;                     // candidates of a tile (192: 1-9% slower, fewer warps fit)
+// candidates of a tile: density kinds, and those whose candidates carry records (larger
+// tiles balance the lanes of phase B better, until fewer warps fit)
+constexpr int kTileD = 160;
+constexpr int kTileR = 128;
 constexpr int kPartMax = 32;                   // members searched at once (one per lane)
 // The walk takes a node of at most this many particles whole instead of opening it.
 constexpr int kWalkWhole = 32;
@@ -197,9 +200,13 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;
 
 // position part shared by all members: coordinates relative to the group centre (the
 // exact fixed-point position is reloaded by the rare paths that need it)
+// Lower decision threshold of members whose physics takes exact differences: no pair lies
+// below it, so every one goes through the decision's slow path (one-sided kinds: h2lo;
+// symmetric ones: -bk).
+constexpr float kAlwaysSlow = -3.0e38f;
+
 struct MemberPos {
     float mx, my, mz;
-    bool precise;       // far from the group centre: physics from exact differences
     int rank;           // -1: slot empty
     int n;              // neighbours found
     int64_t xpos;       // export write position
@@ -227,13 +234,14 @@ __device__ __forceinline__ MemberRec load_member(const SearchArgs& a, int rank) 
     return r;
 }
 
+// precise: far from the group centre, physics from exact differences
 __device__ __forceinline__ bool pos_init(MemberPos& M, const MemberRec& rec, uint32_t cx, uint32_t cy, uint32_t cz,
-                                         float hf) {
+                                         float hf, bool& precise) {
     const int rank = rec.rank;
     M.rank = rank;
     M.n = 0;
     M.xpos = 0;
-    M.precise = false;
+    precise = false;
     if (rank < 0) {
         M.mx = M.my = M.mz = 0.0f;
         return false;
@@ -241,7 +249,7 @@ __device__ __forceinline__ bool pos_init(MemberPos& M, const MemberRec& rec, uin
     M.mx = rel_coord(rec.P.x, rec.O.x, cx);
     M.my = rel_coord(rec.P.y, rec.O.y, cy);
     M.mz = rel_coord(rec.P.z, rec.O.z, cz);
-    M.precise = fmaxf(fabsf(M.mx), fmaxf(fabsf(M.my), fabsf(M.mz))) > kPreciseReach * hf;
+    precise = fmaxf(fabsf(M.mx), fmaxf(fabsf(M.my), fabsf(M.mz))) > kPreciseReach * hf;
     return true;
 }
 
@@ -325,7 +333,8 @@ __device__ __forceinline__ void member_init(DMember& M, const SearchArgs& a, con
     M.p0 = M.p1 = 0.0f;
     const double h = rec.h;
     float hf = (float)h;
-    if (!pos_init(M, rec, cx, cy, cz, hf)) {
+    bool precise;
+    if (!pos_init(M, rec, cx, cy, cz, hf, precise)) {
         M.hinv = 0.0f;
         M.h2lo = M.h2hi = -1.0f;
         M.thr_dot = -3.0e38f;
@@ -336,7 +345,7 @@ __device__ __forceinline__ void member_init(DMember& M, const SearchArgs& a, con
     float m2 = M.mx * M.mx + M.my * M.my + M.mz * M.mz;
     float bk = 8.0f * kBandRel * m2;
     M.h2hi = fmaf(h2, 1.0f + 3.0f * kBandRel, bk);
-    M.h2lo = fmaf(h2, 1.0f - 3.0f * kBandRel, -bk);
+    M.h2lo = precise ? kAlwaysSlow : fmaf(h2, 1.0f - 3.0f * kBandRel, -bk);
     M.thr_dot = M.h2hi - m2;
 }
 
@@ -385,7 +394,8 @@ __device__ __forceinline__ bool sym_init(SymMember& M, const MemberRec& rec, uin
                                          uint32_t cz) {
     const double h = rec.h;
     M.h = (float)h;
-    if (!pos_init(M, rec, cx, cy, cz, M.h)) {
+    bool precise;
+    if (!pos_init(M, rec, cx, cy, cz, M.h, precise)) {
         M.h = 0.0f; M.hinv = 0.0f; M.sk = 0.0f;
         M.h2 = -1.0f; M.bk = -1.0f;
         M.bk_dot = -3.0e38f;
@@ -393,8 +403,8 @@ __device__ __forceinline__ bool sym_init(SymMember& M, const MemberRec& rec, uin
     }
     M.h2 = (float)(h * h);
     float m2 = M.mx * M.mx + M.my * M.my + M.mz * M.mz;
-    M.bk = 8.0f * kBandRel * m2;
-    M.bk_dot = M.bk - m2;
+    M.bk = precise ? -kAlwaysSlow : 8.0f * kBandRel * m2;
+    M.bk_dot = 8.0f * kBandRel * m2 - m2;
     return true;
 }
 
@@ -457,7 +467,8 @@ __device__ __forceinline__ void member_init(VMember& M, const SearchArgs& a, con
     M.rrho = 0.0f;
     const double h = rec.h;
     float hf = (float)h;
-    if (!pos_init(M, rec, cx, cy, cz, hf)) {
+    bool precise;
+    if (!pos_init(M, rec, cx, cy, cz, hf, precise)) {
         M.hinv = 0.0f;
         M.h2lo = M.h2hi = -1.0f;
         M.thr_dot = -3.0e38f;
@@ -468,7 +479,7 @@ __device__ __forceinline__ void member_init(VMember& M, const SearchArgs& a, con
     float m2 = M.mx * M.mx + M.my * M.my + M.mz * M.mz;
     float bk = 8.0f * kBandRel * m2;
     M.h2hi = fmaf(h2, 1.0f + 3.0f * kBandRel, bk);
-    M.h2lo = fmaf(h2, 1.0f - 3.0f * kBandRel, -bk);
+    M.h2lo = precise ? kAlwaysSlow : fmaf(h2, 1.0f - 3.0f * kBandRel, -bk);
     M.thr_dot = M.h2hi - m2;
     const float4 H0 = a.hyd0[rec.rank];
     const float4 H1 = a.hyd1[rec.rank];
@@ -487,56 +498,45 @@ __device__ __forceinline__ float member_radius(const SymMember& M) { return M.ra
 // ---------------------------------------------------------------------------------
 // Candidate tiles in shared memory: the candidates of a group that passed the test
 // against its dilated box, in walk order, as FP32 coordinates relative to the group
-// centre, packed in pairs, with their mass (symmetric kinds: and h^2), rank and the
-// kind's own records.  With S slices the lane of slice s filters the pairs s, s + S,
-// s + 2S, ...  Phase A reads whole rows of pairs past the last candidate (up to 64 pairs,
-// into the arrays behind b) and drops their bits.
+// centre (w = |p|^2), with their mass (symmetric kinds: and h^2), rank and the kind's own
+// records.  With S slices, the candidates go to the slices in turn, four at a time, and a
+// slice's are contiguous (`rows` quads of them), so that phase A reads them by whole
+// quads at constant strides and phase B finds a candidate by adding its number to the
+// slice's start.  Phase A may read one row past the last (the next slice's or array's
+// values) and drops its bits.
 // ---------------------------------------------------------------------------------
 
-struct PlainTile {
-    float4 a[kTile / 2];    // {x0, x1, y0, y1}
-    float4 b[kTile / 2];    // {z0, z1, w0, w1}, w = |p|^2
-    float m[kTile];
-    int r[kTile];           // ranks
-    uint32_t masks[kTile];  // phase-A bit masks [word][lane]
-
-    __device__ __forceinline__ void put(int t, float x, float y, float z) {
-        const int o = 4 * (t >> 1) + (t & 1);
-        float* pa = reinterpret_cast<float*>(a);
-        float* pb = reinterpret_cast<float*>(b);
-        pa[o] = x;
-        pa[o + 2] = y;
-        pb[o] = z;
-        pb[o + 2] = fmaf(x, x, fmaf(y, y, z * z));
-    }
-    __device__ __forceinline__ float3 pos(int t) const {
-        const int o = 4 * (t >> 1) + (t & 1);
-        const float* pa = reinterpret_cast<const float*>(a);
-        return make_float3(pa[o], pa[o + 2], reinterpret_cast<const float*>(b)[o]);
-    }
+template <int N>
+struct alignas(16) PlainTileOf {
+    static constexpr int cap = N;
+    float x[N], y[N], z[N], w[N];
+    float m[N];
+    int r[N];           // ranks
+    uint32_t masks[N];  // phase-A bit masks [word][lane]
 };
-struct SymTile : PlainTile {
-    float h2[kTile];        // h_j^2
+using PlainTile = PlainTileOf<kTileD>;
+struct SymTile : PlainTileOf<kTileR> {
+    float h2[kTileR];       // h_j^2
 };
-struct VelTile : PlainTile {
-    float4 v[kTile];        // hyd0 {vx, vy, vz, -}
+struct VelTile : PlainTileOf<kTileR> {
+    float4 v[kTileR];       // hyd0 {vx, vy, vz, -}
 };
 struct HydroTile : SymTile {
-    float4 v[kTile];        // hyd0 {vx, vy, vz, c}
-    float4 h[kTile];        // hyd1 {A, rho, 1/h, limiter}
+    float4 v[kTileR];       // hyd0 {vx, vy, vz, c}
+    float4 h[kTileR];       // hyd1 {A, rho, 1/h, limiter}
 };
 struct HAdjTile : SymTile {
-    float4 v[kTile];        // hyd0 {vx, vy, vz, c}
-    float4 h[kTile];        // hyd1 {A, rho, 1/h, 8/(pi h^4)}
-    float4 w[kTile];        // wadj {wx, wy, wz, -}
+    float4 v[kTileR];       // hyd0 {vx, vy, vz, c}
+    float4 h[kTileR];       // hyd1 {A, rho, 1/h, 8/(pi h^4)}
+    float4 wt[kTileR];      // wadj {wx, wy, wz, -}
 };
 struct DAdjTile : SymTile {
-    float4 d[kTile];        // dadj {alpha, beta, 1/h, 8/(pi h^4)}
+    float4 d[kTileR];       // dadj {alpha, beta, 1/h, 8/(pi h^4)}
 };
 
 // kind policies; min_blocks: resident blocks per SM (register budget; 0: compiler's choice)
 struct KDens {
-    static constexpr int min_blocks = 7;
+    static constexpr int min_blocks = 8;
     static constexpr int id = 0;
     static constexpr bool sym = false;
     using Member = DMember;
@@ -604,7 +604,7 @@ __device__ __forceinline__ void stage_records(HydroTile& T, const SearchArgs& a,
 __device__ __forceinline__ void stage_records(HAdjTile& T, const SearchArgs& a, int t, int rank) {
     copy16_async(&T.v[t], a.hyd0 + rank);
     copy16_async(&T.h[t], a.hyd1 + rank);
-    copy16_async(&T.w[t], a.wadj + rank);
+    copy16_async(&T.wt[t], a.wadj + rank);
 }
 __device__ __forceinline__ void stage_records(DAdjTile& T, const SearchArgs& a, int t, int rank) {
     copy16_async(&T.d[t], a.dadj + rank);
@@ -685,25 +685,28 @@ __device__ __forceinline__ void density_terms(D2Member& M, float mj, float q) {
     M.p2 = fmaf(mj, fmaf(q * q, d2w, fmaf(8.0f * q, dw, 12.0f * w)), M.p2);
 }
 
-// Decision of the density criterion |r| < h_i, and the pair's difference.  Only the rare
-// slow path branches: the FP64 re-test inside the band, and the exact differences of
-// members far from the centre.
+// Decision of the density criterion |r| < h_i, and the pair's difference.  The caller has
+// counted the candidate in M.n; one that is outside is taken off and false returned.  Only
+// the rare slow path branches: the FP64 re-test inside the band, and the exact
+// differences of members far from the centre.
 template <bool WRAP, class Mem>
-__device__ __forceinline__ bool dens_decide(const Mem& M, const SearchArgs& a, float3 p, int crank, LocalCounters& lc,
+__device__ __forceinline__ bool dens_decide(Mem& M, const SearchArgs& a, float3 p, int crank, LocalCounters& lc,
                                             float& dx, float& dy, float& dz, float& r2) {
     dx = rel_diff<WRAP>(p.x, M.mx);
     dy = rel_diff<WRAP>(p.y, M.my);
     dz = rel_diff<WRAP>(p.z, M.mz);
     r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    bool in = r2 < M.h2lo;
-    if (M.precise || (!in && r2 < M.h2hi)) {
-        if (!in && r2 < M.h2hi) {
+    bool in = true;
+    if (!(r2 < M.h2lo)) {
+        in = false;
+        if (r2 < M.h2hi) {
             const double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
             const double h = a.h64[M.rank];
             in = e < __dmul_rn(h, h);
             lc.retests++;
         }
-        if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
+        if (!in) M.n--;
+        if (M.h2lo == kAlwaysSlow) precise_diff(M, a, crank, dx, dy, dz, r2);
     }
     return in;
 }
@@ -715,6 +718,13 @@ __device__ __forceinline__ void export_pair(MemberPos& M, const SearchArgs& a, i
     else atomicOr(a.err, kErrCap);
 }
 
+// r from r^2 (1 ulp; 0 at 0)
+__device__ __forceinline__ float sqrt_fast(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // density pair: p = candidate's coordinates relative to the member's centre, m_j its mass.
 // A candidate outside enters the sums with mass 0 (phase A leaves few of them).
 template <int MODE, bool WRAP = false, class Mem>
@@ -722,8 +732,7 @@ __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float3
                                              LocalCounters& lc) {
     float dx, dy, dz, r2;
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
-    M.n += in ? 1 : 0;
-    if (MODE == kAcc) density_terms(M, in ? mj : 0.0f, q_of(r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)), M.hinv));
+    if (MODE == kAcc) density_terms(M, in ? mj : 0.0f, q_of(sqrt_fast(r2), M.hinv));
     else if (MODE == kFill && in) export_pair(M, a, crank);
 }
 
@@ -747,9 +756,8 @@ __device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, f
                                              int crank, LocalCounters& lc) {
     float dx, dy, dz, r2;
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
-    M.n += in ? 1 : 0;
     if (MODE != kAcc) return;
-    density_terms(M, in ? mj : 0.0f, q_of(r2 * rsqrt_fast(fmaxf(r2, 1.0e-30f)), M.hinv));
+    density_terms(M, in ? mj : 0.0f, q_of(sqrt_fast(r2), M.hinv));
     if (in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
@@ -774,29 +782,29 @@ __device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float3
                                          LocalCounters& lc) {
     float dx, dy, dz, r2;
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
-    M.n += in ? 1 : 0;
     if (MODE == kAcc && in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
 // decision of the symmetric criterion |r| < max(h_i, h_j), as dens_decide
 template <bool WRAP, class Mem>
-__device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, float3 p, float hj2, int crank,
+__device__ __forceinline__ bool sym_decide(Mem& M, const SearchArgs& a, float3 p, float hj2, int crank,
                                            LocalCounters& lc, float& dx, float& dy, float& dz, float& r2) {
     dx = rel_diff<WRAP>(p.x, M.mx);
     dy = rel_diff<WRAP>(p.y, M.my);
     dz = rel_diff<WRAP>(p.z, M.mz);
     r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
     const float H2 = fmaxf(M.h2, hj2);
-    bool in = r2 < fmaf(H2, 1.0f - 3.0f * kBandRel, -M.bk);
-    const bool band = !in && r2 < fmaf(H2, 1.0f + 3.0f * kBandRel, M.bk);
-    if (M.precise || band) {
-        if (band) {
+    bool in = true;
+    if (!(r2 < fmaf(H2, 1.0f - 3.0f * kBandRel, -M.bk))) {
+        in = false;
+        if (r2 < fmaf(H2, 1.0f + 3.0f * kBandRel, M.bk)) {
             const double e = exact_r2(a.xd, a.yd, a.zd, M.rank, crank);
             const double hi = a.h64[M.rank], hj = a.h64[crank];
             in = e < fmax(__dmul_rn(hi, hi), __dmul_rn(hj, hj));
             lc.retests++;
         }
-        if (M.precise) precise_diff(M, a, crank, dx, dy, dz, r2);
+        if (!in) M.n--;
+        if (M.bk == -kAlwaysSlow) precise_diff(M, a, crank, dx, dy, dz, r2);
     }
     return in;
 }
@@ -807,13 +815,11 @@ __device__ __forceinline__ bool sym_decide(const Mem& M, const SearchArgs& a, fl
 template <int MODE, bool WRAP = false>
 __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float3 p, float2 q,
                                            float4 v, float4 hh, int crank, LocalCounters& lc) {
-    // The member itself is a candidate: the exports skip it by rank; the sums count it
-    // as a pair at r = 0, taken off the neighbour count at the end.
-    if (MODE != kAcc && crank == M.rank) return;
+    // The member itself is a candidate, counted as a pair at r = 0 and taken off the
+    // neighbour count at the end; the export skips it by rank.
     float dx, dy, dz, r2;
     const bool in = sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2);
-    M.n += in ? 1 : 0;
-    if (MODE == kFill && in) export_pair(M, a, crank);
+    if (MODE == kFill && in && crank != M.rank) export_pair(M, a, crank);
     if (MODE != kAcc || !(in && r2 > 0.0f)) return;
     const float rinv = rsqrt_fast(r2);
     const float r = r2 * rinv;
@@ -849,7 +855,6 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     // the member itself enters as a pair at r = 0, which contributes nothing
     float dx, dy, dz, r2;
     if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
-    M.n++;
     if (MODE != kAcc) return;
     if (r2 == 0.0f) return;
     const float rinv = rsqrt_fast(r2);
@@ -924,7 +929,6 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
     // alpha W(0, h) + beta W_h(0, h) = alpha s h - 3 beta s, and no position term.
     float dx, dy, dz, r2;
     if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
-    M.n++;
     if (MODE != kAcc) return;
     const float rinv = r2 > 0.0f ? rsqrt_fast(r2) : 0.0f;
     const float r = r2 * rinv;
@@ -950,42 +954,42 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DMember& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.r[j], lc);
+    density_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(D2Member& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.r[j], lc);
+    density_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DVMember& M, const SearchArgs& a, const VelTile& T, int j,
                                           LocalCounters& lc) {
-    densvel_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.v[j], T.r[j], lc);
+    densvel_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), T.m[j], T.v[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DLMember& M, const SearchArgs& a, const PlainTile& T, int j,
                                           LocalCounters& lc) {
-    density_list_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.r[j], lc);
+    density_list_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), T.m[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(VMember& M, const SearchArgs& a, const VelTile& T, int j,
                                           LocalCounters& lc) {
-    vel_pair<MODE, WRAP>(M, a, T.pos(j), T.m[j], T.v[j], T.r[j], lc);
+    vel_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), T.m[j], T.v[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(HMember& M, const SearchArgs& a, const HydroTile& T, int j,
                                           LocalCounters& lc) {
-    hydro_pair<MODE, WRAP>(M, a, T.pos(j), make_float2(T.h2[j], T.m[j]), T.v[j], T.h[j], T.r[j], lc);
+    hydro_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), make_float2(T.h2[j], T.m[j]), T.v[j], T.h[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(HAMember& M, const SearchArgs& a, const HAdjTile& T, int j,
                                           LocalCounters& lc) {
-    hydro_adj_pair<MODE, WRAP>(M, a, T.pos(j), make_float2(T.h2[j], T.m[j]), T.v[j], T.h[j], T.w[j], T.r[j], lc);
+    hydro_adj_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), make_float2(T.h2[j], T.m[j]), T.v[j], T.h[j], T.wt[j], T.r[j], lc);
 }
 template <int MODE, bool WRAP>
 __device__ __forceinline__ void tile_pair(DAMember& M, const SearchArgs& a, const DAdjTile& T, int j,
                                           LocalCounters& lc) {
-    dens_adj_pair<MODE, WRAP>(M, a, T.pos(j), make_float2(T.h2[j], T.m[j]), T.d[j], T.r[j], lc);
+    dens_adj_pair<MODE, WRAP>(M, a, make_float3(T.x[j], T.y[j], T.z[j]), make_float2(T.h2[j], T.m[j]), T.d[j], T.r[j], lc);
 }
 
 // Phase-A thresholds: of the dot form |p|^2 - 2 p.m (one-sided kinds: a constant of the
@@ -998,7 +1002,7 @@ __device__ __forceinline__ float thr_diff(const DMember& M, float) { return M.h2
 __device__ __forceinline__ float thr_diff(const DLMember& M, float) { return M.h2whi; }
 __device__ __forceinline__ float thr_diff(const VMember& M, float) { return M.h2hi; }
 __device__ __forceinline__ float thr_diff(const SymMember& M, float hj2) {
-    return fmaf(fmaxf(M.h2, hj2), 1.0f + 3.0f * kBandRel, M.bk);
+    return fmaf(fmaxf(M.h2, hj2), 1.0f + 3.0f * kBandRel, M.bk);   // precise members: everything
 }
 
 // combine the slice copies of a member: add the values held o lanes above, where add says so
@@ -1087,7 +1091,7 @@ __device__ __forceinline__ void write_result(const HMember& H, const SearchArgs&
         a.o_dudt[orig] = H.su - H.cu;
         if (a.o_nh) a.o_nh[orig] = H.n - 1;   // the member itself was counted as a pair
     } else if (MODE == kCount) {
-        a.x_cnt[orig] = H.n;
+        a.x_cnt[orig] = H.n - 1;
     }
 }
 template <int MODE>
@@ -1145,11 +1149,13 @@ __device__ __forceinline__ int warp_incl_scan(int v, int lane) {
 // none (its slice is then S or more, or the member has left).
 struct Layout {
     int gw, S, slice, k;
+    int rows;       // quads of candidates a slice holds
     uint32_t inv;   // ceil(2^16 / S): n / S = n * inv >> 16 for the n <= 2^10 used here
 };
 
 // pow2: member slots rounded up to a power of two and at most 4 slices
-__device__ __forceinline__ Layout make_layout(int cnt, int lane, bool allow_slices, int max_slices, bool pow2) {
+__device__ __forceinline__ Layout make_layout(int cnt, int lane, bool allow_slices, int max_slices, bool pow2,
+                                              int tile) {
     Layout L;
     L.gw = pow2 && cnt > 1 ? 1 << (32 - __clz(cnt - 1)) : cnt;
     const uint32_t q = 65536u / (uint32_t)L.gw + 1u;
@@ -1158,6 +1164,7 @@ __device__ __forceinline__ Layout make_layout(int cnt, int lane, bool allow_slic
     const int k = lane - L.slice * L.gw;
     L.k = (L.slice < L.S && k < cnt) ? k : -1;
     L.inv = 65535u / (uint32_t)L.S + 1u;
+    L.rows = (int)(((tile / 4) * L.inv) >> 16);
     return L;
 }
 
@@ -1171,43 +1178,55 @@ __device__ __forceinline__ void slice_sum(Mem& M, const Layout& L) {
     }
 }
 
-// Phase A of one mask word: the lane's next 2 * rows candidates (rows a multiple of 4, at
-// most 16; pairs first, first + S, ...) against the member's FP32 threshold, the first
-// candidate in the top bit of the 2 * rows lowest ones.  Dot form, packed: per pair of
-// candidates two shared-memory loads, three packed FMAs, one packed add and two shifts
-// that collect the signs; its rounding stays inside the FP64 decision band.
+// place of the t-th candidate of a tile
+__device__ __forceinline__ int tile_place(const Layout& L, int t) {
+    const int quad = t >> 2;
+    const int row = (int)((quad * L.inv) >> 16);
+    return ((quad - row * L.S) * L.rows + row) * 4 + (t & 3);
+}
+
+// Phase A of one mask word: 4 * quads of the lane's candidates from place j0 against the
+// member's FP32 threshold, the first in the top bit of the 4 * quads lowest ones (quads
+// even).  Dot form, packed: per quad four 16-byte shared-memory loads, six packed FMAs, two
+// packed adds and four shifts that collect the signs; its rounding stays inside the FP64
+// decision band.
 template <class K, bool WRAP>
-__device__ __forceinline__ uint32_t test_word(const typename K::Tile& T, const typename K::Member& Mb, int first,
-                                              int S, int rows) {
+__device__ __forceinline__ uint32_t test_word(const typename K::Tile& T, const typename K::Member& Mb, int j0,
+                                              int quads) {
     uint32_t mask = 0u;
     if constexpr (!WRAP) {
         const unsigned long long ax = pair_of(-2.0f * Mb.mx, -2.0f * Mb.mx), ay = pair_of(-2.0f * Mb.my, -2.0f * Mb.my),
                                  az = pair_of(-2.0f * Mb.mz, -2.0f * Mb.mz),
                                  at = pair_of(-thr_dot(Mb), -thr_dot(Mb));
-        for (int r = 0; r < rows; r += 4) {
+        for (int r = 0; r < quads; r += 2) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int i = first + (r + q) * S;
-                const ulonglong2 pa = *reinterpret_cast<const ulonglong2*>(&T.a[i]);
-                const ulonglong2 pb = *reinterpret_cast<const ulonglong2*>(&T.b[i]);
-                unsigned long long w = add_pair(pb.y, at);
+            for (int q = 0; q < 2; ++q) {
+                const int j = j0 + 4 * (r + q);
+                const ulonglong2 px = *reinterpret_cast<const ulonglong2*>(&T.x[j]);
+                const ulonglong2 py = *reinterpret_cast<const ulonglong2*>(&T.y[j]);
+                const ulonglong2 pz = *reinterpret_cast<const ulonglong2*>(&T.z[j]);
+                const ulonglong2 pw = *reinterpret_cast<const ulonglong2*>(&T.w[j]);
+                unsigned long long t0 = add_pair(pw.x, at), t1 = add_pair(pw.y, at);
                 if constexpr (K::sym) {
-                    const float2 hj2 = *reinterpret_cast<const float2*>(&T.h2[2 * i]);
+                    const float4 hj2 = *reinterpret_cast<const float4*>(&T.h2[j]);
                     constexpr float kk = -(1.0f + 3.0f * kBandRel);
-                    w = fma_pair(pair_of(fmaxf(Mb.h2, hj2.x), fmaxf(Mb.h2, hj2.y)), pair_of(kk, kk), w);
+                    t0 = fma_pair(pair_of(fmaxf(Mb.h2, hj2.x), fmaxf(Mb.h2, hj2.y)), pair_of(kk, kk), t0);
+                    t1 = fma_pair(pair_of(fmaxf(Mb.h2, hj2.z), fmaxf(Mb.h2, hj2.w)), pair_of(kk, kk), t1);
                 }
-                const unsigned long long t = fma_pair(pa.x, ax, fma_pair(pa.y, ay, fma_pair(pb.x, az, w)));
-                mask = push_sign(mask, (uint32_t)t);
-                mask = push_sign(mask, (uint32_t)(t >> 32));
+                t0 = fma_pair(px.x, ax, fma_pair(py.x, ay, fma_pair(pz.x, az, t0)));
+                t1 = fma_pair(px.y, ax, fma_pair(py.y, ay, fma_pair(pz.y, az, t1)));
+                mask = push_sign(mask, (uint32_t)t0);
+                mask = push_sign(mask, (uint32_t)(t0 >> 32));
+                mask = push_sign(mask, (uint32_t)t1);
+                mask = push_sign(mask, (uint32_t)(t1 >> 32));
             }
         }
     } else {
-        for (int r = 0; r < 2 * rows; ++r) {
-            const int t = 2 * (first + (r >> 1) * S) + (r & 1);
-            const float3 p = T.pos(t);
+        for (int j = j0; j < j0 + 4 * quads; ++j) {
             float hj2 = 0.0f;
-            if constexpr (K::sym) hj2 = T.h2[t];
-            const float dx = rel_diff<true>(p.x, Mb.mx), dy = rel_diff<true>(p.y, Mb.my), dz = rel_diff<true>(p.z, Mb.mz);
+            if constexpr (K::sym) hj2 = T.h2[j];
+            const float dx = rel_diff<true>(T.x[j], Mb.mx), dy = rel_diff<true>(T.y[j], Mb.my),
+                        dz = rel_diff<true>(T.z[j], Mb.mz);
             const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
             mask = (mask << 1) | (r2 < thr_diff(Mb, hj2) ? 1u : 0u);
         }
@@ -1216,44 +1235,50 @@ __device__ __forceinline__ uint32_t test_word(const typename K::Tile& T, const t
 }
 
 // Member x candidate filter of the nt candidates in the tile.  Phase A: bit masks of the
-// lane's slice, a word per 32 candidates.  Phase B: every lane walks its own set bits
-// across all words (no per-word wait for the slowest lane) for the exact decision and the
-// pair terms; forward partial sums are folded into the compensated totals after the
-// tile.
+// lane's slice, a word per 32 candidates; their bits count as neighbours.  Phase B: every
+// lane walks its own set bits across all words (no per-word wait for the slowest lane)
+// for the exact decision and the pair terms; forward partial sums are folded into the
+// compensated totals after the tile.
 template <class K, int MODE, bool WRAP>
 __device__ __forceinline__ void filter_tile(typename K::Tile& T, const Layout& L, typename K::Member& Mb, int nt,
                                             const SearchArgs& a, LocalCounters& lc, int lane) {
     const int S = L.S;
-    const int npair = (nt + 1) >> 1;
-    const int rows = (int)(((npair + S - 1) * L.inv) >> 16);   // of slice 0, the longest
-    // the lane's own candidates: whole pairs, and the last half pair if it is its
+    const int full = nt >> 2;                                             // whole quads
+    const int most = (int)((((nt + 3) >> 2) + S - 1) * L.inv >> 16);      // quads of slice 0, the longest
+    // the lane's own candidates: its whole quads, and the last part quad if it is its
     int mine = 0;
-    if (Mb.rank >= 0)
-        mine = (int)((((nt >> 1) + S - 1 - L.slice) * L.inv) >> 16) +
-               (int)(((npair + S - 1 - L.slice) * L.inv) >> 16);
-    lc.tests += mine;
-    const int nw = (rows + 15) >> 4;
-    const int sl = L.slice < S ? L.slice : 0;   // lanes without a member test slice 0's and drop it
-    for (int c = 0; c < nw; ++c) {
-        const int rw = min(16, (rows - 16 * c + 3) & ~3);
-        const uint32_t mask = test_word<K, WRAP>(T, Mb, sl + 16 * c * S, S, rw) << (32 - 2 * rw);
-        const int own = min(max(mine - 32 * c, 0), 32);
-        T.masks[(c << 5) + lane] = mask & (uint32_t)(0xffffffff00000000ull >> own);
+    if (Mb.rank >= 0) {
+        const int own = (int)((full + S - 1 - L.slice) * L.inv >> 16);
+        const bool part = (int)((full + S - L.slice) * L.inv >> 16) != own;
+        mine = 4 * own + (part ? nt & 3 : 0);
     }
+    lc.tests += mine;
+    const int nw = (most + 7) >> 3;
+    // lanes without a member test slice 0's and drop it
+    const int j0 = (L.slice < S ? L.slice : 0) * L.rows * 4;
+    int hits = 0;
+    for (int c = 0; c < nw; ++c) {
+        const int quads = min(8, (most - 8 * c + 1) & ~1);
+        const int own = min(max(mine - 32 * c, 0), 32);
+        const uint32_t mask = (test_word<K, WRAP>(T, Mb, j0 + 32 * c, quads) << (32 - 4 * quads)) &
+                              (uint32_t)(0xffffffff00000000ull >> own);
+        T.masks[(c << 5) + lane] = mask;
+        hits += __popc(mask);
+    }
+    Mb.n += hits;
     // two words at a time in registers, the second following the first without a branch
     for (int c = 0; c < nw; c += 2) {
         uint32_t cur = T.masks[(c << 5) + lane], nxt = c + 1 < nw ? T.masks[(c << 5) + 32 + lane] : 0u;
-        int l0 = c << 5;
+        int j1 = j0 + (c << 5);
         while (cur | nxt) {
             if (cur == 0u) {
                 cur = nxt;
                 nxt = 0u;
-                l0 += 32;
+                j1 += 32;
             }
             const int q = __clz(cur);
-            cur ^= 0x80000000u >> q;
-            const int l = l0 + q;
-            tile_pair<MODE, WRAP>(Mb, a, T, 2 * ((l >> 1) * S + sl) + (l & 1), lc);
+            cur &= 0x7fffffffu >> q;
+            tile_pair<MODE, WRAP>(Mb, a, T, j1 + q, lc);
         }
     }
     if (MODE == kAcc) flush(Mb);
@@ -1620,13 +1645,14 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
     };
     Walk w = walk_begin();
     walk_visit(a, W, w, walk_start(a, root, cx, cy, cz, reach, lane), kWalkWhole, lane, open_node);
-    int ns = 0;   // candidates in the tile
+    int ns = 0;                                 // candidates in the tile
+    const int room = 4 * L.S * L.rows - 32;     // a window more still fits
     for (;;) {
         while (walk_can_step(a, w) && w.total - w.done < 64) walk_step(a, W, w, kWalkWhole, lane, open_node);
         walk_spill(a, W, w, lane);
         const bool walked = w.empty();
         // candidates by whole windows of 32 while the walk goes on
-        while (ns <= kTile - 32 && (w.total - w.done >= 32 || (walked && w.total > w.done))) {
+        while (ns <= room && (w.total - w.done >= 32 || (walked && w.total > w.done))) {
             int rank;
             const int nt = walk_take(W, w, lane, rank);
             bool in = false;
@@ -1651,8 +1677,11 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
             }
             const unsigned im = __ballot_sync(0xffffffffu, in);
             if (in) {
-                const int t = ns + __popc(im & lt);
-                T.put(t, px, py, pz);
+                const int t = tile_place(L, ns + __popc(im & lt));
+                T.x[t] = px;
+                T.y[t] = py;
+                T.z[t] = pz;
+                T.w[t] = fmaf(px, px, fmaf(py, py, pz * pz));
                 T.m[t] = mj;
                 if constexpr (K::sym) T.h2[t] = hj2;
                 T.r[t] = rank;
@@ -1662,7 +1691,7 @@ __device__ __forceinline__ void group_search(const SearchArgs& a, WalkSmem& W, t
         }
         const bool last = walked && w.total == w.done;
         if (last && lane == 0) W.ctr.cands += w.total;
-        if (ns > kTile - 32 || last) {
+        if (ns > room || last) {
             if (ns > 0) {
                 copies_wait();
                 __syncwarp();
@@ -1692,7 +1721,8 @@ template <class K, int MODE>
 __device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, typename K::Tile& T, const GroupDesc& d,
                                              LocalCounters& lc, int lane) {
     constexpr bool kLists = K::id == kKindDensityList;
-    const Layout L = make_layout(d.cnt, lane, MODE == kAcc, kLists ? min(4, d.smax) : d.smax, kLists);
+    const Layout L = make_layout(d.cnt, lane, MODE == kAcc, kLists ? min(4, d.smax) : d.smax, kLists,
+                                 K::Tile::cap);
     const int entry = member_entry(d, L, W, lane);
     const MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[entry] : -1)};
     uint32_t cx = 0, cy = 0, cz = 0;
@@ -1711,7 +1741,7 @@ __device__ __forceinline__ void process_part(const SearchArgs& a, WalkSmem& W, t
     if (lane == 0) W.ctr.walks++;
     group_search<K, MODE>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
     // the symmetric sums count the member itself as a pair at r = 0 (once, in slice 0)
-    constexpr bool kSelfPair = MODE == kAcc && (K::id == kKindHydro || K::id == kKindHydroAdj);
+    constexpr bool kSelfPair = K::id == kKindHydro || K::id == kKindHydroAdj;
     lc.pairs += mem.n - ((kSelfPair && L.slice == 0 && mem.rank >= 0) ? 1 : 0);
     if constexpr (kLists) {
         // the member's slice-0 lane records its sub-list lengths, S and whether all fit
@@ -1936,7 +1966,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
         if (gid >= ng) break;
         const GroupDesc d = group_desc(a, gid, nlarge);
         if (d.cnt <= 0) continue;
-        const Layout L = make_layout(d.cnt, lane, true, d.smax, false);
+        const Layout L = make_layout(d.cnt, lane, true, d.smax, false, PlainTile::cap);
         const int entry = member_entry(d, L, W, lane);
         MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[entry] : -1)};
         double lo = 0.0, hi = __longlong_as_double(0x7ff0000000000000ll);
@@ -2014,6 +2044,7 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                         const float3 rel = make_float3(rel_coord(Q.x, O.x, cx), rel_coord(Q.y, O.y, cy),
                                                        rel_coord(Q.z, O.z, cz));
                         if (KIND == 0) {
+                            dm.n++;
                             density_pair<MODE>(dm, a, rel, O.w, q, lc);
                         } else {
                             float hj = __uint_as_float(Q.w);
@@ -2022,6 +2053,7 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                             float thr = fmaf(fmaxf(hm.h2, hj * hj), 1.0f + 3.0f * kBandRel, hm.bk);
                             if (r2 < thr) {
                                 float4 H0 = a.hyd0[q], H1 = a.hyd1[q];
+                                hm.n++;
                                 hydro_pair<MODE>(hm, a, rel, make_float2(hj * hj, O.w), H0, H1, q, lc);
                             }
                         }
@@ -2034,7 +2066,7 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
                 node = lk.w;
             }
         }
-        lc.pairs += (KIND == 0) ? dm.n : hm.n;
+        lc.pairs += (KIND == 0) ? dm.n : hm.n - 1;
         if (KIND == 0) write_result<MODE>(dm, a);
         else write_result<MODE>(hm, a);
     }
