@@ -89,7 +89,7 @@ static_assert(kHistWords <= kSortHeadWords, "sort scratch head");
 // The last block to finish turns the digit counts of `passes` passes into each digit's first
 // position (exclusive scan over the bins), so that no launch of its own is needed.
 __device__ __forceinline__ void scan_digit_counts(uint32_t* hist, int passes, uint32_t* done) {
-    __shared__ uint32_t wsum[8];
+    __shared__ uint32_t wsum[kKeyPasses][8];
     __shared__ bool last;
     __threadfence();
     __syncthreads();
@@ -98,22 +98,33 @@ __device__ __forceinline__ void scan_digit_counts(uint32_t* hist, int passes, ui
     if (!last) return;
     __threadfence();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int p = 0; p < passes; ++p) {
-        uint32_t* h = hist + p * kBins;
-        const uint32_t c0 = __ldcg(h + 2 * threadIdx.x), c1 = __ldcg(h + 2 * threadIdx.x + 1);
-        uint32_t v = c0 + c1;
+    uint32_t c0[kKeyPasses], c1[kKeyPasses], v[kKeyPasses];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += t;
+    for (int p = 0; p < kKeyPasses; ++p) {   // all loads in flight together
+        c0[p] = p < passes ? __ldcg(hist + p * kBins + 2 * threadIdx.x) : 0u;
+        c1[p] = p < passes ? __ldcg(hist + p * kBins + 2 * threadIdx.x + 1) : 0u;
+        v[p] = c0[p] + c1[p];
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+        for (int p = 0; p < kKeyPasses; ++p) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, v[p], o);
+            if (lane >= o) v[p] += t;
         }
-        if (lane == 31) wsum[w] = v;
-        __syncthreads();
-        uint32_t off = v - c0 - c1;
-        for (int k = 0; k < w; ++k) off += wsum[k];
-        h[2 * threadIdx.x] = off;
-        h[2 * threadIdx.x + 1] = off + c0;
-        __syncthreads();
+    }
+    if (lane == 31) {
+#pragma unroll
+        for (int p = 0; p < kKeyPasses; ++p) wsum[p][w] = v[p];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < kKeyPasses; ++p) {
+        if (p >= passes) break;
+        uint32_t off = v[p] - c0[p] - c1[p];
+        for (int k = 0; k < w; ++k) off += wsum[p][k];
+        hist[p * kBins + 2 * threadIdx.x] = off;
+        hist[p * kBins + 2 * threadIdx.x + 1] = off + c0[p];
     }
 }
 
@@ -293,6 +304,18 @@ struct SweepArgs {
     unsigned* err;
 };
 
+// lanes with the same digit (kDigitBits bits and the one above them)
+__device__ __forceinline__ uint32_t same_digit(uint32_t d) {
+    uint32_t peers = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b <= kDigitBits; ++b) {
+        const bool set = d >> b & 1u;
+        const uint32_t vote = __ballot_sync(0xffffffffu, set);
+        peers &= set ? vote : ~vote;
+    }
+    return peers;
+}
+
 template <int ITEMS>
 constexpr size_t sweep_smem() {
     return (size_t)256 * ITEMS * 12;
@@ -340,7 +363,7 @@ __global__ void __launch_bounds__(256) k_radix_pass(SweepArgs a) {
     for (int r = 0; r < ITEMS; ++r) {
         const bool valid = base + r * 32 + lane < a.n;
         const uint32_t d = valid ? (uint32_t)(kk[r] >> a.shift) & (kBins - 1) : (uint32_t)kBins;
-        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t peers = same_digit(d);
         const uint32_t prev = valid ? wh[w][d] : 0u;
         __syncwarp();
         if (valid && lane == __ffs(peers) - 1) wh[w][d] = (uint16_t)(prev + __popc(peers));
