@@ -660,7 +660,7 @@ int sphgrp_ctx_destroy(sphgrp_ctx* ctx) {
                     c->acc_s2, c->wadj, c->dadj, c->adj0, c->adj1, c->adj2, c->adj3,
                     c->stack_spill, c->start_tab, c->ctr, c->err, c->work, c->ctr_log, c->tree.ncen, c->tree.next, c->tree.nlink,
                     c->tree.nlevel, c->tree.nparent, c->tree.narrive, c->tree.level_cnt, c->tree.box_lo, c->tree.box_hi,
-                    c->tree.top_cells, c->lst, c->lrec, c->lhw,
+                    c->tree.tile_cnt, c->lst, c->lrec, c->lhw,
                     c->lslot, c->npass};
     for (void* p : ptrs)
         if (p) cudaFree(p);

@@ -66,12 +66,12 @@ struct Tree {
     uint32_t* narrive = nullptr;   // children that arrived in the running bottom-up pass
     uint4* box_lo = nullptr;       // fixed-point boxes (scratch of the bottom-up pass)
     uint4* box_hi = nullptr;
-    int32_t* level_cnt = nullptr;  // nodes per level (device, kTreeLevels)
+    int32_t* level_cnt = nullptr;  // nodes per level (device, kTreeLevels), and wanted in all
+    int32_t* tile_cnt = nullptr;   // nodes per (level, tile of particles) of the build
     int64_t cap = 0;               // allocated nodes
     int64_t count = 0;             // nodes in the current tree (a forest: a bound)
-    int nlevels = 10;              // deepest level of the last build (first: a guess)
+    int nlevels = 0;               // deepest level
     int nroots = 1;
-    int32_t* top_cells = nullptr;  // the top levels' cell table (single-box build)
 };
 
 struct DevCounters {
