@@ -37,14 +37,17 @@ if ROOT not in sys.path:
 METRIC = "SPH density+hydro active particles/s: grouped vs per-particle search, 1 GB300"
 UNIT = "active particles/s"
 
-# algorithmic bytes per unit (candidate, member, node) of the two search kernels
-B_CAND = {"density": 32, "hydro": 64}
+# algorithmic bytes per unit (candidate, member, node) of the two search kernels.  A candidate
+# counts as its 32 B position record: all that every candidate costs.  The further records of
+# the kinds that need them (32 B hydro, 16 B velocity, 48 and 16 B the adjoints) are read only
+# for the candidates that lie in the members' box, which no counter tells apart.
+B_CAND = {"density": 32, "hydro": 32}
 B_MEMBER = {"density": 32 + 16, "hydro": 64 + 16}
 B_NODE = 48
-# the backward's three pair loops and the velocity-derivative loop: (bytes per staged
-# candidate, bytes per member)
-B_BWD = {"density_sums": (32, 48), "hydro_adjoint": (80, 136), "density_adjoint": (48, 72)}
-B_VEL = (48, 92)
+# the backward's three pair loops and the velocity-derivative loop: (bytes per candidate,
+# bytes per member)
+B_BWD = {"density_sums": (32, 48), "hydro_adjoint": (32, 136), "density_adjoint": (32, 72)}
+B_VEL = (32, 92)
 
 
 def launch_gbs(e: dict, b_cand: int, b_member: int) -> float:
@@ -446,6 +449,7 @@ def roofline(collect, peak_gbs, clocks=None, form: str = "grouped"):
     last = collect[-1].get("density_passes") if collect else None
     if last and "density" in detail:
         detail["density"]["passes_of_last_step"] = last
+    # k_indiv is the per-particle form's record name (its loops run k_group on groups of one)
     kernel = f"k_indiv ({dom})" if form == "individual" else f"k_group ({dom})"
     return {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak_gbs,
             "unit": "GB/s", "frac": achieved / peak_gbs, "traffic": traffic,

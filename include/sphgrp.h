@@ -85,9 +85,11 @@ typedef struct sphgrp_params {
                            keeps plain chunks of group_size.  e.g. 2 */
     int iteration;      /* smoothing-length iteration of the grouped density:
                            SPHGRP_ITER_PASSES (default: one search launch per pass over the
-                           still unconverged particles, regrouped), SPHGRP_ITER_IN_GROUP (one
-                           launch; every group repeats walk, filter and update until its
-                           members converge) or SPHGRP_ITER_RECYCLE (the first pass
+                           still unconverged particles, regrouped; lists of at most 4096
+                           particles per SM in count mode iterate as SPHGRP_ITER_IN_GROUP
+                           instead, which is faster there),
+                           SPHGRP_ITER_IN_GROUP (one launch; every group repeats walk, filter
+                           and update until its members converge) or SPHGRP_ITER_RECYCLE (the first pass
                            also keeps, for every member, the candidates of its group's
                            superset within iter_widen * h; later passes of the particles
                            whose h stays within that radius iterate on those candidates in

@@ -908,7 +908,7 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
             return set_error(SPHGRP_ENOCONV, std::to_string(c->host_small[2]) + " particles did not converge");
         return SPHGRP_OK;
     }
-    int64_t walks = 0, members = 0;
+    int64_t members = 0;
     int it = 1;
     const int max_iter = iterate ? c->p.max_iter : 1;
     // Recycled iteration (Sec. 2.2 iteration with the Sec. 2.1 supersets reused): the
@@ -934,7 +934,6 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
         a.g = grouped ? group_size : 1;
         a.ngroups = grouped ? (nu + group_size - 1) / group_size : nu;
         if (grouped && (rc = make_pieces(c, &a, U, nu, group_size, s))) return rc;
-        walks += grouped ? 0 : nu;
         members += nu;
         UpdateArgs ua;
         std::memset(&ua, 0, sizeof(ua));
@@ -1042,7 +1041,7 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
     }
     cudaMemcpyAsync(c->host_small + 2, nfail, sizeof(int), cudaMemcpyDeviceToHost, s);
     rc = finish(c, s, 0);
-    c->last.walks = walks + c->dev_walks;
+    c->last.walks = c->dev_walks;
     c->last.members = members;
     c->last.iterations = std::min(std::max(it, list_passes), max_iter);
     if (rc) return rc;
@@ -1083,7 +1082,7 @@ int hydro_force(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, const dou
         note_launch();
     }
     rc = finish(c, s, 0);
-    c->last.walks = grouped ? c->dev_walks : nu;
+    c->last.walks = c->dev_walks;
     c->last.members = nu;
     return rc;
 }

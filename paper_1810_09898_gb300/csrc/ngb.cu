@@ -1,9 +1,10 @@
 // Neighbour search and the SPH loops that consume it, forward and backward.
 //
 // Two forms (Sec. 1.1 standard search, Sec. 2.1 Neighbour Recycling):
-//  * individual: one thread per active particle walks the octree depth-first with
-//    skip pointers and radius h_i (hydro: max(h_i, node hmax)), testing the particles
-//    of every opened leaf;
+//  * individual: every active particle is searched by itself, a warp walking the octree
+//    for its sphere of radius h_i (hydro: max(h_i, node hmax)): a group of one member.
+//    The calls that export neighbour lists walk with a thread per particle, depth-first
+//    by skip pointers;
 //  * grouped: one warp per group of consecutive active particles (key order).  The
 //    warp walks the octree cooperatively once for the group (32 nodes tested per
 //    step) over the members' box dilated by their largest radius, takes the particles
@@ -1974,12 +1975,12 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, 6) k_group_dens_iter(Sear
         const int entry = member_entry(d, L, W, lane);
         MemberRec rec[1] = {load_member(a, L.k >= 0 ? a.U[entry] : -1)};
         double lo = 0.0, hi = __longlong_as_double(0x7ff0000000000000ll);
+        if (lane == 0) W.ctr.walks++;
         for (int pass = 1;; ++pass) {
             uint32_t cx = 0, cy = 0, cz = 0;
             if (!group_centre<1>(a, rec, cx, cy, cz)) break;
             DMember mem;
             member_init(mem, a, rec[0], cx, cy, cz);
-            if (lane == 0) W.ctr.walks++;
             group_search<KDens, kAcc>(a, W, T, L, mem, cx, cy, cz, d.root, lc, lane);
             lc.pairs += mem.n;
             slice_sum(mem, L);

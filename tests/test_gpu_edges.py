@@ -126,3 +126,19 @@ def test_sort_sizes(cuda_device, n):
         assert np.array_equal(perm.cpu().numpy(), order)
         assert np.array_equal(keys.cpu().numpy().astype(np.uint64), ref[order])
     ctx.close()
+
+
+def test_individual_walks_are_counted_once(cuda_device):
+    """stats: one walk per particle and pass in the individual form, both loops."""
+    d = sphgen.make("uniform", 3001, config=1)
+    G = Gpu(d["pos"], d["m"].astype(np.float32))
+    act = np.arange(0, 3001, 2, dtype=np.int32)
+    h = np.full(3001, d["h0"])
+    st = G.density(act, h, 0, 0, 1)["stats"]
+    assert st["walks"] == st["members"] == len(act)
+    st = G.density(act, h, 1, 0, 1)["stats"]
+    assert st["walks"] == st["members"] > len(act)
+    one = np.ones(3001, np.float32)
+    st = G.hydro(act, h, one, one, np.zeros((3001, 3), np.float32), one, 0, 1)["stats"]
+    assert st["walks"] == st["members"] == len(act)
+    G.ctx.close()
