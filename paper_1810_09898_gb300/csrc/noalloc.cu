@@ -5,8 +5,8 @@
 // budget, and latency-critical paths where the implicit device-wide synchronisation
 // of cudaMalloc / cudaFree is not acceptable.  For them sphgrp_sfc_keys_sort_static
 // runs the same key and radix-sort kernels as sphgrp_sfc_keys_sort, with the sort's
-// scratch (the second ping-pong buffer pair, the digit counts and the error flag) in one file-scope __device__ array of fixed size instead of
-// a context's workspace.  Every GPU that loads the library holds that array until the
+// scratch (the second ping-pong buffer pair, the digit counts and the error flag) in one
+// file-scope __device__ array of fixed size instead of a context's workspace.  Every GPU that loads the library holds that array until the
 // process exits.
 #include <mutex>
 
