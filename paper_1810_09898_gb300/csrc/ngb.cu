@@ -125,12 +125,23 @@ __device__ __forceinline__ float rel_diff(float p, float m) {
 // dW/dr = kSkernel h^-4 dw/dq for the M4 spline W = 8 / (pi h^3) w(r / h)
 constexpr float kSkernel = 2.54647908947032537f;   // 8 / pi
 
-// hardware reciprocal square root and reciprocal (1 ulp; arguments of normal size)
+// hardware reciprocal square root and reciprocal (1 ulp; arguments of normal size: a
+// subnormal one is flushed to zero and gives infinity)
 __device__ __forceinline__ float rsqrt_fast(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// the same, subnormal arguments included (three more instructions)
+__device__ __forceinline__ float rsqrt_any(float x) {
+    float y;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// Least r^2 of normal size: a pair closer than its root, 1.1e-19 of the box, is taken as
+// coincident where its terms vanish with r (kernel gradients); the hydro adjoint, whose
+// derivative of the pair force does not, takes its root by rsqrt_any.
+constexpr float kMinR2 = 1.17549435e-38f;
 __device__ __forceinline__ float rcp_fast(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -741,7 +752,7 @@ __device__ __forceinline__ void density_pair(Mem& M, const SearchArgs& a, float3
 }
 
 // divergence and curl terms of a neighbour at x_j - x_i = d: grad_i W = W'(r, h_i) (x_i -
-// x_j) / r, v_ij = v_i - v_j; r > 0 (at r = 0 grad W = 0)
+// x_j) / r, v_ij = v_i - v_j; r^2 >= kMinR2 (grad W goes to 0 with r)
 template <class Mem>
 __device__ __forceinline__ void velocity_terms(Mem& M, float mj, float4 vj, float dx, float dy, float dz, float r2) {
     const float rinv = rsqrt_fast(r2);
@@ -762,7 +773,7 @@ __device__ __forceinline__ void densvel_pair(DVMember& M, const SearchArgs& a, f
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
     if (MODE != kAcc) return;
     density_terms(M, in ? mj : 0.0f, q_of(sqrt_fast(r2), M.hinv));
-    if (in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
+    if (in && r2 >= kMinR2) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
 // density pair of the recycled iteration: a candidate inside the widened threshold joins
@@ -786,7 +797,7 @@ __device__ __forceinline__ void vel_pair(VMember& M, const SearchArgs& a, float3
                                          LocalCounters& lc) {
     float dx, dy, dz, r2;
     const bool in = dens_decide<WRAP>(M, a, p, crank, lc, dx, dy, dz, r2);
-    if (MODE == kAcc && in && r2 > 0.0f) velocity_terms(M, mj, vj, dx, dy, dz, r2);
+    if (MODE == kAcc && in && r2 >= kMinR2) velocity_terms(M, mj, vj, dx, dy, dz, r2);
 }
 
 // decision of the symmetric criterion |r| < max(h_i, h_j), as dens_decide
@@ -814,7 +825,7 @@ __device__ __forceinline__ bool sym_decide(Mem& M, const SearchArgs& a, float3 p
 }
 
 // hydro pair: p = relative coordinates, q = {h_j^2, m_j}, v = {vx, vy, vz, c_j},
-// hh = {A_j, rho_j, 1/h_j, limiter_j}.  A pair at r = 0 (coincident, or the member itself)
+// hh = {A_j, rho_j, 1/h_j, limiter_j}.  A pair below kMinR2 (coincident, or the member itself)
 // has no kernel gradient.
 template <int MODE, bool WRAP = false>
 __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float3 p, float2 q,
@@ -824,7 +835,7 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
     float dx, dy, dz, r2;
     const bool in = sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2);
     if (MODE == kFill && in && crank != M.rank) export_pair(M, a, crank);
-    if (MODE != kAcc || !(in && r2 > 0.0f)) return;
+    if (MODE != kAcc || !(in && r2 >= kMinR2)) return;
     const float rinv = rsqrt_fast(r2);
     const float r = r2 * rinv;
     const float dWi = M.sk * m4_slope(q_of(r, M.hinv));
@@ -861,7 +872,7 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
     if (MODE != kAcc) return;
     if (r2 == 0.0f) return;
-    const float rinv = rsqrt_fast(r2);
+    const float rinv = rsqrt_any(r2);
     const float r = r2 * rinv;
     const float D0 = -dx, D1 = -dy, D2 = -dz;   // x_k - x_j
     const float e0 = D0 * rinv, e1 = D1 * rinv, e2 = D2 * rinv;
@@ -934,7 +945,7 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
     float dx, dy, dz, r2;
     if (!sym_decide<WRAP>(M, a, p, q.x, crank, lc, dx, dy, dz, r2)) return;
     if (MODE != kAcc) return;
-    const float rinv = r2 > 0.0f ? rsqrt_fast(r2) : 0.0f;
+    const float rinv = r2 >= kMinR2 ? rsqrt_fast(r2) : 0.0f;
     const float r = r2 * rinv;
     float wk_, dwk, d2wk, wj_, dwj, d2wj;
     const float qk = q_of(r, M.hinv), qj = q_of(r, d.z);
@@ -943,7 +954,7 @@ __device__ __forceinline__ void dens_adj_pair(DAMember& M, const SearchArgs& a, 
     // k as a neighbour of j: rho_j gains m_k W(r, h_j), dRho_j/dh_j gains m_k W_h(r, h_j)
     const float hj = q.x * d.z;
     M.mb = fmaf(d.x * d.w, hj * wj_, fmaf(-d.y * d.w, fmaf(qj, dwj, 3.0f * wj_), M.mb));
-    if (r2 == 0.0f) return;
+    if (r2 < kMinR2) return;
     const float Wr_k = M.sk * dwk, Wr_j = d.w * dwj;
     const float Whr_k = -M.sk * M.hinv * fmaf(qk, d2wk, 4.0f * dwk);
     const float Whr_j = -d.w * d.z * fmaf(qj, d2wj, 4.0f * dwj);
