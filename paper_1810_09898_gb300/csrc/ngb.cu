@@ -2374,20 +2374,23 @@ int launch_gather_groups(int nch, int g, const int2* tmp, const int32_t* cnt, co
 // Launchers
 // ---------------------------------------------------------------------------------
 
+// Shared memory of a block: below the 48 KB that a kernel may take on any device without an
+// attribute of its own (attributes belong to a device; a flag per process would leave them
+// unset on the next one).
+constexpr size_t kPlainSmem = 48 * 1024;
+
 template <class K>
-static size_t group_smem() {
-    return kWarpsPerBlock * (sizeof(WalkSmem) + sizeof(typename K::Tile));
+constexpr size_t group_smem() {
+    constexpr size_t sh = kWarpsPerBlock * (sizeof(WalkSmem) + sizeof(typename K::Tile));
+    static_assert(sh <= kPlainSmem, "the kernel would need the opt-in attribute");
+    return sh;
 }
 
 // Persistent grid: every resident block slot of the GPU, but at most one block per four
 // groups (ngroups_host: their number, or a bound on it; -1: unknown).
 template <typename Kern, typename... Args>
-static int launch_persistent(Kern kern, bool& configured, size_t sh, int64_t ngroups_host, int sm_count,
-                             cudaStream_t s, const char* what, Args... args) {
-    if (!configured) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-        configured = true;
-    }
+static int launch_persistent(Kern kern, size_t sh, int64_t ngroups_host, int sm_count, cudaStream_t s,
+                             const char* what, Args... args) {
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarpsPerBlock * 32, sh);
     if (per_sm < 1) per_sm = 1;
@@ -2401,22 +2404,20 @@ static int launch_persistent(Kern kern, bool& configured, size_t sh, int64_t ngr
 
 template <class K, int MODE>
 static int launch_group(const SearchArgs& a, int sm_count, cudaStream_t s) {
-    static bool configured = false;
     if (a.g > 128) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
     SearchArgs b = a;
     b.parts = (a.g + kPartMax - 1) / kPartMax;
     // many single members: several items per counter access (one address serves all warps)
     b.take = a.g == 1 && a.ngroups >= 1 << 16 ? 4 : 1;
-    return launch_persistent(k_group<K, MODE>, configured, group_smem<K>(),
+    return launch_persistent(k_group<K, MODE>, group_smem<K>(),
                              a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s, "grouped search kernel", b);
 }
 
 template <bool SYM, bool FILL>
 static int launch_superset(const SearchArgs& a, int sm_count, cudaStream_t s) {
-    static bool configured = false;
     if (a.g > 32 * kSupSlots) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
-    return launch_persistent(k_superset<SYM, FILL>, configured, kWarpsPerBlock * sizeof(WalkSmem), a.ngroups, sm_count,
-                             s, "superset kernel", a);
+    return launch_persistent(k_superset<SYM, FILL>, kWarpsPerBlock * sizeof(WalkSmem), a.ngroups, sm_count, s,
+                             "superset kernel", a);
 }
 
 template <class K>
@@ -2449,21 +2450,20 @@ int launch_search_dev(const SearchArgs& a, int kind, int max_g, int sm_count, cu
 int launch_density_iter(const SearchArgs& a, const IterArgs& it, int max_g, int sm_count, cudaStream_t s) {
     if (max_g < 1 || max_g > 128) return set_error(SPHGRP_EINVAL, "group size outside [1, 128]");
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
-    static bool configured = false;
     SearchArgs b = a;
     b.parts = (a.g + kPartMax - 1) / kPartMax;
-    return launch_persistent(k_group_dens_iter, configured, group_smem<KDens>(),
+    return launch_persistent(k_group_dens_iter, group_smem<KDens>(),
                              a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s,
                              "grouped density iteration kernel", b, it);
 }
 
 template <class K0, class K1>
 static int launch_pair(const SearchArgs& a0, const SearchArgs& a1, int sm_count, cudaStream_t s) {
-    static bool configured = false;
     constexpr size_t tile = sizeof(typename K0::Tile) > sizeof(typename K1::Tile) ? sizeof(typename K0::Tile)
                                                                                   : sizeof(typename K1::Tile);
-    const size_t sh = kWarpsPerBlock * (sizeof(WalkSmem) + tile);
-    return launch_persistent(k_group_pair<K0, K1>, configured, sh, -1, sm_count, s, "paired search kernel", a0, a1);
+    constexpr size_t sh = kWarpsPerBlock * (sizeof(WalkSmem) + tile);
+    static_assert(sh <= kPlainSmem, "the kernel would need the opt-in attribute");
+    return launch_persistent(k_group_pair<K0, K1>, sh, -1, sm_count, s, "paired search kernel", a0, a1);
 }
 
 int launch_search_pair(const SearchArgs& a0, int kind0, const SearchArgs& a1, int kind1, int max_g, int sm_count,
@@ -2741,13 +2741,11 @@ __global__ void __launch_bounds__(128) k_list_iterate(ListIterArgs a) {
 
 int launch_list_iterate(const ListIterArgs& a, cudaStream_t s) {
     if (a.nu <= 0) return SPHGRP_OK;
-    static bool configured = false;
-    if (!configured) {
-        // no shared memory: all of it as L1, which holds the candidates that neighbouring
-        // particles gather
-        cudaFuncSetAttribute(k_list_iterate, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-        configured = true;
-    }
+    // no shared memory: all of it as L1, which holds the candidates that neighbouring
+    // particles gather (set on each call: the attribute belongs to the current device)
+    int rc = check_cuda(cudaFuncSetAttribute(k_list_iterate, cudaFuncAttributePreferredSharedMemoryCarveout, 0),
+                        "list iteration");
+    if (rc) return rc;
     k_list_iterate<<<blocks_for(a.nu, 128), 128, 0, s>>>(a);
     note_launch();
     return check_cuda(cudaGetLastError(), "list iteration");

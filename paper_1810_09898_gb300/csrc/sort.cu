@@ -475,11 +475,6 @@ static int launch_pass(const SweepArgs& a, cudaStream_t s) {
     const int items = sort_items(a.n);
     const unsigned tiles = (unsigned)((a.n + 256 * items - 1) / (256 * items));
     if (items == 16) {
-        static bool configured = false;
-        if (!configured) {
-            cudaFuncSetAttribute(k_radix_pass<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<16>());
-            configured = true;
-        }
         k_radix_pass<16><<<tiles, 256, sweep_smem<16>(), s>>>(a);
     } else if (items == 8) {
         k_radix_pass<8><<<tiles, 256, sweep_smem<8>(), s>>>(a);
@@ -503,6 +498,13 @@ static int radix_passes(uint64_t* const (&kbuf)[2], int32_t* const (&vbuf)[2], i
                         uint64_t* keys_copy, int32_t* vals_copy, int32_t* rank_of, unsigned* err, cudaStream_t s) {
     const int64_t set = (sort_scratch_words(n) - kSortHeadWords) / 2;
     uint32_t* sets[2] = {scratch + kSortHeadWords, scratch + kSortHeadWords + set};
+    // With its static tables the largest tile is above the 48 KB that need no permission,
+    // which belongs to the current device: given on every call, whichever device that is.
+    if (sort_items(n) == 16) {
+        int rc = check_cuda(cudaFuncSetAttribute(k_radix_pass<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)sweep_smem<16>()), "radix pass shared memory");
+        if (rc) return rc;
+    }
     for (int p = 0; p < passes; ++p) {
         const bool last = p == passes - 1;
         SweepArgs a;
