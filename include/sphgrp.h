@@ -97,8 +97,9 @@ typedef struct sphgrp_params {
                            group_size <= 32; device memory for 192 candidate ranks per
                            particle is allocated by the first such call, and without it the
                            call walks every pass).  The iterates are those of the pass-by-pass
-                           iteration in every mode.  The individual form always iterates in
-                           passes. */
+                           iteration in every mode, except that SPHGRP_ITER_IN_GROUP, where it
+                           is asked for, holds h at 0.49 (the small lists above do not).  The
+                           individual form always iterates in passes. */
     int group_mode;     /* how the grouped form cuts the active list (in key order) into groups:
                            SPHGRP_GROUP_COUNT: chunks of group_size, split as group_split says;
                            SPHGRP_GROUP_RADIUS (Sec. 2.1, the paper's rule): a group starts at an

@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <string>
 
 #include "search_args.cuh"
@@ -881,6 +882,9 @@ int density_call(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, double* 
         it.nngb = c->p.nngb;
         it.tol = c->p.nngb_tol;
         it.max_iter = c->p.max_iter;
+        // asked for, the in-group form holds h where the minimum image is unique; in place of
+        // passes it follows their iterates wherever they go
+        it.h_max = iteration == SPHGRP_ITER_IN_GROUP ? kInGroupHMax : std::numeric_limits<double>::infinity();
         it.h64 = c->h64;
         it.pfix = c->pfix;
         it.h_out = h;

@@ -272,6 +272,7 @@ int issue_step(Batch* b, const sphgrp_batch_io* io, int flags, cudaStream_t s) {
         it.nngb = c->p.nngb;
         it.tol = c->p.nngb_tol;
         it.max_iter = c->p.max_iter;
+        it.h_max = kInGroupHMax;
         it.h64 = c->h64;
         it.pfix = c->pfix;
         it.h_out = io->h;

@@ -1959,7 +1959,7 @@ __device__ __forceinline__ bool hsml_step(const SearchArgs& a, const IterArgs& i
         else if (lo == 0.0) hn = h / cbrt2;
         else hn = cbrt(0.5 * (lo * lo * lo + hi * hi * hi));
     }
-    h = fmin(hn, 0.49);   // the minimum image needs h < 1/2 (such a particle cannot converge)
+    h = hn > it.h_max ? it.h_max : hn;   // (a NaN h stays one: it finds nothing)
     if (writer) {
         it.h64[r] = h;
         it.pfix[r].w = __float_as_uint((float)h);

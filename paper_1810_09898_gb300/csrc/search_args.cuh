@@ -184,10 +184,15 @@ struct CutArgs {
     int* npieces;
 };
 
-// smoothing-length iteration inside the grouped density kernel (batch path)
+// largest h of the in-group iteration: the minimum image needs h < 1/2 (a particle that would
+// go beyond does not converge)
+constexpr double kInGroupHMax = 0.49;
+
+// smoothing-length iteration inside the grouped density kernel
 struct IterArgs {
     double nngb, tol;
     int max_iter;
+    double h_max;         // h is held below this (infinity: not at all, as by passes)
     double* h64;          // rank order, updated in place
     uint4* pfix;          // .w = FP32 copy of h
     // results (original order)

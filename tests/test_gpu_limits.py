@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import sphgen
-from gpu_common import Gpu
+from gpu_common import RHO_TOL, Gpu, dataset
 
 pytestmark = pytest.mark.gpu
 
@@ -76,4 +76,41 @@ def test_close_pairs_gradient(cuda_device):
             assert np.all(np.isfinite(got)), (g, what)
             if g == 1 or what != "x":
                 assert _rel(got, want) <= GRAD_TOL, (g, what)
+    G.ctx.close()
+
+
+# ---------------------------------------------------------------- smoothing lengths
+
+@pytest.mark.parametrize("mode,g", [(0, 1), (1, 1), (1, 16), (1, 64)])
+@pytest.mark.parametrize("n", [104, 116])
+def test_iterated_h_beyond_half_the_box(cuda_device, n, mode, g):
+    """So few particles that the relation holds at h between 0.4 and 0.6: the default
+    iteration follows the oracle's there (an iterate accepted at the edge of the band by one
+    of them and not by the other may differ: two particles are let off)."""
+    rng = np.random.default_rng(sphgen.SEED_BASE + n)
+    pos = rng.random((n, 3))
+    m = np.full(n, 1.0 / n, np.float32)
+    href, ref = oracle.density_iterate(pos, m.astype(np.float64), np.full(n, 0.3))
+    assert ref["failed"] == 0 and (href > 0.5).any() and ((href > 0.49) & (href < 0.5)).any()
+    G = Gpu(pos, m)
+    out = G.density(np.arange(n, dtype=np.int32), np.full(n, 0.3), 1, mode, g)
+    same = np.abs(out["h"] / href - 1.0) <= 1e-5
+    assert same.sum() >= n - 2
+    assert np.max(np.abs(out["rho"][same] / ref["rho"][same] - 1.0)) <= 5 * RHO_TOL   # rho goes as h^-3
+    G.ctx.close()
+
+
+@pytest.mark.parametrize("iteration", [0, 1])
+def test_h_not_a_number_searches_nothing(cuda_device, iteration):
+    """A NaN h is EINVAL, and no pair is found for it on the way there."""
+    import paper_1810_09898_gb300 as sg
+
+    n = 3000
+    d = dataset("uniform", n, 1)
+    G = Gpu(d["pos"], d["m32"], iteration=iteration)
+    with pytest.raises(sg.SphgrpError, match="EINVAL"):
+        G.density(np.arange(n, dtype=np.int32), np.full(n, np.nan), 1, 1, 16)
+    assert G.ctx.stats()["pairs"] == 0
+    out = G.density(np.arange(n, dtype=np.int32), np.full(n, d["h0"]), 0, 1, 16)   # still usable
+    assert np.array_equal(out["nngb"], oracle.density(d["pos"], d["m32"].astype(np.float64), np.full(n, d["h0"]))["nngb"])
     G.ctx.close()
