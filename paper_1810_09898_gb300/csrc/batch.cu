@@ -227,6 +227,7 @@ int make_batch_groups(Batch* b, bool all, int only_cls, const uint8_t* active, c
     ca.windows = b->chunks;
     ca.nwindows_dev = b->dsc + kNWindows;
     ca.box_split = b->box_split;
+    ca.err = c->err;
     ca.pieces4 = all ? b->groups_all : b->groups;
     ca.cap = n;
     ca.npieces = b->dsc + (all ? kNPiecesAll : kNPieces);

@@ -2120,6 +2120,9 @@ __global__ void __launch_bounds__(kCutWarps * 32) k_cut_pieces(CutArgs a) {
     __shared__ int cnt[2][kCutWarps];
     __shared__ int at[2];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // A forest that outgrew its arrays has only its roots: searched, every group would scan
+    // its whole box, and the batch step, which reads nothing back, goes on until its end.
+    if (BATCH && (*a.err & kErrNodes)) return;
     const int nwin = BATCH ? *a.nwindows_dev : a.nwindows;
     for (int w0 = blockIdx.x * kCutWarps; w0 < nwin; w0 += gridDim.x * kCutWarps) {   // block-uniform
         const int win = w0 + w;

@@ -177,6 +177,7 @@ struct CutArgs {
     const int4* windows;
     const int* nwindows_dev;
     const float* box_split;
+    const unsigned* err;   // batch: no pieces are made when the forest did not fit
     // output
     int2* pieces;
     int4* pieces4;

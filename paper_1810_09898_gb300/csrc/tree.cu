@@ -167,8 +167,8 @@ __device__ __forceinline__ int level_first(const TreeArgs& a, int l) { return a.
 
 // Ids of every particle's nodes, linked down to their first child: a warp per tile, lane l
 // holding the next id of level l.  With more nodes than the arrays hold, only the roots are
-// made, as leaves, and the error flag is set (the caller builds again, or reports it);
-// lcnt[kTreeLevels] tells how many there would be.
+// made, as leaves, and the error flag is set (the caller builds again, or makes no search
+// and reports it); lcnt[kTreeLevels] tells how many there would be.
 __global__ void __launch_bounds__(256) k_tree_nodes(TreeArgs a) {
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;

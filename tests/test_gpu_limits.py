@@ -114,3 +114,49 @@ def test_h_not_a_number_searches_nothing(cuda_device, iteration):
     out = G.density(np.arange(n, dtype=np.int32), np.full(n, d["h0"]), 0, 1, 16)   # still usable
     assert np.array_equal(out["nngb"], oracle.density(d["pos"], d["m32"].astype(np.float64), np.full(n, d["h0"]))["nngb"])
     G.ctx.close()
+
+
+# ---------------------------------------------------------------- batches
+
+def _batch_io(pos, h):
+    import torch
+
+    n = len(pos)
+    z = lambda *s: torch.zeros(s, device="cuda")  # noqa: E731
+    return {"pos": torch.as_tensor(pos, device="cuda"), "m": z(n) + 1 / n, "vel": z(n, 3), "u": z(n) + 1,
+            "h": torch.as_tensor(h, device="cuda"), "rho": z(n) + 1, "drhodh": z(n), "fgrad": z(n) + 1,
+            "nngb": torch.zeros(n, dtype=torch.int32, device="cuda"), "acc": z(n, 3), "dudt": z(n),
+            "g_acc": z(n, 3) + 1, "g_rho": z(n), "g_pos": z(n, 3), "g_vel": z(n, 3), "g_m": z(n)}
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_forest_overflow_does_no_search(cuda_device, graph):
+    """Chains that outgrow the forest's arrays in one of two boxes: EOVERFLOW without a
+    search, whose walks would start at leaves as large as the boxes; the next call with
+    positions that fit gives the oracle's counts."""
+    import torch
+
+    import paper_1810_09898_gb300 as sg
+
+    rng = np.random.default_rng(sphgen.SEED_BASE + 74)
+    k = 4000
+    a = rng.random((k, 3)) * 0.99
+    good = rng.random((2 * k, 3))
+    pos = np.concatenate([a, a + 2.0 ** -20, good])
+    n = len(pos)
+    B = sg.Batch([0, 2 * k, n], leaf_size=1)
+    io = _batch_io(pos, np.full(n, 0.05))
+    with pytest.raises(sg.SphgrpError, match="EOVERFLOW"):
+        B.run(io, backward=True, graph=graph)
+    st = B.stats()
+    assert st["pair_tests"] == 0 and st["walks"] == 0
+    B.close()
+    B = sg.Batch([0, 2 * k, n])
+    io["h"].fill_(0.12)
+    B.run(io, backward=True, graph=graph)
+    h = io["h"].cpu().numpy()
+    for s in (slice(0, 2 * k), slice(2 * k, n)):
+        ref = oracle.density(pos[s], np.full(2 * k, 1 / n), h[s])
+        assert np.array_equal(io["nngb"].cpu().numpy()[s], ref["nngb"])
+    assert torch.isfinite(io["g_pos"]).all()
+    B.close()
