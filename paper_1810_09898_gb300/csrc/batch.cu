@@ -439,11 +439,11 @@ int sphgrp_batch_create(sphgrp_batch** out, const sphgrp_params* params, int nbo
     // walk start tables: 1.2 MB per box, so only for batches of up to kMaxTableBoxes
     // boxes (larger batches walk from their boxes' roots)
     if (nbox <= kMaxTableBoxes) rc = rc ? rc : dalloc(&b->start_tabs, (int64_t)nbox * kStartTableSize);
-    rc = rc ? rc : alloc_tree(b->c, node_cap);
     rc = rc ? rc : backward_buffers(b->c);
     if (!rc && cudaMallocHost(&b->host, (2 + kNScalars) * sizeof(int32_t)) != cudaSuccess) rc = SPHGRP_ENOMEM;
     if (!rc && cudaMallocHost(&b->host_ctr, sizeof(DevCounters)) != cudaSuccess) rc = SPHGRP_ENOMEM;
     if (!rc) rc = check_cuda(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking), "capture stream");
+    rc = rc ? rc : alloc_tree(b->c, node_cap, b->cap_stream);   // complete with the synchronisation below
     if (!rc) {
         cudaStream_t s = b->cap_stream;
         rc = check_cuda(cudaMemcpyAsync(b->box_off, box_off, (nbox + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s),

@@ -58,6 +58,7 @@ constexpr int kStartTableSize = start_table_offset(kStartLevels + 1);
 // skip = the node visited after this one's subtree in a depth-first walk (-1 = end).
 constexpr int kTreeLevels = kKeyLevels + 1;   // levels 0 .. 21
 struct Tree {
+    void* block = nullptr;         // holds the arrays below
     uint4* ncen = nullptr;
     float4* next = nullptr;
     int4* nlink = nullptr;
@@ -268,7 +269,7 @@ int refresh_hmax(Ctx* c, cudaStream_t s);                                       
 int sort_keys_boxed(Ctx* c, int64_t n, const double* pos, const int64_t* box_off_dev, int nbox, uint64_t* tmp64a,
                     uint64_t* tmp64b, int32_t* tmp32a, int32_t* tmp32b, int32_t* box_of_rank,
                     cudaStream_t s);                                                        // sort.cu
-int alloc_tree(Ctx* c, int64_t cap);                                                       // tree.cu
+int alloc_tree(Ctx* c, int64_t cap, cudaStream_t s);                                       // tree.cu
 int build_forest(Ctx* c, int nbox, const int64_t* box_off_dev, const int32_t* box_of_rank, int32_t* start_tabs,
                  cudaStream_t s, const int32_t* box_cfg = nullptr);                         // tree.cu
 void note_launches(long long k);                                                           // api.cu

@@ -160,3 +160,34 @@ def test_forest_overflow_does_no_search(cuda_device, graph):
         assert np.array_equal(io["nngb"].cpu().numpy()[s], ref["nngb"])
     assert torch.isfinite(io["g_pos"]).all()
     B.close()
+
+
+# ---------------------------------------------------------------- octree storage
+
+def test_rebuilds_of_one_context(cuda_device):
+    """A context for 20k particles builds octrees of a few particles, of chains that outgrow
+    the node arrays, and of more and fewer particles after that, on two streams."""
+    import torch
+
+    import paper_1810_09898_gb300 as sg
+
+    rng = np.random.default_rng(sphgen.SEED_BASE + 75)
+    a = rng.random((3000, 3)) * 0.99
+    sets = [rng.random((300, 3)), np.concatenate([a, a + 2.0 ** -20]), rng.random((20000, 3)), rng.random((5, 3)),
+            np.concatenate([a, a + 2.0 ** -20])]
+    ctx = sg.Context(20000, leaf_size=1)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for k, pos in enumerate(sets):
+        n = len(pos)
+        h = np.full(n, min(0.3, (20.0 / n) ** (1 / 3)))
+        with torch.cuda.stream(streams[k % 2]):
+            p, m = torch.as_tensor(pos, device="cuda"), torch.full((n,), 1.0 / n, device="cuda")
+            f = [torch.zeros(n, device="cuda") for _ in range(3)]
+            nn = torch.zeros(n, dtype=torch.int32, device="cuda")
+            act = torch.arange(n, dtype=torch.int32, device="cuda")
+            ctx.sfc_keys_sort(p)
+            ctx.tree_build(p, m)
+            ctx.density(act, torch.as_tensor(h, device="cuda"), 0, 1, 16, *f, nn)
+            got = nn.cpu().numpy()
+        assert np.array_equal(got, oracle.density(pos, np.full(n, 1.0 / n), h)["nngb"]), k
+    ctx.close()
