@@ -92,9 +92,10 @@ __global__ void k_gather_h(int64_t n, const int32_t* __restrict__ perm, const do
     pfix[r].w = __float_as_uint((float)v);
 }
 
-// Hydro inputs in key order: hyd0 = {v, c}, hyd1 = {A = f P / rho^2, rho, 1/h, fbal}.
-// fbal is Balsara's viscosity limiter |div v| / (|div v| + |curl v| + 1e-4 c / h) when the
-// caller gives div v and curl v, else 1 (the plain Monaghan viscosity).
+// Hydro inputs in key order: hyd0 = {v, c}, hyd1 = {A = f P / rho^2, rho / 4, 1/h, fbal / 4}
+// (quarters: see hydro_pair).  fbal is Balsara's viscosity limiter
+// |div v| / (|div v| + |curl v| + 1e-4 c / h) when the caller gives div v and curl v, else 1
+// (the plain Monaghan viscosity).
 // One thread per rank: the caller-order inputs are gathered through the permutation and
 // the key-ordered records written coalesced (the scattered-store form, one thread per
 // caller index, measured 1.6x slower: its partial-sector writes cost more than these loads).
@@ -123,7 +124,7 @@ __global__ void k_hydro_prep(int64_t n, const int32_t* __restrict__ perm, const 
         const float cx = curlv[3 * (int64_t)i], cy = curlv[3 * (int64_t)i + 1], cz = curlv[3 * (int64_t)i + 2];
         fb = ad / (ad + sqrtf(fmaf(cx, cx, fmaf(cy, cy, cz * cz))) + 1.0e-4f * cs / hf);
     }
-    hyd1[r] = make_float4(A, rh, 1.0f / hf, fb);
+    hyd1[r] = make_float4(A, 0.25f * rh, 1.0f / hf, 0.25f * fb);
 }
 
 // velocities in key order for the density loop with velocity derivatives: hyd0 = {v, 0}

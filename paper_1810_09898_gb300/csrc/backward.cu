@@ -47,7 +47,7 @@ __device__ __forceinline__ DensityState density_state(double h, float s0, float 
     return d;
 }
 
-// Inputs of the hydro-adjoint loop in key order: hyd0 = {v, c}, hyd1 = {A, rho, 1/h,
+// Inputs of the hydro-adjoint loop in key order: hyd0 = {v, c}, hyd1 = {A, rho / 4, 1/h,
 // 8/(pi h^4)}, wadj = {w, 0}, with A = f (gamma - 1) u / rho, c = sqrt(gamma (gamma - 1) u).
 __global__ void k_bwd_prep(int64_t n, const int32_t* __restrict__ perm, const double* __restrict__ h64,
                            const float* __restrict__ s0, const float* __restrict__ s1,
@@ -62,7 +62,7 @@ __global__ void k_bwd_prep(int64_t n, const int32_t* __restrict__ perm, const do
     const double A = d.f * (gamma - 1.0) * ui * d.irho;
     const double c = sqrt(gamma * (gamma - 1.0) * ui);
     hyd0[r] = make_float4(vel[3 * i], vel[3 * i + 1], vel[3 * i + 2], (float)c);
-    hyd1[r] = make_float4((float)A, (float)d.rho, (float)d.ih, (float)(d.sigma * d.ih));
+    hyd1[r] = make_float4((float)A, 0.25f * (float)d.rho, (float)d.ih, (float)(d.sigma * d.ih));
     wadj[r] = make_float4(w[3 * i], w[3 * i + 1], w[3 * i + 2], 0.0f);
 }
 

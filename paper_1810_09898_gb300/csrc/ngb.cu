@@ -309,7 +309,8 @@ struct SymMember : MemberPos {
 };
 
 struct HMember : SymMember {
-    float vx, vy, vz, cs, A, rho, fb;   // fb: the viscosity limiter (1 without one)
+    float vx, vy, vz, cs, A;
+    float rho4, fb4;   // a quarter of the density and of the viscosity limiter (1 without one)
     float sx, cx_, sy, cy_, sz, cz_, su, cu;   // compensated totals
     float px_, py_, pz_, pu;                   // plain partial sums of the current tile
 };
@@ -317,7 +318,7 @@ struct HMember : SymMember {
 // hydro-adjoint member: the forward hydro state, the weights w_k = dL/da_k, and the
 // adjoint sums of x, v, m, h, rho and A = f P / rho^2
 struct HAMember : SymMember {
-    float vx, vy, vz, cs, A, rho, m;
+    float vx, vy, vz, cs, A, rho4, m;   // rho4: a quarter of the density
     float wx, wy, wz;
     float xb[3], vb[3], mb, hb, rb, Ab;
 };
@@ -427,24 +428,24 @@ __device__ __forceinline__ void member_init(HMember& M, const SearchArgs& a, con
                                             uint32_t cy, uint32_t cz) {
     M.sx = M.cx_ = M.sy = M.cy_ = M.sz = M.cz_ = M.su = M.cu = 0.0f;
     M.px_ = M.py_ = M.pz_ = M.pu = 0.0f;
-    M.vx = M.vy = M.vz = M.cs = M.A = M.rho = 0.0f;
-    M.fb = 1.0f;
+    M.vx = M.vy = M.vz = M.cs = M.A = M.rho4 = 0.0f;
+    M.fb4 = 0.25f;
     if (!sym_init(M, rec, cx, cy, cz)) return;
     float4 H0 = a.hyd0[rec.rank];
-    float4 H1 = a.hyd1[rec.rank];   // {A, rho, 1/h, limiter}
+    float4 H1 = a.hyd1[rec.rank];   // {A, rho / 4, 1/h, limiter / 4}
     M.hinv = H1.z;
     M.sk = kSkernel * (H1.z * H1.z) * (H1.z * H1.z);
-    M.fb = H1.w;
+    M.fb4 = H1.w;
     M.vx = H0.x; M.vy = H0.y; M.vz = H0.z; M.cs = H0.w;
     M.A = H1.x;
-    M.rho = H1.y;
+    M.rho4 = H1.y;
 }
 
 __device__ __forceinline__ void member_init(HAMember& M, const SearchArgs& a, const MemberRec& rec, uint32_t cx,
                                             uint32_t cy, uint32_t cz) {
     for (int k = 0; k < 3; ++k) M.xb[k] = M.vb[k] = 0.0f;
     M.mb = M.hb = M.rb = M.Ab = 0.0f;
-    M.vx = M.vy = M.vz = M.cs = M.A = M.rho = M.m = 0.0f;
+    M.vx = M.vy = M.vz = M.cs = M.A = M.rho4 = M.m = 0.0f;
     M.wx = M.wy = M.wz = 0.0f;
     if (!sym_init(M, rec, cx, cy, cz)) return;
     float4 H0 = a.hyd0[rec.rank];
@@ -454,7 +455,7 @@ __device__ __forceinline__ void member_init(HAMember& M, const SearchArgs& a, co
     M.sk = H1.w;
     M.vx = H0.x; M.vy = H0.y; M.vz = H0.z; M.cs = H0.w;
     M.A = H1.x;
-    M.rho = H1.y;
+    M.rho4 = H1.y;
     M.m = rec.O.w;
     M.wx = Wt.x; M.wy = Wt.y; M.wz = Wt.z;
 }
@@ -538,11 +539,11 @@ struct VelTile : PlainTileOf<kTileR> {
 };
 struct HydroTile : SymTile {
     float4 v[kTileR];       // hyd0 {vx, vy, vz, c}
-    float4 h[kTileR];       // hyd1 {A, rho, 1/h, limiter}
+    float4 h[kTileR];       // hyd1 {A, rho / 4, 1/h, limiter / 4}
 };
 struct HAdjTile : SymTile {
     float4 v[kTileR];       // hyd0 {vx, vy, vz, c}
-    float4 h[kTileR];       // hyd1 {A, rho, 1/h, 8/(pi h^4)}
+    float4 h[kTileR];       // hyd1 {A, rho / 4, 1/h, 8/(pi h^4)}
     float4 wt[kTileR];      // wadj {wx, wy, wz, -}
 };
 struct DAdjTile : SymTile {
@@ -825,7 +826,7 @@ __device__ __forceinline__ bool sym_decide(Mem& M, const SearchArgs& a, float3 p
 }
 
 // hydro pair: p = relative coordinates, q = {h_j^2, m_j}, v = {vx, vy, vz, c_j},
-// hh = {A_j, rho_j, 1/h_j, limiter_j}.  A pair below kMinR2 (coincident, or the member itself)
+// hh = {A_j, rho_j / 4, 1/h_j, limiter_j / 4}.  A pair below kMinR2 (coincident, or the member itself)
 // has no kernel gradient.
 template <int MODE, bool WRAP = false>
 __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, float3 p, float2 q,
@@ -844,11 +845,13 @@ __device__ __forceinline__ void hydro_pair(HMember& M, const SearchArgs& a, floa
     const float vx = M.vx - v.x, vy = M.vy - v.y, vz = M.vz - v.z;
     const float vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
     // Pi = (-alpha cbar mu + beta mu^2) / rhobar for approaching pairs, rhobar = (rho_i +
-    // rho_j) / 2, scaled by the pair mean of the limiter (1 for the plain viscosity)
+    // rho_j) / 2, scaled by the pair mean of the limiter (1 for the plain viscosity).  The
+    // records hold quarters of rho and the limiter, which cancel: the hardware reciprocal
+    // flushes a subnormal result to zero, which 1 / (rho_i + rho_j) is above 2^126.
     const float hb = 0.5f * fmaf(q.x, hh.z, M.h);
     const float mu = hb * vr * rcp_fast(fmaf(a.eps * hb, hb, r2));
     const float cb = 0.5f * (M.cs + v.w);
-    const float pi_ij = fmaf(-a.alpha * cb, mu, a.beta * mu * mu) * rcp_fast(M.rho + hh.y) * (M.fb + hh.w);
+    const float pi_ij = fmaf(-a.alpha * cb, mu, a.beta * mu * mu) * rcp_fast(M.rho4 + hh.y) * (M.fb4 + hh.w);
     const float visc = vr < 0.0f ? pi_ij : 0.0f;
     const float gbar = 0.5f * (dWi + dWj);
     const float mr = q.y * rinv;
@@ -888,7 +891,7 @@ __device__ __forceinline__ void hydro_adj_pair(HAMember& M, const SearchArgs& a,
     const float hbar = 0.5f * fmaf(q.x, hh.z, M.h);
     const float Dn = fmaf(a.eps * hbar, hbar, r2);
     const float iDn = rcp_fast(Dn);
-    const float irbar = 2.0f * rcp_fast(M.rho + hh.y);   // 1 / rhobar
+    const float irbar = 0.5f * rcp_fast(M.rho4 + hh.y);   // 1 / rhobar, from quarters as in hydro_pair
     float Pi = 0.0f, Pmu = 0.0f;
     if (vr < 0.0f) {
         const float cbar = 0.5f * (M.cs + v.w);

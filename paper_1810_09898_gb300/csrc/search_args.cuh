@@ -98,7 +98,7 @@ struct SearchArgs {
     const double *xd, *yd, *zd;
     const double* h64;
     const float4* hyd0;   // {vx, vy, vz, c}
-    const float4* hyd1;   // {A, rho, hinv, s}
+    const float4* hyd1;   // hydro {A, rho / 4, 1/h, limiter / 4}, its adjoint {A, rho / 4, 1/h, s}
     const float4* wadj;   // {wx, wy, wz, -}: weights dL/da of the hydro adjoint
     const float4* dadj;   // {alpha, beta, hinv, s}: coefficients of the density adjoint
     const int32_t* perm;

@@ -22,7 +22,7 @@ namespace sphgrp {
 //   poff      float4   {x 2^32 - X, ..., m}: sub-unit offsets in [0,1) and the mass
 //   h64       double   smoothing length (FP64 master)
 //   hyd0      float4   {vx, vy, vz, c}                        (hydro candidates)
-//   hyd1      float4   {A = f P / rho^2, rho, 1/h, Balsara limiter or 1} (hydro candidates)
+//   hyd1      float4   {A = f P / rho^2, rho / 4, 1/h, (Balsara limiter or 1) / 4} (hydro candidates)
 //
 // A coordinate relative to a fixed-point centre C is
 //   float(int32(X - C)) + off, scaled by 2^-32:

@@ -191,3 +191,25 @@ def test_rebuilds_of_one_context(cuda_device):
             got = nn.cpu().numpy()
         assert np.array_equal(got, oracle.density(pos, np.full(n, 1.0 / n), h)["nngb"]), k
     ctx.close()
+
+
+# ---------------------------------------------------------------- the top of the FP32 range
+
+@pytest.mark.parametrize("mode,g", [(0, 1), (1, 16)])
+def test_viscosity_at_large_densities(cuda_device, mode, g):
+    """rho_i + rho_j above 2^126, whose reciprocal is subnormal: the viscosity of cold gas."""
+    rng = np.random.default_rng(sphgen.SEED_BASE + 72)
+    n = 500
+    pos = rng.random((n, 3))
+    m = np.full(n, 1.0 / n, np.float32)
+    h = np.full(n, 0.2)
+    vel = (1e3 * rng.standard_normal((n, 3))).astype(np.float32)
+    rho = (6e37 * (1.0 + rng.random(n))).astype(np.float32)
+    zero, one = np.zeros(n, np.float32), np.ones(n, np.float32)
+    ref = oracle.hydro(pos, vel.astype(np.float64), m.astype(np.float64), h, rho.astype(np.float64), one, zero)
+    G = Gpu(pos, m)
+    got = G.hydro(np.arange(n, dtype=np.int32), h, rho, one, vel, zero, mode, g)
+    scale = 1e30   # the forces themselves are about 1e-30
+    assert _rel(scale * got["acc"].astype(np.float64), scale * ref["acc"]) <= ACC_TOL
+    assert _rel(scale * got["dudt"].astype(np.float64), scale * ref["dudt"]) <= ACC_TOL
+    G.ctx.close()
