@@ -45,7 +45,7 @@ enum {
     SPHGRP_EINVAL = -1,    /* bad argument: NaN or out-of-box position, h outside (0, 0.5), n = 0 ... */
     SPHGRP_ENOMEM = -2,    /* device allocation failed */
     SPHGRP_ENOCONV = -3,   /* smoothing-length iteration did not converge within max_iter */
-    SPHGRP_ETIMEOUT = -4,  /* a bounded device-side wait gave up */
+    SPHGRP_ETIMEOUT = -4,  /* kept for callers that test for it: no device-side wait fails a call */
     SPHGRP_EOVERFLOW = -5, /* an internal capacity was exceeded (results invalid) */
     SPHGRP_ECUDA = -6,     /* a CUDA runtime call failed */
     SPHGRP_ESTATE = -7     /* calls made out of order (e.g. a search before a tree) */
@@ -372,7 +372,7 @@ int sphgrp_batch_destroy(sphgrp_batch* b);
  * Synchronises the stream to read the device-side status.  Errors: EINVAL (a position
  * or h out of range), ENOCONV (a particle did not converge within max_iter passes;
  * its last values are written), EOVERFLOW (forest capacity or walk stack; results
- * invalid), ETIMEOUT, ECUDA. */
+ * invalid), ECUDA. */
 int sphgrp_batch_run(sphgrp_batch* b, const sphgrp_batch_io* io, int flags, cudaStream_t stream);
 
 /* Autotuner: runs one step (updating io like sphgrp_batch_run), then for every class

@@ -343,7 +343,6 @@ int read_status(Batch* b, int flags) {
     if (err & kErrH) return set_error(SPHGRP_EINVAL, "a smoothing length is outside (0, 0.5)");
     if (err & kErrStack) return set_error(SPHGRP_EOVERFLOW, "walk stack overflow");
     if (err & kErrNodes) return set_error(SPHGRP_EOVERFLOW, "forest capacity exceeded");
-    if (err & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait gave up");
     if (sc[kNFail] > 0) return set_error(SPHGRP_ENOCONV, std::to_string(sc[kNFail]) + " particles did not converge");
     return SPHGRP_OK;
 }

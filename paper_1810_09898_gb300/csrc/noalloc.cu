@@ -83,7 +83,6 @@ extern "C" int sphgrp_sfc_keys_sort_static(int64_t n, const double* pos, uint64_
     if (rc) return rc;
     rc = check_cuda(cudaStreamSynchronize(stream), "stream");
     if (rc) return rc;
-    if (flag & kErrTimeout) return set_error(SPHGRP_ETIMEOUT, "a bounded device wait (radix pass) gave up");
     if (flag & kErrRange) return set_error(SPHGRP_EINVAL, "a position is outside [0,1) or not finite");
     return SPHGRP_OK;
 }

@@ -281,11 +281,13 @@ int exclusive_scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, int64
 //
 // A tile's word of a digit: 0 = not there yet, v + 1 = the tile's own count v, bit 31 set =
 // the count of all tiles up to it.  The earlier tiles were taken by blocks that run
-// already, so a wait ends; it is bounded all the same.
+// already, so a wait ends.  It is bounded all the same, and a thread at the limit counts its
+// digit in the earlier tile's keys itself: the order is right whatever happens, so that the
+// kernels that follow in a step that reads nothing back never index by a part of it.
 // ---------------------------------------------------------------------------------
 
 constexpr uint32_t kTotalBit = 0x80000000u;
-constexpr uint32_t kSpinLimit = 1u << 24;
+constexpr uint32_t kSpinLimit = 1u << 16;   // reads of a word, some 50 ms
 
 struct SweepArgs {
     const uint64_t* kin;
@@ -301,7 +303,6 @@ struct SweepArgs {
     uint32_t* counts;      // published words, kBins per tile (zero)
     uint32_t* counts_next; // those of the next pass, zeroed here
     uint32_t* ticket;
-    unsigned* err;
 };
 
 // lanes with the same digit (kDigitBits bits and the one above them)
@@ -314,6 +315,14 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t d) {
         peers &= set ? vote : ~vote;
     }
     return peers;
+}
+
+// keys of tile t (a whole one: a later tile exists) with digit d
+__device__ __noinline__ uint32_t count_in_tile(const SweepArgs& a, int t, int tile_keys, uint32_t d) {
+    const uint64_t* k = a.kin + (int64_t)t * tile_keys;
+    uint32_t n = 0;
+    for (int e = 0; e < tile_keys; ++e) n += ((uint32_t)(k[e] >> a.shift) & (kBins - 1)) == d ? 1u : 0u;
+    return n;
 }
 
 template <int ITEMS>
@@ -332,12 +341,8 @@ __global__ void __launch_bounds__(256) k_radix_pass(SweepArgs a) {
     __shared__ uint32_t gbase[kBins];    // global position of the digit's run, less lbase
     __shared__ uint32_t wsum[8];
     __shared__ int tile_s;
-    __shared__ bool gave_up;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        tile_s = (int)atomicAdd(a.ticket, 1u);
-        gave_up = false;
-    }
+    if (threadIdx.x == 0) tile_s = (int)atomicAdd(a.ticket, 1u);
     for (int d = threadIdx.x; d < 8 * kBins / 2; d += 256) reinterpret_cast<uint32_t*>(&wh[0][0])[d] = 0u;
     __syncthreads();
     const int tile = tile_s;
@@ -417,7 +422,6 @@ __global__ void __launch_bounds__(256) k_radix_pass(SweepArgs a) {
         const int d = 2 * threadIdx.x + q;
         uint32_t before = 0;
         uint32_t spins = 0;
-        bool ok = true;
         for (int t = tile - 1; t >= 0;) {
             const uint32_t word = *reinterpret_cast<volatile uint32_t*>(a.counts + (int64_t)t * kBins + d);
             if (word & kTotalBit) {
@@ -428,30 +432,24 @@ __global__ void __launch_bounds__(256) k_radix_pass(SweepArgs a) {
                 before += word - 1u;
                 --t;
             } else if (++spins > kSpinLimit) {
-                ok = false;
-                break;
+                before += count_in_tile(a, t, kTileKeys, (uint32_t)d);
+                --t;
             }
-        }
-        if (!ok) {
-            gave_up = true;
-            atomicOr(a.err, kErrTimeout);
         }
         if (tile > 0) pub[d] = kTotalBit | (before + tot[q]);
         gbase[d] = a.start[d] + before - (q ? off + tot[0] : off);
     }
     __syncthreads();
-    if (gave_up) return;   // positions unknown: nothing is written, the call reports the timeout
     const int cnt = (int)min((int64_t)kTileKeys, a.n - tile0);
     for (int e = threadIdx.x; e < cnt; e += 256) {
         const uint64_t key = sk[e];
         const int32_t val = sv[e];
         const uint32_t p = gbase[(uint32_t)(key >> a.shift) & (kBins - 1)] + (uint32_t)e;
-        if (p >= a.n) continue;   // only after a wait gave up in an earlier pass
         a.kout[p] = key;
         a.vout[p] = val;
         if (a.kout2) a.kout2[p] = key;
         if (a.vout2) a.vout2[p] = val;
-        if (a.rank_of && (uint32_t)val < (uint32_t)a.n) a.rank_of[val] = (int32_t)p;
+        if (a.rank_of) a.rank_of[val] = (int32_t)p;
     }
 }
 
@@ -495,7 +493,7 @@ static void zero_scratch(uint32_t* scratch, int64_t n, cudaStream_t s) {
 // Passes over the digits of `bits` bits: (kbuf[0], vbuf[0] or the positions) -> ... ; the
 // result ends in kbuf[passes & 1], vbuf[passes & 1].
 static int radix_passes(uint64_t* const (&kbuf)[2], int32_t* const (&vbuf)[2], int64_t n, int passes, uint32_t* scratch,
-                        uint64_t* keys_copy, int32_t* vals_copy, int32_t* rank_of, unsigned* err, cudaStream_t s) {
+                        uint64_t* keys_copy, int32_t* vals_copy, int32_t* rank_of, cudaStream_t s) {
     const int64_t set = (sort_scratch_words(n) - kSortHeadWords) / 2;
     uint32_t* sets[2] = {scratch + kSortHeadWords, scratch + kSortHeadWords + set};
     // With its static tables the largest tile is above the 48 KB that need no permission,
@@ -521,7 +519,6 @@ static int radix_passes(uint64_t* const (&kbuf)[2], int32_t* const (&vbuf)[2], i
         a.counts = sets[p & 1];
         a.counts_next = sets[(p + 1) & 1];
         a.ticket = scratch + kKeyPasses * kBins + p;
-        a.err = err;
         int rc = launch_pass(a, s);
         if (rc) return rc;
     }
@@ -544,7 +541,7 @@ int sort_keys(Ctx* c, int64_t n, const double* pos, cudaStream_t s, uint64_t* ke
     uint64_t* const kbuf[2] = {c->keys_alt, c->keys};
     int32_t* const vbuf[2] = {c->perm_alt, c->perm};
     static_assert(kKeyPasses % 2 == 1, "the result ends in the second buffers");
-    int rc = radix_passes(kbuf, vbuf, n, kKeyPasses, c->hist, keys_copy, perm_copy, c->rank_of, c->err, s);
+    int rc = radix_passes(kbuf, vbuf, n, kKeyPasses, c->hist, keys_copy, perm_copy, c->rank_of, s);
     if (rc) return rc;
     return check_cuda(cudaGetLastError(), "sort");
 }
@@ -608,7 +605,7 @@ int sort_keys_boxed(Ctx* c, int64_t n, const double* pos, const int64_t* box_off
     note_launch();
     uint64_t* const kbuf[2] = {tmp64a, tmp64b};
     int32_t* const vbuf[2] = {tmp32b, tmp32a};
-    if ((rc = radix_passes(kbuf, vbuf, n, passes, c->hist, nullptr, nullptr, nullptr, c->err, s))) return rc;
+    if ((rc = radix_passes(kbuf, vbuf, n, passes, c->hist, nullptr, nullptr, nullptr, s))) return rc;
     // box digits in (box, key) order, and the rank in key order of every position
     k_box_gather<<<blocks_for(n, 256), 256, 0, s>>>(n, vbuf[passes & 1], c->keys, c->perm, kbuf[passes & 1], c->keys_alt,
                                                      c->perm_alt, c->rank_of, box_of_rank);
@@ -630,7 +627,7 @@ int sort_keys_scratch(int64_t n, const double* pos, uint64_t* keys_out, int32_t*
     launch_keys(n, pos, keys_alt, scratch, err, s);
     uint64_t* const kbuf[2] = {keys_alt, keys_out};
     int32_t* const vbuf[2] = {perm_alt, perm_out};
-    int rc = radix_passes(kbuf, vbuf, n, kKeyPasses, scratch, nullptr, nullptr, nullptr, err, s);
+    int rc = radix_passes(kbuf, vbuf, n, kKeyPasses, scratch, nullptr, nullptr, nullptr, s);
     if (rc) return rc;
     return check_cuda(cudaGetLastError(), "sort (caller buffers)");
 }
