@@ -2408,6 +2408,26 @@ static int launch_persistent(Kern kern, size_t sh, int64_t ngroups_host, int sm_
     return check_cuda(cudaGetLastError(), what);
 }
 
+// Items are numbered by an int, and a listed group of more than 32 members is up to four of
+// them: more than kMaxItems go in several launches (the radius and tree modes on more than
+// 2^29 particles).
+constexpr int kMaxItems = 0x7fffffff - (1 << 20);   // less what the warps take past the end
+
+template <class Launch>
+static int launch_items(const SearchArgs& a, cudaStream_t s, Launch launch) {
+    const int most = kMaxItems / a.parts;
+    if (!a.groups || a.ngroups <= most) return launch(a);
+    int rc = SPHGRP_OK;
+    for (int off = 0; off < a.ngroups && !rc; off += most) {
+        SearchArgs b = a;
+        b.groups = a.groups + off;
+        b.ngroups = std::min(most, a.ngroups - off);
+        if (off > 0) cudaMemsetAsync(a.work, 0, sizeof(int), s);
+        rc = launch(b);
+    }
+    return rc;
+}
+
 template <class K, int MODE>
 static int launch_group(const SearchArgs& a, int sm_count, cudaStream_t s) {
     if (a.g > 128) return set_error(SPHGRP_EINVAL, "group_size must be <= 128");
@@ -2415,8 +2435,10 @@ static int launch_group(const SearchArgs& a, int sm_count, cudaStream_t s) {
     b.parts = (a.g + kPartMax - 1) / kPartMax;
     // many single members: several items per counter access (one address serves all warps)
     b.take = a.g == 1 && a.ngroups >= 1 << 16 ? 4 : 1;
-    return launch_persistent(k_group<K, MODE>, group_smem<K>(),
-                             a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s, "grouped search kernel", b);
+    return launch_items(b, s, [&](const SearchArgs& c) {
+        return launch_persistent(k_group<K, MODE>, group_smem<K>(),
+                                 c.npieces ? c.nu : (int64_t)c.ngroups * c.parts, sm_count, s, "grouped search kernel", c);
+    });
 }
 
 template <bool SYM, bool FILL>
@@ -2458,9 +2480,11 @@ int launch_density_iter(const SearchArgs& a, const IterArgs& it, int max_g, int 
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     SearchArgs b = a;
     b.parts = (a.g + kPartMax - 1) / kPartMax;
-    return launch_persistent(k_group_dens_iter, group_smem<KDens>(),
-                             a.npieces ? a.nu : (int64_t)a.ngroups * b.parts, sm_count, s,
-                             "grouped density iteration kernel", b, it);
+    return launch_items(b, s, [&](const SearchArgs& c) {
+        return launch_persistent(k_group_dens_iter, group_smem<KDens>(),
+                                 c.npieces ? c.nu : (int64_t)c.ngroups * c.parts, sm_count, s,
+                                 "grouped density iteration kernel", c, it);
+    });
 }
 
 template <class K0, class K1>

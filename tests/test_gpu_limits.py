@@ -213,3 +213,34 @@ def test_viscosity_at_large_densities(cuda_device, mode, g):
     assert _rel(scale * got["acc"].astype(np.float64), scale * ref["acc"]) <= ACC_TOL
     assert _rel(scale * got["dudt"].astype(np.float64), scale * ref["dudt"]) <= ACC_TOL
     G.ctx.close()
+
+
+# ---------------------------------------------------------------- groups above 32 members
+
+@pytest.mark.parametrize("params", [{"group_mode": 1, "group_f": 2.0}, {"group_mode": 2, "group_level": 3},
+                                    {"group_split": 0.0}], ids=["radius", "tree", "chunks"])
+@pytest.mark.parametrize("g", [33, 64, 100, 128])
+def test_large_groups_in_every_mode(cuda_device, params, g):
+    """Groups of more than 32 members are searched in parts of 32."""
+    d = dataset("clustered", 9001, 2)
+    n = 9001
+    G = Gpu(d["pos"], d["m32"], **params)
+    h = np.full(n, 0.8 * d["h0"])
+    act = np.sort(G.perm.cpu().numpy()[np.arange(n) % 11 < 9]).astype(np.int32)
+    m64 = d["m32"].astype(np.float64)
+    out = G.density(act, h, 0, 1, g)
+    ref = oracle.density(d["pos"], m64, h, targets=act)
+    assert np.array_equal(out["nngb"][act], ref["nngb"])
+    assert np.max(np.abs(out["rho"][act] / ref["rho"] - 1.0)) <= RHO_TOL
+    one = np.ones(n, np.float32)
+    hy = G.hydro(act, h, one, one, d["vel32"], d["u32"], 1, g)
+    href = oracle.hydro(d["pos"], d["vel32"].astype(np.float64), m64, h, one, one, d["u32"].astype(np.float64),
+                        targets=act)
+    assert np.array_equal(hy["nngb"][act], href["nngb"])
+    assert _rel(hy["acc"][act], href["acc"]) <= ACC_TOL
+    off, idx = G.ngb_sets(act, h, 1, 1, g)
+    roff, ridx = oracle.ngb_sets(d["pos"], h, act, 1)
+    assert np.array_equal(off, roff)
+    for k in range(len(act)):
+        assert np.array_equal(np.sort(idx[off[k]:off[k + 1]]), np.sort(ridx[roff[k]:roff[k + 1]]))
+    G.ctx.close()
