@@ -1,11 +1,15 @@
-"""Inputs at the limits of what the calls take.  References are the FP64 oracle's."""
+"""Inputs at the limits of what the calls take: pairs closer than FP32 squares reach,
+densities near the top of the FP32 range, smoothing lengths beyond half the box or not a
+number, forests that outgrow their arrays, box counts around the digits of the box sort,
+lists on either side of the in-group iteration's size rule, several octrees of one context,
+and groups above 32 members in every grouping mode.  References are the FP64 oracle's."""
 
 import numpy as np
 import pytest
 
 import oracle
 import sphgen
-from gpu_common import RHO_TOL, Gpu, dataset
+from gpu_common import NEFF_TOL, RHO_TOL, Gpu, dataset
 
 pytestmark = pytest.mark.gpu
 
@@ -116,6 +120,36 @@ def test_h_not_a_number_searches_nothing(cuda_device, iteration):
     G.ctx.close()
 
 
+def test_iteration_on_both_sides_of_the_size_rule(cuda_device):
+    """Lists of 4096 particles per SM iterate inside their groups, longer ones by passes:
+    the same iterates, both converged under the oracle's arithmetic."""
+    import torch
+
+    edge = 4096 * torch.cuda.get_device_properties(0).multi_processor_count
+    n = edge + 1000
+    d = dataset("clustered", n, 2)
+    G = Gpu(d["pos"], d["m32"])
+    # from h around the converged ones, so that a pass or two settles most of them
+    rng = np.random.default_rng(sphgen.SEED_BASE + 73)
+    order = G.perm.cpu().numpy()
+    h0 = np.full(n, d["h0"])
+    h0 = G.density(np.arange(n, dtype=np.int32), h0, 1, 1, 16)["h"] * np.exp(0.05 * rng.standard_normal(n))
+    h0 = np.minimum(h0, 0.49)
+    out = [G.density(np.sort(order[:nu]).astype(np.int32), h0, 1, 1, 16) for nu in (edge, edge + 1)]
+    assert out[0]["stats"]["search_launches"] == 1 and out[1]["stats"]["search_launches"] > 1
+    both = order[:edge]
+    a, b = (o["h"][both] for o in out)
+    assert np.mean(np.abs(a / b - 1.0) <= 1e-5) > 0.999
+    t = np.sort(order[rng.integers(0, edge, 2048)]).astype(np.int32)
+    for o in out:
+        chk = oracle.density(d["pos"], d["m32"].astype(np.float64), o["h"], targets=t)
+        neff = 4.0 * np.pi / 3.0 * o["h"][t] ** 3 * chk["rho"] / d["m32"][t].astype(np.float64)
+        assert np.all(np.abs(neff - 64.0) <= NEFF_TOL)
+        assert np.array_equal(o["nngb"][t], chk["nngb"])
+        assert np.max(np.abs(o["rho"][t] / chk["rho"] - 1.0)) <= RHO_TOL
+    G.ctx.close()
+
+
 # ---------------------------------------------------------------- batches
 
 def _batch_io(pos, h):
@@ -160,6 +194,31 @@ def test_forest_overflow_does_no_search(cuda_device, graph):
         assert np.array_equal(io["nngb"].cpu().numpy()[s], ref["nngb"])
     assert torch.isfinite(io["g_pos"]).all()
     B.close()
+
+
+@pytest.mark.parametrize("nbox", [512, 513, 600, 1100])
+def test_box_counts_around_the_sort_digit(cuda_device, nbox):
+    """The box sort takes 9 bits of the box index a pass: one pass up to 512 boxes, two above
+    (the result then ends in the other pair of buffers); every box's counts and densities
+    are the oracle's on that box alone."""
+    import paper_1810_09898_gb300 as sg
+
+    rng = np.random.default_rng(sphgen.SEED_BASE + nbox)
+    sizes = rng.integers(300, 500, nbox)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(off[-1])
+    pos = rng.random((n, 3))
+    io = _batch_io(pos, np.full(n, 0.3))
+    B = sg.Batch(off)
+    B.run({k: v for k, v in io.items() if not k.startswith("g_")})
+    h, rho, nn = (io[k].cpu().numpy() for k in ("h", "rho", "nngb"))
+    B.close()
+    for k in [*rng.integers(0, nbox, 20), 0, 255, 256, 511, nbox - 1]:
+        s = slice(int(off[k]), int(off[k + 1]))
+        ref = oracle.density(pos[s], np.full(sizes[k], np.float32(1 / n), np.float64), h[s])
+        assert np.all(np.abs(ref["neff"] - 64.0) <= NEFF_TOL), k
+        assert np.array_equal(nn[s], ref["nngb"]), k
+        assert np.max(np.abs(rho[s] / ref["rho"] - 1.0)) <= RHO_TOL, k
 
 
 # ---------------------------------------------------------------- octree storage
