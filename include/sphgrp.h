@@ -54,8 +54,11 @@ enum {
 /* Neighbour-search forms. */
 enum {
     SPHGRP_INDIVIDUAL = 0, /* one walk per active particle with radius h_i (Sec. 1.1) */
-    SPHGRP_GROUPED = 1     /* Neighbour Recycling: one walk per group of group_size
-                              consecutive active particles in key order (Sec. 2.1) */
+    SPHGRP_GROUPED = 1     /* Neighbour Recycling: one walk per group of consecutive active
+                              particles in key order (Sec. 2.1).  group_size is the most a
+                              group holds; the calls that compute search groups of more than
+                              32 in parts of 32 and cut short lists into smaller chunks
+                              (sphgrp_stats.walks counts the walks made) */
 };
 
 /* Neighbour definitions (Sec. 1.1, last paragraph). */
@@ -193,15 +196,18 @@ int sphgrp_ngb_search(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active, con
 
 /* The candidate superset of every group of the grouped form (Sec. 2.1), for
  * inspection.  Groups are runs of consecutive active particles in key order: chunks
- * of group_size, each cut in halves while its members are spread wider than
- * params.group_split times their smallest h.
+ * of group_size, each cut while it is too wide as params.group_split says (or by the rule of
+ * params.group_mode), and the superset is that of the paper's search sphere around the
+ * group.  The calls that compute use the same rule on chunks of at most 32 (fewer on short
+ * lists) and search the members' box dilated by their largest radius, so their groups are
+ * finer and their candidates fewer than those listed here.
  * group_offsets: device, n_act + 1 int64 offsets of every group's candidates in cand;
  * group_first:   device, n_act + 1 int32 (may be NULL): group k's members are
  *                members[group_first[k] .. group_first[k+1]);
  * members:       device, n_act int32 (may be NULL): the active original indices in
  *                key order;
  * cand:          device, cap int32 original indices, or NULL to count only;
- * n_groups, n_cand: host, number of groups (walks) and total candidates.
+ * n_groups, n_cand: host, number of groups listed and total candidates.
  * kind selects the density or hydro radius. */
 int sphgrp_group_supersets(sphgrp_ctx* ctx, int64_t n_act, const int32_t* active,
                            const double* h, int kind, int group_size, int64_t cap,
@@ -405,7 +411,8 @@ int sphgrp_batch_stats(sphgrp_batch* b, sphgrp_stats* out);
 int sphgrp_get_stats(sphgrp_ctx* ctx, sphgrp_stats* out);
 
 /* Per-launch record of the search kernels of the most recent call, in launch order
- * (one entry per smoothing-length pass for sphgrp_density): particles processed,
+ * (sphgrp_density: one entry per smoothing-length pass made as a launch; one in all where
+ * the groups iterate inside one launch, see sphgrp_params.iteration): particles processed,
  * candidates staged, member x candidate tests, node tests and device time in ms
  * (CUDA events).  All arrays are host arrays of cap entries and may be NULL;
  * count receives the number of entries written.  No device work. */

@@ -832,8 +832,13 @@ namespace sphgrp {
 
 // Work lists of at most this many particles per SM iterate inside their groups (one launch)
 // instead of by passes: there a pass costs its launches and its read-back, and the
-// regrouping gains little.  Passes / in groups, uniform sets from the uniform guess: 32k 600 /
-// 356 us, 131k 950 / 690, 524k 1950 / 1750, 1.0M 3530 / 3470, 4.2M 11.7 / 12.1 ms.
+// regrouping gains little.  Passes / in groups, us, |N_eff - 64| within 2, from the uniform
+// guess and from h scattered by 5% about the converged one:
+//   uniform    5k 396 / 203, 321 / 185   32k 448 / 263, 371 / 250   131k 625 / 475, 583 / 414
+//              623k 1371 / 1304, 1221 / 1182
+//   clustered  5k 1446 / 385, 406 / 217   32k 2197 / 1179, 809 / 577   131k 6523 / 6030, 1486 / 1152
+//              623k 35273 / 29937, 1987 / 1859
+// Above, uniform sets from the uniform guess within 1e-3: 1.0M 3530 / 3470 us, 4.2M 11.7 / 12.1 ms.
 constexpr int kInGroupPerSM = 4096;
 
 // The density with the smoothing-length iteration; with vel (not NULL) the same density

@@ -139,8 +139,10 @@ __device__ __forceinline__ float rsqrt_any(float x) {
     return y;
 }
 // Least r^2 of normal size: a pair closer than its root, 1.1e-19 of the box, is taken as
-// coincident where its terms vanish with r (kernel gradients); the hydro adjoint, whose
-// derivative of the pair force does not, takes its root by rsqrt_any.
+// coincident where its terms vanish with r (kernel gradients; the viscosity's with a
+// softening eps > 0); the hydro adjoint, whose derivative of the pair force does not, takes
+// its root by rsqrt_any.  Hydro of 4.2M 6.46 ms with and without; subnormal roots everywhere
+// cost it 1.3% and backward of 2.1M 1.1%, in the adjoint alone 0.5% (9.72 -> 9.77 ms).
 constexpr float kMinR2 = 1.17549435e-38f;
 __device__ __forceinline__ float rcp_fast(float x) {
     float y;
@@ -1122,16 +1124,8 @@ __device__ __forceinline__ void write_result(const HAMember& H, const SearchArgs
 template <int MODE>
 __device__ __forceinline__ void write_result(const VMember& V, const SearchArgs& a) {
     if (MODE != kAcc) return;
-    if (a.o_res4) {
-        a.o_res4[V.rank] = make_float4(V.rrho * (V.sd - V.cd), V.rrho * (V.sx - V.cx_), V.rrho * (V.sy - V.cy_),
-                                       V.rrho * (V.sz - V.cz_));
-        return;
-    }
-    const int orig = a.perm[V.rank];
-    a.o_divv[orig] = V.rrho * (V.sd - V.cd);
-    a.o_curl[3 * (int64_t)orig] = V.rrho * (V.sx - V.cx_);
-    a.o_curl[3 * (int64_t)orig + 1] = V.rrho * (V.sy - V.cy_);
-    a.o_curl[3 * (int64_t)orig + 2] = V.rrho * (V.sz - V.cz_);
+    a.o_res4[V.rank] = make_float4(V.rrho * (V.sd - V.cd), V.rrho * (V.sx - V.cx_), V.rrho * (V.sy - V.cy_),
+                                   V.rrho * (V.sz - V.cz_));
 }
 template <int MODE>
 __device__ __forceinline__ void write_result(const DAMember& D, const SearchArgs& a) {
@@ -1616,7 +1610,8 @@ __device__ __noinline__ bool meets_members(float3 d, float4 ext, float hnode, fl
 // around C that covers every member's sphere is up to a third larger in volume for a
 // cubic box and far larger for an elongated one.
 //
-// Bound by instruction issue (71% of issue slots, L2 hit 97%).  Of the about 900 particles
+// Bound by instruction issue (84% of the issue slots in the density loop, 74% in hydro; L2 hit
+// 94%).  Of the about 900 particles
 // that the opened nodes hold (16.8M clustered particles, g = 16) fewer than half lie in
 // the dilated box: they are dropped here, at a few instructions per 32 of them, before
 // the members' filter, and only the kept ones fetch the kind's own records.  Against
@@ -2099,16 +2094,18 @@ __global__ void __launch_bounds__(128) k_indiv(SearchArgs a) {
 
 // ---------------------------------------------------------------------------------
 // Pieces of the searches that compute (count mode): one warp per window of up to 32
-// consecutive work-list entries, whole chunks of g (g > 32: chunks of 32).  Every chunk is
-// cut as k_split_groups cuts the exported groups: (recursively) while its members' search
-// sphere, ((sqrt(3)/2) box width + h_min)^3, exceeds split * (members) member spheres
-// h_min^3, at the largest gap in key order between consecutive members (ties: nearest the
-// middle; the middle when they are contiguous); in a batch, whose active particles are
-// not runs, in the middle (gap cuts peel off single members there: a 16-box step 22.7 ->
-// 23.5 ms).
+// consecutive work-list entries, whole chunks of g (g > 32: chunks of 32).  A chunk is cut
+// (recursively) by the volume rule of k_split_groups, which cuts the exported groups: while
+// its members' search sphere, ((sqrt(3)/2) box width + h_min)^3, exceeds split * (members)
+// member spheres h_min^3, at the largest gap in key order between consecutive members (ties:
+// nearest the middle; the middle when they are contiguous).  The pieces are not those groups:
+// chunks are at most 32 and smaller on small lists, and every cut may be at a gap, where
+// k_split_groups, which keeps a stack, halves a chunk after eight pending ranges.  In a batch,
+// whose active particles are not runs, cuts are in the middle (gap cuts peel off single
+// members there: a 16-box step 22.7 -> 23.5 ms).
 //
-// Pieces that reach far beyond their smallest h have the most candidates; they are listed
-// from the end of the list, which the search kernels take first.
+// Pieces that reach far beyond their smallest h have the most candidates: they are stored
+// from the end of the list downwards, and the search kernels take them first.
 //
 // The pieces go straight to the list, a block's together, with one atomic each for the
 // large ones and the others: no scan of counts, and their number stays on the device.

@@ -129,12 +129,9 @@ struct SearchArgs {
     float4* o_adj1;       // hydro adjoint {vb, -}
     float4* o_adj2;       // hydro adjoint {hb, rhob, Ab, n}
     float4* o_adj3;       // density adjoint {xb, mb}
-    // velocity derivatives (original order)
-    float* o_divv;
-    float* o_curl;        // n x 3
     // hydro / velocity-derivative results in key order (rank space, one float4 per
-    // member: {a, du/dt} or {div v, curl v}) and the hydro neighbour counts; null: the
-    // results go straight to the caller's order below
+    // member: {a, du/dt} or {div v, curl v}) and the hydro neighbour counts; null (hydro in
+    // a batch): the results go straight to the caller's order below
     float4* o_res4;
     int32_t* o_rcnt;
     // hydro results (original order)

@@ -268,16 +268,19 @@ int exclusive_scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, int64
 // ---------------------------------------------------------------------------------
 // LSD radix sort, 9-bit digits, stable, one kernel per pass.  The digit counts of all
 // passes come from the kernel that makes the keys.  A pass's block takes the next tile
-// (in ticket order), ranks its keys by warp matching -- warp w owns a contiguous part of
-// the tile and goes through it 32 keys at a time, so ranks follow the input order --
+// (in ticket order), ranks its keys by ballots of their digits' bits -- warp w owns a
+// contiguous part of the tile and goes through it 32 keys at a time, so ranks follow the
+// input order --
 // publishes the tile's digit counts, sorts the tile by digit in shared memory, and finds
 // for every digit how many such keys the earlier tiles hold by looking back through their
 // published counts until one has its total (decoupled look-back).  Then every digit's
 // run goes out with consecutive threads on consecutive addresses.
 //
-// Every key and value is read and written once per pass: bound by HBM on large sets, by the
-// launches on small ones (8 launches where counting, scanning and scattering 8-bit
-// digits took 25): 20k particles by the allocation-free call 182 -> 114 us.
+// Every key and value is read and written once per pass.  On large sets a pass is bound by
+// the dependent steps of a block, of which 60 KB of shared memory leave three on an SM: a
+// pass over 4.0M keys takes about 70 us (97 the last), where its 96 MB take 14 at the measured
+// 6791 GB/s.  On small ones it is bound by the launches (8 where counting, scanning and
+// scattering 8-bit digits took 25): 20k particles by the allocation-free call 182 -> 101 us.
 //
 // A tile's word of a digit: 0 = not there yet, v + 1 = the tile's own count v, bit 31 set =
 // the count of all tiles up to it.  The earlier tiles were taken by blocks that run
@@ -525,9 +528,12 @@ static int radix_passes(uint64_t* const (&kbuf)[2], int32_t* const (&vbuf)[2], i
     return SPHGRP_OK;
 }
 
+// Blocks of the kernels that count digits: at least 4 keys a thread and four blocks for each
+// of the chip's 152 SMs, so that few of them add their counts to memory.
+constexpr int64_t kCountBlocks = 152 * 4;
+
 static void launch_keys(int64_t n, const double* pos, uint64_t* keys, uint32_t* hist, unsigned* err, cudaStream_t s) {
-    // at least 4 keys a thread, so that the digit counts are added to memory by few blocks
-    const int64_t blocks = std::min<int64_t>((n + 1023) / 1024, 152 * 4);
+    const int64_t blocks = std::min<int64_t>((n + 1023) / 1024, kCountBlocks);
     k_keys<<<(unsigned)blocks, 256, 0, s>>>(n, pos, keys, hist, err);
     note_launch();
 }
@@ -600,8 +606,8 @@ int sort_keys_boxed(Ctx* c, int64_t n, const double* pos, const int64_t* box_off
     int passes = 1;
     while ((int64_t)nbox > (int64_t)1 << (passes * kDigitBits)) ++passes;
     zero_scratch(c->hist, n, s);
-    k_box_digit<<<(unsigned)std::min<int64_t>((n + 1023) / 1024, 152 * 4), 256, 0, s>>>(n, c->perm, box_off_dev, nbox,
-                                                                                          tmp64a, passes, c->hist);
+    k_box_digit<<<(unsigned)std::min<int64_t>((n + 1023) / 1024, kCountBlocks), 256, 0, s>>>(
+        n, c->perm, box_off_dev, nbox, tmp64a, passes, c->hist);
     note_launch();
     uint64_t* const kbuf[2] = {tmp64a, tmp64b};
     int32_t* const vbuf[2] = {tmp32b, tmp32a};
