@@ -470,8 +470,12 @@ int make_groups(Ctx* c, SearchArgs* a, const int32_t* U, int nu, int g, cudaStre
     return SPHGRP_OK;
 }
 
-// A small work list is cut into smaller chunks while it would make fewer pieces than this
-// many per SM: below that the launch lasts as long as its slowest piece.
+// A small work list is cut into smaller chunks, of at least 4, while it would make fewer pieces
+// than this many per SM: below that the launch lasts as long as its slowest piece.  Clustered
+// sets, us, limit 0 / 8 / 16 / 32 pieces: hydro of 8k at g = 32 315 / 177 / 174 / 175, of 39k
+// active of 131k 556 / 561 / 417 / 327, density with derivatives of 8k 290 / 156 / 155 / 158;
+// longer lists do not change (hydro of 524k 1132 / 1134 / 1130 / 1135).  Least chunk 2 / 4 / 8:
+// hydro of 8k 180 / 177 / 193, derivatives of 8k 155 / 155 / 175.
 constexpr int kSmallPieces = 16;
 
 // Work items of a search that computes: in count mode the pieces of the chunks (their number
